@@ -1,121 +1,415 @@
 // Per-head dense algebra of Orthogonal BackFill (Eq. 2-6), one thread block per
-// (cache, layer, KV head), everything in fp32 in shared memory.
+// (cache, layer, KV head), everything in fp32.
 //
-// Inputs (from the streaming pass): Gram of the deleted values G_del, Gram of the
-// retained values G_keep (only when k_eff >= d), u = sum_del A_j v_j, the demand
-// sums, and the retained rows themselves (read back from v_out).  The tuned streaming
-// pass delivers G and u over ALL rows instead (it runs before the selection is known):
-// P G_all P = P G_del P because P annihilates the retained rows; the retained rows'
-// share of u and of the trace of G is subtracted here, while they are read for the basis.
+// Inputs (from the streaming pass): Gram of the deleted values G_del, u = sum_del A_j v_j, the demand sums, and the
+// retained rows themselves (read back from v_out).  The tuned streaming pass delivers G and u over ALL rows instead (it
+// runs before the selection is known): P G_all P = P G_del P because P annihilates the retained rows; the retained
+// rows' share of u and of the trace of G is subtracted here.
 //
-//   1. k_eff >= d: k_span_test has factorised G_keep (Cholesky).  If every pivot
-//      stayed above 1e-3 of its diagonal entry the retained values span R^d, the
-//      residual of Eq. 3 is identically zero and delta = 0.
-//   2. Otherwise: orthonormal basis Q of span(V_keep) (Eq. 2) by Gram-Schmidt over
-//      the retained rows, iterated a second time for a row that lost more than half
-//      of its squared norm in the first pass; a row adds a direction when what is
-//      left of it exceeds 1e-4 of its own norm.
-//   3. M = P G P = R^T R with P = I - Q^T Q (Eq. 3 in Gram form, App. H), formed without P as two rank-m
-//      updates with the m basis rows in Q: X <- X - Q^T (Q X) from the left, then the same from the right
-//      (8 m d^2 flops instead of the 4 d^3 of two full products),
-//      r_bar = P u / (A_del + eps) = (u - Q^T (Q u)) / (A_del + eps)  (Eq. 4).
-//   4. C = eigenvectors of the `rank` largest eigenvalues of M above 1e-5 of the
-//      largest.  For rank <= ALG_TRI_MAX_RANK: Householder reduction of M to
-//      tridiagonal form (two block barriers per column), the rank + 1 largest
-//      eigenvalues by 33-way multisection on Sturm counts, their vectors by inverse
-//      iteration (neighbours closer than 1e-3 of the largest eigenvalue are kept
-//      orthogonal during the iteration), mapped back through the reflectors two at a
-//      time.  For larger ranks: full eigen-decomposition by
-//      parallel-order Jacobi rotations run to convergence.
-//   5. Delta = C^T C r_bar (Eq. 5), delta = A_del / (A_keep + eps) * Delta (Eq. 6), projected once more off the
-//      basis rows (the subtractions that form M leave rounding noise of the size of G's largest entries),
-//      V_out = V_keep + delta on the head's retained rows (Eq. 7).
+//   1. k_eff >= d: k_span_test has factorised G_keep (Cholesky).  If every pivot stayed above 1e-3 of its diagonal
+//      entry the retained values span R^d, the residual of Eq. 3 is identically zero and delta = 0.
+//   2. Otherwise the retained rows are reduced by Householder reflectors H_0 .. H_{m-1} (Eq. 2 as a QR factorisation:
+//      reflector j maps row after row onto the coordinates 0 .. j); a row adds a reflector when what is left of it
+//      beyond the coordinates reached so far exceeds 1e-4 of its own norm.  The same reflectors are then applied to G
+//      from both sides.  With H = H_0 .. H_{m-1} the span of the retained values is the first m coordinates
+//      of the rotated space, so the trailing block of H^T G H IS the residual's Gram matrix R^T R (Eq. 3 in Gram form,
+//      App. H) in the d - m coordinates of the complement: no basis, no projector and no product P G P is formed, and
+//      whatever is computed in those coordinates is orthogonal to the retained values to rounding.
+//      r_bar (Eq. 4) is the tail of H^T u / (A_del + eps).
+//   3. C = eigenvectors of the `rank` largest eigenvalues above 1e-5 of the largest.  For rank <= ALG_TRI_MAX_RANK the
+//      reflectors simply go on: H_{m+1} .. H_{d-2} take the trailing block to tridiagonal form (so the basis and the
+//      tridiagonal form together cost the d - 2 steps that the tridiagonal form of the full matrix would), the wanted
+//      eigenvalues come from multisection on Sturm counts, their vectors from twisted factorisations (neighbours closer
+//      than 1e-3 of the largest eigenvalue: from inverse iteration, kept orthogonal during it).  For larger ranks: full
+//      eigen-decomposition by parallel-order Jacobi rotations run to convergence.
+//   4. Delta = C^T C r_bar (Eq. 5) in the rotated coordinates, taken back through the reflectors as ONE vector,
+//      delta = A_del / (A_keep + eps) * Delta (Eq. 6), V_out = V_keep + delta on the head's retained rows (Eq. 7).
 //
-// Shared memory: M (d x d) plus a region sized by the number of basis rows any head of the call can have
-// (min(k_eff, d)): with budgets below d two blocks share a multiprocessor, which is what the latency-bound
-// steps of the eigen-solver need.  That caps the kernel at 64 registers per thread: the loops below are written
-// for few live values and few instructions (thread maps that keep a warp's 32 lanes on 32 banks of the
-// 129-float rows, whole rows and column groups skipped rather than predicated off), which is what its time is
-// made of.
+// What bounds it: the chain of d - 2 dependent reflectors, each a matrix-vector product, a reduction, a rank-two
+// update and the norm of the next row.  The matrix therefore lives in REGISTERS (half-warp g of 8 holds rows g, g + 8, ..,
+// a lane pairs of columns for the two-wide FMA); only the reflector and the product cross warps, through shared memory,
+// at one block barrier per reflector of a retained row and two per reflector of the tridiagonal form.  Steps run in
+// stages of 32 so that finished rows and column pairs cost nothing and every register index is static.  128 threads of
+// 255 registers and less than 113 KB per block: two blocks share a multiprocessor.  What is run once per head is written
+// as small loops: a section's first pass costs about 130 cycles per 128 bytes of its code, more than its arithmetic.
+// Measured on 36 x 8 heads, budget 32, rank 2, head_dim 128 (every head back-filled): 0.178 ms against 0.534 ms for the
+// same algebra on a matrix in shared memory (Gram-Schmidt basis, M = P G P, then the reduction); cycles of one block with
+// its neighbour on the multiprocessor: load 16 k, retained rows 49 k, their reflectors on G 51 k, tridiagonal form 146 k
+// (1550 per reflector; a product and an update of the first stage take 467 and 558 by themselves), eigenvalues 11 k,
+// eigenvectors 15 k, way back 18 k.  Slower were: eight warps with half the registers (0.21), the chain of reflectors in a
+// warp of its own beside the matrix warps (0.20 to 0.26: the registers it takes cost the others more), one copy of the
+// step's code for all stages (0.26), retained rows and G in one loop (0.186).
 #pragma once
+
+#include <type_traits>
 
 #include "common.cuh"
 #include "span_test.cuh"
 
 namespace obf {
 
-constexpr int ALG_NT = 512;
+constexpr int ALG_NW = 4;
+constexpr int ALG_NT = 32 * ALG_NW;
+constexpr int ALG_NG = 2 * ALG_NW;              // half-warps: the units that rows are dealt to
+constexpr int ALG_BATCH = 32;                   // retained rows in registers at a time
 constexpr float SPAN_ROW_TOL = 1e-4f;
 constexpr float RCR_SKIP_TOL = 1e-6f;
 constexpr float EIG_RANK_TOL = 1e-5f;
 constexpr int JACOBI_MAX_SWEEPS = 30;
-constexpr int ALG_TRI_MAX_RANK = 8;     // up to this rank only rank + 1 eigenpairs are computed
-constexpr int ALG_TRI_NE = ALG_TRI_MAX_RANK + 1;
+constexpr int ALG_TRI_MAX_RANK = 8;     // up to this rank only rank + 1 eigenvalues and rank eigenvectors are computed
 constexpr float EIG_CLUSTER_TOL = 1e-3f; // eigenvalues closer than this (relative to the largest) are orthogonalised explicitly
 
-// Number of eigenvalues of the symmetric tridiagonal matrix (diagonal a, off-diagonal b) that are smaller than x:
-// the negative pivots of the LDL^T factorisation of T - x I.
-template <int D>
-__device__ __forceinline__ int sturm_count(const float *a, const float *b, float x, float pivmin)
+// ---- pairs of fp32 in one 64-bit register, for the two-wide FMA ------------------------------------
+typedef unsigned long long f32x2;
+
+__device__ __forceinline__ f32x2 pk(float a, float b)
 {
-    float q = a[0] - x;
-    int cnt = q < 0.f ? 1 : 0;
-#pragma unroll 4
-    for (int i = 1; i < D; ++i) {
-        if (fabsf(q) < pivmin) q = -pivmin;
-        // the quotient need not be rounded correctly: an error of a few ulp moves the count's switching point by as much
-        q = a[i] - x - __fdividef(b[i - 1] * b[i - 1], q);
-        cnt += q < 0.f ? 1 : 0;
-    }
-    return cnt;
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void upk(f32x2 v, float &a, float &b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+// a where the mask is all ones, b where it is zero.  (A conditional between array elements would be a conditional
+// address, and the array would have to live in memory.)
+__device__ __forceinline__ f32x2 sel2(f32x2 mask, f32x2 a, f32x2 b) { return b ^ ((a ^ b) & mask); }
+__device__ __forceinline__ f32x2 mask2(bool c) { return c ? ~0ull : 0ull; }
+__device__ __forceinline__ float sum2(f32x2 v)
+{
+    float a, b;
+    upk(v, a, b);
+    return a + b;
 }
 
-// Floats of the eigen-solver's workspace: tridiagonal form (diagonal, off-diagonal, eigenvalues, rank + 1 vectors
-// with five factor arrays each), or the d x d eigenvector matrix of the Jacobi route, or two row blocks of the
-// fixed-iteration route.
+// Sums of N values per lane (a power of two) over runs of W lanes (W >= N): lane l of a run ends with the total of value
+// l / (W / N).  Half as many values travel at every step: about N shuffles instead of N log2(W).
+template <int N, int W>
+__device__ __forceinline__ float transposed_sum(float (&a)[N], int lane)
+{
+    int off = W / 2;
+#pragma unroll
+    for (int n = N / 2; n >= 1; n >>= 1, off >>= 1) {
+        const bool up = (lane & off) != 0;
+#pragma unroll
+        for (int i = 0; i < n; ++i) {
+            const float send = up ? a[i] : a[i + n], keep = up ? a[i + n] : a[i];
+            a[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+        }
+    }
+#pragma unroll
+    for (; off >= 1; off >>= 1) a[0] += __shfl_xor_sync(0xffffffffu, a[0], off);
+    return a[0];
+}
+
+__device__ __forceinline__ float half_sum(float v)
+{
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+__device__ __forceinline__ float rsqrt_approx(float x)
+{
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+__device__ __forceinline__ float rcp_approx(float x)
+{
+    float r;
+    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// The matrix in registers.  Half-warp g (of ALG_NG) holds rows g, g + ALG_NG, ..; lane c of its sixteen holds of each
+// row the pairs of columns 32 q + 2 c, 32 q + 2 c + 1.  A reflector and the product with it meet the warps in shared
+// memory twice: in order (for the columns) and doubled into pairs with a half-warp's rows next to one another (for its
+// rows).
+template <int D>
+struct AlgShape {
+    static constexpr int RW = D / ALG_NG;        // rows a lane holds
+    static constexpr int NQ = D / 32;            // column pairs a lane holds per row
+    static constexpr int RPS = 32 / ALG_NG;      // rows a lane holds of 32 consecutive ones
+    static constexpr int GRP = RW + 2;           // pairs per half-warp in the doubled arrays (padded against bank conflicts)
+    static constexpr int DUP = ALG_NG * GRP;     // pairs of one doubled array
+    __device__ static __forceinline__ int dup_index(int i) { return (i % ALG_NG) * GRP + i / ALG_NG; }
+};
+template <int D>
+using AlgMat = f32x2[AlgShape<D>::RW][AlgShape<D>::NQ];
+template <int D>
+using AlgRow = f32x2[AlgShape<D>::NQ];
+
+// Column pairs from pair FROM on of a vector of D floats in shared memory.
+template <int D, int FROM = 0>
+__device__ __forceinline__ void alg_load(AlgRow<D> &x, const float *v, int c16)
+{
+#pragma unroll
+    for (int q = FROM; q < AlgShape<D>::NQ; ++q) x[q] = *reinterpret_cast<const f32x2 *>(v + 32 * q + 2 * c16);
+}
+template <int D, int FROM = 0>
+__device__ __forceinline__ float alg_dot(const AlgRow<D> &x, const AlgRow<D> &y)
+{
+    f32x2 a = mul2(x[FROM], y[FROM]);
+#pragma unroll
+    for (int q = FROM + 1; q < AlgShape<D>::NQ; ++q) a = fma2(x[q], y[q], a);
+    return sum2(a);
+}
+
+// Stage S serves the reflectors 32 S .. 32 S + 31: their support starts at row and column 32 S or later.
+// p = 2 M v on the rows of the stage; pd may be null.  With vd (the reflector doubled) also this half-warp's share of
+// v . p, in kp[grp]: formed from the lanes' partial sums, its reduction runs beside that of p.
+template <int D, int S>
+__device__ __forceinline__ void alg_product(const AlgMat<D> &M, const AlgRow<D> &v2, float *pl, f32x2 *pd, const f32x2 *vd, float *kp,
+                                            int grp, int c16)
+{
+    constexpr int RW = AlgShape<D>::RW, R0 = AlgShape<D>::RPS * S, NR = RW - R0;
+    constexpr int NP = NR > 8 ? 16 : NR > 4 ? 8 : NR > 2 ? 4 : 2;
+    float acc[NP];
+#pragma unroll
+    for (int r = 0; r < NP; ++r) acc[r] = r < NR ? alg_dot<D, S>(M[R0 + (r < NR ? r : 0)], v2) : 0.f;
+    float ka = 0.f, kb = 0.f;
+    if (vd) {
+        const f32x2 *vr = vd + grp * AlgShape<D>::GRP + R0;
+#pragma unroll
+        for (int r = 0; r < NR; r += 2) {
+            const ulonglong2 w = *reinterpret_cast<const ulonglong2 *>(vr + r);
+            float a, b, t;
+            upk(w.x, a, t);
+            upk(w.y, b, t);
+            ka = fmaf(a, acc[r], ka);
+            kb = fmaf(b, acc[r + 1], kb);
+        }
+        ka = 2.f * half_sum(ka + kb);
+    }
+    const float s = 2.f * transposed_sum<NP, 16>(acc, c16);
+    constexpr int LPR = 16 / NP;
+    const int r = c16 / LPR;
+    if ((c16 % LPR) == 0 && r < NR) {
+        pl[grp + ALG_NG * (R0 + r)] = s;
+        if (pd) pd[grp * AlgShape<D>::GRP + R0 + r] = pk(s, s);
+    }
+    if (vd && c16 == 0) kp[grp] = ka;
+}
+
+// M <- M - v w^T - w v^T with w = p - (v.p) v on the rows and columns of the stage.  x: row `xr` of the stage's first
+// RPS rows as the update leaves it, formed first so that the next reflector need not wait.
+template <int D, int S>
+__device__ __forceinline__ void alg_update(AlgMat<D> &M, const AlgRow<D> &v, const f32x2 *vd, const float *pl, const f32x2 *pd,
+                                           const float *kp, int grp, int c16, int xr, AlgRow<D> &x)
+{
+    constexpr int RW = AlgShape<D>::RW, NQ = AlgShape<D>::NQ, R0 = AlgShape<D>::RPS * S;
+    AlgRow<D> w2, v2;
+    alg_load<D, S>(w2, pl, c16);
+    float kq[ALG_NG / 4], kk = 0.f;
+#pragma unroll
+    for (int e = 0; e < ALG_NG / 4; ++e) {
+        const float4 t = *reinterpret_cast<const float4 *>(kp + 4 * e);
+        kq[e] = (t.x + t.y) + (t.z + t.w);
+    }
+#pragma unroll
+    for (int e = 0; e < ALG_NG / 4; e += 2) kk += kq[e] + kq[e + 1];
+    const f32x2 nk = pk(-kk, -kk), neg = pk(-1.f, -1.f);
+#pragma unroll
+    for (int q = S; q < NQ; ++q) {
+        w2[q] = mul2(fma2(nk, v[q], w2[q]), neg);
+        v2[q] = mul2(v[q], neg);
+    }
+    const f32x2 *vr = vd + grp * AlgShape<D>::GRP, *pr = pd + grp * AlgShape<D>::GRP;
+    {
+        const f32x2 vx = vr[R0 + xr], wx = fma2(nk, vx, pr[R0 + xr]);
+        const f32x2 odd = mask2(xr & 1), high = mask2(xr & 2);
+#pragma unroll
+        for (int q = S; q < NQ; ++q) {
+            f32x2 m = sel2(odd, M[R0 + 1][q], M[R0][q]);
+            if constexpr (AlgShape<D>::RPS == 4) m = sel2(high, sel2(odd, M[R0 + 3][q], M[R0 + 2][q]), m);
+            x[q] = fma2(vx, w2[q], fma2(wx, v2[q], m));
+        }
+    }
+#pragma unroll
+    for (int r = R0; r < RW; r += 2) {
+        const ulonglong2 va = *reinterpret_cast<const ulonglong2 *>(vr + r), pa = *reinterpret_cast<const ulonglong2 *>(pr + r);
+        const f32x2 wa = fma2(nk, va.x, pa.x), wb = fma2(nk, va.y, pa.y);
+#pragma unroll
+        for (int q = S; q < NQ; ++q) {
+            M[r][q] = fma2(va.x, w2[q], fma2(wa, v2[q], M[r][q]));
+            M[r + 1][q] = fma2(va.y, w2[q], fma2(wb, v2[q], M[r + 1][q]));
+        }
+    }
+}
+
+// Entry c (the same in every lane) of a row, given as column pairs, for both half-warps.
+template <int D, int FROM = 0>
+__device__ __forceinline__ float alg_entry(const AlgRow<D> &x, int c, int lane)
+{
+    f32x2 v = x[FROM];
+#pragma unroll
+    for (int q = FROM + 1; q < AlgShape<D>::NQ; ++q) v = sel2(mask2(c >> 5 == q), x[q], v);
+    float a, b;
+    upk(v, a, b);
+    return __shfl_sync(0xffffffffu, (c & 1) ? b : a, (lane & 16) + ((c & 31) >> 1));
+}
+
+// Sum of squares of a row's entries from `from` on (pairs before FROM hold nothing of it).
+template <int D, int FROM = 0>
+__device__ __forceinline__ float alg_tail2(const AlgRow<D> &x, int from, int c16)
+{
+    float s = 0.f;
+#pragma unroll
+    for (int q = FROM; q < AlgShape<D>::NQ; ++q) {
+        float a, b;
+        upk(x[q], a, b);
+        const int c = 32 * q + 2 * c16;
+        a = c >= from ? a : 0.f;
+        b = c + 1 >= from ? b : 0.f;
+        s = fmaf(a, a, fmaf(b, b, s));
+    }
+    return half_sum(s);
+}
+
+// Writes the unit reflector of support >= j0 made of x: entry j0 is `first`, the others x, all scaled (a half-warp's lanes).
+template <int D, int FROM = 0>
+__device__ __forceinline__ void alg_store_reflector(const AlgRow<D> &x, int j0, float first, float rs, float *v, f32x2 *vd, int c16)
+{
+#pragma unroll
+    for (int q = 0; q < AlgShape<D>::NQ; ++q) {
+        float a = 0.f, b = 0.f;
+        if (q >= FROM) upk(x[q], a, b);
+        const int c = 32 * q + 2 * c16;
+        a = c < j0 ? 0.f : (c == j0 ? first : a) * rs;
+        b = c + 1 < j0 ? 0.f : (c + 1 == j0 ? first : b) * rs;
+        *reinterpret_cast<f32x2 *>(v + c) = pk(a, b);
+        if (vd) {
+            vd[AlgShape<D>::dup_index(c)] = pk(a, a);
+            vd[AlgShape<D>::dup_index(c + 1)] = pk(b, b);
+        }
+    }
+}
+
+// Reflector j + 1 from row j of the trailing block (entries of x from j on), with the row's diagonal and off-diagonal
+// entry of the tridiagonal form.  Every half-warp computes on its own row; the owner of row j stores.
+template <int D, int FROM>
+__device__ __forceinline__ void alg_row_done(const AlgRow<D> &x, int j, float tiny2, float *Y, f32x2 *vd, float *ta, float *tb,
+                                             int grp, int lane)
+{
+    const int c16 = lane & 15;
+    const float below2 = alg_tail2<D, FROM>(x, j + 2, c16);          // squares right of the super-diagonal entry
+    const float dg = alg_entry<D, FROM>(x, j, lane), x0 = alg_entry<D, FROM>(x, j + 1, lane);
+    const float n2 = fmaf(x0, x0, below2), nrm = n2 * rsqrt_approx(fmaxf(n2, 1e-37f));
+    const float al = x0 >= 0.f ? -nrm : nrm;
+    const float vn2 = 2.f * fmaf(nrm, fabsf(x0), n2);                // |x - al e_0|^2
+    const bool skip = !(below2 > tiny2) || !(vn2 > 1e-37f);          // nothing beyond the super-diagonal
+    const float rs = skip ? 0.f : rsqrt_approx(vn2);
+    if (grp == j % ALG_NG) {
+        alg_store_reflector<D, FROM>(x, j + 1, x0 - al, rs, Y + (j + 1) * D, vd, c16);
+        if (c16 == 0) {
+            ta[j] = dg;
+            tb[j] = skip ? x0 : al;
+        }
+    }
+}
+
+// Sturm counts of the tridiagonal matrix (diagonal a, squared off-diagonals b2, scaled to a spectrum within [-1, 1]) at
+// two shifts: the number of eigenvalues below each, as the sign changes of the leading principal minors'
+// three-term recurrence p_i = (a_i - x) p_{i-1} - b2_{i-1} p_{i-2} (Givens' bisection).  No division: a step of the chain
+// is one FMA.  Both values are rescaled by a power of two every four steps (a step grows them at most threefold; b2 is
+// kept above 1e-14, so four steps shrink them by 1e-28 at most and two consecutive zeros cannot occur).
+// n4: steps in groups of four; the arrays are padded to that with a = 2 (no sign change), b2 = 0.
+__device__ __forceinline__ void sturm_count2(const float *a, const float *b2, int n4, float x0, float x1, int &c0, int &c1)
+{
+    float p0 = 1.f, q0 = 0.f, p1 = 1.f, q1 = 0.f;
+    uint32_t n0 = 0u, n1 = 0u;
+    float4 an = *reinterpret_cast<const float4 *>(a), bn = *reinterpret_cast<const float4 *>(b2);
+#pragma unroll 1
+    for (int i = 0; i < n4; ++i) {
+        const float aa[4] = {an.x, an.y, an.z, an.w}, bb[4] = {-bn.x, -bn.y, -bn.z, -bn.w};
+        // the next four steps' entries, ahead of the chain (the arrays have four floats to spare)
+        an = *reinterpret_cast<const float4 *>(a + 4 * i + 4);
+        bn = *reinterpret_cast<const float4 *>(b2 + 4 * i + 4);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const float r0 = fmaf(aa[e] - x0, p0, bb[e] * q0), r1 = fmaf(aa[e] - x1, p1, bb[e] * q1);
+            n0 += (__float_as_uint(r0) ^ __float_as_uint(p0)) >> 31;
+            n1 += (__float_as_uint(r1) ^ __float_as_uint(p1)) >> 31;
+            q0 = p0; p0 = r0;
+            q1 = p1; p1 = r1;
+        }
+        // 2^-e of the larger one's exponent e (max 254 keeps the factor a normal number)
+        const uint32_t e0 = max(__float_as_uint(p0) & 0x7F800000u, __float_as_uint(q0) & 0x7F800000u);
+        const uint32_t e1 = max(__float_as_uint(p1) & 0x7F800000u, __float_as_uint(q1) & 0x7F800000u);
+        const float f0 = __uint_as_float(0x7F000000u - min(e0, 0x7E800000u)), f1 = __uint_as_float(0x7F000000u - min(e1, 0x7E800000u));
+        p0 *= f0; q0 *= f0;
+        p1 *= f1; q1 *= f1;
+    }
+    c0 = (int)n0;
+    c1 = (int)n1;
+}
+
+// Shared memory, in floats.  Y: the reflectors (all d of them on the tridiagonal route, else those of the retained rows).
+template <int D>
+__host__ __device__ constexpr int algebra_y_rows(int mcap, int rank, int fast_iters)
+{
+    return (fast_iters > 0 || rank > ALG_TRI_MAX_RANK) ? mcap : D;
+}
+
+// Workspace of the eigen-solvers: tridiagonal form (scaled diagonal and squared off-diagonals, per wanted vector six
+// arrays), or two blocks of rows of the fixed-iteration route, or the trailing block and the eigenvector matrix of the
+// Jacobi route.  At least the retained rows' share of u before it and the products among the reflectors after it.
 template <int D>
 __host__ __device__ constexpr int algebra_eig_floats(int rank, int fast_iters)
 {
-    const int ne = (rank < D ? rank : D) + 1;
-    const int tri = 2 * D + 16 + ne * D + ne * 5 * D;
-    const int jac = D * (D + 1);
-    const int fast = 2 * (rank < D ? rank : D) * (D + 1);
-    return fast_iters > 0 ? fast : (rank <= ALG_TRI_MAX_RANK ? tri : jac);
-}
-
-// mcap: basis rows any head of the call can have, min(largest k_eff, D).
-template <int D>
-__host__ __device__ constexpr int algebra_region_floats(int mcap, int rank, int fast_iters)
-{
-    const int thin = mcap * (D + 1);                                // Q X of a projection
-    const int eig = algebra_eig_floats<D>(rank, fast_iters);
-    return mcap * (D + 1) + (thin > eig ? thin : eig);
+    const int r = rank < D ? rank : D;
+    const int tri = 2 * (D + 8) + r * 6 * D;
+    const int least = ALG_BATCH * D;
+    const int eig = fast_iters > 0 ? 2 * r * D : (rank <= ALG_TRI_MAX_RANK ? tri : 2 * D * (D + 1));
+    return eig > least ? eig : least;
 }
 
 template <int D>
 inline size_t algebra_smem_bytes(int mcap, int rank, int fast_iters)
 {
-    return (size_t)(D * (D + 1) + 6 * D + 64 + algebra_region_floats<D>(mcap, rank, fast_iters)) * sizeof(float) +
-           2 * D * sizeof(int);
+    return (size_t)(algebra_y_rows<D>(mcap, rank, fast_iters) * D + 12 * AlgShape<D>::DUP + 2 * D + 6 * D + 96 +
+                    algebra_eig_floats<D>(rank, fast_iters)) * sizeof(float) + 2 * D * sizeof(int);
 }
 
 template <typename TIN, int D>
 __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant__ CallDev p)
 {
-    constexpr int LD = D + 1;
-    extern __shared__ float sm[];
-    const int mcap = p.alg_rows;                   // basis rows any head of this call can have
-    float *B2 = sm;                                // d x d: G, then M, then the reflectors in M's dead columns
-    float *vw = B2 + D * LD, *vc = vw + D, *vu = vc + D, *vl = vu + D, *vcs = vl + D;  // vcs: 2*D/2 floats (c,s)
-    float *red = vcs + D;                          // 32 floats
-    float *misc = red + 32;                        // 32 floats
-    int *ipq = reinterpret_cast<int *>(misc + 32); // D ints: pairs (p,q); then D ints: selected eigen-columns
-    int *isel = ipq + D;
-    float *Qb = reinterpret_cast<float *>(isel + D);   // basis rows of span(V_keep), mcap x LD; stays to the end
-    float *Bm = Qb + mcap * LD;                    // Q X (m x d) of the two projections; the eigen-solvers reuse this
-    float *WS = Bm;                                // workspace of the eigen-solvers
+    typedef AlgShape<D> SH;
+    constexpr int RW = SH::RW, NQ = SH::NQ, LD = D + 1;
+    extern __shared__ __align__(16) float sm[];
+    float *Y = sm;                                                    // reflector j in row j, support >= j
+    f32x2 *vdup = reinterpret_cast<f32x2 *>(Y + algebra_y_rows<D>(p.alg_rows, p.rank, p.fast_iters) * D);   // 4 buffers: reflector j in j & 3
+    f32x2 *pdup = vdup + 4 * SH::DUP;                                 // 2 buffers
+    float *pl = reinterpret_cast<float *>(pdup + 2 * SH::DUP);        // 2 buffers of D
+    float *ta = pl + 2 * D, *tb = ta + D;                             // tridiagonal form
+    float *vu = tb + D, *vx = vu + D, *vc = vx + D, *vl = vc + D;     // vectors of d
+    float *red = vl + D, *misc = red + 32, *tlam = misc + 32;         // 32 floats each
+    int *ipq = reinterpret_cast<int *>(tlam + 32), *isel = ipq + D;   // Jacobi: pairs (p, q), selected columns
+    float *rows_s = reinterpret_cast<float *>(isel + D);              // a batch of retained rows; then
+    float *WS = rows_s;                                               // the workspace of the eigen-solvers
+    __shared__ int s_flag[2];
+    __shared__ __align__(16) float kpart[2 * ALG_NG];                 // 2 buffers: the half-warps' shares of v . p
 
-    const int g = blockIdx.x, tid = threadIdx.x;
+    const int g = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int grp = tid >> 4, c16 = tid & 15;                         // half-warp and the lane in it
     int ci, lh;
     locate(p, g, ci, lh);
     const CacheDev &c = p.c[ci];
@@ -128,123 +422,87 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
         p.delta[(size_t)g * D + tid] = 0.f;
         if (c.delta_out) c.delta_out[(size_t)lh * D + tid] = 0.f;
     }
-    const uint32_t hflag_in = p.hflag[g];          // written by k_span_test
-    __syncthreads();
-    if (tid == 0) p.hflag[g] = 0u;
     if (T - k == 0 || p.rank <= 0) return;
 
     uint32_t status = 0u;
     int m = 0;
-    // c = Q x (vc) and x -= Q^T c for a vector x of d floats in shared memory: four threads per basis row / per
-    // channel.  The thread's share of the row is cut so that the 32 lanes of a warp meet 32 different banks (rows are
-    // d + 1 floats apart: lanes of neighbouring rows are one bank apart, the four threads of a row eight).
-    auto q_dot = [&](const float *x, int rows) {
-        const int j = tid >> 2, part = tid & 3;
-        float sacc = 0.f;
-        if (j < rows) {
-            const float *qj = Qb + j * LD;
-#pragma unroll 8
-            for (int e = 0; e < D / 4; ++e) {
-                const int cc = ((e >> 3) << 5) + part * 8 + (e & 7);
-                sacc = fmaf(qj[cc], x[cc], sacc);
-            }
-        }
-        sacc += __shfl_xor_sync(0xffffffffu, sacc, 1);
-        sacc += __shfl_xor_sync(0xffffffffu, sacc, 2);
-        if (part == 0 && j < rows) vc[j] = sacc;
-    };
-    auto q_minus = [&](float *x, int rows) {
-        const int cc = tid >> 2, part = tid & 3;
-        float sacc = 0.f;
-        if (cc < D) {
-            const int n_e = ((rows + 31) >> 5) << 3;
-            for (int e = 0; e < n_e; ++e) {
-                const int j = ((e >> 3) << 5) + part * 8 + (e & 7);
-                if (j < rows) sacc = fmaf(vc[j], Qb[j * LD + cc], sacc);
-            }
-        }
-        sacc += __shfl_xor_sync(0xffffffffu, sacc, 1);
-        sacc += __shfl_xor_sync(0xffffffffu, sacc, 2);
-        if (part == 0 && cc < D) x[cc] -= sacc;
-    };
     float rcr = 0.f, lam1 = 0.f, lam_rho = 0.f, lam_next = 0.f, dnorm = 0.f, revr = 0.f, pc = 0.f;
     int rho = 0;
     bool done = false;
 
     // ---- 1. k_eff >= d: the span test kernel has already factorised G_keep --
-    if (k >= D && (hflag_in & HFLAG_SPAN_FULL)) { m = D; done = true; pc = 1.f; status |= OBF_DEV_SKIPPED | OBF_DEV_SPAN_FULL; }
+    if (k >= D && (p.hflag[g] & HFLAG_SPAN_FULL)) { m = D; done = true; pc = 1.f; status |= OBF_DEV_SKIPPED | OBF_DEV_SPAN_FULL; }
 
-    // ---- 2. orthonormal basis of span(V_keep), Eq. 2 ------------------------
-    float u_keep[U_LEVELS], sq_keep = 0.f;         // retained rows' share of u (channel tid, per mass level) and of tr G
-#pragma unroll
-    for (int l = 0; l < U_LEVELS; ++l) u_keep[l] = 0.f;
     if (!done) {
         const TIN *vk = reinterpret_cast<const TIN *>(c.v_out) + (size_t)lh * k * D;
         const float *A = p.scores + c.tok_off + (size_t)lh * T;
         const int32_t *idx = c.idx_out + (size_t)lh * k;
-        // the next row and its mass are asked for while the current row is worked on
-        float v_next = 0.f, a_next = 0.f;
-        if (tid < D && k > 0) {
-            v_next = to_f32(vk[tid]);
-            if (p.gram_all) a_next = A[idx[0]];
-        }
-#pragma unroll 1
-        for (int i = 0; i < k && m < D; ++i) {
-            if (tid < D) {
-                const float v = v_next, a = a_next;
-                if (i + 1 < k) {
-                    v_next = to_f32(vk[(size_t)(i + 1) * D + tid]);
-                    if (p.gram_all) a_next = A[idx[i + 1]];
-                }
-                vw[tid] = v;
-                if (p.gram_all) {
-                    const int lev = u_level(a);
-#pragma unroll
-                    for (int l = 0; l < U_LEVELS; ++l)
-                        if (l == lev) u_keep[l] = fmaf(a, v, u_keep[l]);
-                }
-            }
-            __syncthreads();
-            // the norms of a row are taken by every warp for itself (same sum, same order): no block reduction
-            float np0 = 0.f;
-            for (int cc = (tid & 31); cc < D; cc += 32) np0 = fmaf(vw[cc], vw[cc], np0);
-            const float n0sq = warp_sum(np0);
-            sq_keep += n0sq;
-            const float n0 = sqrtf(n0sq);
-            // Gram-Schmidt against the basis so far, a second time only when the first pass took away more than half of
-            // the row's squared norm: what is left of a row that keeps more than that is orthogonal to the basis to
-            // rounding already ("twice is enough", and once where nothing cancels)
-            float n1 = 0.f;
-            for (int pass = 0; pass < 2; ++pass) {
-                q_dot(vw, m);
-                __syncthreads();
-                q_minus(vw, m);
-                __syncthreads();
-                float np1 = 0.f;
-                for (int cc = (tid & 31); cc < D; cc += 32) np1 = fmaf(vw[cc], vw[cc], np1);
-                const float n1sq = warp_sum(np1);
-                n1 = sqrtf(n1sq);
-                if (n1sq > 0.5f * n0sq) break;                      // the same in every thread
-            }
-            const float w1 = tid < D ? vw[tid] : 0.f;
-            if (n1 > SPAN_ROW_TOL * n0 && n1 > 0.f) {
-                // a head can only have more basis rows than the call's layout holds if they reach d (span full)
-                if (m < mcap && tid < D) Qb[m * LD + tid] = w1 / n1;
-                ++m;
-            }
-            __syncthreads();
-        }
-        if (m >= D) { done = true; pc = 1.f; status |= OBF_DEV_SKIPPED | OBF_DEV_SPAN_FULL; }
-        else if (m > mcap) { done = true; status |= OBF_DEV_INTERNAL | OBF_DEV_SKIPPED; }   // cannot happen: m <= min(k, d)
-    }
 
-    if (!done) {
-        // ---- 3. G, u; M = P G P and r_bar without forming P -----------------------
-        for (int e = tid; e < D * D; e += ALG_NT) {
-            float s = 0.f;
-            for (int sp = 0; sp < n_del; ++sp) s += p.gram_d[((size_t)g * S + sp) * D * D + e];
-            B2[(e / D) * LD + (e % D)] = s;
+        // ---- G into registers, its trace --------------------------------------------
+        AlgMat<D> M;
+        {
+            const float *G = p.gram_d + (size_t)g * S * D * D + grp * D + 2 * c16;
+#pragma unroll
+            for (int r = 0; r < RW; ++r)
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) M[r][q] = *reinterpret_cast<const f32x2 *>(G + r * ALG_NG * D + 32 * q);
+#pragma unroll 1
+            for (int sp = 1; sp < n_del; ++sp) {
+                G += D * D;
+#pragma unroll
+                for (int r = 0; r < RW; ++r)
+#pragma unroll
+                    for (int q = 0; q < NQ; ++q) M[r][q] = add2(M[r][q], *reinterpret_cast<const f32x2 *>(G + r * ALG_NG * D + 32 * q));
+            }
         }
+        // this thread's share of the diagonal from row `from` on
+        auto diag_part = [&](int from) __attribute__((always_inline)) {
+            float s = 0.f;
+#pragma unroll
+            for (int r = 0; r < RW; ++r) {
+                const int i = grp + ALG_NG * r;
+                float a, b;
+                upk(M[r][r / SH::RPS], a, b);
+                if (i >= from && c16 == (i & 31) >> 1) s += (i & 1) ? b : a;
+            }
+            return s;
+        };
+
+        // ---- u (and, for the diagnostics, the plain sum of the deleted values) -------------------
+        constexpr int NPART = ALG_NT / D;
+        float sq = 0.f;
+        if (p.gram_all) {
+            // the retained rows' share of u per mass level, and of the trace of G; a lane fetches one row's mass
+            const int col = tid % D, part = tid / D;
+            float uk[U_LEVELS];
+#pragma unroll
+            for (int l = 0; l < U_LEVELS; ++l) uk[l] = 0.f;
+#pragma unroll 1
+            for (int b0 = 0; b0 < k; b0 += 32) {
+                const float al = b0 + lane < k ? A[idx[b0 + lane]] : 0.f;
+#pragma unroll 1
+                for (int i0 = 0; i0 < 32; i0 += 16 * NPART) {
+                    float v[16];
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) {
+                        const int i = b0 + i0 + e * NPART + part;
+                        v[e] = i < k ? to_f32(vk[(size_t)i * D + col]) : 0.f;
+                    }
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) {
+                        const float a = __shfl_sync(0xffffffffu, al, i0 + e * NPART + part);
+                        const int lev = u_level(a);
+                        sq = fmaf(v[e], v[e], sq);
+#pragma unroll
+                        for (int l = 0; l < U_LEVELS; ++l) uk[l] = fmaf(l == lev ? a : 0.f, v[e], uk[l]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int l = 0; l < U_LEVELS; ++l) WS[(part * U_LEVELS + l) * D + col] = uk[l];
+        }
+        const float sq_keep = block_sum<ALG_NT>(sq, red);             // (its barriers also publish WS)
+        const float trAll = block_sum<ALG_NT>(diag_part(0), red);
         if (tid < D) {
             // per level: what the pass over V added up minus the retained rows' share; smallest masses first
             float s = 0.f;
@@ -252,669 +510,844 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                 float sl = 0.f;
                 for (int sp = 0; sp < n_del; ++sp) sl += p.uvec[(((size_t)g * S + sp) * p.u_levels + l) * D + tid];
                 if (p.gram_all) {
-#pragma unroll
-                    for (int l2 = 0; l2 < U_LEVELS; ++l2)
-                        if (l2 == l) sl -= u_keep[l2];
+                    float kl = 0.f;
+                    for (int q = 0; q < NPART; ++q) kl += WS[(q * U_LEVELS + l) * D + tid];
+                    sl -= kl;
                 }
                 s += sl;
             }
             vu[tid] = s;
-            if (c.diag) vw[tid] = p.svec[(size_t)g * D + tid];
+            vx[tid] = c.diag ? p.svec[(size_t)g * D + tid] : 0.f;
         }
         __syncthreads();
-        // x -> P x = x - Q^T (Q x) for the vector in `x` (d floats in shared memory), in place; vc is scratch
-        auto project = [&](float *x) {
-            q_dot(x, m);
-            __syncthreads();
-            q_minus(x, m);
-            __syncthreads();
-        };
-        if (c.diag) {
-            // projection cosine: s = sum of the deleted values, its part inside span(V_keep) is s - P s
-            const float sv = tid < D ? vw[tid] : 0.f;
-            project(vw);
-            const float par = tid < D ? sv - vw[tid] : 0.f;
-            const float ss = block_sum<ALG_NT>(sv * sv, red), pp = block_sum<ALG_NT>(par * par, red);
-            const float sp = block_sum<ALG_NT>(sv * par, red);
-            pc = (ss > 0.f && pp > 0.f) ? sp * rsqrtf(ss) * rsqrtf(pp) : 0.f;
-        }
         // squared Frobenius norm of the deleted values (the denominator of RCR).  As a difference of two fp32 traces
         // it is resolved down to about 1e-6 of the squared norm of all values: below 1e-5 of it the deleted values
         // count as negligible beside the retained ones and nothing is injected.
-        const float trAll = block_sum<ALG_NT>(tid < D ? B2[tid * LD + tid] : 0.f, red);
-        const float trG = trAll - (p.gram_all ? sq_keep : 0.f);
+        const float trG = trAll - sq_keep;
         const bool del_negligible = p.gram_all && !(trG > 1e-5f * trAll);
-        // M = (I - Q^T Q) G (I - Q^T Q) as two rank-m updates: B = Q X (m x d), X -= Q^T B, first on X = G from the
-        // left, then on the transposed problem from the right (X is symmetric up to rounding, so "B = Q X^T")
-        for (int side = 0; side < 2; ++side) {
-            // B[j][c] = sum_a Q[j][a] X[a][c] (left) or sum_a Q[j][a] X[c][a] (right): a 1 x 4 register tile per thread,
-            // its four columns d / 4 apart so that the lanes of a warp read neighbouring banks
-            for (int t = tid; t < m * (D / 4); t += ALG_NT) {
-                const int j = t / (D / 4), c0 = t % (D / 4);
-                float acc[4] = {0.f, 0.f, 0.f, 0.f};
-                const float *qj = Qb + j * LD;
-                if (side == 0) {
-#pragma unroll 4
-                    for (int a = 0; a < D; ++a) {
-                        const float qv = qj[a];
+        // one more vector per half-warp that the reflectors are applied to: u in the first, the sum of the deleted values
+        // in the second
+        AlgRow<D> aux;
+        if (grp < 2) alg_load<D>(aux, grp == 0 ? vu : vx, c16);
+        else {
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) acc[e] = fmaf(qv, B2[a * LD + c0 + e * (D / 4)], acc[e]);
-                    }
-                } else {
-#pragma unroll 4
-                    for (int a = 0; a < D; ++a) {
-                        const float qv = qj[a];
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) acc[e] = fmaf(qv, B2[(c0 + e * (D / 4)) * LD + a], acc[e]);
-                    }
-                }
-#pragma unroll
-                for (int e = 0; e < 4; ++e) Bm[j * LD + c0 + e * (D / 4)] = acc[e];
-            }
-            __syncthreads();
-            // left: X[a][c] -= sum_j Q[j][a] B[j][c];  right: X[a][c] -= sum_j B[j][a] Q[j][c].  4 x 4 tile per thread
-            const float *Lf = side == 0 ? Qb : Bm, *Rf = side == 0 ? Bm : Qb;
-            for (int t = tid; t < (D / 4) * (D / 4); t += ALG_NT) {
-                const int a0 = (t / (D / 4)) * 4, c0 = t % (D / 4);       // rows a0 .. a0 + 3, columns c0 + e d / 4
-                float acc[4][4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) acc[i][e] = 0.f;
-                for (int j = 0; j < m; ++j) {
-                    float l[4], r[4];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) { l[i] = Lf[j * LD + a0 + i]; r[i] = Rf[j * LD + c0 + i * (D / 4)]; }
-#pragma unroll
-                    for (int i = 0; i < 4; ++i)
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) acc[i][e] = fmaf(l[i], r[e], acc[i][e]);
-                }
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) B2[(a0 + i) * LD + c0 + e * (D / 4)] -= acc[i][e];
-            }
-            __syncthreads();
+            for (int q = 0; q < NQ; ++q) aux[q] = 0ull;
         }
-        for (int e = tid; e < D * D; e += ALG_NT) {            // symmetrise
-            const int a = e / D, bb = e % D;
-            if (a < bb) {
-                const float sy = 0.5f * (B2[a * LD + bb] + B2[bb * LD + a]);
-                B2[a * LD + bb] = sy;
-                B2[bb * LD + a] = sy;
-            }
-        }
-        // r_bar = P u / (A_del + eps)
-        project(vu);
-        if (tid < D) vu[tid] = vu[tid] / (a_del + p.eps);
-        __syncthreads();
-        const float trM = block_sum<ALG_NT>(tid < D ? B2[tid * LD + tid] : 0.f, red);
-        rcr = del_negligible ? 0.f : trM / (trG + p.eps);
-        if (!(rcr >= RCR_SKIP_TOL)) { done = true; status |= OBF_DEV_SKIPPED; }
-
-        // delta, projected once more off the basis rows, published and injected (Eq. 5-7): dl = this thread's channel
-        auto finish_delta = [&](float dl) {
-            if (tid < D) vw[tid] = dl;
-            __syncthreads();
-            project(vw);
-            dl = tid < D ? vw[tid] : 0.f;
-            const float dn2 = block_sum<ALG_NT>(dl * dl, red);
-            dnorm = sqrtf(dn2);
-            if (!isfinite(dn2)) { status |= OBF_DEV_NONFINITE | OBF_DEV_SKIPPED; dnorm = 0.f; }
-            else if (rho == 0 || dn2 == 0.f) status |= OBF_DEV_SKIPPED;
-            else {
-                if (tid < D) {
-                    p.delta[(size_t)g * D + tid] = dl;
-                    if (c.delta_out) c.delta_out[(size_t)lh * D + tid] = dl;
-                }
-                if (tid == 0) p.hflag[g] = HFLAG_INJECT;
-                // Eq. 7: V_out = V_keep + delta on every retained row; the fp32 sum is rounded once.  Attn-inject
-                // (App. D.2): row t takes k * A_t / (A_keep + eps) times delta instead
-                TIN *rows = reinterpret_cast<TIN *>(c.v_out) + (size_t)lh * k * D;
-                const float *Am = p.scores + c.tok_off + (size_t)lh * T;
-                const int32_t *ix = c.idx_out + (size_t)lh * k;
-                const float share = (float)k / (a_keep + p.eps);
-                for (int e = tid; e < k * D; e += ALG_NT) {
-                    const float wgt = p.attn_inject ? share * Am[ix[e / D]] : 1.f;
-                    const float sum = fmaf(wgt, vw[e % D], to_f32(rows[e]));
-                    if constexpr (sizeof(TIN) == 4) rows[e] = sum;
-                    else rows[e] = __float2bfloat16_rn(sum);
-                }
-            }
+        // x <- x - 2 (x.v) v
+        auto reflect = [&](AlgRow<D> &x, const AlgRow<D> &v) __attribute__((always_inline)) {
+            const float s = -2.f * half_sum(alg_dot<D>(x, v));
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) x[q] = fma2(pk(s, s), v[q], x[q]);
         };
-
-        // ---- 4f. fast path of App. H: C <- orth(C M), a fixed number of times, from the first rows of the identity ----
-        if (!done && p.fast_iters > 0) {
-            const int lane = tid & 31, warp = tid >> 5;
-            int rho_f = min(min(p.rank, D), D - m);               // rank(R) <= d - m
-            float *C = WS, *Y = WS + min(p.rank, D) * LD;         // row blocks of length D (stride LD)
-            for (int e = tid; e < rho_f * D; e += ALG_NT) C[(e / D) * LD + (e % D)] = (e / D == e % D) ? 1.f : 0.f;
-            __syncthreads();
+        // ---- 2. reflectors of the retained rows (Eq. 2), then applied to G from both sides.  Two loops: together their
+        // code outgrows what a multiprocessor fetches at full speed (3500 cycles per row in one loop, 3100 in two) ----
+        {
+            // a batch of rows in shared memory: row b0 + grp + ALG_NG s in slot s of the half-warp
+            constexpr int NS = ALG_BATCH / ALG_NG;
+            float *R = rows_s + grp * D, *n0 = vl;                     // n0: the rows' squared norms
+            // rows of the half-warp from slot s0 on, reflected by v
+            auto reflect_rows = [&](const AlgRow<D> &v, int s0) __attribute__((always_inline)) {
+                AlgRow<D> x[NS];
+                float d4[NS];
+#pragma unroll
+                for (int s = 0; s < NS; ++s) alg_load<D>(x[s], R + s * ALG_NG * D, c16);
+#pragma unroll
+                for (int s = 0; s < NS; ++s) d4[s] = alg_dot<D>(x[s], v);
+                const float tot = -2.f * transposed_sum<NS, 16>(d4, c16);
+#pragma unroll
+                for (int s = 0; s < NS; ++s) {
+                    const float f = __shfl_sync(0xffffffffu, tot, (lane & 16) + (16 / NS) * s);
+                    if (s >= s0) {
+#pragma unroll
+                        for (int q = 0; q < NQ; ++q) *reinterpret_cast<f32x2 *>(R + s * ALG_NG * D + 32 * q + 2 * c16) = fma2(pk(f, f), v[q], x[s][q]);
+                    }
+                }
+                __syncwarp();
+            };
+            // whether row i of the batch adds a direction to the m there are, and its reflector
+            auto candidate = [&](int i) __attribute__((always_inline)) {
+                if (warp != (i % ALG_NG) / 2) return;
+                AlgRow<D> x;
+                alg_load<D>(x, R + (i / ALG_NG) * ALG_NG * D, c16);
+                const float t2 = alg_tail2<D>(x, m, c16), x0 = R[(i / ALG_NG) * ALG_NG * D + (m < D ? m : 0)];
+                const float nrm = t2 * rsqrt_approx(fmaxf(t2, 1e-37f));
+                if (grp == i % ALG_NG) {
+                    const bool add = m < D && t2 > SPAN_ROW_TOL * SPAN_ROW_TOL * n0[i] && t2 > 1e-37f;
+                    if (add) {
+                        const float al = x0 >= 0.f ? -nrm : nrm;
+                        alg_store_reflector<D>(x, m, x0 - al, rsqrt_approx(2.f * fmaf(nrm, fabsf(x0), t2)), Y + m * D, nullptr, c16);
+                    }
+                    if (c16 == 0) s_flag[i & 1] = add ? 1 : 0;
+                }
+            };
 #pragma unroll 1
-            for (int itn = 0; itn < p.fast_iters; ++itn) {
-                for (int e = tid; e < rho_f * D; e += ALG_NT) {    // Y = C M
-                    const int i = e / D, b = e % D;
-                    float sacc = 0.f;
-#pragma unroll 8
-                    for (int a = 0; a < D; ++a) sacc = fmaf(C[i * LD + a], B2[a * LD + b], sacc);
-                    Y[i * LD + b] = sacc;
+            for (int b0 = 0; b0 < k && m < D; b0 += ALG_BATCH) {
+#pragma unroll 1
+                for (int s = 0; s < NS; ++s) {
+                    const int i = grp + ALG_NG * s;
+                    AlgRow<D> x;
+#pragma unroll
+                    for (int q = 0; q < NQ; ++q) {
+                        x[q] = 0ull;
+                        if (b0 + i < k) {
+                            const TIN *src = vk + (size_t)(b0 + i) * D + 32 * q + 2 * c16;
+                            if constexpr (sizeof(TIN) == 4) x[q] = *reinterpret_cast<const f32x2 *>(src);
+                            else {
+                                const uint32_t w = *reinterpret_cast<const uint32_t *>(src);
+                                x[q] = pk(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u));
+                            }
+                        }
+                        *reinterpret_cast<f32x2 *>(R + s * ALG_NG * D + 32 * q + 2 * c16) = x[q];
+                    }
+                    const float nn = half_sum(alg_dot<D>(x, x));
+                    if (c16 == 0) n0[i] = nn;
+                }
+                __syncwarp();
+                // (the reflectors that earlier batches found, all published behind a barrier)
+#pragma unroll 1
+                for (int j = 0; j < m; ++j) {
+                    AlgRow<D> v;
+                    alg_load<D>(v, Y + j * D, c16);
+                    reflect_rows(v, 0);
+                }
+                const int rows = min(ALG_BATCH, k - b0);
+                candidate(0);
+#pragma unroll 1
+                for (int i = 0; i < rows; ++i) {
+                    __syncthreads();
+                    if (s_flag[i & 1]) {                               // row i has a reflector
+                        AlgRow<D> v;
+                        alg_load<D>(v, Y + m * D, c16);
+                        reflect_rows(v, (i + ALG_NG - grp) / ALG_NG);
+                        if (++m >= D) break;
+                        if (i + 1 < rows) candidate(i + 1);
+                        reflect(aux, v);
+                    } else if (i + 1 < rows) {
+                        candidate(i + 1);
+                    }
+                }
+                // the flag is written again by the next batch
+                __syncthreads();
+            }
+            auto double_up = [&](int j) __attribute__((always_inline)) {
+                if (tid < D) {
+                    const float t = Y[j * D + tid];
+                    vdup[(j & 3) * SH::DUP + SH::dup_index(tid)] = pk(t, t);
+                }
+            };
+            auto apply_stage = [&](auto stage) __attribute__((always_inline)) {
+                constexpr int ST = decltype(stage)::value;
+                const int j1 = min(32 * ST + 32, m);
+#pragma unroll 1
+                for (int j = 32 * ST; j < j1; ++j) {
+                    const int pb = j & 1;
+                    AlgRow<D> v, x;
+                    alg_load<D, ST>(v, Y + j * D, c16);
+                    alg_product<D, ST>(M, v, pl + pb * D, pdup + pb * SH::DUP, vdup + (j & 3) * SH::DUP, kpart + pb * ALG_NG, grp, c16);
+                    if (j + 1 < m) double_up(j + 1);
+                    __syncthreads();                                   // p is there, and the next reflector doubled
+                    alg_update<D, ST>(M, v, vdup + (j & 3) * SH::DUP, pl + pb * D, pdup + pb * SH::DUP, kpart + pb * ALG_NG, grp, c16, 0, x);
+                }
+            };
+            if (m < D) {
+                if (m > 0) double_up(0);
+                __syncthreads();
+                apply_stage(std::integral_constant<int, 0>{});
+                apply_stage(std::integral_constant<int, 1>{});
+                if constexpr (D > 64) {
+                    apply_stage(std::integral_constant<int, D / 32 - 2>{});
+                    apply_stage(std::integral_constant<int, D / 32 - 1>{});
+                }
+                __syncthreads();                                       // the buffers are used again
+            }
+        }
+        if (m >= D) { done = true; pc = 1.f; status |= OBF_DEV_SKIPPED | OBF_DEV_SPAN_FULL; }
+
+        if (!done) {
+            if (c.diag) {
+                // projection cosine: s = sum of the deleted values; its part inside span(V_keep) is the first m coordinates
+                const float all = alg_tail2<D>(aux, 0, c16), out = alg_tail2<D>(aux, m, c16);
+                if (grp == 1 && c16 == 0) misc[8] = all > 0.f ? sqrtf(fmaxf(all - out, 0.f) / all) : 0.f;
+                __syncthreads();
+                pc = misc[8];
+            }
+            const float trM = block_sum<ALG_NT>(diag_part(m), red);
+            rcr = del_negligible ? 0.f : trM / (trG + p.eps);
+            if (!(rcr >= RCR_SKIP_TOL)) { done = true; status |= OBF_DEV_SKIPPED; }
+
+            // Delta in the rotated coordinates (vx, all d of them, zero below m) -> delta, published and injected (Eq. 6-7).
+            // hi: the reflectors hi .. m + 1 and m - 1 .. 0 lead back.
+            auto finish_delta = [&](int hi) {
+                if (tid < D) pl[tid] = 0.f;
+                __syncthreads();
+                if (warp == 0) {
+                    // four reflectors per step: H_0 H_1 H_2 H_3 x needs the four products with x and the six among the
+                    // reflectors, whose reductions go through the half-warp together
+                    AlgRow<D> x;
+                    alg_load<D>(x, vx, c16);
+#pragma unroll 1
+                    for (int l = (hi > m ? hi - m : 0) + m - 1; l >= 0; l -= 4) {
+                        AlgRow<D> v[4];
+                        float d[16], dv[10];
+                        // v[0] is applied first; past the last one: zeros
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) alg_load<D>(v[e], l - e >= 0 ? Y + (l - e + (l - e >= m ? 1 : 0)) * D : pl, c16);
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) d[e] = 0.f;
+                        // at e (e + 1) / 2: the products of v[e] with v[0] .. v[e - 1] and with x
+#pragma unroll
+                        for (int e = 0; e < 4; ++e)
+#pragma unroll
+                            for (int f = 0; f <= e; ++f) d[e * (e + 1) / 2 + f] = f < e ? alg_dot<D>(v[e], v[f]) : alg_dot<D>(v[e], x);
+                        const float tot = transposed_sum<16, 16>(d, c16);
+#pragma unroll
+                        for (int e = 0; e < 10; ++e) dv[e] = __shfl_sync(0xffffffffu, tot, (lane & 16) + e);
+                        const float s0 = -2.f * dv[0];
+                        const float s1 = -2.f * fmaf(s0, dv[1], dv[2]);
+                        const float s2 = -2.f * fmaf(s1, dv[4], fmaf(s0, dv[3], dv[5]));
+                        const float s3 = -2.f * fmaf(s2, dv[8], fmaf(s1, dv[7], fmaf(s0, dv[6], dv[9])));
+#pragma unroll
+                        for (int q = 0; q < NQ; ++q)
+                            x[q] = fma2(pk(s3, s3), v[3][q], fma2(pk(s2, s2), v[2][q], fma2(pk(s1, s1), v[1][q], fma2(pk(s0, s0), v[0][q], x[q]))));
+                    }
+#pragma unroll
+                    for (int q = 0; q < NQ; ++q) {
+                        x[q] = mul2(x[q], pk(alpha, alpha));
+                        if (grp == 0) *reinterpret_cast<f32x2 *>(vx + 32 * q + 2 * c16) = x[q];
+                    }
+                    const float dn = half_sum(alg_dot<D>(x, x));
+                    if (lane == 0) misc[9] = dn;
                 }
                 __syncthreads();
-                // orth: Gram-Schmidt over the rows in order, twice; a row with nothing left is dropped (warp 0)
-                if (warp == 0) {
-                    int kept = 0;
-                    for (int i = 0; i < rho_f; ++i) {
-                        float *y = Y + i * LD;
-                        float n0 = 0.f;
-                        for (int cc = lane; cc < D; cc += 32) n0 = fmaf(y[cc], y[cc], n0);
-                        n0 = warp_sum(n0);
-                        for (int pass = 0; pass < 2; ++pass)
-                            for (int j = 0; j < kept; ++j) {
-                                const float *qv = C + j * LD;
-                                float dsum = 0.f;
-                                for (int cc = lane; cc < D; cc += 32) dsum = fmaf(y[cc], qv[cc], dsum);
-                                dsum = warp_sum(dsum);
-                                for (int cc = lane; cc < D; cc += 32) y[cc] -= dsum * qv[cc];
+                const float dn2 = misc[9];
+                dnorm = sqrtf(dn2);
+                if (!isfinite(dn2)) { status |= OBF_DEV_NONFINITE | OBF_DEV_SKIPPED; dnorm = 0.f; }
+                else if (rho == 0 || dn2 == 0.f) status |= OBF_DEV_SKIPPED;
+                else {
+                    if (tid < D) {
+                        p.delta[(size_t)g * D + tid] = vx[tid];
+                        if (c.delta_out) c.delta_out[(size_t)lh * D + tid] = vx[tid];
+                    }
+                    // Eq. 7: V_out = V_keep + delta on every retained row; the fp32 sum is rounded once.  Attn-inject
+                    // (App. D.2): row t takes k * A_t / (A_keep + eps) times delta instead
+                    constexpr int EPT = 16 / (int)sizeof(TIN);
+                    TIN *rows = reinterpret_cast<TIN *>(c.v_out) + (size_t)lh * k * D;
+                    const float share = (float)k / (a_keep + p.eps);
+                    for (int e0 = tid * EPT; e0 < k * D; e0 += ALG_NT * EPT) {
+                        const float wgt = p.attn_inject ? share * A[idx[e0 / D]] : 1.f;
+                        uint4 raw = *reinterpret_cast<const uint4 *>(rows + e0);
+                        const float *dl = vx + e0 % D;
+                        if constexpr (sizeof(TIN) == 4) {
+                            raw.x = __float_as_uint(fmaf(wgt, dl[0], __uint_as_float(raw.x)));
+                            raw.y = __float_as_uint(fmaf(wgt, dl[1], __uint_as_float(raw.y)));
+                            raw.z = __float_as_uint(fmaf(wgt, dl[2], __uint_as_float(raw.z)));
+                            raw.w = __float_as_uint(fmaf(wgt, dl[3], __uint_as_float(raw.w)));
+                        } else {
+                            uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) {
+                                const float lo = fmaf(wgt, dl[2 * q], __uint_as_float(w[q] << 16));
+                                const float hi2 = fmaf(wgt, dl[2 * q + 1], __uint_as_float(w[q] & 0xFFFF0000u));
+                                w[q] = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(lo)) |
+                                       ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(hi2)) << 16);
+                            }
+                            raw = make_uint4(w[0], w[1], w[2], w[3]);
+                        }
+                        *reinterpret_cast<uint4 *>(rows + e0) = raw;
+                    }
+                }
+            };
+            const float inv_del = 1.f / (a_del + p.eps);
+
+            // ---- 3a. few eigenpairs wanted: tridiagonal form, multisection, inverse iteration ----
+            if (!done && p.fast_iters == 0 && p.rank <= ALG_TRI_MAX_RANK) {
+                const float tiny2 = 1e-20f * trM * trM;
+                const int n = D - m;                                   // size of the trailing block
+                if (n > 1) {
+                    // reflector m + 1 from row m as it stands
+                    AlgRow<D> x;
+#pragma unroll
+                    for (int q = 0; q < NQ; ++q) {
+                        x[q] = M[0][q];
+#pragma unroll
+                        for (int r = 1; r < RW; ++r) x[q] = sel2(mask2(r == m / ALG_NG), M[r][q], x[q]);
+                    }
+                    alg_row_done<D, 0>(x, m, tiny2, Y, vdup + ((m + 1) & 3) * SH::DUP, ta, tb, grp, lane);
+                }
+                auto reduce_stage = [&](auto stage) __attribute__((always_inline)) {
+                    constexpr int ST = decltype(stage)::value;
+                    const int j1 = min(32 * ST + 31, D - 2);
+#pragma unroll 1
+                    for (int j = max(m + 1, 32 * ST); j <= j1; ++j) {
+                        const int pb = j & 1;
+                        AlgRow<D> v, x;
+                        __syncthreads();                               // reflector j is there
+                        alg_load<D, ST>(v, Y + j * D, c16);
+                        alg_product<D, ST>(M, v, pl + pb * D, pdup + pb * SH::DUP, vdup + (j & 3) * SH::DUP, kpart + pb * ALG_NG, grp, c16);
+                        {
+                            const float s = -2.f * half_sum(alg_dot<D, ST>(aux, v));
+#pragma unroll
+                            for (int q = ST; q < NQ; ++q) aux[q] = fma2(pk(s, s), v[q], aux[q]);
+                        }
+                        __syncthreads();                               // p is there
+                        alg_update<D, ST>(M, v, vdup + (j & 3) * SH::DUP, pl + pb * D, pdup + pb * SH::DUP, kpart + pb * ALG_NG,
+                                          grp, c16, (j / ALG_NG) & (SH::RPS - 1), x);
+                        alg_row_done<D, ST>(x, j, tiny2, Y, vdup + ((j + 1) & 3) * SH::DUP, ta, tb, grp, lane);
+                    }
+                };
+                reduce_stage(std::integral_constant<int, 0>{});
+                reduce_stage(std::integral_constant<int, 1>{});
+                if constexpr (D > 64) {
+                    reduce_stage(std::integral_constant<int, D / 32 - 2>{});
+                    reduce_stage(std::integral_constant<int, D / 32 - 1>{});
+                }
+                {
+                    // the last diagonal entry
+                    float a, b;
+                    upk(M[RW - 1][NQ - 1], a, b);
+                    if (grp == (D - 1) % ALG_NG && c16 == 15) ta[D - 1] = b;
+                }
+                if (grp == 0) {
+#pragma unroll
+                    for (int q = 0; q < NQ; ++q) *reinterpret_cast<f32x2 *>(vu + 32 * q + 2 * c16) = aux[q];
+                }
+                __syncthreads();
+                const int ne = min(min(p.rank, D) + 1, n);             // eigenvalues computed: the wanted ones and the next
+                const int rmax = min(min(p.rank, D), n);
+                const int n4 = (n + 3) / 4;
+                const float *da = ta + m, *db = tb + m;                // db[i] couples i and i + 1, i < n - 1
+                // bounds of the spectrum (Gershgorin); the recurrences run on the matrix scaled by their larger one
+                float gb = 0.f;
+                if (tid < n) gb = fabsf(da[tid]) + (tid > 0 ? fabsf(db[tid - 1]) : 0.f) + (tid < n - 1 ? fabsf(db[tid]) : 0.f);
+                const float bound = fmaxf(block_max<ALG_NT>(gb, red), 1e-30f), scl = 1.f / bound;
+                float *sa = WS, *sb2 = WS + D + 8, *vec = WS + 2 * (D + 8);   // vec: per wanted eigenvector dd, dl, du, du2, pv, y of D each
+                if (tid < 4 * n4) {
+                    sa[tid] = tid < n ? da[tid] * scl : 2.f;
+                    const float b = (tid > 0 && tid < n) ? db[tid - 1] * scl : 0.f;        // couples tid - 1 and tid
+                    sb2[tid] = (tid > 0 && tid < n) ? fmaxf(b * b, 1e-14f) : 0.f;
+                }
+                __syncthreads();
+                // eigenvalue e (largest first) by 65-way multisection, one warp each, two shifts per lane
+                for (int e = warp; e < ne; e += ALG_NW) {
+                    const int want = n - 1 - e;                        // it has exactly `want` eigenvalues below it
+                    float lo = -0.001f, hi = 1.001f;                   // (R^T R has no negative eigenvalues beyond rounding)
+#pragma unroll 1
+                    for (int round = 0; round < 4; ++round) {          // 65^-4 of the interval: 5.6e-8 of the largest eigenvalue's bound
+                        const float step = (hi - lo) * (1.f / 65.f);
+                        const float x0 = fmaf(step, (float)(2 * lane + 1), lo), x1 = fmaf(step, (float)(2 * lane + 2), lo);
+                        int c0, c1;
+                        sturm_count2(sa, sb2, n4, x0, x1, c0, c1);
+                        // shifts not above the eigenvalue: the counts are monotone in x
+                        const int nl = __popc(__ballot_sync(0xffffffffu, c0 <= want)) + __popc(__ballot_sync(0xffffffffu, c1 <= want));
+                        const float nlo = fmaf(step, (float)nl, lo), nhi = fmaf(step, (float)(nl + 1), lo);
+                        if (nl > 0) lo = nlo;
+                        if (nl < 64) hi = nhi;
+                    }
+                    if (lane == 0) tlam[e] = 0.5f * (lo + hi);         // in units of `bound`
+                }
+                __syncthreads();
+                const float l1 = tlam[0];
+                while (rho < rmax && tlam[rho] > EIG_RANK_TOL * l1 && tlam[rho] > 0.f) ++rho;
+                lam1 = l1 * bound;
+                lam_rho = rho > 0 ? tlam[rho - 1] * bound : 0.f;
+                lam_next = rho < ne ? fmaxf(tlam[rho] * bound, 0.f) : 0.f;
+                for (int t = 0; t < rho; ++t) revr += tlam[t];
+                revr *= bound / (trM + p.eps);                         // trace of R^T R = sum of all its eigenvalues
+                bool clustered = false;
+                for (int t = 1; t < rho; ++t) clustered = clustered || tlam[t - 1] - tlam[t] <= EIG_CLUSTER_TOL * fabsf(l1);
+                // Close neighbours: inverse iteration on the scaled T: factor T - lambda I once (LU with row interchanges), three solves; the operands of four steps are fetched together, ahead of the chain that needs them
+                constexpr float PERT = 4e-7f;
+                if (!clustered) {
+                    // Isolated eigenvalues: twisted factorisation.  Lane 0 eliminates from the top, lane 1 from the bottom, at
+                    // the same time; where the two meet with the smallest remainder gamma the eigenvector has its largest
+                    // entry, and its other entries follow outwards by multiplication alone (Fernando's method).  The residual
+                    // is gamma over the vector's length; should it exceed 2e-7 of the spectrum's bound the inverse iteration
+                    // below takes over.  Each lane's operands lie in the order it needs them, four to a load.
+                    constexpr float PIV = 1e-10f;
+                    if (tid == 0) misc[7] = 0.f;
+                    __syncthreads();
+                    for (int e = warp; e < rho; e += ALG_NW) {
+                        float *pa = vec + e * 6 * D, *pb = pa + D, *qa = pb + D, *qb = qa + D, *y = pa + 5 * D;
+                        const float lam = tlam[e];
+                        for (int i = lane; i < 4 * n4; i += 32) {
+                            const bool on = i < n - 1;
+                            const float bu = on ? db[i] * scl : 0.f, bd = on ? db[n - 2 - i] * scl : 0.f;
+                            pa[i] = i < n ? sa[i] - lam : 1.f;
+                            qa[i] = i < n ? sa[n - 1 - i] - lam : 1.f;
+                            pb[i] = bu * bu;
+                            qb[i] = bd * bd;
+                        }
+                        __syncwarp();
+                        if (lane < 2) {
+                            float *a = lane ? qa : pa;
+                            const float *b = lane ? qb : pb;
+                            float4 an = *reinterpret_cast<const float4 *>(a);
+                            float d = an.x;
+#pragma unroll 1
+                            for (int t = 0; t < n4; ++t) {
+                                const float4 ac = an, bc = *reinterpret_cast<const float4 *>(b + 4 * t);
+                                an = *reinterpret_cast<const float4 *>(a + 4 * t + 4);
+                                const float ax[4] = {ac.y, ac.z, ac.w, an.x}, bx[4] = {bc.x, bc.y, bc.z, bc.w};
+                                float o[4];
+#pragma unroll
+                                for (int q = 0; q < 4; ++q) {
+                                    d = copysignf(fmaxf(fabsf(d), PIV), d);
+                                    o[q] = d;
+                                    d = fmaf(-bx[q], rcp_approx(d), ax[q]);
+                                }
+                                *reinterpret_cast<float4 *>(a + 4 * t) = make_float4(o[0], o[1], o[2], o[3]);
+                            }
+                        }
+                        __syncwarp();
+                        float best = INFINITY;
+                        int at = 0;
+                        for (int i = lane; i < n; i += 32) {
+                            const float gm = fabsf(pa[i] + qa[n - 1 - i] - (sa[i] - lam));
+                            if (gm < best) { best = gm; at = i; }
+                        }
+#pragma unroll
+                        for (int o = 16; o > 0; o >>= 1) {
+                            const float ob = __shfl_xor_sync(0xffffffffu, best, o);
+                            const int oa = __shfl_xor_sync(0xffffffffu, at, o);
+                            if (ob < best || (ob == best && oa < at)) { best = ob; at = oa; }
+                        }
+                        // the multipliers along both arms, from the twist outwards
+                        for (int i = lane; i < 4 * n4; i += 32) {
+                            const int u = at - 1 - i, w = at + 1 + i;
+                            pb[i] = u >= 0 ? -db[u] * scl * rcp_approx(pa[u]) : 0.f;
+                            qb[i] = w < n ? -db[w - 1] * scl * rcp_approx(qa[n - 1 - w]) : 0.f;
+                        }
+                        __syncwarp();
+                        if (lane < 2) {
+                            float *mu = lane ? qb : pb;
+                            float x = 1.f;
+#pragma unroll 1
+                            for (int t = (lane ? n - 1 - at : at); t > 0; t -= 4, mu += 4) {
+                                const float4 mv = *reinterpret_cast<const float4 *>(mu);
+                                float4 o;
+                                o.x = mv.x * x; o.y = mv.y * o.x; o.z = mv.z * o.y; x = o.w = mv.w * o.z;
+                                *reinterpret_cast<float4 *>(mu) = o;
+                            }
+                        }
+                        __syncwarp();
+                        float n2 = 0.f;
+                        for (int i = lane; i < n; i += 32) {
+                            const float t = i == at ? 1.f : i < at ? pb[at - 1 - i] : qb[i - at - 1];
+                            y[i] = t;
+                            n2 = fmaf(t, t, n2);
+                        }
+                        n2 = warp_sum(n2);
+                        const float inv = rsqrtf(n2);
+                        for (int i = lane; i < n; i += 32) y[i] *= inv;
+                        if (lane == 0 && !(best * inv <= 2e-7f)) misc[7] = 1.f;
+                    }
+                    __syncthreads();
+                    clustered = misc[7] != 0.f;
+                }
+                for (int e = warp; clustered && e < rho; e += ALG_NW) {
+                    float *dd = vec + e * 6 * D, *dl = dd + D, *du = dl + D, *du2 = du + D, *pv = du2 + D, *y = pv + D;
+                    const float lam = tlam[e];
+                    for (int i = lane; i < 4 * n4; i += 32) {
+                        dd[i] = i < n ? sa[i] - lam : 1.f;
+                        du[i] = i < n - 1 ? db[i] * scl : 0.f;         // entry (i, i + 1), and (i + 1, i)
+                        // a start vector without structure
+                        const uint32_t hsh = ((uint32_t)i * 2654435761u + (uint32_t)e * 40503u + 12345u) >> 8;
+                        y[i] = i < n ? (float)(hsh & 0xFFFFu) * (1.f / 65536.f) - 0.5f : 0.f;
+                    }
+                    __syncwarp();
+                    if (lane == 0) {
+                        // the running pivot (di) and the entry right of it (ui)
+                        float di = dd[0], ui = du[0];
+                        float4 dn4 = *reinterpret_cast<const float4 *>(dd), un4 = *reinterpret_cast<const float4 *>(du);
+#pragma unroll 1
+                        for (int q = 0; q < n4; ++q) {
+                            const float4 dc = dn4, uc = un4;
+                            if (q + 1 < n4) {
+                                dn4 = *reinterpret_cast<const float4 *>(dd + 4 * q + 4);
+                                un4 = *reinterpret_cast<const float4 *>(du + 4 * q + 4);
+                            }
+                            const float li_[4] = {uc.x, uc.y, uc.z, uc.w};
+                            const float dx[4] = {dc.y, dc.z, dc.w, dn4.x}, ux[4] = {uc.y, uc.z, uc.w, un4.x};
+                            float o_d[4], o_l[4], o_u[4], o_u2[4], o_p[4];
+#pragma unroll
+                            for (int t = 0; t < 4; ++t) {
+                                const int i = 4 * q + t;
+                                const float li = i < n - 1 ? li_[t] : 0.f;
+                                const float dn = i < n - 1 ? dx[t] : 1.f, un = i < n - 2 ? ux[t] : 0.f;
+                                const bool keep = fabsf(di) >= fabsf(li);
+                                float den = keep ? di : li;
+                                if (fabsf(den) < PERT) den = den < 0.f ? -PERT : PERT;
+                                const float num = keep ? li : di;
+                                const float rc = rcp_approx(den), f = num * rc;
+                                o_d[t] = rc;                           // the solves multiply by the pivots' reciprocals
+                                o_l[t] = f;
+                                o_p[t] = keep ? 0.f : 1.f;
+                                o_u[t] = keep ? ui : dn;
+                                o_u2[t] = keep ? 0.f : un;
+                                const float nd = keep ? fmaf(-f, ui, dn) : fmaf(-f, dn, ui);
+                                ui = keep ? un : -f * un;
+                                di = nd;
+                            }
+                            *reinterpret_cast<float4 *>(dd + 4 * q) = make_float4(o_d[0], o_d[1], o_d[2], o_d[3]);
+                            *reinterpret_cast<float4 *>(dl + 4 * q) = make_float4(o_l[0], o_l[1], o_l[2], o_l[3]);
+                            *reinterpret_cast<float4 *>(du + 4 * q) = make_float4(o_u[0], o_u[1], o_u[2], o_u[3]);
+                            *reinterpret_cast<float4 *>(du2 + 4 * q) = make_float4(o_u2[0], o_u2[1], o_u2[2], o_u2[3]);
+                            *reinterpret_cast<float4 *>(pv + 4 * q) = make_float4(o_p[0], o_p[1], o_p[2], o_p[3]);
+                        }
+                    }
+                    __syncwarp();
+                }
+#pragma unroll 1
+                for (int itn = 0; itn < (clustered ? 3 : 0); ++itn) {
+                    for (int e = warp; e < rho; e += ALG_NW) {
+                        float *dd = vec + e * 6 * D, *dl = dd + D, *du = dl + D, *du2 = du + D, *pv = du2 + D, *y = pv + D;
+                        if (lane == 0) {
+                            float yi = y[0];
+                            float4 yn4 = *reinterpret_cast<const float4 *>(y), ln4 = *reinterpret_cast<const float4 *>(dl);
+                            float4 pn4 = *reinterpret_cast<const float4 *>(pv);
+#pragma unroll 1
+                            for (int q = 0; q < n4; ++q) {
+                                const float4 yc = yn4, lc = ln4, pc4 = pn4;
+                                if (q + 1 < n4) {
+                                    yn4 = *reinterpret_cast<const float4 *>(y + 4 * q + 4);
+                                    ln4 = *reinterpret_cast<const float4 *>(dl + 4 * q + 4);
+                                    pn4 = *reinterpret_cast<const float4 *>(pv + 4 * q + 4);
+                                } else {
+                                    yn4.x = 0.f;
+                                }
+                                const float yx[4] = {yc.y, yc.z, yc.w, yn4.x}, ll[4] = {lc.x, lc.y, lc.z, lc.w}, pp[4] = {pc4.x, pc4.y, pc4.z, pc4.w};
+                                float o[4];
+#pragma unroll
+                                for (int t = 0; t < 4; ++t) {
+                                    const float a0 = fmaf(-ll[t], yi, yx[t]), b0 = fmaf(-ll[t], yx[t], yi);
+                                    o[t] = pp[t] == 0.f ? yi : yx[t];
+                                    yi = pp[t] == 0.f ? a0 : b0;
+                                }
+                                *reinterpret_cast<float4 *>(y + 4 * q) = make_float4(o[0], o[1], o[2], o[3]);
+                            }
+                            float y0 = 0.f, y1 = 0.f;                  // y[i + 1], y[i + 2]
+                            float4 yb = *reinterpret_cast<const float4 *>(y + 4 * n4 - 4), db4 = *reinterpret_cast<const float4 *>(dd + 4 * n4 - 4);
+                            float4 ub = *reinterpret_cast<const float4 *>(du + 4 * n4 - 4), vb = *reinterpret_cast<const float4 *>(du2 + 4 * n4 - 4);
+#pragma unroll 1
+                            for (int q = n4 - 1; q >= 0; --q) {
+                                const float yy[4] = {yb.x, yb.y, yb.z, yb.w}, iv[4] = {db4.x, db4.y, db4.z, db4.w};
+                                const float uu[4] = {ub.x, ub.y, ub.z, ub.w}, u2[4] = {vb.x, vb.y, vb.z, vb.w};
+                                if (q > 0) {
+                                    yb = *reinterpret_cast<const float4 *>(y + 4 * q - 4);
+                                    db4 = *reinterpret_cast<const float4 *>(dd + 4 * q - 4);
+                                    ub = *reinterpret_cast<const float4 *>(du + 4 * q - 4);
+                                    vb = *reinterpret_cast<const float4 *>(du2 + 4 * q - 4);
+                                }
+                                float o[4];
+#pragma unroll
+                                for (int t = 3; t >= 0; --t) {
+                                    const float s = fmaf(-uu[t], y0, fmaf(-u2[t], y1, yy[t])) * iv[t];
+                                    o[t] = s;
+                                    y1 = y0;
+                                    y0 = s;
+                                }
+                                *reinterpret_cast<float4 *>(y + 4 * q) = make_float4(o[0], o[1], o[2], o[3]);
+                            }
+                        }
+                        __syncwarp();
+                        // scaled to largest entry 1, then to unit length, by the whole warp (padding entries are zero)
+                        float mx = 0.f;
+                        for (int i = lane; i < n; i += 32) mx = fmaxf(mx, fabsf(y[i]));
+                        mx = warp_max(mx);
+                        const float sc1 = mx > 0.f ? 1.f / mx : 1.f;
+                        float n2 = 0.f;
+                        for (int i = lane; i < n; i += 32) { const float t = y[i] * sc1; n2 = fmaf(t, t, n2); }
+                        n2 = warp_sum(n2);
+                        const float inv = n2 > 0.f ? rsqrtf(n2) * sc1 : 0.f;
+                        for (int i = lane; i < 4 * n4; i += 32) y[i] = i < n ? y[i] * inv : 0.f;
+                        __syncwarp();
+                    }
+                    if (clustered) {
+                        __syncthreads();
+                        if (warp == 0) {
+                            // in order of the eigenvalues: orthogonal to the close neighbours before it, unit length
+                            for (int j = 1; j < rho; ++j) {
+                                float *y = vec + (j * 6 + 5) * D;
+                                for (int i2 = 0; i2 < j; ++i2) {
+                                    if (fabsf(tlam[i2] - tlam[j]) > EIG_CLUSTER_TOL * fabsf(l1)) continue;
+                                    const float *z = vec + (i2 * 6 + 5) * D;
+                                    float dsum = 0.f;
+                                    for (int cc = lane; cc < n; cc += 32) dsum = fmaf(y[cc], z[cc], dsum);
+                                    dsum = warp_sum(dsum);
+                                    for (int cc = lane; cc < n; cc += 32) y[cc] -= dsum * z[cc];
+                                    __syncwarp();
+                                }
+                                float n2 = 0.f;
+                                for (int cc = lane; cc < n; cc += 32) n2 = fmaf(y[cc], y[cc], n2);
+                                n2 = warp_sum(n2);
+                                const float inv = n2 > 0.f ? rsqrtf(n2) : 0.f;
+                                for (int cc = lane; cc < n; cc += 32) y[cc] *= inv;
                                 __syncwarp();
                             }
-                        float n1 = 0.f;
-                        for (int cc = lane; cc < D; cc += 32) n1 = fmaf(y[cc], y[cc], n1);
-                        n1 = warp_sum(n1);
-                        if (n1 > 1e-10f * n0 && n1 > 0.f) {
-                            const float inv = rsqrtf(n1);
-                            for (int cc = lane; cc < D; cc += 32) C[kept * LD + cc] = y[cc] * inv;
-                            ++kept;
                         }
-                        __syncwarp();
+                        __syncthreads();
                     }
-                    if (lane == 0) misc[6] = (float)kept;
+                }
+                // r_bar's products with the eigenvectors, in the coordinates of the tridiagonal form
+                for (int e = warp; e < rho; e += ALG_NW) {
+                    const float *y = vec + (e * 6 + 5) * D;
+                    float s = 0.f;
+                    for (int i = lane; i < n; i += 32) s = fmaf(y[i], vu[m + i], s);
+                    s = warp_sum(s);
+                    if (lane == 0) vc[e] = s * inv_del;
                 }
                 __syncthreads();
-                rho_f = (int)misc[6];
+                if (tid < D) {
+                    float s = 0.f;
+                    if (tid >= m)
+                        for (int t = 0; t < rho; ++t) s = fmaf(vc[t], vec[(t * 6 + 5) * D + tid - m], s);
+                    vx[tid] = s;
+                }
+                finish_delta(D - 2);
+                done = true;
             }
-            rho = rho_f;
-            // Rayleigh quotients of the rows (for the diagnostics), then Delta and delta
-            if (warp < 16) {
-                for (int i = warp; i < rho; i += 16) {
-                    float rq = 0.f;
+
+            // r_bar in the rotated coordinates, for the other two routes
+            if (!done) {
+                if (grp == 0) {
+#pragma unroll
+                    for (int q = 0; q < NQ; ++q) {
+                        const int cc = 32 * q + 2 * c16;
+                        float a, b;
+                        upk(aux[q], a, b);
+                        vu[cc] = cc >= m ? a * inv_del : 0.f;
+                        vu[cc + 1] = cc + 1 >= m ? b * inv_del : 0.f;
+                    }
+                }
+                __syncthreads();
+            }
+
+            // ---- 3f. fast path of App. H: C <- orth(C M), a fixed number of times, from the first rows of the identity ----
+            if (!done && p.fast_iters > 0) {
+                int rho_f = min(min(p.rank, D), D - m);               // rank(R) <= d - m
+                float *C = WS, *Yb = WS + min(p.rank, D) * D;         // row blocks; entries below m stay zero in C
+                // the rows of the identity in the rotated coordinates: e_i H_0 .. H_{m-1} (what lies below m meets only zeros of M)
+#pragma unroll 1
+                for (int i0 = 0; i0 < rho_f; i0 += ALG_NG) {
+                    const int i = i0 + grp;
+                    AlgRow<D> x, v;
+#pragma unroll
+                    for (int q = 0; q < NQ; ++q) x[q] = pk(32 * q + 2 * c16 == i ? 1.f : 0.f, 32 * q + 2 * c16 + 1 == i ? 1.f : 0.f);
+#pragma unroll 1
+                    for (int j = 0; j < m; ++j) { alg_load<D>(v, Y + j * D, c16); reflect(x, v); }
+#pragma unroll
+                    for (int q = 0; q < NQ; ++q) {
+                        const int cc = 32 * q + 2 * c16;
+                        float a, b;
+                        upk(x[q], a, b);
+                        if (i < rho_f) *reinterpret_cast<f32x2 *>(C + i * D + cc) = pk(cc >= m ? a : 0.f, cc + 1 >= m ? b : 0.f);
+                    }
+                }
+                // Y = 2 C M from the registers (the factor drops out of the directions)
+                auto times_m = [&](int rows) __attribute__((always_inline)) {
+                    __syncthreads();
+#pragma unroll 1
+                    for (int i = 0; i < rows; ++i) {
+                        AlgRow<D> v;
+                        alg_load<D>(v, C + i * D, c16);
+                        auto one = [&](auto stage) __attribute__((always_inline)) {
+                            alg_product<D, decltype(stage)::value>(M, v, Yb + i * D, nullptr, nullptr, nullptr, grp, c16);
+                        };
+                        if (D > 64 && m >= 96) one(std::integral_constant<int, D / 32 - 1>{});
+                        else if (D > 64 && m >= 64) one(std::integral_constant<int, D / 32 - 2>{});
+                        else if (m >= 32) one(std::integral_constant<int, 1>{});
+                        else one(std::integral_constant<int, 0>{});
+                    }
+                    __syncthreads();
+                };
+#pragma unroll 1
+                for (int itn = 0; itn < p.fast_iters; ++itn) {
+                    times_m(rho_f);
+                    // orth: Gram-Schmidt over the rows in order, twice; a row with nothing left is dropped (warp 0)
+                    if (warp == 0) {
+                        int kept = 0;
+                        for (int i = 0; i < rho_f; ++i) {
+                            // a lane's entries: lane, lane + 32, ..
+                            float y[NQ], n0 = 0.f, n1 = 0.f;
+#pragma unroll
+                            for (int q = 0; q < NQ; ++q) { y[q] = 32 * q + lane >= m ? Yb[i * D + 32 * q + lane] : 0.f; n0 = fmaf(y[q], y[q], n0); }
+                            n0 = warp_sum(n0);
+                            for (int pass = 0; pass < 2; ++pass)
+                                for (int j = 0; j < kept; ++j) {
+                                    float dsum = 0.f;
+#pragma unroll
+                                    for (int q = 0; q < NQ; ++q) dsum = fmaf(y[q], C[j * D + 32 * q + lane], dsum);
+                                    dsum = warp_sum(dsum);
+#pragma unroll
+                                    for (int q = 0; q < NQ; ++q) y[q] = fmaf(-dsum, C[j * D + 32 * q + lane], y[q]);
+                                }
+#pragma unroll
+                            for (int q = 0; q < NQ; ++q) n1 = fmaf(y[q], y[q], n1);
+                            n1 = warp_sum(n1);
+                            if (n1 > 1e-10f * n0 && n1 > 0.f) {
+                                const float inv = rsqrtf(n1);
+#pragma unroll
+                                for (int q = 0; q < NQ; ++q) C[kept * D + 32 * q + lane] = y[q] * inv;
+                                ++kept;
+                            }
+                        }
+                        if (lane == 0) misc[6] = (float)kept;
+                    }
+                    __syncthreads();
+                    rho_f = (int)misc[6];
+                }
+                rho = rho_f;
+                // Rayleigh quotients of the rows (for the diagnostics), then Delta and delta
+                if (c.diag) times_m(rho);
+                for (int i = warp; i < rho; i += ALG_NW) {
+                    float rq = 0.f, cu = 0.f;
                     for (int a = lane; a < D; a += 32) {
-                        float sacc = 0.f;
-                        for (int b = 0; b < D; ++b) sacc = fmaf(B2[a * LD + b], C[i * LD + b], sacc);
-                        rq = fmaf(C[i * LD + a], sacc, rq);
+                        if (c.diag && a >= m) rq = fmaf(C[i * D + a], 0.5f * Yb[i * D + a], rq);
+                        cu = fmaf(C[i * D + a], vu[a], cu);
                     }
                     rq = warp_sum(rq);
-                    if (lane == 0) vl[i] = rq;
+                    cu = warp_sum(cu);
+                    if (lane == 0) { vl[i] = rq; vc[i] = cu; }
                 }
+                __syncthreads();
+                for (int t = 0; t < rho; ++t) revr += vl[t];
+                revr /= trM + p.eps;
+                lam1 = rho > 0 ? vl[0] : 0.f; lam_rho = rho > 0 ? vl[rho - 1] : 0.f; lam_next = 0.f;
+                if (tid < D) {
+                    float sacc = 0.f;
+                    for (int t = 0; t < rho; ++t) sacc = fmaf(vc[t], C[t * D + tid], sacc);
+                    vx[tid] = sacc;
+                }
+                finish_delta(0);
+                done = true;
             }
-            if (tid < rho) {
-                float sacc = 0.f;
-                for (int cc = 0; cc < D; ++cc) sacc = fmaf(C[tid * LD + cc], vu[cc], sacc);
-                vc[tid] = sacc;
-            }
-            __syncthreads();
-            for (int t = 0; t < rho; ++t) revr += vl[t];
-            revr /= trM + p.eps;
-            lam1 = rho > 0 ? vl[0] : 0.f; lam_rho = rho > 0 ? vl[rho - 1] : 0.f; lam_next = 0.f;
-            float dl = 0.f;
-            if (tid < D) {
-                float sacc = 0.f;
-                for (int t = 0; t < rho; ++t) sacc = fmaf(vc[t], C[t * LD + tid], sacc);
-                dl = alpha * sacc;
-            }
-            __syncthreads();                                        // vc is scratch of the projection that follows
-            finish_delta(dl);
-            done = true;
-        }
 
-        // ---- 4a. few eigenpairs wanted: tridiagonal form, bisection, inverse iteration ----
-        if (!done && p.rank <= ALG_TRI_MAX_RANK) {
-            const int lane = tid & 31, warp = tid >> 5;
-            const int ne = min(min(p.rank, D) + 1, D);             // eigenpairs computed: the wanted ones and the next
-            float *ta = WS, *tb = WS + D;                          // diagonal, off-diagonal (tb[i] couples i and i + 1)
-            float *tlam = tb + D;                                  // ne <= ALG_TRI_NE eigenvalues, largest first (16 floats)
-            float *tz = tlam + 16;                                 // [ne][D] eigenvectors
-            float *twk = tz + ne * D;                              // [ne][5][D] factors of T - lambda I
-            // Householder reduction: reflector k (a unit vector) zeroes column k below the sub-diagonal.  During its step it
-            // sits in one of two vectors (vl, vcs); afterwards in the part of column k of M that the step has emptied
-            // (rows k + 1 .. d - 1).
-            //
-            // Two block barriers per column.  Step k:
-            //   B  p = 2 M v_k on the trailing block (rows and columns > k), four threads per row;
-            //   C  kk = v_k . p and w = p - kk v_k (every warp for itself), then
-            //      - row k + 1 as the update M - v w^T - w v^T leaves it, formed by every warp for itself from the old row:
-            //        its first entry is the next diagonal entry, the rest gives reflector k + 1 (norm, sign) at once, so
-            //        no barrier stands between the update and the next reflector;
-            //      - the update itself on rows and columns > k + 1 (row and column k + 1 are dead from here on; column
-            //        k + 1 takes its reflector a step later);
-            //      - reflector k into column k.
-            // The loop starts at k = -1 with v = 0: that step only forms reflector 0 from row 0.
-            const float tiny2 = 1e-20f * trM * trM;
-            constexpr int RPW = (D + ALG_NT / 32 - 2) / (ALG_NT / 32 - 1);   // rows a warp of the update handles
-            constexpr int CPL = (D + 31) / 32;                           // columns per lane
-            if (tid < D) { vl[tid] = 0.f; vcs[tid] = 0.f; vc[tid] = 0.f; }
-            __syncthreads();
-#pragma unroll 1
-            for (int k = -1; k < D - 2; ++k) {
-                const float *v = (k & 1) ? vl : vcs;                // v_k; v_{k+1} goes to the other vector
-                float *vnext = (k & 1) ? vcs : vl;
-                if (k >= 0) {                                       // B: p = 2 M v on the trailing block -> vc
-                    const int j = tid >> 2, part = tid & 3;
-                    const bool on = j > k && j < D;
-                    float s0 = 0.f, s1 = 0.f;
-                    if (on) {
-                        const float *row = B2 + j * LD;
-                        // columns from the 32-column group of k + 1 on (v is zero up to k); the four threads of a row
-                        // take eight columns of a group each, which keeps the lanes of a warp on different banks
-#pragma unroll 1
-                        for (int g32 = (k + 1) >> 5; g32 < D / 32; ++g32) {
-                            const float *rw = row + (g32 << 5) + part * 8, *vv = v + (g32 << 5) + part * 8;
+            // The last route works on the trailing block in shared memory (zero outside rows and columns >= m)
+            float *B2 = WS;
+            if (!done) {
 #pragma unroll
-                            for (int i = 0; i < 8; i += 2) {
-                                s0 = fmaf(rw[i], vv[i], s0);
-                                s1 = fmaf(rw[i + 1], vv[i + 1], s1);
+                for (int r = 0; r < RW; ++r)
+#pragma unroll
+                    for (int q = 0; q < NQ; ++q) {
+                        const int i = grp + ALG_NG * r, cc = 32 * q + 2 * c16;
+                        float a, b;
+                        upk(M[r][q], a, b);
+                        B2[i * LD + cc] = (i >= m && cc >= m) ? a : 0.f;
+                        B2[i * LD + cc + 1] = (i >= m && cc + 1 >= m) ? b : 0.f;
+                    }
+                __syncthreads();
+                for (int e = tid; e < D * D; e += ALG_NT) {            // symmetrise
+                    const int a = e / D, bb = e % D;
+                    if (a < bb) {
+                        const float sy = 0.5f * (B2[a * LD + bb] + B2[bb * LD + a]);
+                        B2[a * LD + bb] = sy;
+                        B2[bb * LD + a] = sy;
+                    }
+                }
+                __syncthreads();
+            }
+
+            // ---- 3b. Jacobi eigen-decomposition of the block (B2), eigenvectors in U -----
+            if (!done) {
+                float *vcs = vx;                                        // (c, s) of d / 2 pairs
+                float *U = B2 + D * LD;                                 // d x d, starts as the identity
+                for (int e = tid; e < D * D; e += ALG_NT) U[(e / D) * LD + (e % D)] = (e / D == e % D) ? 1.f : 0.f;
+                __syncthreads();
+                // rotations below the fp32 noise level of the largest eigenvalue never settle: stop there
+                const float floor_abs = 2e-7f * block_max<ALG_NT>(tid < D ? B2[tid * LD + tid] : 0.f, red);
+                bool converged = false;
+#pragma unroll 1
+                for (int sweep = 0; sweep < JACOBI_MAX_SWEEPS && !converged; ++sweep) {
+                    if (tid == 0) misc[0] = 0.f;
+                    __syncthreads();
+#pragma unroll 1
+                    for (int r = 0; r < D - 1; ++r) {
+                        if (tid < D / 2) {
+                            int pp, qq;
+                            if (tid == 0) { pp = D - 1; qq = r; }
+                            else { pp = (r + tid) % (D - 1); qq = (r - tid + (D - 1)) % (D - 1); }
+                            if (pp > qq) { const int t = pp; pp = qq; qq = t; }
+                            const float app = B2[pp * LD + pp], aqq = B2[qq * LD + qq], apq = B2[pp * LD + qq];
+                            float cs = 1.f, sn = 0.f;
+                            if (fabsf(apq) > 1e-7f * sqrtf(fabsf(app * aqq)) + floor_abs) {
+                                const float theta = (aqq - app) / (2.f * apq);
+                                const float t = (theta >= 0.f ? 1.f : -1.f) / (fabsf(theta) + sqrtf(theta * theta + 1.f));
+                                cs = rsqrtf(t * t + 1.f);
+                                sn = t * cs;
+                                misc[0] = 1.f;
+                            }
+                            vcs[2 * tid] = cs; vcs[2 * tid + 1] = sn;
+                            ipq[2 * tid] = pp; ipq[2 * tid + 1] = qq;
+                        }
+                        __syncthreads();
+                        for (int e = tid; e < D * (D / 2); e += ALG_NT) {      // columns of M and U
+                            const int i = e / (D / 2), t = e % (D / 2);
+                            const float cs = vcs[2 * t], sn = vcs[2 * t + 1];
+                            if (sn != 0.f) {
+                                const int pp = ipq[2 * t], qq = ipq[2 * t + 1];
+                                const float mp = B2[i * LD + pp], mq = B2[i * LD + qq];
+                                B2[i * LD + pp] = cs * mp - sn * mq;
+                                B2[i * LD + qq] = sn * mp + cs * mq;
+                                const float up = U[i * LD + pp], uq = U[i * LD + qq];
+                                U[i * LD + pp] = cs * up - sn * uq;
+                                U[i * LD + qq] = sn * up + cs * uq;
                             }
                         }
-                    }
-                    float sacc = s0 + s1;
-                    sacc += __shfl_xor_sync(0xffffffffu, sacc, 1);
-                    sacc += __shfl_xor_sync(0xffffffffu, sacc, 2);
-                    if (on && part == 0) vc[j] = 2.f * sacc;
-                    __syncthreads();
-                }
-                // C
-                float kpart = 0.f;
-                for (int cc = k + 1 + lane; cc < D; cc += 32) kpart = fmaf(v[cc], vc[cc], kpart);
-                const float kk = warp_sum(kpart);                   // v . p, the same sum in every warp
-                // groups of 32 columns the trailing block has (the same in every thread: whole groups are skipped)
-                const int nc = (D - (k + 1) + 31) >> 5;
-                float vj[CPL], wj[CPL];
-#pragma unroll
-                for (int cI = 0; cI < CPL; ++cI) {
-                    vj[cI] = 0.f;
-                    wj[cI] = 0.f;
-                    if (cI < nc) {
-                        const int j = k + 1 + lane + 32 * cI;
-                        vj[cI] = j < D ? v[j] : 0.f;
-                        wj[cI] = j < D ? vc[j] - kk * vj[cI] : 0.f;
-                    }
-                }
-                if (warp == 0) {
-                    // warp 0 forms reflector k + 1; the other warps share the update
-                    float xj[CPL];
-                    const float vr = v[k + 1], wr = vc[k + 1] - kk * vr;     // entries k + 1 of v and w
-                    float part2 = 0.f;
-#pragma unroll
-                    for (int cI = 0; cI < CPL; ++cI) {
-                        xj[cI] = 0.f;
-                        if (cI < nc) {
-                            const int j = k + 1 + lane + 32 * cI;
-                            // row k + 1 after the update (the same expression as the update below)
-                            xj[cI] = j < D ? B2[(k + 1) * LD + j] - (vr * wj[cI] + wr * vj[cI]) : 0.f;
-                            if (j >= k + 3) part2 = fmaf(xj[cI], xj[cI], part2);
-                        }
-                    }
-                    const float below2 = warp_sum(part2);              // squares right of the super-diagonal entry
-                    const float dg = __shfl_sync(0xffffffffu, xj[0], 0);    // entry (k + 1, k + 1)
-                    const float x0 = __shfl_sync(0xffffffffu, xj[0], 1);    // entry (k + 1, k + 2)
-                    const float nrm2 = below2 + x0 * x0;
-                    const float nrm = sqrtf(nrm2);
-                    const float al = x0 >= 0.f ? -nrm : nrm;
-                    const float vn2 = 2.f * nrm * (nrm + fabsf(x0));   // |x - al e_0|^2
-                    const bool skip = !(below2 > tiny2) || !(vn2 > 0.f);   // nothing beyond the super-diagonal
-                    const float rs = skip ? 0.f : rsqrtf(vn2);
-#pragma unroll
-                    for (int cI = 0; cI < CPL; ++cI) {
-                        const int j = k + 1 + lane + 32 * cI;
-                        if (cI < nc && j < D) vnext[j] = j == k + 1 ? 0.f : (j == k + 2 ? x0 - al : xj[cI]) * rs;
-                    }
-                    if (lane == 0) {
-                        if (k >= 0) vnext[k] = 0.f;
-                        ta[k + 1] = dg;
-                        tb[k + 1] = skip ? x0 : al;
-                    }
-                }
-                if (k >= 0 && warp > 0) {
-                    // M <- H M H = M - v w^T - w v^T on rows and columns > k + 1; a warp's rows are read before the first
-                    // is written back (the compiler cannot tell that they do not overlap), RB at a time
-                    // RB = 1 measured fastest (0.60 ms on the paper's regime; 2: 0.63, 3: 0.66, 4: 0.68): registers, not
-                    // the stores, are what the loop is short of
-                    constexpr int RB = 1;
-#pragma unroll
-                    for (int r0 = 0; r0 < RPW; r0 += RB) {
-                        // (the same in every lane of the warp: rows and column groups outside the block cost nothing)
-                        if (k + 2 + (warp - 1) + r0 * (ALG_NT / 32 - 1) < D) {
-                            float m_[RB][CPL], vi[RB], wi[RB];
-#pragma unroll
-                            for (int r = 0; r < RB; ++r) {
-                                const int i = k + 2 + (warp - 1) + (r0 + r) * (ALG_NT / 32 - 1);
-                                const bool on = r0 + r < RPW && i < D;
-                                vi[r] = on ? v[i] : 0.f;
-                                wi[r] = on ? vc[i] - kk * vi[r] : 0.f;
-#pragma unroll
-                                for (int cI = 0; cI < CPL; ++cI) {
-                                    m_[r][cI] = 0.f;
-                                    if (cI < nc) {
-                                        const int j = k + 1 + lane + 32 * cI;
-                                        m_[r][cI] = (on && j < D) ? B2[i * LD + j] : 0.f;
-                                    }
-                                }
-                            }
-#pragma unroll
-                            for (int r = 0; r < RB; ++r) {
-                                const int i = k + 2 + (warp - 1) + (r0 + r) * (ALG_NT / 32 - 1);
-                                const bool on = r0 + r < RPW && i < D;
-#pragma unroll
-                                for (int cI = 0; cI < CPL; ++cI) {
-                                    if (cI < nc) {
-                                        const int j = k + 1 + lane + 32 * cI;
-                                        if (on && j > k + 1 && j < D) B2[i * LD + j] = m_[r][cI] - (vi[r] * wj[cI] + wi[r] * vj[cI]);
-                                    }
-                                }
+                        __syncthreads();
+                        for (int e = tid; e < D * (D / 2); e += ALG_NT) {      // rows of M
+                            const int t = e / D, j = e % D;
+                            const float cs = vcs[2 * t], sn = vcs[2 * t + 1];
+                            if (sn != 0.f) {
+                                const int pp = ipq[2 * t], qq = ipq[2 * t + 1];
+                                const float mp = B2[pp * LD + j], mq = B2[qq * LD + j];
+                                B2[pp * LD + j] = cs * mp - sn * mq;
+                                B2[qq * LD + j] = sn * mp + cs * mq;
                             }
                         }
+                        __syncthreads();
                     }
+                    converged = (misc[0] == 0.f);
+                    __syncthreads();
                 }
-                // reflector k into the column it has emptied
-                if (k >= 0 && tid > k && tid < D) B2[tid * LD + k] = v[tid];
-                __syncthreads();
-            }
-            if (tid == 0) { ta[D - 1] = B2[(D - 1) * LD + D - 1]; tb[D - 1] = 0.f; }
-            __syncthreads();
-            // bounds of the spectrum (Gershgorin) and the pivot floor of the Sturm counts
-            float gl = INFINITY, gh = -INFINITY, b2 = 0.f;
-            if (tid < D) {
-                const float r = (tid > 0 ? fabsf(tb[tid - 1]) : 0.f) + fabsf(tb[tid]);
-                gl = ta[tid] - r; gh = ta[tid] + r; b2 = tb[tid] * tb[tid];
-            }
-            const float g_hi = block_max<ALG_NT>(gh, red), g_lo = -block_max<ALG_NT>(-gl, red);
-            const float pivmin = 1e-30f * fmaxf(1.f, block_max<ALG_NT>(b2, red));
-            const float span = fmaxf(g_hi - g_lo, 1e-30f);
-            // eigenvalue j (largest first) by 32-way multisection, one warp per eigenvalue
-            if (warp < ne) {
-                const int want = D - 1 - warp;                      // it has exactly `want` eigenvalues below it
-                float lo = g_lo - 1e-3f * span, hi = g_hi + 1e-3f * span;
-#pragma unroll 1
-                for (int round = 0; round < 6; ++round) {                // 33^-6 of the spectrum's width: below fp32 resolution
-                    const float x = lo + (hi - lo) * (float)(lane + 1) * (1.f / 33.f);
-                    const bool below = sturm_count<D>(ta, tb, x, pivmin) <= want;     // x is not above the eigenvalue
-                    const int nl = __popc(__ballot_sync(0xffffffffu, below));        // counts are monotone in x
-                    const float x_lo = __shfl_sync(0xffffffffu, x, max(nl - 1, 0));
-                    const float x_hi = __shfl_sync(0xffffffffu, x, min(nl, 31));
-                    if (nl > 0) lo = x_lo;
-                    if (nl < 32) hi = x_hi;
-                }
-                if (lane == 0) tlam[warp] = 0.5f * (lo + hi);
-            }
-            __syncthreads();
-            const float l1 = tlam[0];
-            // inverse iteration on T: factor T - lambda_j I once (LU with row interchanges), three solves
-            if (warp < ne) {
-                const float lam = tlam[warp];
-                float *dd = twk + (warp * 5) * D, *dl = dd + D, *du = dl + D, *du2 = du + D, *pv = du2 + D;
-                const float pert = 4e-7f * fmaxf(fabsf(g_hi), fabsf(g_lo)) + 1e-30f;
-                for (int i = lane; i < D; i += 32) { dd[i] = ta[i] - lam; dl[i] = tb[i]; du[i] = tb[i]; du2[i] = 0.f; }
-                __syncwarp();
-                if (lane == 0) {
-                    // the running pivot and the entry above the next one travel in registers: a step of the chain is a
-                    // reciprocal and two multiply-adds, not a round trip through shared memory
-                    float di = dd[0], ui = du[0];
-                    for (int i = 0; i < D - 1; ++i) {
-                        const float li = dl[i];
-                        float dn = dd[i + 1], un = i < D - 2 ? du[i + 1] : 0.f;
-                        if (fabsf(di) >= fabsf(li)) {
-                            if (di == 0.f) di = pert;
-                            const float f = __fdividef(li, di);
-                            dd[i] = di; dl[i] = f; pv[i] = 0.f;
-                            dn -= f * ui;
-                        } else {
-                            const float f = __fdividef(di, li);
-                            dd[i] = li; dl[i] = f; du[i] = dn;
-                            dn = ui - f * dn;
-                            if (i < D - 2) { du2[i] = un; un = -f * un; }
-                            pv[i] = 1.f;
-                        }
-                        di = dn; ui = un;
-                        if (i < D - 2) du[i + 1] = un;
-                    }
-                    dd[D - 1] = di == 0.f ? pert : di;
-                }
-                __syncwarp();
-                // the solves multiply by the pivots' reciprocals
-                for (int i = lane; i < D; i += 32) {
-                    float dv = dd[i];
-                    if (fabsf(dv) < pert) dv = dv < 0.f ? -pert : pert;
-                    dd[i] = 1.f / dv;
-                }
-            }
-            if (warp < ne) {
-                float *y = tz + warp * D;
-                for (int i = lane; i < D; i += 32) {                // a start vector without structure
-                    const uint32_t hsh = ((uint32_t)i * 2654435761u + (uint32_t)warp * 40503u + 12345u) >> 8;
-                    y[i] = (float)(hsh & 0xFFFFu) * (1.f / 65536.f) - 0.5f;
-                }
-            }
-            __syncthreads();
-#pragma unroll 1
-            for (int itn = 0; itn < 3; ++itn) {
-                if (warp < ne) {
-                    float *y = tz + warp * D;
-                    if (lane == 0) {
-                        // dd holds the reciprocals of the pivots; the value a step hands to the next stays in a register
-                        const float *dd = twk + (warp * 5) * D, *dl = dd + D, *du = dl + D, *du2 = du + D, *pv = du2 + D;
-                        float yi = y[0];
-                        for (int i = 0; i < D - 1; ++i) {
-                            const float yn = y[i + 1];
-                            if (pv[i] == 0.f) { y[i] = yi; yi = yn - dl[i] * yi; }
-                            else { y[i] = yn; yi = yi - dl[i] * yn; }
-                        }
-                        float y1 = yi * dd[D - 1];                               // y[i + 1]
-                        y[D - 1] = y1;
-                        float y0 = (y[D - 2] - du[D - 2] * y1) * dd[D - 2];      // y[i]
-                        y[D - 2] = y0;
-                        for (int i = D - 3; i >= 0; --i) {
-                            const float t = (y[i] - du[i] * y0 - du2[i] * y1) * dd[i];
-                            y[i] = t;
-                            y1 = y0;
-                            y0 = t;
-                        }
-                    }
-                    __syncwarp();
-                    // scaled to largest entry 1 by the whole warp
-                    float mx = 0.f;
-                    for (int i = lane; i < D; i += 32) mx = fmaxf(mx, fabsf(y[i]));
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-                    const float sc1 = mx > 0.f ? 1.f / mx : 1.f;
-                    for (int i = lane; i < D; i += 32) y[i] *= sc1;
-                }
-                __syncthreads();
-                if (warp == 0) {
-                    // in order of the eigenvalues: orthogonal to the close neighbours before it, unit length
-                    for (int j = 0; j < ne; ++j) {
-                        float *y = tz + j * D;
-                        for (int i2 = 0; i2 < j; ++i2) {
-                            if (fabsf(tlam[i2] - tlam[j]) > EIG_CLUSTER_TOL * fabsf(l1)) continue;
-                            const float *z = tz + i2 * D;
-                            float dsum = 0.f;
-                            for (int cc = lane; cc < D; cc += 32) dsum = fmaf(y[cc], z[cc], dsum);
-                            dsum = warp_sum(dsum);
-                            for (int cc = lane; cc < D; cc += 32) y[cc] -= dsum * z[cc];
-                            __syncwarp();
-                        }
-                        float n2 = 0.f;
-                        for (int cc = lane; cc < D; cc += 32) n2 = fmaf(y[cc], y[cc], n2);
-                        n2 = warp_sum(n2);
-                        const float inv = n2 > 0.f ? rsqrtf(n2) : 0.f;
-                        for (int cc = lane; cc < D; cc += 32) y[cc] *= inv;
-                        __syncwarp();
-                    }
-                }
-                __syncthreads();
-            }
-            // back through the reflectors: z = H_0 H_1 ... H_{D-3} y, one warp per vector, two reflectors per step:
-            // H_{k-1} H_k z = z - 2 a v_k - 2 (b - 2 c a) v_{k-1} with a = v_k . z, b = v_{k-1} . z, c = v_{k-1} . v_k,
-            // so that the three sums of a pair go through the warp together (half as many dependent reductions)
-            static_assert(D % 2 == 0, "the reflectors are taken in pairs");
-            if (warp < ne) {
-                float *y = tz + warp * D;
-                constexpr int CPLB = (D + 31) / 32;
-#pragma unroll 1
-                for (int k = D - 3; k >= 1; k -= 2) {
-                    // reflector k: column k of B2 below the diagonal; reflector k - 1: column k - 1 from row k on
-                    float vk[CPLB], vm[CPLB], zz[CPLB];
-                    float a = 0.f, b = 0.f, cdot = 0.f;
-#pragma unroll
-                    for (int cI = 0; cI < CPLB; ++cI) {
-                        const int cc = k + lane + 32 * cI;
-                        vk[cI] = (cc > k && cc < D) ? B2[cc * LD + k] : 0.f;
-                        vm[cI] = cc < D ? B2[cc * LD + k - 1] : 0.f;
-                        zz[cI] = cc < D ? y[cc] : 0.f;
-                        a = fmaf(vk[cI], zz[cI], a);
-                        b = fmaf(vm[cI], zz[cI], b);
-                        cdot = fmaf(vm[cI], vk[cI], cdot);
-                    }
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) {
-                        a += __shfl_xor_sync(0xffffffffu, a, o);
-                        b += __shfl_xor_sync(0xffffffffu, b, o);
-                        cdot += __shfl_xor_sync(0xffffffffu, cdot, o);
-                    }
-                    const float fa = 2.f * a, fb = 2.f * (b - 2.f * cdot * a);
-#pragma unroll
-                    for (int cI = 0; cI < CPLB; ++cI) {
-                        const int cc = k + lane + 32 * cI;
-                        if (cc < D) y[cc] = zz[cI] - fa * vk[cI] - fb * vm[cI];
-                    }
-                    __syncwarp();
-                }
-            }
-            __syncthreads();
-            // ---- 5a. Delta, delta from the wanted eigenvectors ----------------------------------
-            const int rmax = min(p.rank, D);
-            rho = 0;
-            while (rho < rmax && rho < ne && tlam[rho] > EIG_RANK_TOL * l1 && tlam[rho] > 0.f) ++rho;
-            lam1 = l1; lam_rho = rho > 0 ? tlam[rho - 1] : 0.f; lam_next = rho < ne ? fmaxf(tlam[rho], 0.f) : 0.f;
-            for (int t = 0; t < rho; ++t) revr += tlam[t];
-            revr /= trM + p.eps;                                    // trace of M = sum of all its eigenvalues
-            if (tid < rho) {
-                float sacc = 0.f;
-                for (int cc = 0; cc < D; ++cc) sacc = fmaf(tz[tid * D + cc], vu[cc], sacc);
-                vc[tid] = sacc;
-            }
-            __syncthreads();
-            float dl = 0.f;
-            if (tid < D) {
-                float sacc = 0.f;
-                for (int t = 0; t < rho; ++t) sacc = fmaf(vc[t], tz[t * D + tid], sacc);
-                dl = alpha * sacc;
-            }
-            __syncthreads();                                        // vc is scratch of the projection that follows
-            finish_delta(dl);
-            done = true;
-        }
+                if (!converged) status |= OBF_DEV_NO_CONVERGE;
 
-        // ---- 4b. Jacobi eigen-decomposition of M (B2), eigenvectors in U (workspace) -----
-        if (!done) {
-            float *U = WS;                                          // d x d, starts as the identity
-            for (int e = tid; e < D * D; e += ALG_NT) U[(e / D) * LD + (e % D)] = (e / D == e % D) ? 1.f : 0.f;
-            __syncthreads();
-            // rotations below the fp32 noise level of the largest eigenvalue never settle: stop there
-            const float floor_abs = 2e-7f * block_max<ALG_NT>(tid < D ? B2[tid * LD + tid] : 0.f, red);
-            bool converged = false;
-#pragma unroll 1
-            for (int sweep = 0; sweep < JACOBI_MAX_SWEEPS && !converged; ++sweep) {
-                if (tid == 0) misc[0] = 0.f;
+                // ---- 5. top-rank eigenvectors, Delta, delta ----------------------
+                if (tid < D) vl[tid] = B2[tid * LD + tid];
                 __syncthreads();
-#pragma unroll 1
-                for (int r = 0; r < D - 1; ++r) {
-                    if (tid < D / 2) {
-                        int pp, qq;
-                        if (tid == 0) { pp = D - 1; qq = r; }
-                        else { pp = (r + tid) % (D - 1); qq = (r - tid + (D - 1)) % (D - 1); }
-                        if (pp > qq) { const int t = pp; pp = qq; qq = t; }
-                        const float app = B2[pp * LD + pp], aqq = B2[qq * LD + qq], apq = B2[pp * LD + qq];
-                        float cs = 1.f, sn = 0.f;
-                        if (fabsf(apq) > 1e-7f * sqrtf(fabsf(app * aqq)) + floor_abs) {
-                            const float theta = (aqq - app) / (2.f * apq);
-                            const float t = (theta >= 0.f ? 1.f : -1.f) / (fabsf(theta) + sqrtf(theta * theta + 1.f));
-                            cs = rsqrtf(t * t + 1.f);
-                            sn = t * cs;
-                            misc[0] = 1.f;
-                        }
-                        vcs[2 * tid] = cs; vcs[2 * tid + 1] = sn;
-                        ipq[2 * tid] = pp; ipq[2 * tid + 1] = qq;
+                if (tid == 0) {
+                    float l1 = 0.f;
+                    for (int i = 0; i < D; ++i) l1 = fmaxf(l1, vl[i]);
+                    int n = 0;
+                    float last = 0.f, kept = 0.f;
+                    const int rmax = min(p.rank, D);
+                    while (n < rmax) {
+                        int b = -1; float best = EIG_RANK_TOL * l1;
+                        for (int i = 0; i < D; ++i) if (vl[i] > best) { best = vl[i]; b = i; }
+                        if (b < 0) break;
+                        isel[n++] = b; last = vl[b]; kept += vl[b]; vl[b] = -1.f;
                     }
-                    __syncthreads();
-                    for (int e = tid; e < D * (D / 2); e += ALG_NT) {      // columns of M and U
-                        const int i = e / (D / 2), t = e % (D / 2);
-                        const float cs = vcs[2 * t], sn = vcs[2 * t + 1];
-                        if (sn != 0.f) {
-                            const int pp = ipq[2 * t], qq = ipq[2 * t + 1];
-                            const float mp = B2[i * LD + pp], mq = B2[i * LD + qq];
-                            B2[i * LD + pp] = cs * mp - sn * mq;
-                            B2[i * LD + qq] = sn * mp + cs * mq;
-                            const float up = U[i * LD + pp], uq = U[i * LD + qq];
-                            U[i * LD + pp] = cs * up - sn * uq;
-                            U[i * LD + qq] = sn * up + cs * uq;
-                        }
-                    }
-                    __syncthreads();
-                    for (int e = tid; e < D * (D / 2); e += ALG_NT) {      // rows of M
-                        const int t = e / D, j = e % D;
-                        const float cs = vcs[2 * t], sn = vcs[2 * t + 1];
-                        if (sn != 0.f) {
-                            const int pp = ipq[2 * t], qq = ipq[2 * t + 1];
-                            const float mp = B2[pp * LD + j], mq = B2[qq * LD + j];
-                            B2[pp * LD + j] = cs * mp - sn * mq;
-                            B2[qq * LD + j] = sn * mp + cs * mq;
-                        }
-                    }
-                    __syncthreads();
+                    float nxt = 0.f;
+                    for (int i = 0; i < D; ++i) nxt = fmaxf(nxt, vl[i]);
+                    misc[1] = l1; misc[2] = last; misc[3] = nxt; misc[4] = (float)n; misc[5] = kept;
                 }
-                converged = (misc[0] == 0.f);
                 __syncthreads();
-            }
-            if (!converged) status |= OBF_DEV_NO_CONVERGE;
-
-            // ---- 5. top-rank eigenvectors, Delta, delta ----------------------
-            if (tid < D) vl[tid] = B2[tid * LD + tid];
-            __syncthreads();
-            if (tid == 0) {
-                float l1 = 0.f;
-                for (int i = 0; i < D; ++i) l1 = fmaxf(l1, vl[i]);
-                int n = 0;
-                float last = 0.f, kept = 0.f;
-                const int rmax = min(p.rank, D);
-                while (n < rmax) {
-                    int b = -1; float best = EIG_RANK_TOL * l1;
-                    for (int i = 0; i < D; ++i) if (vl[i] > best) { best = vl[i]; b = i; }
-                    if (b < 0) break;
-                    isel[n++] = b; last = vl[b]; kept += vl[b]; vl[b] = -1.f;
+                lam1 = misc[1]; lam_rho = misc[2]; lam_next = misc[3]; rho = (int)misc[4];
+                revr = misc[5] / (trM + p.eps);
+                if (tid < rho) {
+                    const int col = isel[tid];
+                    float s = 0.f;
+                    for (int cc = 0; cc < D; ++cc) s = fmaf(U[cc * LD + col], vu[cc], s);
+                    vc[tid] = s;
                 }
-                float nxt = 0.f;
-                for (int i = 0; i < D; ++i) nxt = fmaxf(nxt, vl[i]);
-                misc[1] = l1; misc[2] = last; misc[3] = nxt; misc[4] = (float)n; misc[5] = kept;
+                __syncthreads();
+                if (tid < D) {
+                    float s = 0.f;
+                    for (int t = 0; t < rho; ++t) s = fmaf(vc[t], U[tid * LD + isel[t]], s);
+                    vx[tid] = s;
+                }
+                finish_delta(0);
             }
-            __syncthreads();
-            lam1 = misc[1]; lam_rho = misc[2]; lam_next = misc[3]; rho = (int)misc[4];
-            revr = misc[5] / (trM + p.eps);
-            if (tid < rho) {
-                const int col = isel[tid];
-                float s = 0.f;
-                for (int cc = 0; cc < D; ++cc) s = fmaf(U[cc * LD + col], vu[cc], s);
-                vc[tid] = s;
             }
-            __syncthreads();
-            float dl = 0.f;
-            if (tid < D) {
-                float s = 0.f;
-                for (int t = 0; t < rho; ++t) s = fmaf(vc[t], U[tid * LD + isel[t]], s);
-                dl = alpha * s;
-            }
-            __syncthreads();                                        // vc is scratch of the projection that follows
-            finish_delta(dl);
-        }
     }
 
     if (tid == 0) {

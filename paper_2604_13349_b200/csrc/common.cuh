@@ -10,11 +10,10 @@
 
 namespace obf {
 
-// One cache as the kernels see it (device pointers, resolved sizes).
 // Per-head flags in the workspace (hflag).
-constexpr uint32_t HFLAG_INJECT = 1u;      // delta != 0: the injection kernel has work for this head
 constexpr uint32_t HFLAG_SPAN_FULL = 2u;   // span(V_keep) = R^d
 
+// One cache as the kernels see it (device pointers, resolved sizes).
 struct CacheDev {
     const void *k, *v, *q;
     void *k_out, *v_out;
@@ -96,7 +95,7 @@ struct CallDev {
     float *uvec;              // [heads_total, gram_slots, u_levels, d] partial sum_j A_j v_j over the same rows as gram_d, per mass level
     float *delta;             // [heads_total, d]
     float *svec;              // [heads_total, d] sum of the deleted value rows (only filled when diagnostics are asked for)
-    uint32_t *hflag;          // [heads_total] bit0: delta != 0 -> inject
+    uint32_t *hflag;          // [heads_total] HFLAG_*
 };
 
 __device__ __forceinline__ void locate(const CallDev &p, int g, int &ci, int &lh)

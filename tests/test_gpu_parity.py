@@ -120,6 +120,15 @@ def test_codimension_one():
     assert all(dg["span_rank"] == 63 and dg["rho_eff"] == 1 for dg in diags)
 
 
+@pytest.mark.parametrize("budget,rank", [(2, 8), (31, 1), (32, 2), (33, 4), (64, 8), (65, 2), (95, 3), (97, 9), (126, 2), (127, 2)])
+def test_basis_sizes_around_the_batches_and_stages_of_the_dense_algebra(budget, rank):
+    # retained rows come in batches of 32, reflectors in stages of 32, the tridiagonal form of what they leave ends at one
+    # or two rows, more than eight eigenpairs take the Jacobi route
+    w = small("basis", d=128, dtype="bf16", rank=rank, caches=((333, budget),), n_outlier=3, seed=budget)
+    outs, reps, _ = run_and_check(w)
+    assert all(dg["span_rank"] == budget for dg in P.parse_diag(outs[0]["diag"]))
+
+
 def test_budget_above_head_dim_full_rank_is_bit_exact_eviction():
     w = small("full", d=64, dtype="bf16", rank=3, caches=((400, 90),))
     outs, reps, _ = run_and_check(w)
