@@ -501,10 +501,15 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
     }
     if (cd.merge) {
         // cache-merging baseline (App. E): route the deleted positions, then add their values into the retained rows
-        const size_t sm_mg = merge_smem_bytes<D>();
-        if ((s = set_smem(k_merge_assign<TIN, D>, sm_mg)) != OBF_OK) return s;
-        dim3 ga((T_max + MG_TILE - 1) / MG_TILE, heads);
-        k_merge_assign<TIN, D><<<ga, 256, sm_mg, st>>>(cd);
+        if constexpr (sizeof(TIN) == 2) {
+            dim3 ga((T_max + MGT_ROWS - 1) / MGT_ROWS, heads);
+            k_merge_assign_mma<D><<<ga, MGT_NT, 0, st>>>(cd);
+        } else {
+            const size_t sm_mg = merge_smem_bytes<D>();
+            if ((s = set_smem(k_merge_assign<TIN, D>, sm_mg)) != OBF_OK) return s;
+            dim3 ga((T_max + MG_TILE - 1) / MG_TILE, heads);
+            k_merge_assign<TIN, D><<<ga, 256, sm_mg, st>>>(cd);
+        }
         mark(st, "k_merge_assign");
         dim3 gm((k_max + 7) / 8, heads);
         k_merge_apply<TIN, D><<<gm, 256, 0, st>>>(cd);

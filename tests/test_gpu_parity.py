@@ -800,6 +800,12 @@ def test_cache_merging_baseline(dtype, d, caches, flags):
     print("\n[merge] near-tie routings %d, of which the GPU chose another near-best slot %d" % (near_ties, flips))
 
 
+@pytest.mark.parametrize("d,caches", [(64, ((65, 1), (257, 64), (300, 65))), (128, ((255, 63), (129, 8), (513, 200)))])
+def test_cache_merging_around_the_tiles_of_the_tensor_core_routing(d, caches):
+    # positions come in tiles of 16, 64 and 256, slots in groups of 8 and 64
+    test_cache_merging_baseline("bf16", d, caches, 0)
+
+
 # ---------------------------------------------------------------------------
 # int8 copy of the compacted relay (post-hoc quantisation stacked on the compression, App. E)
 # ---------------------------------------------------------------------------
