@@ -114,7 +114,7 @@ typedef enum { OBF_F32 = 0, OBF_BF16 = 1 } obf_dtype_t;
                                       20 ms, so every wait for them runs out, the kernels return by themselves, the
                                       status word carries OBF_DEV_TIMEOUT and the outputs hold valid positions but no
                                       meaningful selection.  Accepted only for at most 4 (layer, KV head) pairs in all,
-                                      every T <= 2048, on the tuned bf16 / head_dim 128 path; else
+                                      every T <= 2048, on the tuned bf16 path; else
                                       OBF_ERR_INVALID_ARG                                                         */
 
 #define OBF_MAX_CACHES 32          /* caches per call                                              */

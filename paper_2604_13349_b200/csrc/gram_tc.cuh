@@ -1,4 +1,4 @@
-// Tuned streaming pass of Orthogonal BackFill for bf16 caches with head_dim 128:
+// Tuned streaming pass of Orthogonal BackFill for bf16 caches (head_dim 64 or 128):
 // one pass over V on the tensor cores that needs no selection result.
 //
 // With Q an orthonormal basis of the retained values' span and P = I - Q Q^T (Eq. 2-3), every
@@ -17,9 +17,9 @@
 // (b - first block touching that head).
 //
 // Block = 10 warps:
-//   warp 0       TMA producer: 128 x 128 bf16 tiles (two 128-byte-swizzled column halves) into a ring
-//   warp 1       issues tcgen05.mma: [G | u] (+)= tile^T [tile | a] in ONE instruction per 16 tokens (N = 144): the
-//                B operand is the value tile followed, as a third 64-column block of the same MN-major layout, by
+//   warp 0       TMA producer: 128 x d bf16 tiles (128-byte-swizzled blocks of 64 columns) into a ring
+//   warp 1       issues tcgen05.mma: [G | u] (+)= tile^T [tile | a] in ONE instruction per 16 tokens (N = d + 16): the
+//                B operand is the value tile followed, as one more 64-column block of the same MN-major layout, by
 //                the tile's 128 masses as bf16 columns: high, middle and low part of the fp32 mass (their sum is
 //                the mass exactly, and bf16 x bf16 products are exact in fp32), so that the CUDA cores never read
 //                a value tile; the three columns exist once per mass level (common.cuh: u_level), a token filling
@@ -33,15 +33,20 @@
 
 namespace obf {
 
-constexpr int GT_STAGES = 3;
 constexpr int GT_TILE = 128;                       // tokens per tile
-constexpr int GT_TILE_BYTES = GT_TILE * 128 * 2;   // 32 KiB
-constexpr int GT_ABLOCK_BYTES = GT_TILE * 128;     // mass block: [128 tokens][64 columns] bf16 like a column block of the tile; columns 3 * level + part in use
-constexpr int GT_STAGE_BYTES = GT_TILE_BYTES + GT_ABLOCK_BYTES;   // the mass block sits right behind its value tile
+constexpr int GT_BLOCK_BYTES = GT_TILE * 128;      // a 64-channel column block of a tile: 16 KiB; the mass block has the same layout, columns 3 * level + part in use
+// Ring stages: three of 48 KiB (head_dim 128), four of 32 KiB (head_dim 64): as many mass warps, and little enough
+// shared memory that the side stream's blocks find room.  The mass block sits right behind its value tile.
+template <int D>
+struct GramShape {
+    static constexpr int STAGES = D == 128 ? 3 : 4;
+    static constexpr int TILE_BYTES = GT_TILE * D * 2;
+    static constexpr int STAGE_BYTES = TILE_BYTES + GT_BLOCK_BYTES;
+    static constexpr size_t SMEM_BYTES = 1024 + (size_t)STAGES * STAGE_BYTES + 64;
+};
 constexpr int GT_NU = 16;                          // columns of the mass block that enter the MMA
 static_assert(3 * U_LEVELS <= GT_NU, "the mass columns must fit the MMA's extra columns");
 constexpr int GT_THREADS = 64 + 128 + 128;
-constexpr size_t GT_SMEM_BYTES = 1024 + (size_t)GT_STAGES * GT_STAGE_BYTES + 64;
 constexpr uint32_t GT_TMEM_COLS = 512;             // 2 accumulators of 128 + 16 columns at a stride of 256
 constexpr uint32_t GT_TMEM_STRIDE = 256;
 
@@ -85,15 +90,17 @@ struct TileRun {
     }
 };
 
-// G_all and u_all from V.
+// G_all and u_all from V.  With head_dim 64 the instruction still has M = 128: the second 64 rows of its A operand are
+// the mass block (the column block behind the tile), and what they produce is never read.
 // One block per multiprocessor; the launch bound of three only caps the registers at 64 per thread, so that the
 // blocks of the selection and the gather, which run on a side stream at the same time, find registers beside it.
+template <int D>
 __global__ void __launch_bounds__(GT_THREADS, 3) k_gram_tc(const __grid_constant__ CallDev p, const __grid_constant__ TcMaps tm)
 {
-    constexpr int D = 128;
+    constexpr int GT_STAGES = GramShape<D>::STAGES, GT_TILE_BYTES = GramShape<D>::TILE_BYTES, GT_STAGE_BYTES = GramShape<D>::STAGE_BYTES;
     extern __shared__ uint8_t gt_smem_raw[];
     uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(gt_smem_raw) + 1023) & ~(uintptr_t)1023);
-    uint8_t *tiles = base;                                                // GT_STAGES x (32 KiB tile + 16 KiB mass block), 1024-byte aligned
+    uint8_t *tiles = base;                                                // GT_STAGES x (tile + mass block), 1024-byte aligned
     __shared__ uint64_t bar_full[GT_STAGES], bar_ready[GT_STAGES], bar_empty[GT_STAGES];
     __shared__ uint64_t bar_acc_full[2], bar_acc_empty[2];
     __shared__ uint32_t s_tmem, s_abort;
@@ -132,8 +139,8 @@ __global__ void __launch_bounds__(GT_THREADS, 3) k_gram_tc(const __grid_constant
                     if (!tc::mbar_wait(&bar_empty[s], ph ^ 1u, wc)) break;
                     tc::mbar_expect_tx(&bar_full[s], GT_TILE_BYTES);
                     const uint32_t dst = tc::smem_u32(tiles + s * GT_STAGE_BYTES);
-                    tc::tma_load_3d(dst, map, &bar_full[s], 0, (sub0 + t) * GT_TILE, lh);
-                    tc::tma_load_3d(dst + GT_TILE_BYTES / 2, map, &bar_full[s], 64, (sub0 + t) * GT_TILE, lh);
+                    for (int h = 0; h < D / 64; ++h)
+                        tc::tma_load_3d(dst + h * GT_BLOCK_BYTES, map, &bar_full[s], 64 * h, (sub0 + t) * GT_TILE, lh);
                 }
                 if (s_abort) break;
             }
@@ -145,7 +152,7 @@ __global__ void __launch_bounds__(GT_THREADS, 3) k_gram_tc(const __grid_constant
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
         if (lane == 0) {
-            constexpr uint32_t idesc = tc::idesc_bf16(128, 128 + GT_NU, 1, 1);
+            constexpr uint32_t idesc = tc::idesc_bf16(128, D + GT_NU, 1, 1);
             TileRun run;
             run.init(p, blockIdx.x);
             int cache, lh, sub0, nsub, slot;
@@ -166,8 +173,8 @@ __global__ void __launch_bounds__(GT_THREADS, 3) k_gram_tc(const __grid_constant
 #pragma unroll
                     for (int kk = 0; kk < 8; ++kk) {
                         // 16 tokens per instruction: rows kk*16.. of the tile; the column blocks of 64 follow one another
-                        // at 16 KiB: two of the value tile and, for the B operand, the mass block
-                        const uint64_t dv = tc::smem_desc_sw128(tile + kk * 2048, GT_TILE_BYTES / 2, 1024);
+                        // at 16 KiB: one or two of the value tile, then the mass block
+                        const uint64_t dv = tc::smem_desc_sw128(tile + kk * 2048, GT_BLOCK_BYTES, 1024);
                         tc::umma_bf16(acc, dv, dv, idesc, (t > 0 || kk > 0) ? 1u : 0u);
                     }
                     tc::umma_commit(&bar_empty[s]);
@@ -268,8 +275,9 @@ __global__ void __launch_bounds__(GT_THREADS, 3) k_gram_tc(const __grid_constant
             tc::tc_fence_after();
             const uint32_t tl = tmem + ((uint32_t)(q * 32) << 16);
             float *dst = p.gram_d + ((size_t)g * p.gram_slots + slot) * D * D + (size_t)row * D;
+            if (q * 32 < D) {                          // (the same in every lane of the warp)
 #pragma unroll 1
-            for (int cb = 0; cb < 4; ++cb) {
+            for (int cb = 0; cb < D / 32; ++cb) {
                 uint32_t r[32];
                 tc::tmem_ld32(tl + buf * GT_TMEM_STRIDE + cb * 32u, r);
                 tc::tmem_ld_wait();
@@ -282,12 +290,13 @@ __global__ void __launch_bounds__(GT_THREADS, 3) k_gram_tc(const __grid_constant
             {
                 // u of value channel `row`, per mass level: three columns add up the products with the three parts of the masses
                 uint32_t r[32];
-                tc::tmem_ld32(tl + buf * GT_TMEM_STRIDE + 128u, r);
+                tc::tmem_ld32(tl + buf * GT_TMEM_STRIDE + (uint32_t)D, r);
                 tc::tmem_ld_wait();
 #pragma unroll
                 for (int l = 0; l < U_LEVELS; ++l)
                     p.uvec[(((size_t)g * p.gram_slots + slot) * U_LEVELS + l) * D + row] =
                         (__uint_as_float(r[3 * l]) + __uint_as_float(r[3 * l + 1])) + __uint_as_float(r[3 * l + 2]);
+            }
             }
             tc::tc_fence_before();
             __syncwarp();

@@ -106,10 +106,10 @@ static int sm_count()
     return cached[dev];
 }
 
-// The tensor-core kernels cover bf16 caches with head_dim 128 and at least one full 128-token tile.
+// The tensor-core kernels cover bf16 caches with at least one full 128-token tile.
 static bool tuned_path_applies(const obf_params_t *p, const obf_cache_t *caches, int32_t n)
 {
-    if (p->dtype != OBF_BF16 || p->head_dim != 128 || (p->flags & OBF_FLAG_GENERIC_PATH)) return false;
+    if (p->dtype != OBF_BF16 || (p->flags & OBF_FLAG_GENERIC_PATH)) return false;
     for (int i = 0; i < n; ++i)
         if (caches[i].T < GT_TILE) return false;
     return true;
@@ -296,14 +296,14 @@ static EncodeTiledFn tensor_map_encoder()
     return fn;
 }
 
-// Tensor map of a bf16 array [heads, rows, 128] for box_rows x 64-column boxes with the
+// Tensor map of a bf16 array [heads, rows, d] for box_rows x 64-column boxes with the
 // 128-byte swizzle; rows past `rows` read as zero.
-static obf_status_t encode_rows_map(CUtensorMap *m, const void *ptr, uint64_t rows, uint64_t heads, uint32_t box_rows = GT_TILE)
+static obf_status_t encode_rows_map(CUtensorMap *m, const void *ptr, uint64_t d, uint64_t rows, uint64_t heads, uint32_t box_rows = GT_TILE)
 {
     EncodeTiledFn enc = tensor_map_encoder();
     if (!enc) return OBF_ERR_CUDA;
-    cuuint64_t dims[3] = {128, rows, heads};
-    cuuint64_t strides[2] = {128 * 2, rows * 128 * 2};
+    cuuint64_t dims[3] = {d, rows, heads};
+    cuuint64_t strides[2] = {d * 2, rows * d * 2};
     cuuint32_t box[3] = {64, (cuuint32_t)box_rows, 1};
     cuuint32_t es[3] = {1, 1, 1};
     const CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(ptr), dims, strides, box, es,
@@ -316,42 +316,44 @@ static obf_status_t encode_rows_map(CUtensorMap *m, const void *ptr, uint64_t ro
     return OBF_OK;
 }
 
-// Streaming pass of OBF on the tensor cores (bf16, head_dim 128): Gram matrix and mass-weighted sum over all rows
+// Streaming pass of OBF on the tensor cores (bf16): Gram matrix and mass-weighted sum over all rows
 // of V (needs the masses, not the selection).
+template <int D>
 static obf_status_t launch_gram_tc(const CallDev &cd, const Layout &L, cudaStream_t st)
 {
     static thread_local TcMaps m;
     if (L.tc_blocks == 0) return OBF_OK;
     const uint64_t hpc = (uint64_t)cd.heads_per_cache;
     for (int i = 0; i < cd.n_caches; ++i) {
-        const obf_status_t s = encode_rows_map(&m.a[i], cd.c[i].v, (uint64_t)cd.c[i].T, hpc);
+        const obf_status_t s = encode_rows_map(&m.a[i], cd.c[i].v, D, (uint64_t)cd.c[i].T, hpc);
         if (s != OBF_OK) return s;
     }
-    OBF_CUDA_TRY(cudaFuncSetAttribute(k_gram_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GT_SMEM_BYTES));
     // the whole shared-memory capacity, so that the side stream's blocks find room beside this kernel's
-    OBF_CUDA_TRY(cudaFuncSetAttribute(k_gram_tc, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared));
-    k_gram_tc<<<L.tc_blocks, GT_THREADS, GT_SMEM_BYTES, st>>>(cd, m);
+    const obf_status_t sa = set_smem(k_gram_tc<D>, GramShape<D>::SMEM_BYTES);
+    if (sa != OBF_OK) return sa;
+    k_gram_tc<D><<<L.tc_blocks, GT_THREADS, GramShape<D>::SMEM_BYTES, st>>>(cd, m);
     mark(st, "k_gram_tc");
     return OBF_OK;
 }
 
-// Attention mass on the tensor cores (bf16, head_dim 128): one persistent launch.
+// Attention mass on the tensor cores (bf16): one persistent launch.
+template <int D>
 static obf_status_t launch_score_tc(const CallDev &cd, const Layout &L, cudaStream_t st)
 {
     static thread_local TcMaps maps;
     const uint64_t hpc = (uint64_t)cd.heads_per_cache;
     for (int i = 0; i < cd.n_caches; ++i) {
-        obf_status_t s = encode_rows_map(&maps.a[i], cd.c[i].k, (uint64_t)cd.c[i].T, hpc);
+        obf_status_t s = encode_rows_map(&maps.a[i], cd.c[i].k, D, (uint64_t)cd.c[i].T, hpc);
         if (s != OBF_OK) return s;
-        if ((s = encode_rows_map(&maps.b[i], cd.c[i].q, (uint64_t)cd.n_q, hpc)) != OBF_OK) return s;
+        if ((s = encode_rows_map(&maps.b[i], cd.c[i].q, D, (uint64_t)cd.n_q, hpc)) != OBF_OK) return s;
     }
-    const size_t smem = ST_SMEM_BYTES;
-    OBF_CUDA_TRY(cudaFuncSetAttribute(k_score_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const size_t smem = score_tc_smem_bytes<D>();
+    OBF_CUDA_TRY(cudaFuncSetAttribute(k_score_tc<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     OBF_CUDA_TRY(cudaMemsetAsync(cd.sc_head, 0, (L.off_sc_sync - L.off_sc_head) + (size_t)cd.heads_total * L.sc_qt * sizeof(uint32_t), st));
     // The blocks of a head's team wait for one another, so the whole grid has to be resident at once: a
     // cooperative launch starts only when it is (the grid never exceeds one block per multiprocessor).
     void *args[2] = {const_cast<CallDev *>(&cd), &maps};
-    OBF_CUDA_TRY(cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(k_score_tc), dim3(L.sc_blocks), dim3(ST_THREADS),
+    OBF_CUDA_TRY(cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(k_score_tc<D>), dim3(L.sc_blocks), dim3(ST_THREADS),
                                              args, smem, st));
     mark(st, "k_score_tc");
     if (L.sc_qt == 2) {
@@ -371,7 +373,7 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
     const size_t sm_sc = score_smem_bytes<D>();
     obf_status_t s;
     if (L.sc_on) {
-        if ((s = launch_score_tc(cd, L, st)) != OBF_OK) return s;
+        if ((s = launch_score_tc<D>(cd, L, st)) != OBF_OK) return s;
     } else {
         if ((s = set_smem(k_score_stats<TIN, D>, sm_sc)) != OBF_OK) return s;
         if ((s = set_smem(k_score_pool<TIN, D>, sm_sc)) != OBF_OK) return s;
@@ -392,7 +394,7 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
     if (side) {
         OBF_CUDA_TRY(cudaEventRecord(side->fork, st));
         OBF_CUDA_TRY(cudaStreamWaitEvent(side->stream, side->fork, 0));
-        if ((s = launch_gram_tc(cd, L, st)) != OBF_OK) return s;
+        if ((s = launch_gram_tc<D>(cd, L, st)) != OBF_OK) return s;
     }
     if (cd.layerwise) {
         // masses of a layer's KV heads added up, then every head's block selects on its layer's sums
@@ -431,7 +433,7 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
         k_gather<D * (int)sizeof(TIN), 1><<<g4, 256, 0, sel>>>(cd);
         mark(sel, "k_gather");
         OBF_CUDA_TRY(cudaEventRecord(side->rows_done, side->stream));
-        if constexpr (sizeof(TIN) == 2 && D == 128) {
+        if constexpr (sizeof(TIN) == 2) {
             // the span test reads the gathered rows only (it forms G_keep itself): it runs here, beside the pass over
             // V, whose persistent blocks leave room for one of its blocks per multiprocessor
             const size_t sm_span = span_smem_bytes<D>();
@@ -454,7 +456,7 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
         const size_t sm_alg = algebra_smem_bytes<D>(cd.alg_rows, cd.rank, cd.fast_iters);
         if ((s = set_smem(k_obf_algebra<TIN, D>, sm_alg)) != OBF_OK) return s;
         if (tuned_obf) {
-            if constexpr (sizeof(TIN) == 2 && D == 128) {
+            if constexpr (sizeof(TIN) == 2) {
                 if (cd.skip_full) {
                     // the span test before the pass over V, which then skips the heads whose retained values span R^d
                     const size_t sm_span0 = span_smem_bytes<D>();
@@ -463,7 +465,7 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
                     mark(st, "k_span_test");
                 }
             }
-            if (!side && (s = launch_gram_tc(cd, L, st)) != OBF_OK) return s;
+            if (!side && (s = launch_gram_tc<D>(cd, L, st)) != OBF_OK) return s;
         } else {
             dim3 g5(cd.splits, heads);
             k_gram<TIN, D><<<g5, 256, 0, st>>>(cd);
@@ -482,7 +484,7 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
         if (side || cd.skip_full) {
             // the span test has been enqueued already: on the side stream (this stream has waited for it) or, with
             // OBF_FLAG_EARLY_OUT, before the pass over V
-        } else if constexpr (sizeof(TIN) == 2 && D == 128) {
+        } else if constexpr (sizeof(TIN) == 2) {
             if (tuned_obf) {
                 // the tuned path forms G_keep inside the span test, from the gathered rows
                 if ((s = set_smem(k_span_test<D, true>, sm_span)) != OBF_OK) return s;

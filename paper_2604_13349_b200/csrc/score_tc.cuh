@@ -1,5 +1,5 @@
 // Tuned attention-mass kernel (step a1, Eq. 1 with the softmax of App. L.1) for bf16
-// caches with head_dim 128 and up to 256 query rows per KV head (above 128 rows a head is
+// caches with head_dim 64 or 128 and up to 256 query rows per KV head (above 128 rows a head is
 // worked on as two items of up to 128 rows whose masses are added afterwards).
 //
 //   A_j = sum_t softmax_j(q_t . K_j / sqrt(d)),  t over the n_q query rows of the KV head.
@@ -53,14 +53,14 @@ constexpr int ST_CHUNK = ST_TILES * 128;
 constexpr int ST_STAGES = 4;                        // K tiles in flight in shared memory
 constexpr int ST_TBUF = 4;                          // accumulator tiles in tensor memory
 constexpr int ST_LAG = 1;                           // rounds between a chunk's statistics pass and its pooling pass
-constexpr int ST_TILE_BYTES = 128 * 128 * 2;
+constexpr int ST_BOX_BYTES = 128 * 128;              // a 64-channel column block of a tile: 128 rows of 128 bytes
 constexpr int ST_GROUPS = 4;                        // consumer groups of four warps, one accumulator tile each
 constexpr int ST_CONSUMERS = ST_GROUPS * 128;
 constexpr int ST_THREADS = 64 + ST_CONSUMERS + 64;
 constexpr int ST_MAX_NQ = 256;                      // two query tiles of 128 rows
 constexpr float ST_LOG2E = 1.4426950408889634f;
-constexpr size_t ST_SMEM_BYTES = 1024 + (size_t)2 * ST_TILE_BYTES + (size_t)ST_STAGES * ST_TILE_BYTES +
-                                 (2 * 2 * ST_GROUPS * 128 + 2 * 128) * sizeof(float) + 64;
+template <int D>
+constexpr size_t score_tc_smem_bytes() { return 1024 + (size_t)(2 + ST_STAGES) * 128 * D * 2 + (2 * 2 * ST_GROUPS * 128 + 2 * 128) * sizeof(float) + 64; }
 static_assert(ST_STAGES == ST_TBUF, "a ring stage is released by the accumulator barrier of the same index");
 
 struct ScoreItem {
@@ -200,8 +200,10 @@ __device__ __forceinline__ float pool_piece(const uint32_t (&rr)[32], const floa
     return (a0 + a1) + (a2 + a3);
 }
 
+template <int D>
 __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constant__ CallDev p, const __grid_constant__ TcMaps tm)
 {
+    constexpr int ST_TILE_BYTES = 128 * D * 2, NBOX = D / 64;
     extern __shared__ uint8_t st_smem_raw[];
     uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(st_smem_raw) + 1023) & ~(uintptr_t)1023);
     uint8_t *q_s = base;                                           // 2 x [128 x 128] bf16: Q of a statistics pass, Q of a pooling pass; two 64-column halves each
@@ -261,8 +263,8 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constan
                 if (nq[kind] > 0 && !tc::mbar_wait(&bar_q_free[kind], (nq[kind] - 1) & 1u, wc, 64)) return false;
                 const uint32_t qdst = tc::smem_u32(q_s + kind * ST_TILE_BYTES);
                 tc::mbar_expect_tx(&bar_q_full[kind], ST_TILE_BYTES);
-                tc::tma_load_3d(qdst, &tm.b[item.cache], &bar_q_full[kind], 0, item.qt * 128, item.lh);      // rows past n_q read as zero
-                tc::tma_load_3d(qdst + ST_TILE_BYTES / 2, &tm.b[item.cache], &bar_q_full[kind], 64, item.qt * 128, item.lh);
+                for (int h = 0; h < NBOX; ++h)                                   // rows past n_q read as zero
+                    tc::tma_load_3d(qdst + h * ST_BOX_BYTES, &tm.b[item.cache], &bar_q_full[kind], 64 * h, item.qt * 128, item.lh);
                 ++nq[kind];
                 return true;
             };
@@ -276,10 +278,9 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constan
                     // the next statistics pass reads its tiles from HBM: ask for them now
                     ScoreItem nx;
                     if (item.r + 1 < R && score_item(p, s_tab, item.r + 1, nx)) {
-                        for (int t = 0; t < nx.nt; ++t) {
-                            tc::tma_prefetch_l2_3d(&tm.a[nx.cache], 0, nx.chunk * ST_CHUNK + t * 128, nx.lh);
-                            tc::tma_prefetch_l2_3d(&tm.a[nx.cache], 64, nx.chunk * ST_CHUNK + t * 128, nx.lh);
-                        }
+                        for (int t = 0; t < nx.nt; ++t)
+                            for (int h = 0; h < NBOX; ++h)
+                                tc::tma_prefetch_l2_3d(&tm.a[nx.cache], 64 * h, nx.chunk * ST_CHUNK + t * 128, nx.lh);
                     }
                 }
                 for (int t = 0; t < item.nt; ++t, ++it) {
@@ -293,8 +294,8 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constan
                     tc::mbar_expect_tx(&bar_full[s], ST_TILE_BYTES);
                     const uint32_t dst = tc::smem_u32(ring + s * ST_TILE_BYTES);
                     const int row0 = item.chunk * ST_CHUNK + t * 128;
-                    tc::tma_load_3d(dst, &tm.a[item.cache], &bar_full[s], 0, row0, item.lh);
-                    tc::tma_load_3d(dst + ST_TILE_BYTES / 2, &tm.a[item.cache], &bar_full[s], 64, row0, item.lh);
+                    for (int h = 0; h < NBOX; ++h)
+                        tc::tma_load_3d(dst + h * ST_BOX_BYTES, &tm.a[item.cache], &bar_full[s], 64 * h, row0, item.lh);
                 }
                 if (dead) break;
                 // Q of the next pass, while the tiles just asked for are worked on
@@ -344,9 +345,9 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constan
                     // pass A: queries on the lanes (S = Q K^T); pass B: keys on the lanes (S^T = K Q^T)
                     const uint64_t da0 = kind == 0 ? dq0 : dk0, db0 = kind == 0 ? dk0 : dq0;
 #pragma unroll
-                    for (int kk = 0; kk < 8; ++kk) {
-                        // 16 channels per instruction: 32 bytes along the swizzled row, second half after 4 steps
-                        constexpr uint32_t HALF16 = (ST_TILE_BYTES / 2) >> 4;
+                    for (int kk = 0; kk < D / 16; ++kk) {
+                        // 16 channels per instruction: 32 bytes along the swizzled row, next column block after 4 steps
+                        constexpr uint32_t HALF16 = ST_BOX_BYTES >> 4;
                         const uint64_t off16 = (uint64_t)((kk >> 2) * HALF16 + (kk & 3) * 2);
                         tc::umma_bf16(acc, da0 + off16, db0 + off16, IDESC, kk > 0 ? 1u : 0u);
                     }
@@ -368,7 +369,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constan
         const int grp = (warp - 2) >> 2;               // tiles with index == grp (mod ST_GROUPS) are this warp's
         const int row = q * 32 + lane;                 // lane of the accumulator tile: a query (pass A) or a key (pass B)
         const uint32_t tlane = tmem + ((uint32_t)(q * 32) << 16);
-        const float sc = ST_LOG2E * rsqrtf(128.0f);
+        const float sc = ST_LOG2E * rsqrtf((float)D);
         uint32_t it = 0, n_a[2] = {0u, 0u}, n_b[2] = {0u, 0u};
 
         // The four 32-column pieces of an accumulator tile, `work(piece, registers)` on each; the tile is handed

@@ -12,8 +12,7 @@
 // 8x4 register tiles.
 // Result: bit 1 of hflag[head].
 //
-// FROM_ROWS (tuned path: bf16, head_dim 128): G_keep is not read from the workspace but formed here from the
-// first 256 gathered rows of the head (any subset of the retained rows that spans R^d certifies the test), with
+// FROM_ROWS (tuned path): G_keep is not read from the workspace but formed here from the first 2 d gathered rows of the head (any subset of the retained rows that spans R^d certifies the test), with
 // warp-level mma (bf16 products are exact, fp32 accumulation) while the rows sit in the memory the matrix then takes.
 #pragma once
 
@@ -26,8 +25,6 @@ constexpr float CHOL_PIVOT_TOL = 1e-3f;
 
 template <int D>
 constexpr size_t span_smem_bytes() { return (size_t)(D * (D + 1) + 32 * 33 + 32 + D + 64 + 256 + 3) * sizeof(float); }
-
-constexpr int SPAN_ROWS = 256;          // retained rows that enter G_keep with FROM_ROWS
 
 template <int D, bool FROM_ROWS = false>
 __global__ void __launch_bounds__(ST_NT, 3) k_span_test(const __grid_constant__ CallDev p)
@@ -52,26 +49,28 @@ __global__ void __launch_bounds__(ST_NT, 3) k_span_test(const __grid_constant__ 
         return;
     }
     if constexpr (FROM_ROWS) {
-        static_assert(D == 128, "the row-based Gram matrix is written for head_dim 128");
+        // the first 2 d rows (what fits the matrix's memory), in 16-byte chunks
+        constexpr int SPAN_ROWS = 2 * D, CH = D / 8;
         static_assert(SPAN_ROWS * D * 2 <= D * (D + 1) * 4, "the rows are staged in the matrix's memory");
-        // X: the first rows of the head's compacted values, [SPAN_ROWS][128] bf16, rows past the end zero; the
+        // X: the first rows of the head's compacted values, [SPAN_ROWS][D] bf16, rows past the end zero; the
         // 16-byte chunks of a row are permuted by the row number so that 8 x 8 matrix loads hit distinct banks
         uint8_t *X = reinterpret_cast<uint8_t *>(A);
         const int n_rows = c.k_eff < SPAN_ROWS ? c.k_eff : SPAN_ROWS;
         const uint4 *src = reinterpret_cast<const uint4 *>(reinterpret_cast<const __nv_bfloat16 *>(c.v_out) + (size_t)lh * c.k_eff * D);
         // eight 16-byte loads in flight per thread
 #pragma unroll 1
-        for (int i0 = tid; i0 < SPAN_ROWS * 16; i0 += 8 * ST_NT) {
+        static_assert(SPAN_ROWS * CH % ST_NT == 0, "whole passes");
+        for (int i0 = tid; i0 < SPAN_ROWS * CH; i0 += 8 * ST_NT) {
             uint4 v[8];
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
-                const int i = i0 + u * ST_NT, r = i >> 4, ch = i & 15;
-                v[u] = r < n_rows ? __ldg(src + (size_t)r * 16 + ch) : make_uint4(0u, 0u, 0u, 0u);
+                const int i = i0 + u * ST_NT, r = i / CH, ch = i % CH;
+                v[u] = r < n_rows ? __ldg(src + (size_t)r * CH + ch) : make_uint4(0u, 0u, 0u, 0u);
             }
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
-                const int i = i0 + u * ST_NT, r = i >> 4, ch = i & 15;
-                *reinterpret_cast<uint4 *>(X + r * 256 + (((ch & 8) | ((ch ^ r) & 7)) << 4)) = v[u];
+                const int i = i0 + u * ST_NT, r = i / CH, ch = i % CH;
+                if (i < SPAN_ROWS * CH) *reinterpret_cast<uint4 *>(X + r * (2 * D) + (((ch & 8) | ((ch ^ r) & 7)) << 4)) = v[u];
             }
         }
         __syncthreads();
@@ -79,22 +78,24 @@ __global__ void __launch_bounds__(ST_NT, 3) k_span_test(const __grid_constant__ 
         // B = X both read with transposing 8 x 8 loads from the row-major X)
         const uint32_t xbase = (uint32_t)__cvta_generic_to_shared(X);
         const int mi = lane >> 3, rr = lane & 7;
-        float acc[2][8][4];
+        constexpr int NHF = D / 64;
+        float acc[NHF][8][4];
 #pragma unroll
-        for (int hf = 0; hf < 2; ++hf)
+        for (int hf = 0; hf < NHF; ++hf)
 #pragma unroll
             for (int nt = 0; nt < 8; ++nt)
 #pragma unroll
                 for (int e = 0; e < 4; ++e) acc[hf][nt][e] = 0.f;
+        if (D == 128 || 16 * warp < D)
 #pragma unroll
-        for (int hf = 0; hf < 2; ++hf) {
+        for (int hf = 0; hf < NHF; ++hf) {
 #pragma unroll 1
             for (int k0 = 0; k0 < SPAN_ROWS; k0 += 16) {
                 uint32_t a[4];
                 {
                     // matrices: (tokens k0.., dims i0..), (tokens k0.., dims i0 + 8..), (tokens k0 + 8.., dims i0..), (k0 + 8.., i0 + 8..)
                     const int tok = k0 + (mi >> 1) * 8 + rr, chn = (16 * warp + (mi & 1) * 8) >> 3;
-                    const uint32_t addr = xbase + tok * 256 + (((chn & 8) | ((chn ^ tok) & 7)) << 4);
+                    const uint32_t addr = xbase + tok * (2 * D) + (((chn & 8) | ((chn ^ tok) & 7)) << 4);
                     asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
                                  : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]) : "r"(addr));
                 }
@@ -104,7 +105,7 @@ __global__ void __launch_bounds__(ST_NT, 3) k_span_test(const __grid_constant__ 
                     const int n0 = hf * 64 + np * 16;
                     if (n0 > 16 * warp) continue;              // right of the diagonal: only the lower triangle is ever read
                     const int tok = k0 + (mi & 1) * 8 + rr, chn = (n0 + (mi >> 1) * 8) >> 3;
-                    const uint32_t addr = xbase + tok * 256 + (((chn & 8) | ((chn ^ tok) & 7)) << 4);
+                    const uint32_t addr = xbase + tok * (2 * D) + (((chn & 8) | ((chn ^ tok) & 7)) << 4);
                     uint32_t b[4];
                     asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
                                  : "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3]) : "r"(addr));
@@ -119,8 +120,9 @@ __global__ void __launch_bounds__(ST_NT, 3) k_span_test(const __grid_constant__ 
             }
         }
         __syncthreads();                                   // every warp is done reading X: the matrix takes its place
+        if (D == 128 || 16 * warp < D)
 #pragma unroll
-        for (int hf = 0; hf < 2; ++hf)
+        for (int hf = 0; hf < NHF; ++hf)
 #pragma unroll
             for (int nt = 0; nt < 8; ++nt) {
                 const int row = 16 * warp + (lane >> 2), col = hf * 64 + nt * 8 + 2 * (lane & 3);

@@ -181,6 +181,20 @@ def test_tuned_path_ragged_batches_match_oracle_and_generic_path(caches):
     assert any(not r.oracle_skipped for r in reps) or all(c[1] >= 128 for c in caches)
 
 
+@pytest.mark.parametrize("G,n_obs,caches", [(2, 9, ((128, 16), (129, 64), (300, 63), (777, 100))),
+                                            (2, 65, ((513, 30), (1025, 32))),       # two query tiles per head
+                                            (4, 32, ((2048, 200),))])               # budget above head_dim: the span test's rows
+def test_tuned_path_with_heads_of_64_channels(G, n_obs, caches):
+    w = small("tuned64", layers=2, kv_heads=3, G=G, n_obs=n_obs, d=64, dtype="bf16", rank=2, caches=caches, n_outlier=3,
+              n_sink=2, seed=40 + G)
+    a, reps, arrays = run_and_check(w)
+    names = [n for n, _ in P.obf_compress_profiled(par.params_for(w), a[0]["cache_structs"], a[0]["workspace"])]
+    assert "k_score_tc" in names and "k_gram_tc" in names
+    b, _, _ = run_and_check(w, arrays=arrays, flags=P.binding.OBF_FLAG_GENERIC_PATH)
+    for x, y in zip(a, b):
+        assert torch.equal(x["K_out"], y["K_out"])
+
+
 def test_tuned_path_with_many_caches_of_different_lengths():
     # twelve caches in one call: every role of the score kernel walks the per-cache table
     Ts = [128, 131, 200, 256, 300, 511, 512, 513, 640, 777, 900, 1025]
