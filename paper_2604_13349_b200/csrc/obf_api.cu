@@ -388,6 +388,8 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
     // on the caller's stream while selection and gather run on a side stream of the library.  (Not while
     // profiling per launch, where every kernel is timed alone.)
     const bool tuned_obf = cd.rank > 0 && L.tc_per > 0;
+    // retained values can only span R^d where there are d of them: with smaller budgets there is nothing to test
+    const bool span = cd.rank > 0 && k_max >= D;
     // With OBF_FLAG_EARLY_OUT the span test comes first and the pass over V skips what it found full: one stream.
     SideStream *side = (tuned_obf && !g_prof.active && !cd.skip_full) ? side_stream() : nullptr;
     cudaStream_t sel = side ? side->stream : st;       // stream of selection and gather
@@ -433,7 +435,7 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
         k_gather<D * (int)sizeof(TIN), 1><<<g4, 256, 0, sel>>>(cd);
         mark(sel, "k_gather");
         OBF_CUDA_TRY(cudaEventRecord(side->rows_done, side->stream));
-        if constexpr (sizeof(TIN) == 2) {
+        if constexpr (sizeof(TIN) == 2) if (span) {
             // the span test reads the gathered rows only (it forms G_keep itself): it runs here, beside the pass over
             // V, whose persistent blocks leave room for one of its blocks per multiprocessor
             const size_t sm_span = span_smem_bytes<D>();
@@ -481,8 +483,8 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
             mark(st, "k_vsum");
         }
         const size_t sm_span = span_smem_bytes<D>();
-        if (side || cd.skip_full) {
-            // the span test has been enqueued already: on the side stream (this stream has waited for it) or, with
+        if (side || cd.skip_full || !span) {
+            // nothing to test, or the span test has been enqueued already: on the side stream (this stream has waited for it) or, with
             // OBF_FLAG_EARLY_OUT, before the pass over V
         } else if constexpr (sizeof(TIN) == 2) {
             if (tuned_obf) {
@@ -497,7 +499,7 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
             if ((s = set_smem(k_span_test<D>, sm_span)) != OBF_OK) return s;
             k_span_test<D><<<heads, ST_NT, sm_span, st>>>(cd);
         }
-        if (!side && !cd.skip_full) mark(st, "k_span_test");
+        if (!side && !cd.skip_full && span) mark(st, "k_span_test");
         k_obf_algebra<TIN, D><<<heads, ALG_NT, sm_alg, st>>>(cd);
         mark(st, "k_obf_algebra");
     }
@@ -619,7 +621,7 @@ static obf_status_t run(const obf_params_t *p, const obf_cache_t *caches, int32_
     cd.n_sink = (int32_t)OBF_FLAG_SINK_OF(p->flags);
     cd.fast_iters = (p->flags & OBF_FLAG_FAST_PATH) ? 3 : 0;
     cd.attn_inject = (p->flags & OBF_FLAG_ATTN_INJECT) ? 1 : 0;
-    cd.skip_full = (p->flags & OBF_FLAG_EARLY_OUT) && L.tc_per > 0 && rank > 0 ? 1 : 0;
+    cd.skip_full = (p->flags & OBF_FLAG_EARLY_OUT) && L.tc_per > 0 && rank > 0 && k_max >= p->head_dim ? 1 : 0;
     cd.alg_rows = k_max < p->head_dim ? k_max : p->head_dim;
     cd.wait_limit_ns = tc::WAIT_LIMIT_NS;
     cd.debug_drop_publish = 0;

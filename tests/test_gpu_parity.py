@@ -129,6 +129,17 @@ def test_basis_sizes_around_the_batches_and_stages_of_the_dense_algebra(budget, 
     assert all(dg["span_rank"] == budget for dg in P.parse_diag(outs[0]["diag"]))
 
 
+@pytest.mark.parametrize("dtype,d,budgets", [("bf16", 128, (128, 129, 255, 257)), ("bf16", 64, (64, 65, 127, 129)),
+                                             ("f32", 128, (128, 140)), ("f32", 64, (64, 65)), ("bf16", 128, (127, 128))])
+def test_span_test_at_budgets_around_head_dim_and_its_row_limit(dtype, d, budgets):
+    # full spans with few rows to spare, down to none (tiny pivots: the reflectors then decide): delta = 0 bit for bit;
+    # one row short of head_dim: nothing to test
+    w = small("span", d=d, dtype=dtype, rank=2, caches=tuple((700, b) for b in budgets), n_outlier=3, seed=d + len(budgets))
+    outs, reps, _ = run_and_check(w)
+    for o, b in zip(outs, budgets):
+        assert all(dg["span_rank"] == min(b, d) for dg in P.parse_diag(o["diag"]))
+
+
 def test_budget_above_head_dim_full_rank_is_bit_exact_eviction():
     w = small("full", d=64, dtype="bf16", rank=3, caches=((400, 90),))
     outs, reps, _ = run_and_check(w)
