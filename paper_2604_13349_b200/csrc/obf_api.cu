@@ -67,7 +67,7 @@ static inline void mark(cudaStream_t st, const char *name)
 static inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 struct Layout {
-    size_t off_status, off_scores, off_keep, off_stats, off_sums, off_lscores, off_scores2;
+    size_t off_status, off_scores, off_keep, off_stats, off_sums, off_lscores, clear_end;
     size_t off_gram_d, off_gram_k, off_uvec, off_delta, off_hflag, off_svec, off_assign;
     size_t total;
     int splits;
@@ -86,7 +86,7 @@ struct Layout {
     int sc_nq, sc_subs, sc_blocks, sc_rounds, sc_qt;
     int sc_team[OBF_MAX_CACHES], sc_hpr[OBF_MAX_CACHES], sc_round_base[OBF_MAX_CACHES];
     size_t sc_part_off[OBF_MAX_CACHES], sc_part_pairs;
-    size_t off_sc_part, off_sc_head, off_sc_sync;
+    size_t off_sc_part;
 };
 
 // Streaming multiprocessors of the current device (148 on a B200 when no device can be asked).
@@ -226,22 +226,18 @@ static void make_layout(const obf_params_t *p, const obf_cache_t *caches, int32_
         L.sc_part_pairs = pairs;
     }
     size_t o = 0;
+    // cleared before every call, in this order: the status word, the score kernel's chunk statistics and, where two query
+    // tiles add their masses up, the masses
     L.off_status = o; o += 256;
-    L.off_scores = o; o = align_up(o + tok * sizeof(float), 256);
+    L.off_sc_part = o; if (L.sc_on) o = align_up(o + L.sc_part_pairs * 2 * sizeof(float), 256);
+    L.off_scores = o; L.clear_end = o;
+    o = align_up(o + tok * sizeof(float), 256);
+    if (L.sc_on && L.sc_qt == 2) L.clear_end = o;
     L.off_keep = o;   o = align_up(o + tok, 256);
     L.off_stats = o;  o = align_up(o + (size_t)L.heads_total * n_q * 2 * sizeof(float), 256);
     L.off_sums = o;   o = align_up(o + (size_t)L.heads_total * 4 * sizeof(float), 256);
-    L.off_scores2 = o;
-    if (L.sc_on && L.sc_qt == 2) o = align_up(o + tok * sizeof(float), 256);
     L.off_lscores = o;
     if (p->flags & OBF_FLAG_LAYERWISE) o = align_up(o + tok / p->kv_heads * sizeof(float), 256);
-    L.off_sc_part = L.off_sc_head = L.off_sc_sync = o;
-    if (L.sc_on) {
-        L.off_sc_part = o; o = align_up(o + L.sc_part_pairs * 2 * sizeof(float), 256);
-        // sc_head and sc_cnt are cleared together before every launch
-        L.off_sc_head = o; o = align_up(o + (size_t)L.heads_total * L.sc_qt * 128 * sizeof(unsigned long long), 256);
-        L.off_sc_sync = o; o = align_up(o + (size_t)L.heads_total * L.sc_qt * sizeof(uint32_t), 256);
-    }
     L.off_gram_d = L.off_gram_k = L.off_uvec = L.off_delta = L.off_hflag = L.off_svec = o;
     if (rank > 0) {
         const size_t gsz = (size_t)L.heads_total * L.gram_slots * d * d * sizeof(float);
@@ -349,14 +345,15 @@ static obf_status_t launch_score_tc(const CallDev &cd, const Layout &L, cudaStre
     }
     const size_t smem = score_tc_smem_bytes<D>();
     OBF_CUDA_TRY(cudaFuncSetAttribute(k_score_tc<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    OBF_CUDA_TRY(cudaMemsetAsync(cd.sc_head, 0, (L.off_sc_sync - L.off_sc_head) + (size_t)cd.heads_total * L.sc_qt * sizeof(uint32_t), st));
     // The blocks of a head's team wait for one another, so the whole grid has to be resident at once: a
     // cooperative launch starts only when it is (the grid never exceeds one block per multiprocessor).
     void *args[2] = {const_cast<CallDev *>(&cd), &maps};
     OBF_CUDA_TRY(cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(k_score_tc<D>), dim3(L.sc_blocks), dim3(ST_THREADS),
                                              args, smem, st));
     mark(st, "k_score_tc");
-    if (L.sc_qt == 2) {
+    bool any_out = false;
+    for (int i = 0; i < cd.n_caches; ++i) any_out = any_out || cd.c[i].scores_out != nullptr;
+    if (L.sc_qt == 2 && any_out) {
         int T_max = 1;
         for (int i = 0; i < cd.n_caches; ++i) T_max = cd.c[i].T > T_max ? cd.c[i].T : T_max;
         dim3 gj((T_max + 255) / 256, cd.heads_total);
@@ -615,7 +612,6 @@ static obf_status_t run(const obf_params_t *p, const obf_cache_t *caches, int32_
     cd.stats = reinterpret_cast<float *>(ws + L.off_stats);
     cd.sums = reinterpret_cast<float *>(ws + L.off_sums);
     cd.lscores = reinterpret_cast<float *>(ws + L.off_lscores);
-    cd.scores2 = reinterpret_cast<float *>(ws + L.off_scores2);
     cd.kv_heads = p->kv_heads;
     cd.layerwise = (p->flags & OBF_FLAG_LAYERWISE) ? 1 : 0;
     cd.n_sink = (int32_t)OBF_FLAG_SINK_OF(p->flags);
@@ -630,8 +626,6 @@ static obf_status_t run(const obf_params_t *p, const obf_cache_t *caches, int32_
         cd.debug_drop_publish = 1;
     }
     cd.sc_part = reinterpret_cast<float *>(ws + L.off_sc_part);
-    cd.sc_head = reinterpret_cast<float *>(ws + L.off_sc_head);
-    cd.sc_cnt = reinterpret_cast<uint32_t *>(ws + L.off_sc_sync);
     cd.gram_d = reinterpret_cast<float *>(ws + L.off_gram_d);
     cd.gram_k = reinterpret_cast<float *>(ws + L.off_gram_k);
     cd.uvec = reinterpret_cast<float *>(ws + L.off_uvec);
@@ -642,7 +636,8 @@ static obf_status_t run(const obf_params_t *p, const obf_cache_t *caches, int32_
     cd.merge = (p->flags & OBF_FLAG_MERGE) ? 1 : 0;
 
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (!g_keep_status) OBF_CUDA_TRY(cudaMemsetAsync(cd.status, 0, 256, st));     // a slab of a larger job adds to the job's status
+    const size_t clear_from = g_keep_status ? 256 : 0;                           // a slab of a larger job adds to the job's status
+    if (L.clear_end > clear_from) OBF_CUDA_TRY(cudaMemsetAsync(ws + clear_from, 0, L.clear_end - clear_from, st));
     if (g_prof.active) cudaEventRecord(g_prof.ev[0], st);
 
     if (p->dtype == OBF_F32) {

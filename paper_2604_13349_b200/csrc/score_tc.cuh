@@ -12,8 +12,8 @@
 //       tensor-memory lanes: a thread owns one query and keeps its running maximum m_t
 //       and sum z_t = sum_j exp2(s_tj c - m_t) (c = log2(e)/sqrt(d)) over the block's
 //       chunk of keys; nothing crosses lanes.  Per (head, chunk) the block publishes
-//       (m_t, z_t); the last block of the head to arrive folds all chunks into
-//       M'_t = M_t + log2(Z_t) and publishes that.
+//       (m_t, z_t); every block of the head's team folds all of them into
+//       M'_t = M_t + log2(Z_t).
 //   pass B (pooling)     S^T = K_tile Q^T with the KEYS on the lanes: a thread owns one
 //       key and sums exp2(s_tj c - M'_t) = softmax_j over all queries of the tile;
 //       again nothing crosses lanes, and a key's mass is complete in one thread.
@@ -40,8 +40,8 @@
 // every form), a share of the exponentials evaluated as a polynomial on the FMA pipe (the
 // special-function unit is busy about half of the time: it is not what the warps wait for).
 // Warp 18 is the messenger: it publishes the chunk statistics the consumers leave in shared
-// memory, folds a head's chunks when its block is the last to arrive, and then fetches the
-// head's M' for the pooling pass a round later, so that the consumers never wait for global memory.
+// memory and collects and folds the team's into the head's M' for the pooling pass a round later, so
+// that the consumers never wait for global memory.
 #pragma once
 
 #include "tc_common.cuh"
@@ -66,6 +66,7 @@ static_assert(ST_STAGES == ST_TBUF, "a ring stage is released by the accumulator
 struct ScoreItem {
     int r, cache, lh, chunk, nt;   // r: round; lh: KV head in the cache; nt: tiles of the chunk that hold at least one key
     int lv, qt;                    // lv = lh * query tiles + qt: the (head, query tile) pair; qt: which 128 query rows
+    int nq;                        // query rows of the item (at most 128)
 };
 
 // What a block needs of a cache to find its work of a round (kept in shared memory).
@@ -91,6 +92,7 @@ __device__ __forceinline__ bool score_item(const CallDev &p, const ScoreTab *tab
     it.lv = lv;
     it.lh = p.sc_qt == 2 ? lv >> 1 : lv;
     it.qt = p.sc_qt == 2 ? lv & 1 : 0;
+    it.nq = min(128, p.n_q - 128 * it.qt);
     it.chunk = c.chunk;
     const int tiles = (c.T - c.chunk * ST_CHUNK + 127) >> 7;
     it.nt = tiles < ST_TILES ? tiles : ST_TILES;
@@ -129,13 +131,6 @@ __device__ __forceinline__ float lg2_approx(float x)
     float y;
     asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
-}
-
-__device__ __forceinline__ uint32_t atom_add_acq_rel_gpu(uint32_t *addr, uint32_t v)
-{
-    uint32_t old;
-    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(addr), "r"(v) : "memory");
-    return old;
 }
 
 __device__ __forceinline__ void st_relaxed_gpu_u64(unsigned long long *addr, unsigned long long v)
@@ -317,7 +312,6 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constan
         // issuers on separate warps overlap that.  Tiles are independent: different accumulators and ring
         // stages, and a commit only covers its own thread's instructions.
         if (lane == 0) {
-            constexpr uint32_t IDESC = tc::idesc_bf16(128, 128, 0, 0);
             const uint32_t me = warp == 1 ? 0u : 1u;
             uint32_t it = 0, nq[2] = {0u, 0u};
             const uint32_t ring_addr = tc::smem_u32(ring);
@@ -330,6 +324,8 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constan
                 ++nq[kind];
                 // operand descriptors: the k-step only moves the start address (in 16-byte units, low word)
                 const uint64_t dq0 = tc::smem_desc_sw128(tc::smem_u32(q_s + kind * ST_TILE_BYTES), 16, 1024);
+                // a pooling pass needs as many columns as the item has query rows, in pieces of 32
+                const uint32_t idesc = tc::idesc_bf16(128, kind == 0 ? 128u : (uint32_t)(item.nq + 31) & ~31u, 0, 0);
                 bool issued = false;
                 for (int t = 0; t < item.nt; ++t) {
                     const uint32_t ti = it + t;
@@ -349,7 +345,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constan
                         // 16 channels per instruction: 32 bytes along the swizzled row, next column block after 4 steps
                         constexpr uint32_t HALF16 = ST_BOX_BYTES >> 4;
                         const uint64_t off16 = (uint64_t)((kk >> 2) * HALF16 + (kk & 3) * 2);
-                        tc::umma_bf16(acc, da0 + off16, db0 + off16, IDESC, kk > 0 ? 1u : 0u);
+                        tc::umma_bf16(acc, da0 + off16, db0 + off16, idesc, kk > 0 ? 1u : 0u);
                     }
                     tc::umma_commit(&bar_t_full[tb]);
                     issued = true;
@@ -372,24 +368,30 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constan
         const float sc = ST_LOG2E * rsqrtf((float)D);
         uint32_t it = 0, n_a[2] = {0u, 0u}, n_b[2] = {0u, 0u};
 
-        // The four 32-column pieces of an accumulator tile, `work(piece, registers)` on each; the tile is handed
-        // back as soon as its last piece is in registers.
-        auto walk_tile = [&](uint32_t ti, auto &&work) {
+        // The first `pieces` (at most four) 32-column pieces of an accumulator tile, `work(piece, registers)` on each; the
+        // tile is handed back as soon as its last piece is in registers.  An item with fewer than 128 query rows (the
+        // second one of a head with, say, 160) costs by what it has: a warp whose lanes hold no query walks no piece of a
+        // statistics pass, and a pooling pass walks the columns that hold queries.
+        auto walk_tile = [&](uint32_t ti, int pieces, auto &&work) {
             const uint32_t tb = ti % ST_TBUF;
             tc::mbar_wait(&bar_t_full[tb], (ti / ST_TBUF) & 1u, wc, 20);
             tc::tc_fence_after();
             const uint32_t ta = tlane + tb * 128u;
             uint32_t rr[32];
 #pragma unroll 1
-            for (int pc = 0; pc < 4; ++pc) {
+            for (int pc = 0; pc < pieces; ++pc) {
                 tc::tmem_ld32(ta + 32u * pc, rr);
                 tc::tmem_ld_wait();
-                if (pc == 3) {
+                if (pc == pieces - 1) {
                     tc::tc_fence_before();
                     __syncwarp();
                     if (lane == 0) tc::mbar_arrive(&bar_t_empty[tb]);
                 }
                 work(pc, rr);
+            }
+            if (pieces == 0) {
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(&bar_t_empty[tb]);
             }
         };
 
@@ -408,7 +410,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constan
                     if ((int)(ti % ST_GROUPS) != grp) continue;
                     my_t = t;
                     const int key0 = item.chunk * ST_CHUNK + t * 128;                     // key of column 0 of the tile
-                    walk_tile(ti, [&](int pc, uint32_t (&rr)[32]) {
+                    walk_tile(ti, 32 * q < item.nq ? 4 : 0, [&](int pc, uint32_t (&rr)[32]) {
                         // two copies of the update: the one that masks missing keys runs for a head's ragged last tile only
                         const int k0 = key0 + 32 * pc;
                         if (k0 + 32 > T) stats_update<true>(rr, T - k0, sc, m, z);
@@ -433,19 +435,21 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constan
                 const int T = s_tab[item.cache].T, buf = (i - ST_LAG) & 1;
                 tc::mbar_wait(&bar_mp_ready[buf], n_b[buf] & 1u, wc, 20);
                 const float *mp = s_mp + buf * 128;
-                // with two query tiles per head each writes its own plane; a small kernel adds them up afterwards
-                float *dst = (item.qt ? p.scores2 : p.scores) + c.tok_off + (size_t)item.lh * T;
+                // with two query tiles per head the masses of both are added onto zeros: a sum of two terms, the same in
+                // either order
+                float *dst = p.scores + c.tok_off + (size_t)item.lh * T;
                 float *out = (c.scores_out && p.sc_qt == 1) ? c.scores_out + (size_t)item.lh * T : nullptr;
 #pragma unroll 1
                 for (int t = 0; t < item.nt; ++t) {
                     const uint32_t ti = it + t;
                     if ((int)(ti % ST_GROUPS) != grp) continue;
                     float a = 0.f;
-                    walk_tile(ti, [&](int pc, uint32_t (&rr)[32]) { a += pool_piece(rr, mp + 32 * pc, sc); });
+                    walk_tile(ti, (item.nq + 31) >> 5, [&](int pc, uint32_t (&rr)[32]) { a += pool_piece(rr, mp + 32 * pc, sc); });
                     const int j = item.chunk * ST_CHUNK + t * 128 + row;
                     if (j < T) {
                         if (!isfinite(a)) atomicOr(p.status, OBF_DEV_NONFINITE);
-                        dst[j] = a;
+                        if (p.sc_qt == 1) dst[j] = a;
+                        else atomicAdd(dst + j, a);
                         if (out) out[j] = a;
                     }
                 }
@@ -456,121 +460,123 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constan
             }
         }
     } else {
-        // ---------------- messenger: chunk statistics out, a head's chunks folded by the last block to arrive, M' in ----------------
+        // ---------------- messenger: the chunk's statistics out, the head's in, folded into M' ----------------
+        // Per (head, chunk, query) one 64-bit word, (maximum, sum): zero (as cleared before the launch) until it is
+        // published, never zero afterwards (the sum of a maximum's own exponential is one; a chunk without a finite logit
+        // has the maximum -inf or a NaN).  A word vouches for itself, so nothing is counted and nothing fenced: every
+        // block of a team polls the team's words and folds the head for itself, one trip through the L2 cache after the
+        // last one is written.  (Counting the blocks in, folding in the last one and polling its result took 13000 cycles
+        // a round, as long as the round's arithmetic.)
         uint32_t n_a[2] = {0u, 0u}, n_b[2] = {0u, 0u};
         for (int i = 0; i < R; ++i) {
             ScoreItem item;
             if (!score_item(p, s_tab, i, item)) continue;
             const CacheDev &c = p.c[item.cache];
-            const int buf = i & 1, team = c.sc_team;
-            const int g = c.head_base * p.sc_qt + item.lv;                     // index of the (head, query tile) pair
-            const int nq = min(128, p.n_q - 128 * item.qt);                    // query rows of this item
+            const int buf = i & 1, team = c.sc_team, nq = item.nq;
+            unsigned long long *words = reinterpret_cast<unsigned long long *>(p.sc_part) + (c.sc_part_off + (size_t)item.lv * team * 128);
             tc::mbar_wait(&bar_st_ready[buf], n_a[buf] & 1u, wc, 32);
-            float2 *partials = reinterpret_cast<float2 *>(p.sc_part) + (c.sc_part_off + ((size_t)item.lv * team + item.chunk) * 128);
+            {
+                float m[4][ST_TILES], z[4][ST_TILES];
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+#pragma unroll
+                    for (int e = 0; e < ST_TILES; ++e) {
+                        const int at = (buf * ST_TILES + e) * 128 + lane + 32 * k;
+                        m[k][e] = e < item.nt ? s_m[at] : -INFINITY;
+                        z[k][e] = e < item.nt ? s_z[at] : 0.f;
+                    }
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(&bar_st_free[buf]);
+                ++n_a[buf];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    float M = m[k][0], Z = 0.f;
+#pragma unroll
+                    for (int e = 1; e < ST_TILES; ++e) M = fmaxf(M, m[k][e]);
+                    const float Mf = fmaxf(M, -3e38f);                         // (-inf - -inf would be a NaN)
+#pragma unroll
+                    for (int e = 0; e < ST_TILES; ++e) Z += z[k][e] * ex2_approx(m[k][e] - Mf);
+                    const int t = lane + 32 * k;
+                    if (t < nq && !p.debug_drop_publish)
+                        st_relaxed_gpu_u64(words + (size_t)item.chunk * 128 + t, ((unsigned long long)__float_as_uint(Z) << 32) | __float_as_uint(M));
+                }
+            }
+            float M[4], Z[4], extra[4];
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
+                M[k] = -INFINITY;
+                Z[k] = 0.f;
                 const int t = lane + 32 * k;
-                const float *sm = s_m + buf * ST_TILES * 128 + t, *sz = s_z + buf * ST_TILES * 128 + t;
-                float M = sm[0];
-                for (int e = 1; e < item.nt; ++e) M = fmaxf(M, sm[e * 128]);
-                float Z = 0.f;
-                for (int e = 0; e < item.nt; ++e)
-                    if (sm[e * 128] > -INFINITY) Z += sz[e * 128] * ex2_approx(sm[e * 128] - M);
-                if (t < nq) __stcg(&partials[t], make_float2(M, Z));
+                extra[k] = (c.lse_extra && t < nq) ? c.lse_extra[(size_t)item.lh * p.n_q + 128 * item.qt + t] : -INFINITY;
             }
-            __syncwarp();
-            uint32_t last = 0u;
-            if (lane == 0) {
-                tc::mbar_arrive(&bar_st_free[buf]);
-                // the warp barrier orders the lanes' stores before this release; the acquire side mirrors it
-                last = (atom_add_acq_rel_gpu(&p.sc_cnt[g], 1u) == (uint32_t)(team - 1)) ? 1u : 0u;
-            }
-            last = __shfl_sync(0xffffffffu, last, 0);
-            ++n_a[buf];
-            if (last) {
-                // every lane reads other blocks' statistics below: each orders its own loads behind lane 0's acquire
-                asm volatile("fence.acq_rel.gpu;" ::: "memory");
-                // this block is the last of its head: fold all chunks, eight chunks of the lane's four queries per sweep
-                // (32 loads in flight: the fold is a few round trips long, whatever the team's size)
-                const float2 *hp = reinterpret_cast<const float2 *>(p.sc_part) + (c.sc_part_off + (size_t)item.lv * team * 128);
-                unsigned long long *words = reinterpret_cast<unsigned long long *>(p.sc_head) + (size_t)g * 128;
-                float M[4], Z[4];
+            bool gave_up = false;
+            // eight chunks of the lane's four queries per sweep: 32 loads in flight
+#pragma unroll 1
+            for (int c0 = 0; c0 < team && !gave_up; c0 += 8) {
+                unsigned long long w[4][8];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) { M[k] = -INFINITY; Z[k] = 0.f; }
-                for (int c0 = 0; c0 < team; c0 += 8) {
-                    float2 v[4][8];
+                for (int k = 0; k < 4; ++k)
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) w[k][e] = (c0 + e < team && lane + 32 * k < nq) ? 0ull : 0xff800000ull;   // (-inf, 0)
+                uint64_t t0 = 0ull;
+                for (;;) {
 #pragma unroll
                     for (int k = 0; k < 4; ++k)
 #pragma unroll
                         for (int e = 0; e < 8; ++e)
-                            v[k][e] = (c0 + e < team && lane + 32 * k < nq) ? __ldcg(&hp[(size_t)(c0 + e) * 128 + lane + 32 * k])
-                                                                               : make_float2(-INFINITY, 0.f);
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        float Mn = M[k];
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) Mn = fmaxf(Mn, v[k][e].x);
-                        if (Mn > -INFINITY) {
-                            Z[k] *= ex2_approx(M[k] - Mn);
-#pragma unroll
-                            for (int e = 0; e < 8; ++e)
-                                if (v[k][e].x > -INFINITY) Z[k] += v[k][e].y * ex2_approx(v[k][e].x - Mn);
-                            M[k] = Mn;
-                        }
-                    }
-                }
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const int t = lane + 32 * k;
-                    if (t >= nq) continue;
-                    // the keys outside the prompt take their share of the normaliser
-                    if (c.lse_extra) fold_lse_extra(c.lse_extra[(size_t)item.lh * p.n_q + 128 * item.qt + t], M[k], Z[k]);
-                    float mp = M[k] + lg2_approx(Z[k]);
-                    if (!(Z[k] > 0.f) || !isfinite(mp)) {
-                        atomicOr(p.status, OBF_DEV_NONFINITE);
-                        mp = __int_as_float(0x7fc00000);
-                    }
-                    // one 64-bit word per query: low = M'_t, high = 1 once it is valid
-                    if (!p.debug_drop_publish) st_relaxed_gpu_u64(words + t, (1ull << 32) | __float_as_uint(mp));
-                }
-            }
-            // M'_t of this head for the pooling pass one round on; the team has a round to get there
-            {
-                const int fb = i & 1;
-                if (n_b[fb] > 0) tc::mbar_wait(&bar_mp_free[fb], (n_b[fb] - 1) & 1u, wc, 32);
-                const unsigned long long *words = reinterpret_cast<const unsigned long long *>(p.sc_head) + (size_t)g * 128;
-                // the four words of this lane are polled together: one round trip, not four
-                unsigned long long v[4] = {0ull, 0ull, 0ull, 0ull};
-                const uint64_t t0 = tc::global_ns();
-                for (;;) {
+                            if (w[k][e] == 0ull) w[k][e] = ld_relaxed_gpu_u64(words + (size_t)(c0 + e) * 128 + lane + 32 * k);
                     bool all = true;
 #pragma unroll
                     for (int k = 0; k < 4; ++k)
-                        if (lane + 32 * k < nq && (v[k] >> 32) == 0ull) v[k] = ld_relaxed_gpu_u64(words + lane + 32 * k);
 #pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        if (lane + 32 * k < nq && (v[k] >> 32) == 0ull) all = false;
+                        for (int e = 0; e < 8; ++e) all = all && w[k][e] != 0ull;
                     // the warp leaves the loop as one: votes, not per-lane exits
-                    if (__all_sync(0xffffffffu, all) || __any_sync(0xffffffffu, *(volatile uint32_t *)&s_abort != 0u)) break;
-                    if (__any_sync(0xffffffffu, tc::global_ns() - t0 > p.wait_limit_ns)) {
+                    if (__all_sync(0xffffffffu, all)) break;
+                    const uint64_t now = tc::global_ns();
+                    if (t0 == 0ull) t0 = now;
+                    if (__any_sync(0xffffffffu, *(volatile uint32_t *)&s_abort != 0u || now - t0 > p.wait_limit_ns)) {
                         if (lane == 0) {
+                            if (s_abort == 0u) atomicOr(p.status, OBF_DEV_TIMEOUT);
                             s_abort = 1u;
-                            atomicOr(p.status, OBF_DEV_TIMEOUT);
                         }
+                        gave_up = true;
                         break;
                     }
                     __nanosleep(64);
                 }
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    const int t = lane + 32 * k;
-                    // exp2(-inf) = 0 for padding columns
-                    s_mp[fb * 128 + t] = t < nq ? __uint_as_float((uint32_t)v[k]) : INFINITY;
+                    float Mn = M[k];
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) Mn = fmaxf(Mn, __uint_as_float((uint32_t)w[k][e]));
+                    const float Mf = fmaxf(Mn, -3e38f);
+                    Z[k] *= ex2_approx(M[k] - Mf);
+#pragma unroll
+                    for (int e = 0; e < 8; ++e)
+                        Z[k] += __uint_as_float((uint32_t)(w[k][e] >> 32)) * ex2_approx(__uint_as_float((uint32_t)w[k][e]) - Mf);
+                    M[k] = Mn;
                 }
-                __syncwarp();
-                if (lane == 0) tc::mbar_arrive(&bar_mp_ready[fb]);
-                ++n_b[fb];
             }
+            if (n_b[buf] > 0) tc::mbar_wait(&bar_mp_free[buf], (n_b[buf] - 1) & 1u, wc, 32);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int t = lane + 32 * k;
+                float mp = INFINITY;                                           // exp2(-inf) = 0 for padding columns
+                if (t < nq) {
+                    // the keys outside the prompt take their share of the normaliser
+                    fold_lse_extra(extra[k], M[k], Z[k]);
+                    mp = M[k] + lg2_approx(Z[k]);
+                    if (gave_up) mp = 0.f;
+                    else if (!(Z[k] > 0.f) || !isfinite(mp)) {
+                        if (item.chunk == 0) atomicOr(p.status, OBF_DEV_NONFINITE);
+                        mp = __int_as_float(0x7fc00000);
+                    }
+                }
+                s_mp[buf * 128 + t] = mp;
+            }
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&bar_mp_ready[buf]);
+            ++n_b[buf];
         }
     }
 
@@ -579,7 +585,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constan
     if (warp == 1) tc::tmem_dealloc(tmem, 512);
 }
 
-// Heads with two query tiles: the masses of the second tile's rows are added to the first tile's.
+// Heads with two query tiles (their masses are joined in the workspace) whose masses the caller wants: a copy.
 // grid = (ceil(T_max / 256), heads_total).
 __global__ void __launch_bounds__(256) k_score_join(const __grid_constant__ CallDev p)
 {
@@ -587,11 +593,7 @@ __global__ void __launch_bounds__(256) k_score_join(const __grid_constant__ Call
     locate(p, blockIdx.y, ci, lh);
     const CacheDev &c = p.c[ci];
     const int j = blockIdx.x * 256 + threadIdx.x;
-    if (j >= c.T) return;
-    const size_t e = c.tok_off + (size_t)lh * c.T + j;
-    const float a = p.scores[e] + p.scores2[e];
-    p.scores[e] = a;
-    if (c.scores_out) c.scores_out[(size_t)lh * c.T + j] = a;
+    if (j < c.T && c.scores_out) c.scores_out[(size_t)lh * c.T + j] = p.scores[c.tok_off + (size_t)lh * c.T + j];
 }
 
 }  // namespace obf
