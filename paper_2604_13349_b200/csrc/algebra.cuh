@@ -59,45 +59,10 @@ constexpr int JACOBI_MAX_SWEEPS = 30;
 constexpr int ALG_TRI_MAX_RANK = 8;     // up to this rank only rank + 1 eigenvalues and rank eigenvectors are computed
 constexpr float EIG_CLUSTER_TOL = 1e-3f; // eigenvalues closer than this (relative to the largest) are orthogonalised explicitly
 
-// ---- pairs of fp32 in one 64-bit register, for the two-wide FMA ------------------------------------
-typedef unsigned long long f32x2;
-
-__device__ __forceinline__ f32x2 pk(float a, float b)
-{
-    f32x2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ void upk(f32x2 v, float &a, float &b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
-{
-    f32x2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b)
-{
-    f32x2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
-{
-    f32x2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
 // a where the mask is all ones, b where it is zero.  (A conditional between array elements would be a conditional
 // address, and the array would have to live in memory.)
 __device__ __forceinline__ f32x2 sel2(f32x2 mask, f32x2 a, f32x2 b) { return b ^ ((a ^ b) & mask); }
 __device__ __forceinline__ f32x2 mask2(bool c) { return c ? ~0ull : 0ull; }
-__device__ __forceinline__ float sum2(f32x2 v)
-{
-    float a, b;
-    upk(v, a, b);
-    return a + b;
-}
-
 // Sums of N values per lane (a power of two) over runs of W lanes (W >= N): lane l of a run ends with the total of value
 // l / (W / N).  Half as many values travel at every step: about N shuffles instead of N log2(W).
 template <int N, int W>

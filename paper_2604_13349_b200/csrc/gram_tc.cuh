@@ -139,8 +139,7 @@ __global__ void __launch_bounds__(GT_THREADS, 3) k_gram_tc(const __grid_constant
                     if (!tc::mbar_wait(&bar_empty[s], ph ^ 1u, wc)) break;
                     tc::mbar_expect_tx(&bar_full[s], GT_TILE_BYTES);
                     const uint32_t dst = tc::smem_u32(tiles + s * GT_STAGE_BYTES);
-                    for (int h = 0; h < D / 64; ++h)
-                        tc::tma_load_3d(dst + h * GT_BLOCK_BYTES, map, &bar_full[s], 64 * h, (sub0 + t) * GT_TILE, lh);
+                    tc::tma_load_rows(dst, map, &bar_full[s], (sub0 + t) * GT_TILE, lh);
                 }
                 if (s_abort) break;
             }

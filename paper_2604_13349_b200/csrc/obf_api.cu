@@ -292,17 +292,17 @@ static EncodeTiledFn tensor_map_encoder()
     return fn;
 }
 
-// Tensor map of a bf16 array [heads, rows, d] for box_rows x 64-column boxes with the
-// 128-byte swizzle; rows past `rows` read as zero.
-static obf_status_t encode_rows_map(CUtensorMap *m, const void *ptr, uint64_t d, uint64_t rows, uint64_t heads, uint32_t box_rows = GT_TILE)
+// Tensor map of a bf16 array [heads, rows, d] as [heads][64-column blocks][rows][64]: a box is GT_TILE rows of all
+// blocks with the 128-byte swizzle, block after block; rows past `rows` read as zero.
+static obf_status_t encode_rows_map(CUtensorMap *m, const void *ptr, uint64_t d, uint64_t rows, uint64_t heads)
 {
     EncodeTiledFn enc = tensor_map_encoder();
     if (!enc) return OBF_ERR_CUDA;
-    cuuint64_t dims[3] = {d, rows, heads};
-    cuuint64_t strides[2] = {d * 2, rows * d * 2};
-    cuuint32_t box[3] = {64, (cuuint32_t)box_rows, 1};
-    cuuint32_t es[3] = {1, 1, 1};
-    const CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(ptr), dims, strides, box, es,
+    cuuint64_t dims[4] = {64, rows, d / 64, heads};
+    cuuint64_t strides[3] = {d * 2, 128, rows * d * 2};
+    cuuint32_t box[4] = {64, (cuuint32_t)GT_TILE, (cuuint32_t)(d / 64), 1};
+    cuuint32_t es[4] = {1, 1, 1, 1};
+    const CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(ptr), dims, strides, box, es,
                            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) {

@@ -26,10 +26,10 @@
 // of the L2 cache before its second visit).
 // The wait for M' is bounded like every other wait (tc_common.cuh).
 //
-// Block = 20 warps: warp 0 TMA producer (K tiles through a 4-stage ring, asked into L2 one
+// Block = 23 warps: warp 0 TMA producer (K tiles through a 4-stage ring, asked into L2 one
 // round ahead; Q of a pass is loaded while the pass before it runs, into the buffer of its
 // kind: one for the statistics passes, one for the pooling passes, which read Q again),
-// warps 1 and 19 MMA issuers, alternate tiles (accumulators in a 4-deep ring of 128 tensor-memory columns),
+// warps 1 and 22 MMA issuers, alternate tiles (accumulators in a 4-deep ring of 128 tensor-memory columns),
 // warps 2..17 consumers in four groups of four, group g taking the tiles with index g (mod 4), so
 // that every scheduler holds one warp of each group and the four are at different points of
 // their tiles: a warp owns the 32 tensor-memory lanes of its quarter and walks the 128 columns
@@ -39,8 +39,8 @@
 // piece in flight behind the arithmetic of the piece before it (the unrolled code was slower in
 // every form), a share of the exponentials evaluated as a polynomial on the FMA pipe (the
 // special-function unit is busy about half of the time: it is not what the warps wait for).
-// Warp 18 is the messenger: it publishes the chunk statistics the consumers leave in shared
-// memory and collects and folds the team's into the head's M' for the pooling pass a round later, so
+// Warps 18..21 are the messengers, a query per lane: they publish the chunk statistics the consumers leave in
+// shared memory and collect and fold the team's into the head's M' for the pooling pass a round later, so
 // that the consumers never wait for global memory.
 #pragma once
 
@@ -56,7 +56,8 @@ constexpr int ST_LAG = 1;                           // rounds between a chunk's 
 constexpr int ST_BOX_BYTES = 128 * 128;              // a 64-channel column block of a tile: 128 rows of 128 bytes
 constexpr int ST_GROUPS = 4;                        // consumer groups of four warps, one accumulator tile each
 constexpr int ST_CONSUMERS = ST_GROUPS * 128;
-constexpr int ST_THREADS = 64 + ST_CONSUMERS + 64;
+constexpr int ST_MESSENGERS = 4;                    // messenger warps, a query per lane
+constexpr int ST_THREADS = 64 + ST_CONSUMERS + 32 * ST_MESSENGERS + 32;
 constexpr int ST_MAX_NQ = 256;                      // two query tiles of 128 rows
 constexpr float ST_LOG2E = 1.4426950408889634f;
 template <int D>
@@ -145,70 +146,82 @@ __device__ __forceinline__ unsigned long long ld_relaxed_gpu_u64(const unsigned 
     return v;
 }
 
-// Pass A on one thread's 32 logits of a piece: running maximum m (log2 domain) and sum z of
-// exp2(s c - m) of one query.  With MASKED only the first n_valid columns are keys.
+__device__ __forceinline__ float max3(float a, float b, float c)
+{
+    float r;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+
+// Two logits at a time: exp2(s c + o), added to an accumulator pair.  The multiply-add and the sum are two-wide.
+__device__ __forceinline__ void exp2_add(f32x2 &acc, uint32_t s0, uint32_t s1, f32x2 sc, f32x2 o)
+{
+    float a, b;
+    upk(fma2(pk(__uint_as_float(s0), __uint_as_float(s1)), sc, o), a, b);
+    acc = add2(acc, pk(ex2_approx(a), ex2_approx(b)));
+}
+
+// Pass A on one thread's 16 logits of a piece: reference m (log2 domain) and sum z of exp2(s c - m) of one query.  The
+// reference is the largest logit up to the last piece that exceeded it by 64: no more is needed for a sum that neither
+// overflows nor loses its small terms, and the step that changes it is then a branch hardly ever taken.  z >= 1 wherever a
+// finite logit was met.  With MASKED only the first n_valid columns are keys.
 template <bool MASKED>
-__device__ __forceinline__ void stats_update(uint32_t (&rr)[32], int n_valid, float sc, float &m, float &z)
+__device__ __forceinline__ void stats_update(uint32_t (&rr)[16], int n_valid, float sc, float &m, float &z)
 {
     if (MASKED) {
 #pragma unroll
-        for (int e = 0; e < 32; ++e)
+        for (int e = 0; e < 16; ++e)
             if (e >= n_valid) rr[e] = 0xff800000u;                                     // -inf: no such key
     }
-    float t0 = __uint_as_float(rr[0]), t1 = __uint_as_float(rr[1]);
-    float t2 = __uint_as_float(rr[2]), t3 = __uint_as_float(rr[3]);
+    float t0 = fmaxf(__uint_as_float(rr[0]), __uint_as_float(rr[1])), t1 = fmaxf(__uint_as_float(rr[2]), __uint_as_float(rr[3]));
 #pragma unroll
-    for (int e = 4; e < 32; e += 4) {
-        t0 = fmaxf(t0, __uint_as_float(rr[e]));
-        t1 = fmaxf(t1, __uint_as_float(rr[e + 1]));
-        t2 = fmaxf(t2, __uint_as_float(rr[e + 2]));
-        t3 = fmaxf(t3, __uint_as_float(rr[e + 3]));
+    for (int e = 4; e < 16; e += 4) {
+        t0 = max3(t0, __uint_as_float(rr[e]), __uint_as_float(rr[e + 1]));
+        t1 = max3(t1, __uint_as_float(rr[e + 2]), __uint_as_float(rr[e + 3]));
     }
-    const float mn = fmaxf(m, fmaxf(fmaxf(t0, t1), fmaxf(t2, t3)) * sc);
-    if (mn > -INFINITY) {
-        float z0 = 0.f, z1 = 0.f, z2 = 0.f, z3 = 0.f;
+    const float t = fmaxf(t0, t1) * sc;
+    if (t > m + 64.f) {
+        z *= ex2_approx(m - t);                                                        // (0 * exp2(-inf) at first)
+        m = t;
+    }
+    const float mf = fmaxf(m, -3e38f);                                                 // (no key yet: -inf - -inf would be a NaN)
+    const f32x2 sc2 = pk(sc, sc), o = pk(-mf, -mf);
+    f32x2 z0 = 0ull, z1 = 0ull;
 #pragma unroll
-        for (int e = 0; e < 32; e += 4) {
-            z0 += ex2_approx(fmaf(__uint_as_float(rr[e]), sc, -mn));
-            z1 += ex2_approx(fmaf(__uint_as_float(rr[e + 1]), sc, -mn));
-            z2 += ex2_approx(fmaf(__uint_as_float(rr[e + 2]), sc, -mn));
-            z3 += ex2_approx(fmaf(__uint_as_float(rr[e + 3]), sc, -mn));
-        }
-        z = z * ex2_approx(m - mn) + ((z0 + z1) + (z2 + z3));
-        m = mn;
+    for (int e = 0; e < 16; e += 4) {
+        exp2_add(z0, rr[e], rr[e + 1], sc2, o);
+        exp2_add(z1, rr[e + 2], rr[e + 3], sc2, o);
     }
+    z += sum2(add2(z0, z1));
 }
 
-// Pass B on one thread's 32 logits of a piece: the softmax weights of one key under 32 queries, added up.
-// mp: M'_t of those queries (shared memory, the same address for every lane).
-__device__ __forceinline__ float pool_piece(const uint32_t (&rr)[32], const float *mp, float sc)
+// Pass B on one thread's 16 logits of a piece: the softmax weights of one key under 16 queries, added to a0, a1.
+// mp: -M'_t of those queries (shared memory, the same address for every lane).
+__device__ __forceinline__ void pool_piece(const uint32_t (&rr)[16], const float *mp, float sc, f32x2 &a0, f32x2 &a1)
 {
-    float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+    const f32x2 sc2 = pk(sc, sc);
 #pragma unroll
-    for (int e = 0; e < 32; e += 4) {
-        const float4 v = *reinterpret_cast<const float4 *>(mp + e);
-        a0 += ex2_approx(fmaf(__uint_as_float(rr[e]), sc, -v.x));
-        a1 += ex2_approx(fmaf(__uint_as_float(rr[e + 1]), sc, -v.y));
-        a2 += ex2_approx(fmaf(__uint_as_float(rr[e + 2]), sc, -v.z));
-        a3 += ex2_approx(fmaf(__uint_as_float(rr[e + 3]), sc, -v.w));
+    for (int e = 0; e < 16; e += 4) {
+        const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(mp + e);
+        exp2_add(a0, rr[e], rr[e + 1], sc2, v.x);
+        exp2_add(a1, rr[e + 2], rr[e + 3], sc2, v.y);
     }
-    return (a0 + a1) + (a2 + a3);
 }
 
 template <int D>
 __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constant__ CallDev p, const __grid_constant__ TcMaps tm)
 {
-    constexpr int ST_TILE_BYTES = 128 * D * 2, NBOX = D / 64;
+    constexpr int ST_TILE_BYTES = 128 * D * 2;
     extern __shared__ uint8_t st_smem_raw[];
     uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(st_smem_raw) + 1023) & ~(uintptr_t)1023);
     uint8_t *q_s = base;                                           // 2 x [128 x 128] bf16: Q of a statistics pass, Q of a pooling pass; two 64-column halves each
     uint8_t *ring = q_s + 2 * ST_TILE_BYTES;                       // ST_STAGES x 32 KiB
     float *s_m = reinterpret_cast<float *>(ring + ST_STAGES * ST_TILE_BYTES);   // [2][tile of the chunk][128 queries] tile maxima
     float *s_z = s_m + 2 * ST_GROUPS * 128;                        // [2][tile of the chunk][128 queries] tile sums
-    float *s_mp = s_z + 2 * ST_GROUPS * 128;                       // [2][128] M'_t of the head being pooled
+    float *s_mp = s_z + 2 * ST_GROUPS * 128;                       // [2][128] -M'_t of the head being pooled
     __shared__ uint64_t bar_q_full[2], bar_q_free[2], bar_full[ST_STAGES];
     __shared__ uint64_t bar_t_full[ST_TBUF], bar_t_empty[ST_TBUF];
-    __shared__ uint64_t bar_st_ready[2], bar_st_free[2], bar_mp_ready[2], bar_mp_free[2];
+    __shared__ uint64_t bar_st_ready[2], bar_mp_ready[2];
     __shared__ ScoreTab s_tab[OBF_MAX_CACHES];
     __shared__ uint32_t s_tmem, s_abort;
 
@@ -226,9 +239,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constan
         }
         for (int b = 0; b < 2; ++b) {
             tc::mbar_init(&bar_st_ready[b], ST_CONSUMERS / 32);
-            tc::mbar_init(&bar_st_free[b], 1);
-            tc::mbar_init(&bar_mp_ready[b], 1);
-            tc::mbar_init(&bar_mp_free[b], ST_CONSUMERS / 32);
+            tc::mbar_init(&bar_mp_ready[b], ST_MESSENGERS);
         }
         tc::mbar_init_fence();
     }
@@ -258,8 +269,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constan
                 if (nq[kind] > 0 && !tc::mbar_wait(&bar_q_free[kind], (nq[kind] - 1) & 1u, wc, 64)) return false;
                 const uint32_t qdst = tc::smem_u32(q_s + kind * ST_TILE_BYTES);
                 tc::mbar_expect_tx(&bar_q_full[kind], ST_TILE_BYTES);
-                for (int h = 0; h < NBOX; ++h)                                   // rows past n_q read as zero
-                    tc::tma_load_3d(qdst + h * ST_BOX_BYTES, &tm.b[item.cache], &bar_q_full[kind], 64 * h, item.qt * 128, item.lh);
+                tc::tma_load_rows(qdst, &tm.b[item.cache], &bar_q_full[kind], item.qt * 128, item.lh);      // rows past n_q read as zero
                 ++nq[kind];
                 return true;
             };
@@ -273,9 +283,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constan
                     // the next statistics pass reads its tiles from HBM: ask for them now
                     ScoreItem nx;
                     if (item.r + 1 < R && score_item(p, s_tab, item.r + 1, nx)) {
-                        for (int t = 0; t < nx.nt; ++t)
-                            for (int h = 0; h < NBOX; ++h)
-                                tc::tma_prefetch_l2_3d(&tm.a[nx.cache], 64 * h, nx.chunk * ST_CHUNK + t * 128, nx.lh);
+                        for (int t = 0; t < nx.nt; ++t) tc::tma_prefetch_rows(&tm.a[nx.cache], nx.chunk * ST_CHUNK + t * 128, nx.lh);
                     }
                 }
                 for (int t = 0; t < item.nt; ++t, ++it) {
@@ -289,8 +297,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constan
                     tc::mbar_expect_tx(&bar_full[s], ST_TILE_BYTES);
                     const uint32_t dst = tc::smem_u32(ring + s * ST_TILE_BYTES);
                     const int row0 = item.chunk * ST_CHUNK + t * 128;
-                    for (int h = 0; h < NBOX; ++h)
-                        tc::tma_load_3d(dst + h * ST_BOX_BYTES, &tm.a[item.cache], &bar_full[s], 64 * h, row0, item.lh);
+                    tc::tma_load_rows(dst, &tm.a[item.cache], &bar_full[s], row0, item.lh);
                 }
                 if (dead) break;
                 // Q of the next pass, while the tiles just asked for are worked on
@@ -366,28 +373,34 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constan
         const int row = q * 32 + lane;                 // lane of the accumulator tile: a query (pass A) or a key (pass B)
         const uint32_t tlane = tmem + ((uint32_t)(q * 32) << 16);
         const float sc = ST_LOG2E * rsqrtf((float)D);
-        uint32_t it = 0, n_a[2] = {0u, 0u}, n_b[2] = {0u, 0u};
+        uint32_t it = 0, n_b[2] = {0u, 0u};
 
-        // The first `pieces` (at most four) 32-column pieces of an accumulator tile, `work(piece, registers)` on each; the
-        // tile is handed back as soon as its last piece is in registers.  An item with fewer than 128 query rows (the
-        // second one of a head with, say, 160) costs by what it has: a warp whose lanes hold no query walks no piece of a
-        // statistics pass, and a pooling pass walks the columns that hold queries.
+        // The first `pieces` 32-column pieces of an accumulator tile (at most four), `work(half piece, registers)` on each 16
+        // columns while the next 16 are on their way; the tile is handed back as soon as its last columns are in
+        // registers.  An item with fewer than 128 query rows (the second one of a head with, say, 160) costs by what it
+        // has: a warp whose lanes hold no query walks no piece of a statistics pass, and a pooling pass walks the columns
+        // that hold queries.
         auto walk_tile = [&](uint32_t ti, int pieces, auto &&work) {
             const uint32_t tb = ti % ST_TBUF;
             tc::mbar_wait(&bar_t_full[tb], (ti / ST_TBUF) & 1u, wc, 20);
             tc::tc_fence_after();
             const uint32_t ta = tlane + tb * 128u;
-            uint32_t rr[32];
+            uint32_t ra[16], rb[16];
+            if (pieces > 0) tc::tmem_ld16(ta, ra);
 #pragma unroll 1
             for (int pc = 0; pc < pieces; ++pc) {
-                tc::tmem_ld32(ta + 32u * pc, rr);
-                tc::tmem_ld_wait();
-                if (pc == pieces - 1) {
+                tc::tmem_ld_wait16(ra);
+                tc::tmem_ld16(ta + 32u * pc + 16u, rb);
+                work(2 * pc, ra);
+                tc::tmem_ld_wait16(rb);
+                if (pc + 1 < pieces) {
+                    tc::tmem_ld16(ta + 32u * pc + 32u, ra);
+                } else {
                     tc::tc_fence_before();
                     __syncwarp();
                     if (lane == 0) tc::mbar_arrive(&bar_t_empty[tb]);
                 }
-                work(pc, rr);
+                work(2 * pc + 1, rb);
             }
             if (pieces == 0) {
                 __syncwarp();
@@ -395,68 +408,65 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constan
             }
         };
 
+        ScoreItem item, prev;
+        bool have = false, have_prev = false;
         for (int i = 0; i < R + ST_LAG; ++i) {
+            static_assert(ST_LAG == 1, "the item pooled is the one of the round before");
+            prev = item;
+            have_prev = have;
             // ======== pass A of round i: maximum and sum per query over the keys of this group's tiles ========
-            ScoreItem item;
-            if (i < R && score_item(p, s_tab, i, item)) {
+            have = i < R && score_item(p, s_tab, i, item);
+            if (have) {
                 const int T = s_tab[item.cache].T, buf = i & 1;
                 // a chunk has at most as many tiles as there are groups: this group meets at most one of them
                 static_assert(ST_GROUPS == ST_TILES, "one tile of a chunk per consumer group");
+                const int my_t = (int)((uint32_t)(grp - (int)it) % ST_GROUPS);
                 float m = -INFINITY, z = 0.f;
-                int my_t = -1;
-#pragma unroll 1
-                for (int t = 0; t < item.nt; ++t) {
-                    const uint32_t ti = it + t;
-                    if ((int)(ti % ST_GROUPS) != grp) continue;
-                    my_t = t;
-                    const int key0 = item.chunk * ST_CHUNK + t * 128;                     // key of column 0 of the tile
-                    walk_tile(ti, 32 * q < item.nq ? 4 : 0, [&](int pc, uint32_t (&rr)[32]) {
+                if (my_t < item.nt) {
+                    const int key0 = item.chunk * ST_CHUNK + my_t * 128;                  // key of column 0 of the tile
+                    walk_tile(it + my_t, 32 * q < item.nq ? 4 : 0, [&](int hp, uint32_t (&rr)[16]) {
                         // two copies of the update: the one that masks missing keys runs for a head's ragged last tile only
-                        const int k0 = key0 + 32 * pc;
-                        if (k0 + 32 > T) stats_update<true>(rr, T - k0, sc, m, z);
-                        else stats_update<false>(rr, 32, sc, m, z);
+                        const int k0 = key0 + 16 * hp;
+                        if (k0 + 16 > T) stats_update<true>(rr, T - k0, sc, m, z);
+                        else stats_update<false>(rr, 16, sc, m, z);
                     });
-                }
-                it += item.nt;
-                // hand (m, z) of the tile to the messenger, filed under the tile's place in the chunk: the messenger
-                // merges a chunk's tiles in that order whichever groups worked on them
-                if (n_a[buf] > 0) tc::mbar_wait(&bar_st_free[buf], (n_a[buf] - 1) & 1u, wc, 20);
-                if (my_t >= 0) {
+                    // hand (m, z) of the tile to the messengers, filed under the tile's place in the chunk: they merge a
+                    // chunk's tiles in that order whichever groups worked on them.  (The buffer is free: what the
+                    // messengers made of its last contents has been waited for in the pooling pass since.)
                     s_m[(buf * ST_TILES + my_t) * 128 + row] = m;
                     s_z[(buf * ST_TILES + my_t) * 128 + row] = z;
                 }
-                __syncwarp();
-                if (lane == 0) tc::mbar_arrive(&bar_st_ready[buf]);
-                ++n_a[buf];
-            }
-            // ======== pass B of round i - ST_LAG: pooled mass per key over all queries of the tile ========
-            if (i >= ST_LAG && score_item(p, s_tab, i - ST_LAG, item)) {
-                const CacheDev &c = p.c[item.cache];
-                const int T = s_tab[item.cache].T, buf = (i - ST_LAG) & 1;
-                tc::mbar_wait(&bar_mp_ready[buf], n_b[buf] & 1u, wc, 20);
-                const float *mp = s_mp + buf * 128;
-                // with two query tiles per head the masses of both are added onto zeros: a sum of two terms, the same in
-                // either order
-                float *dst = p.scores + c.tok_off + (size_t)item.lh * T;
-                float *out = (c.scores_out && p.sc_qt == 1) ? c.scores_out + (size_t)item.lh * T : nullptr;
-#pragma unroll 1
-                for (int t = 0; t < item.nt; ++t) {
-                    const uint32_t ti = it + t;
-                    if ((int)(ti % ST_GROUPS) != grp) continue;
-                    float a = 0.f;
-                    walk_tile(ti, (item.nq + 31) >> 5, [&](int pc, uint32_t (&rr)[32]) { a += pool_piece(rr, mp + 32 * pc, sc); });
-                    const int j = item.chunk * ST_CHUNK + t * 128 + row;
-                    if (j < T) {
-                        if (!isfinite(a)) atomicOr(p.status, OBF_DEV_NONFINITE);
-                        if (p.sc_qt == 1) dst[j] = a;
-                        else atomicAdd(dst + j, a);
-                        if (out) out[j] = a;
-                    }
-                }
                 it += item.nt;
                 __syncwarp();
-                if (lane == 0) tc::mbar_arrive(&bar_mp_free[buf]);
+                if (lane == 0) tc::mbar_arrive(&bar_st_ready[buf]);
+            }
+            // ======== pass B of the round before: pooled mass per key over all queries of the tile ========
+            if (have_prev) {
+                const CacheDev &c = p.c[prev.cache];
+                const int T = s_tab[prev.cache].T, buf = (i - 1) & 1;
+                tc::mbar_wait(&bar_mp_ready[buf], n_b[buf] & 1u, wc, 20);
                 ++n_b[buf];
+                const float *mp = s_mp + buf * 128;
+                const int my_t = (int)((uint32_t)(grp - (int)it) % ST_GROUPS);
+                if (my_t < prev.nt) {
+                    f32x2 a0 = 0ull, a1 = 0ull;
+                    walk_tile(it + my_t, (prev.nq + 31) >> 5, [&](int hp, uint32_t (&rr)[16]) { pool_piece(rr, mp + 16 * hp, sc, a0, a1); });
+                    const float a = sum2(add2(a0, a1));
+                    const int j = prev.chunk * ST_CHUNK + my_t * 128 + row;
+                    if (j < T) {
+                        // with two query tiles per head the masses of both are added onto zeros: a sum of two terms, the
+                        // same in either order
+                        float *dst = p.scores + c.tok_off + (size_t)prev.lh * T;
+                        if (!isfinite(a)) atomicOr(p.status, OBF_DEV_NONFINITE);
+                        if (p.sc_qt == 1) {
+                            dst[j] = a;
+                            if (c.scores_out) c.scores_out[(size_t)prev.lh * T + j] = a;
+                        } else {
+                            atomicAdd(dst + j, a);
+                        }
+                    }
+                }
+                it += prev.nt;
             }
         }
     } else {
@@ -467,116 +477,89 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constan
         // block of a team polls the team's words and folds the head for itself, one trip through the L2 cache after the
         // last one is written.  (Counting the blocks in, folding in the last one and polling its result took 13000 cycles
         // a round, as long as the round's arithmetic.)
-        uint32_t n_a[2] = {0u, 0u}, n_b[2] = {0u, 0u};
+        uint32_t n_a[2] = {0u, 0u};
+        const int t = (warp - 2 - ST_CONSUMERS / 32) * 32 + lane;                  // this lane's query
         for (int i = 0; i < R; ++i) {
             ScoreItem item;
             if (!score_item(p, s_tab, i, item)) continue;
             const CacheDev &c = p.c[item.cache];
-            const int buf = i & 1, team = c.sc_team, nq = item.nq;
-            unsigned long long *words = reinterpret_cast<unsigned long long *>(p.sc_part) + (c.sc_part_off + (size_t)item.lv * team * 128);
-            tc::mbar_wait(&bar_st_ready[buf], n_a[buf] & 1u, wc, 32);
+            const int buf = i & 1, team = c.sc_team;
+            const bool mine = t < item.nq;
+            unsigned long long *words = reinterpret_cast<unsigned long long *>(p.sc_part) + (c.sc_part_off + (size_t)item.lv * team * 128) + t;
+            const float extra = (c.lse_extra && mine) ? c.lse_extra[(size_t)item.lh * p.n_q + 128 * item.qt + t] : -INFINITY;
+            tc::mbar_wait(&bar_st_ready[buf], n_a[buf] & 1u, wc, 20);
+            float M = -INFINITY, Z = 0.f;
             {
-                float m[4][ST_TILES], z[4][ST_TILES];
+                float m[ST_TILES], z[ST_TILES];
 #pragma unroll
-                for (int k = 0; k < 4; ++k)
-#pragma unroll
-                    for (int e = 0; e < ST_TILES; ++e) {
-                        const int at = (buf * ST_TILES + e) * 128 + lane + 32 * k;
-                        m[k][e] = e < item.nt ? s_m[at] : -INFINITY;
-                        z[k][e] = e < item.nt ? s_z[at] : 0.f;
-                    }
-                __syncwarp();
-                if (lane == 0) tc::mbar_arrive(&bar_st_free[buf]);
-                ++n_a[buf];
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    float M = m[k][0], Z = 0.f;
-#pragma unroll
-                    for (int e = 1; e < ST_TILES; ++e) M = fmaxf(M, m[k][e]);
-                    const float Mf = fmaxf(M, -3e38f);                         // (-inf - -inf would be a NaN)
-#pragma unroll
-                    for (int e = 0; e < ST_TILES; ++e) Z += z[k][e] * ex2_approx(m[k][e] - Mf);
-                    const int t = lane + 32 * k;
-                    if (t < nq && !p.debug_drop_publish)
-                        st_relaxed_gpu_u64(words + (size_t)item.chunk * 128 + t, ((unsigned long long)__float_as_uint(Z) << 32) | __float_as_uint(M));
+                for (int e = 0; e < ST_TILES; ++e) {
+                    const int at = (buf * ST_TILES + e) * 128 + t;
+                    m[e] = e < item.nt ? s_m[at] : -INFINITY;
+                    z[e] = e < item.nt ? s_z[at] : 0.f;
+                    M = fmaxf(M, m[e]);
                 }
-            }
-            float M[4], Z[4], extra[4];
+                ++n_a[buf];
+                const float Mf = fmaxf(M, -3e38f);                             // (-inf - -inf would be a NaN)
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                M[k] = -INFINITY;
-                Z[k] = 0.f;
-                const int t = lane + 32 * k;
-                extra[k] = (c.lse_extra && t < nq) ? c.lse_extra[(size_t)item.lh * p.n_q + 128 * item.qt + t] : -INFINITY;
+                for (int e = 0; e < ST_TILES; ++e) Z += z[e] * ex2_approx(m[e] - Mf);
+                if (mine && !p.debug_drop_publish)
+                    st_relaxed_gpu_u64(words + (size_t)item.chunk * 128, ((unsigned long long)__float_as_uint(Z) << 32) | __float_as_uint(M));
             }
+            M = -INFINITY;
+            Z = 0.f;
             bool gave_up = false;
-            // eight chunks of the lane's four queries per sweep: 32 loads in flight
+            // sixteen chunks in flight per sweep
 #pragma unroll 1
-            for (int c0 = 0; c0 < team && !gave_up; c0 += 8) {
-                unsigned long long w[4][8];
+            for (int c0 = 0; c0 < team && !gave_up; c0 += 16) {
+                unsigned long long w[16];
 #pragma unroll
-                for (int k = 0; k < 4; ++k)
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) w[k][e] = (c0 + e < team && lane + 32 * k < nq) ? 0ull : 0xff800000ull;   // (-inf, 0)
+                for (int e = 0; e < 16; ++e) w[e] = (c0 + e < team && mine) ? 0ull : 0xff800000ull;   // (-inf, 0)
                 uint64_t t0 = 0ull;
                 for (;;) {
 #pragma unroll
-                    for (int k = 0; k < 4; ++k)
-#pragma unroll
-                        for (int e = 0; e < 8; ++e)
-                            if (w[k][e] == 0ull) w[k][e] = ld_relaxed_gpu_u64(words + (size_t)(c0 + e) * 128 + lane + 32 * k);
+                    for (int e = 0; e < 16; ++e)
+                        if (w[e] == 0ull) w[e] = ld_relaxed_gpu_u64(words + (size_t)(c0 + e) * 128);
                     bool all = true;
 #pragma unroll
-                    for (int k = 0; k < 4; ++k)
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) all = all && w[k][e] != 0ull;
+                    for (int e = 0; e < 16; ++e) all = all && w[e] != 0ull;
                     // the warp leaves the loop as one: votes, not per-lane exits
                     if (__all_sync(0xffffffffu, all)) break;
                     const uint64_t now = tc::global_ns();
                     if (t0 == 0ull) t0 = now;
                     if (__any_sync(0xffffffffu, *(volatile uint32_t *)&s_abort != 0u || now - t0 > p.wait_limit_ns)) {
                         if (lane == 0) {
-                            if (s_abort == 0u) atomicOr(p.status, OBF_DEV_TIMEOUT);
                             s_abort = 1u;
+                            atomicOr(p.status, OBF_DEV_TIMEOUT);
                         }
                         gave_up = true;
                         break;
                     }
-                    __nanosleep(64);
+                    __nanosleep(32);
                 }
+                float Mn = M;
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    float Mn = M[k];
+                for (int e = 0; e < 16; ++e) Mn = fmaxf(Mn, __uint_as_float((uint32_t)w[e]));
+                const float Mf = fmaxf(Mn, -3e38f);
+                Z *= ex2_approx(M - Mf);
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) Mn = fmaxf(Mn, __uint_as_float((uint32_t)w[k][e]));
-                    const float Mf = fmaxf(Mn, -3e38f);
-                    Z[k] *= ex2_approx(M[k] - Mf);
-#pragma unroll
-                    for (int e = 0; e < 8; ++e)
-                        Z[k] += __uint_as_float((uint32_t)(w[k][e] >> 32)) * ex2_approx(__uint_as_float((uint32_t)w[k][e]) - Mf);
-                    M[k] = Mn;
+                for (int e = 0; e < 16; ++e) Z += __uint_as_float((uint32_t)(w[e] >> 32)) * ex2_approx(__uint_as_float((uint32_t)w[e]) - Mf);
+                M = Mn;
+            }
+            // (the buffer is free: every consumer has pooled with its last contents before it handed in this round's statistics)
+            float mp = INFINITY;                                               // exp2(-inf) = 0 for padding columns
+            if (mine) {
+                // the keys outside the prompt take their share of the normaliser
+                fold_lse_extra(extra, M, Z);
+                mp = M + lg2_approx(Z);
+                if (gave_up) mp = 0.f;
+                else if (!(Z > 0.f) || !isfinite(mp)) {
+                    if (item.chunk == 0) atomicOr(p.status, OBF_DEV_NONFINITE);
+                    mp = __int_as_float(0x7fc00000);
                 }
             }
-            if (n_b[buf] > 0) tc::mbar_wait(&bar_mp_free[buf], (n_b[buf] - 1) & 1u, wc, 32);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int t = lane + 32 * k;
-                float mp = INFINITY;                                           // exp2(-inf) = 0 for padding columns
-                if (t < nq) {
-                    // the keys outside the prompt take their share of the normaliser
-                    fold_lse_extra(extra[k], M[k], Z[k]);
-                    mp = M[k] + lg2_approx(Z[k]);
-                    if (gave_up) mp = 0.f;
-                    else if (!(Z[k] > 0.f) || !isfinite(mp)) {
-                        if (item.chunk == 0) atomicOr(p.status, OBF_DEV_NONFINITE);
-                        mp = __int_as_float(0x7fc00000);
-                    }
-                }
-                s_mp[buf * 128 + t] = mp;
-            }
+            s_mp[buf * 128 + t] = -mp;
             __syncwarp();
             if (lane == 0) tc::mbar_arrive(&bar_mp_ready[buf]);
-            ++n_b[buf];
         }
     }
 
