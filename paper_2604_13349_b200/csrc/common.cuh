@@ -69,6 +69,7 @@ struct CallDev {
     int32_t sc_rounds;        // rounds of the persistent score kernel
     int32_t sc_qt;            // tuned score kernel: 128-row query tiles per head (1 or 2)
     float *sc_part;           // per (head, chunk, query of 128): chunk maximum and normaliser as one 64-bit word, zero until published
+    int32_t sc_splits;        // shape-generic statistics kernel: key splits per (head, 64 queries)
     float eps;
     int32_t kv_heads;         // KV heads per layer
     int32_t layerwise;        // 1: one retained set per layer (masses summed over its KV heads)
@@ -85,7 +86,7 @@ struct CallDev {
     float *lscores;           // layerwise selector: [sum layers*T] masses summed over a layer's KV heads (cache offset tok_off / kv_heads)
     uint8_t *keep;            // [sum heads*T] 1 = retained
     int32_t *assign;          // [sum heads*T] cache-merging baseline: slot a deleted position is routed to, -1 = retained
-    float *stats;             // [heads_total, n_q, 2] softmax row max (log2 domain) and normaliser
+    float *stats;             // [heads_total, sc_splits, n_q, 2] softmax row max (log2 domain) and normaliser of a split's keys (shape-generic kernels)
     float *sums;              // [heads_total, 4] a_keep, a_del, kth, next
     float *gram_d;            // [heads_total, gram_slots, d, d] partial Gram of the deleted (gram_all: of all) values
     float *gram_k;            // [heads_total, gram_slots, d, d] partial Gram of retained values (shape-generic path only)
@@ -246,6 +247,39 @@ __device__ __forceinline__ float block_max(float v, float *red)
     t = red[0];
     __syncthreads();
     return t;
+}
+
+// 64 x 64 tile of dot products of D-channel rows on a 16 x 16 thread grid: thread (ty, tx) owns rows ty + 16 i of A and
+// tx + 16 j of B.  Rows lie TD_LD floats apart: four channels are read at a time, the sixteen rows of B that a warp's lanes
+// read then meet every bank twice, which is what 256 bytes cost, and the multiply-adds are two-wide (with scalar reads
+// every pair of multiply-adds waited for one).
+template <int D>
+constexpr int TD_LD = D + 4;
+
+template <int D>
+__device__ __forceinline__ void tile_dots(const float *A, const float *B, int ty, int tx, float (&acc)[4][4])
+{
+    f32x2 s[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) s[i][j] = 0ull;
+#pragma unroll 4
+    for (int c = 0; c < D; c += 4) {
+        ulonglong2 a[4], b[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const ulonglong2 *>(A + (ty + 16 * i) * TD_LD<D> + c);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) b[j] = *reinterpret_cast<const ulonglong2 *>(B + (tx + 16 * j) * TD_LD<D> + c);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) s[i][j] = fma2(a[i].y, b[j].y, fma2(a[i].x, b[j].x, s[i][j]));
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = sum2(s[i][j]);
 }
 
 // Folds the out-of-prompt softmax mass of a query row (natural log of the sum of exp(logit) over the keys outside

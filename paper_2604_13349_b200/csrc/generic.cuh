@@ -10,42 +10,21 @@ namespace obf {
 
 constexpr int SC_TILE = 64;           // queries x keys per score tile
 constexpr int SC_NT = 256;
+constexpr int SC_MAX_SPLITS = 32;     // key splits of the statistics kernel
 constexpr float LOG2E = 1.4426950408889634f;
 
 template <int D>
-constexpr size_t score_smem_bytes() { return 2 * SC_TILE * (D + 1) * sizeof(float) + 2 * SC_TILE * sizeof(float)
+constexpr size_t score_smem_bytes() { return 2 * SC_TILE * TD_LD<D> * sizeof(float) + 2 * SC_TILE * sizeof(float)
                                              + 16 * SC_TILE * sizeof(float); }
 
-// 64x64 tile of Q K^T on a 16x16 thread grid: thread (ty,tx) owns rows ty+16i, cols tx+16j.
-template <int D>
-__device__ __forceinline__ void score_tile(const float *Qs, const float *Ks, int ty, int tx, float (&acc)[4][4])
-{
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-#pragma unroll 4
-    for (int c = 0; c < D; ++c) {
-        float a[4], b[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) a[i] = Qs[(ty + 16 * i) * (D + 1) + c];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) b[j] = Ks[(tx + 16 * j) * (D + 1) + c];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-    }
-}
-
 // Step a1, first pass (Eq. 1): for every query row the running maximum of the
-// scaled logits (log2 domain) and the softmax normaliser over all T keys.
-// grid = (ceil(n_q/64), heads_total).
+// scaled logits (log2 domain) and the softmax normaliser over the keys of a split (the pooling kernel folds the splits).
+// grid = (ceil(n_q/64), heads_total, key splits).
 template <typename TIN, int D>
 __global__ void __launch_bounds__(SC_NT) k_score_stats(const __grid_constant__ CallDev p)
 {
-    extern __shared__ float sm[];
-    float *Qs = sm, *Ks = sm + SC_TILE * (D + 1);
+    extern __shared__ __align__(16) float sm[];
+    float *Qs = sm, *Ks = sm + SC_TILE * TD_LD<D>;
     int ci, lh;
     locate(p, blockIdx.y, ci, lh);
     const CacheDev &c = p.c[ci];
@@ -56,17 +35,19 @@ __global__ void __launch_bounds__(SC_NT) k_score_stats(const __grid_constant__ C
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
     const float sc = LOG2E * rsqrtf((float)D);
 
-    load_rows_f32<TIN, D, SC_NT>(Qs, D + 1, Qh, q0, n_q, SC_TILE);
+    load_rows_f32<TIN, D, SC_NT>(Qs, TD_LD<D>, Qh, q0, n_q, SC_TILE);
     float m[4], Z[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) { m[i] = -INFINITY; Z[i] = 0.f; }
 
-    for (int j0 = 0; j0 < T; j0 += SC_TILE) {
+    const int per = ((T + SC_TILE - 1) / SC_TILE + p.sc_splits - 1) / p.sc_splits * SC_TILE;
+    const int j_end = min(T, ((int)blockIdx.z + 1) * per);
+    for (int j0 = blockIdx.z * per; j0 < j_end; j0 += SC_TILE) {
         __syncthreads();
-        load_rows_f32<TIN, D, SC_NT>(Ks, D + 1, Kh, j0, T, SC_TILE);
+        load_rows_f32<TIN, D, SC_NT>(Ks, TD_LD<D>, Kh, j0, T, SC_TILE);
         __syncthreads();
         float acc[4][4];
-        score_tile<D>(Qs, Ks, ty, tx, acc);
+        tile_dots<D>(Qs, Ks, ty, tx, acc);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             float tm = -INFINITY;
@@ -92,8 +73,8 @@ __global__ void __launch_bounds__(SC_NT) k_score_stats(const __grid_constant__ C
         for (int i = 0; i < 4; ++i) {
             const int row = q0 + ty + 16 * i;
             if (row < n_q) {
-                if (c.lse_extra) fold_lse_extra(c.lse_extra[(size_t)lh * n_q + row], m[i], Z[i]);
-                float *st = p.stats + ((size_t)blockIdx.y * n_q + row) * 2;
+                if (c.lse_extra && blockIdx.z == 0) fold_lse_extra(c.lse_extra[(size_t)lh * n_q + row], m[i], Z[i]);
+                float *st = p.stats + (((size_t)blockIdx.y * p.sc_splits + blockIdx.z) * n_q + row) * 2;
                 st[0] = m[i];
                 st[1] = Z[i];
             }
@@ -106,9 +87,9 @@ __global__ void __launch_bounds__(SC_NT) k_score_stats(const __grid_constant__ C
 template <typename TIN, int D>
 __global__ void __launch_bounds__(SC_NT) k_score_pool(const __grid_constant__ CallDev p)
 {
-    extern __shared__ float sm[];
-    float *Qs = sm, *Ks = sm + SC_TILE * (D + 1);
-    float *rm = Ks + SC_TILE * (D + 1), *rz = rm + SC_TILE, *red = rz + SC_TILE;
+    extern __shared__ __align__(16) float sm[];
+    float *Qs = sm, *Ks = sm + SC_TILE * TD_LD<D>;
+    float *rm = Ks + SC_TILE * TD_LD<D>, *rz = rm + SC_TILE, *red = rz + SC_TILE;
     int ci, lh;
     locate(p, blockIdx.y, ci, lh);
     const CacheDev &c = p.c[ci];
@@ -120,20 +101,32 @@ __global__ void __launch_bounds__(SC_NT) k_score_pool(const __grid_constant__ Ca
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
     const float sc = LOG2E * rsqrtf((float)D);
 
-    load_rows_f32<TIN, D, SC_NT>(Ks, D + 1, Kh, j0, T, SC_TILE);
+    load_rows_f32<TIN, D, SC_NT>(Ks, TD_LD<D>, Kh, j0, T, SC_TILE);
     float colsum[4] = {0.f, 0.f, 0.f, 0.f};
     for (int q0 = 0; q0 < n_q; q0 += SC_TILE) {
         __syncthreads();
-        load_rows_f32<TIN, D, SC_NT>(Qs, D + 1, Qh, q0, n_q, SC_TILE);
+        load_rows_f32<TIN, D, SC_NT>(Qs, TD_LD<D>, Qh, q0, n_q, SC_TILE);
         if (threadIdx.x < SC_TILE) {
+            // the row's statistics over all keys, from the splits' (an empty split has the maximum -inf and the sum 0)
             const int row = q0 + threadIdx.x;
-            const float *st = p.stats + ((size_t)blockIdx.y * n_q + min(row, n_q - 1)) * 2;
-            rm[threadIdx.x] = row < n_q ? st[0] : 0.f;
-            rz[threadIdx.x] = row < n_q ? 1.0f / st[1] : 0.f;
+            const float2 *st = reinterpret_cast<const float2 *>(p.stats) + (size_t)blockIdx.y * p.sc_splits * n_q + min(row, n_q - 1);
+            float M = -INFINITY, Z = 0.f;
+            for (int s0 = 0; s0 < p.sc_splits; s0 += 4) {
+                float2 v[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) v[e] = s0 + e < p.sc_splits ? st[(size_t)(s0 + e) * n_q] : make_float2(-INFINITY, 0.f);
+                const float Mn = fmaxf(fmaxf(fmaxf(v[0].x, v[1].x), fmaxf(v[2].x, v[3].x)), M), Mf = fmaxf(Mn, -3e38f);
+                Z *= exp2f(M - Mf);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) Z = fmaf(v[e].y, exp2f(v[e].x - Mf), Z);
+                M = Mn;
+            }
+            rm[threadIdx.x] = row < n_q ? M : 0.f;
+            rz[threadIdx.x] = row < n_q ? 1.0f / Z : 0.f;
         }
         __syncthreads();
         float acc[4][4];
-        score_tile<D>(Qs, Ks, ty, tx, acc);
+        tile_dots<D>(Qs, Ks, ty, tx, acc);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const float mi = rm[ty + 16 * i], zi = rz[ty + 16 * i];
@@ -692,47 +685,77 @@ __global__ void __launch_bounds__(256) k_gram(const __grid_constant__ CallDev p)
     const int per = (tiles + p.splits - 1) / p.splits;
     const int t_begin = blockIdx.x * per, t_end = min(tiles, t_begin + per);
 
-    float accD[MT][MT], accK[MT][MT];
+    // accumulators as pairs of columns for the two-wide multiply-add
+    f32x2 accD[MT][MT / 2], accK[MT][MT / 2];
 #pragma unroll
     for (int i = 0; i < MT; ++i)
 #pragma unroll
-        for (int j = 0; j < MT; ++j) { accD[i][j] = 0.f; accK[i][j] = 0.f; }
+        for (int j = 0; j < MT / 2; ++j) { accD[i][j] = 0ull; accK[i][j] = 0ull; }
     float u = 0.f;
 
-    for (int t = t_begin; t < t_end; ++t) {
+    // a tile's rows are on their way in registers while the tile before is worked on
+    constexpr int VEC = 16 / (int)sizeof(TIN), CH = D / VEC, NPV = GR_ROWS * CH / 256;
+    static_assert(NPV >= 1 && GR_ROWS * CH % 256 == 0, "whole passes");
+    uint4 raw[NPV];
+    float a_next = 0.f;
+    int f_next = 2;
+    auto fetch = [&](int t) {
         const int r0 = t * GR_ROWS;
-        __syncthreads();
-        load_rows_f32<TIN, D, 256>(Vs, D, Vh, r0, T, GR_ROWS);
+#pragma unroll
+        for (int u2 = 0; u2 < NPV; ++u2) {
+            const int i = threadIdx.x + 256 * u2, r = i / CH, ch = i % CH;
+            raw[u2] = r0 + r < T ? *reinterpret_cast<const uint4 *>(Vh + (size_t)(r0 + r) * D + ch * VEC) : make_uint4(0u, 0u, 0u, 0u);
+        }
         if (threadIdx.x < GR_ROWS) {
             const int j = r0 + threadIdx.x;
-            Fs[threadIdx.x] = j < T ? (int)keep[j] : 2;
-            As[threadIdx.x] = j < T ? A[j] : 0.f;
+            f_next = j < T ? (int)keep[j] : 2;
+            a_next = j < T ? A[j] : 0.f;
         }
+    };
+    if (t_begin < t_end) fetch(t_begin);
+    for (int t = t_begin; t < t_end; ++t) {
         __syncthreads();
+#pragma unroll
+        for (int u2 = 0; u2 < NPV; ++u2) {
+            const int i = threadIdx.x + 256 * u2;
+            float x[VEC];
+            unpack16<TIN>(raw[u2], x);
+            float4 *dst = reinterpret_cast<float4 *>(Vs + i * VEC);
+#pragma unroll
+            for (int e = 0; e < VEC / 4; ++e) dst[e] = make_float4(x[4 * e], x[4 * e + 1], x[4 * e + 2], x[4 * e + 3]);
+        }
+        if (threadIdx.x < GR_ROWS) { Fs[threadIdx.x] = f_next; As[threadIdx.x] = a_next; }
+        __syncthreads();
+        if (t + 1 < t_end) fetch(t + 1);
 #pragma unroll 1
         for (int r = 0; r < GR_ROWS; ++r) {
             const int f = Fs[r];
             if (f == 2) break;
             if (f == 1 && !need_k) continue;
-            float a[MT], b[MT];
+            float a[MT];
+            f32x2 b[MT / 2];
 #pragma unroll
             for (int v = 0; v < NV; ++v) {
                 const float4 fa = *reinterpret_cast<const float4 *>(&Vs[r * D + v * 64 + ty * 4]);
-                const float4 fb = *reinterpret_cast<const float4 *>(&Vs[r * D + v * 64 + tx * 4]);
+                const ulonglong2 fb = *reinterpret_cast<const ulonglong2 *>(&Vs[r * D + v * 64 + tx * 4]);
                 a[4 * v] = fa.x; a[4 * v + 1] = fa.y; a[4 * v + 2] = fa.z; a[4 * v + 3] = fa.w;
-                b[4 * v] = fb.x; b[4 * v + 1] = fb.y; b[4 * v + 2] = fb.z; b[4 * v + 3] = fb.w;
+                b[2 * v] = fb.x; b[2 * v + 1] = fb.y;
             }
             if (f == 0) {
 #pragma unroll
-                for (int i = 0; i < MT; ++i)
+                for (int i = 0; i < MT; ++i) {
+                    const f32x2 ai = pk(a[i], a[i]);
 #pragma unroll
-                    for (int j = 0; j < MT; ++j) accD[i][j] = fmaf(a[i], b[j], accD[i][j]);
+                    for (int j = 0; j < MT / 2; ++j) accD[i][j] = fma2(ai, b[j], accD[i][j]);
+                }
                 if (threadIdx.x < D) u = fmaf(As[r], Vs[r * D + threadIdx.x], u);
             } else {
 #pragma unroll
-                for (int i = 0; i < MT; ++i)
+                for (int i = 0; i < MT; ++i) {
+                    const f32x2 ai = pk(a[i], a[i]);
 #pragma unroll
-                    for (int j = 0; j < MT; ++j) accK[i][j] = fmaf(a[i], b[j], accK[i][j]);
+                    for (int j = 0; j < MT / 2; ++j) accK[i][j] = fma2(ai, b[j], accK[i][j]);
+                }
             }
         }
     }
@@ -744,11 +767,8 @@ __global__ void __launch_bounds__(256) k_gram(const __grid_constant__ CallDev p)
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
             const int col = v * 64 + tx * 4;
-            *reinterpret_cast<float4 *>(&gd[row * D + col]) =
-                make_float4(accD[i][4 * v], accD[i][4 * v + 1], accD[i][4 * v + 2], accD[i][4 * v + 3]);
-            if (need_k)
-                *reinterpret_cast<float4 *>(&gk[row * D + col]) =
-                    make_float4(accK[i][4 * v], accK[i][4 * v + 1], accK[i][4 * v + 2], accK[i][4 * v + 3]);
+            *reinterpret_cast<ulonglong2 *>(&gd[row * D + col]) = make_ulonglong2(accD[i][2 * v], accD[i][2 * v + 1]);
+            if (need_k) *reinterpret_cast<ulonglong2 *>(&gk[row * D + col]) = make_ulonglong2(accK[i][2 * v], accK[i][2 * v + 1]);
         }
     }
     if (threadIdx.x < D) p.uvec[slot * D + threadIdx.x] = u;

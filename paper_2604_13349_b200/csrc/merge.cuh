@@ -12,7 +12,7 @@ namespace obf {
 constexpr int MG_TILE = 64;                 // fp32 keys: deleted positions per block, retained positions per inner tile
 
 template <int D>
-constexpr size_t merge_smem_bytes() { return (size_t)(2 * MG_TILE * (D + 1) + 2 * MG_TILE) * sizeof(float); }
+constexpr size_t merge_smem_bytes() { return (size_t)(2 * MG_TILE * TD_LD<D> + 2 * MG_TILE) * sizeof(float); }
 
 // Larger similarity wins, the lower slot among equals.
 __device__ __forceinline__ void merge_better(float &best, int &best_r, float s, int r)
@@ -26,8 +26,8 @@ __device__ __forceinline__ void merge_better(float &best, int &best_r, float s, 
 template <typename TIN, int D>
 __global__ void __launch_bounds__(256) k_merge_assign(const __grid_constant__ CallDev p)
 {
-    constexpr int LD = D + 1;
-    extern __shared__ float mg_sm[];
+    constexpr int LD = TD_LD<D>;
+    extern __shared__ __align__(16) float mg_sm[];
     float *Kj = mg_sm, *Kt = Kj + MG_TILE * LD, *inv_j = Kt + MG_TILE * LD, *inv_t = inv_j + MG_TILE;
     int ci, lh;
     locate(p, blockIdx.y, ci, lh);
@@ -63,20 +63,7 @@ __global__ void __launch_bounds__(256) k_merge_assign(const __grid_constant__ Ca
         inv_norms(Kt, inv_t, k - r0);
         __syncthreads();
         float acc[4][4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int jj = 0; jj < 4; ++jj) acc[i][jj] = 0.f;
-#pragma unroll 4
-        for (int e = 0; e < D; ++e) {
-            float a[4], b[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) { a[i] = Kj[(ty + 16 * i) * LD + e]; b[i] = Kt[(tx + 16 * i) * LD + e]; }
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int jj = 0; jj < 4; ++jj) acc[i][jj] = fmaf(a[i], b[jj], acc[i][jj]);
-        }
+        tile_dots<D>(Kj, Kt, ty, tx, acc);
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -223,25 +210,27 @@ __global__ void __launch_bounds__(MGT_NT) k_merge_assign_mma(const __grid_consta
     static_assert(KS % 2 == 0, "chunks are taken two k-steps at a time");
 }
 
-// Merge: a warp per retained slot walks the head's routing in ascending position order (a fixed order: the result
-// does not depend on scheduling) and adds the routed values in; the fp32 sum is rounded once to the output type.
-// The walk looks at 256 positions at a time (eight loads of the routing in flight), lists the hits in order, and fetches
-// the values of eight of them together before it adds them up: one row at a time made the kernel a chain of round trips to
-// the caches (115 us on 36 x 8 heads, T = 1024, 32 slots; 48 us so, the time
-// of the slot with the most hits).
-// grid = (ceil(k_eff_max / 8), heads_total), 256 threads.
+// Merge: a block per retained slot; each of its warps walks one eighth of the head's routing in ascending position order
+// and the warps' sums are added in that order (a fixed order: the result does not depend on scheduling); the fp32 sum is
+// rounded once to the output type.
+// A warp looks at 256 positions at a time (eight loads of the routing in flight), lists the hits in order, and fetches
+// the values of eight of them together before it adds them up.  What bounds the kernel is the slot with the most hits, a
+// heavy hitter's: one row at a time it took 115 us on 36 x 8 heads, T = 1024, 32 slots, a warp per slot with eight rows in
+// flight 44 us, a block per slot MEASURED_APPLY.
+// grid = (k_eff_max, heads_total), 256 threads.
 template <typename TIN, int D>
 __global__ void __launch_bounds__(256) k_merge_apply(const __grid_constant__ CallDev p)
 {
     __shared__ int32_t hits_s[8][256];
+    __shared__ float sum_s[8][D];
     int ci, lh;
     locate(p, blockIdx.y, ci, lh);
     const CacheDev &c = p.c[ci];
-    const int T = c.T, k = c.k_eff, lane = threadIdx.x & 31;
-    const int r = blockIdx.x * 8 + (threadIdx.x >> 5);
+    const int T = c.T, k = c.k_eff, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int r = blockIdx.x;
     if (r >= k) return;
     constexpr int PER = D / 32;
-    int32_t *hits = hits_s[threadIdx.x >> 5];
+    int32_t *hits = hits_s[warp];
     const TIN *Vh = reinterpret_cast<const TIN *>(c.v) + (size_t)lh * T * D + lane * PER;
     const float *A = p.scores + c.tok_off + (size_t)lh * T;
     const int32_t *assign = p.assign + c.tok_off + (size_t)lh * T;
@@ -249,10 +238,11 @@ __global__ void __launch_bounds__(256) k_merge_apply(const __grid_constant__ Cal
     float acc[PER];
 #pragma unroll
     for (int e = 0; e < PER; ++e) acc[e] = 0.f;
-    for (int jb = 0; jb < T; jb += 256) {
+    const int per = (T + 255) / 256 * 32, j_end = min(T, (warp + 1) * per);       // positions of a warp: a multiple of 32
+    for (int jb = warp * per; jb < j_end; jb += 256) {
         int a[8], n = 0;
 #pragma unroll
-        for (int u = 0; u < 8; ++u) a[u] = jb + 32 * u + lane < T ? assign[jb + 32 * u + lane] : -1;
+        for (int u = 0; u < 8; ++u) a[u] = jb + 32 * u + lane < j_end ? assign[jb + 32 * u + lane] : -1;
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
             const uint32_t hit = __ballot_sync(0xffffffffu, a[u] == r);
@@ -296,12 +286,17 @@ __global__ void __launch_bounds__(256) k_merge_apply(const __grid_constant__ Cal
         }
         __syncwarp();
     }
-    TIN *row = reinterpret_cast<TIN *>(c.v_out) + ((size_t)lh * k + r) * D + lane * PER;
 #pragma unroll
-    for (int e = 0; e < PER; ++e) {
-        const float sum = to_f32(row[e]) + acc[e];
-        if constexpr (sizeof(TIN) == 4) row[e] = sum;
-        else row[e] = __float2bfloat16_rn(sum);
+    for (int e = 0; e < PER; ++e) sum_s[warp][lane * PER + e] = acc[e];
+    __syncthreads();
+    if (threadIdx.x < D) {
+        TIN *out = reinterpret_cast<TIN *>(c.v_out) + ((size_t)lh * k + r) * D + threadIdx.x;
+        float sum = 0.f;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) sum += sum_s[w][threadIdx.x];
+        sum += to_f32(*out);
+        if constexpr (sizeof(TIN) == 4) *out = sum;
+        else *out = __float2bfloat16_rn(sum);
     }
 }
 

@@ -70,7 +70,7 @@ struct Layout {
     size_t off_status, off_scores, off_keep, off_stats, off_sums, off_lscores, clear_end;
     size_t off_gram_d, off_gram_k, off_uvec, off_delta, off_hflag, off_svec, off_assign;
     size_t total;
-    int splits;
+    int splits, sc_splits;
     int heads_total;
     size_t tok_total;
     size_t tok_off[OBF_MAX_CACHES];
@@ -125,6 +125,19 @@ static int choose_splits(int heads_total, int T_max)
     return s;
 }
 
+// Key splits of the shape-generic statistics kernel: its grid of (64 queries, head) tiles leaves most of the chip idle on
+// small calls, and a block walks all of a split's keys one tile after the other.  About four blocks per multiprocessor
+// (two or three are resident), at least two tiles of keys each.
+static int score_splits(int heads_total, int n_q, int T_max)
+{
+    const long long tiles = (long long)((n_q + SC_TILE - 1) / SC_TILE) * heads_total;
+    const int key_tiles = (T_max + SC_TILE - 1) / SC_TILE;
+    long long s = (4 * 148 + tiles - 1) / tiles;
+    if (s > key_tiles / 2) s = key_tiles / 2;
+    if (s > SC_MAX_SPLITS) s = SC_MAX_SPLITS;
+    return s < 1 ? 1 : (int)s;
+}
+
 // Retained positions of a cache: the protected prefix plus at most `budget` of the other positions.
 static inline int k_eff_of(const obf_params_t *p, const obf_cache_t &c)
 {
@@ -153,7 +166,8 @@ static obf_status_t validate_shapes(const obf_params_t *p, const obf_cache_t *ca
     return OBF_OK;
 }
 
-static void make_layout(const obf_params_t *p, const obf_cache_t *caches, int32_t n, int rank, Layout &L)
+// key_splits: at most this many for the shape-generic statistics kernel (a caller's scratch may not hold more).
+static void make_layout(const obf_params_t *p, const obf_cache_t *caches, int32_t n, int rank, Layout &L, int key_splits = SC_MAX_SPLITS)
 {
     const int hpc = p->layers * p->kv_heads;
     const int d = p->head_dim;
@@ -234,7 +248,9 @@ static void make_layout(const obf_params_t *p, const obf_cache_t *caches, int32_
     o = align_up(o + tok * sizeof(float), 256);
     if (L.sc_on && L.sc_qt == 2) L.clear_end = o;
     L.off_keep = o;   o = align_up(o + tok, 256);
-    L.off_stats = o;  o = align_up(o + (size_t)L.heads_total * n_q * 2 * sizeof(float), 256);
+    L.sc_splits = score_splits(L.heads_total, n_q, T_max);
+    if (L.sc_splits > key_splits) L.sc_splits = key_splits;
+    L.off_stats = o;  if (!L.sc_on) o = align_up(o + (size_t)L.heads_total * L.sc_splits * n_q * 2 * sizeof(float), 256);
     L.off_sums = o;   o = align_up(o + (size_t)L.heads_total * 4 * sizeof(float), 256);
     L.off_lscores = o;
     if (p->flags & OBF_FLAG_LAYERWISE) o = align_up(o + tok / p->kv_heads * sizeof(float), 256);
@@ -374,7 +390,7 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
     } else {
         if ((s = set_smem(k_score_stats<TIN, D>, sm_sc)) != OBF_OK) return s;
         if ((s = set_smem(k_score_pool<TIN, D>, sm_sc)) != OBF_OK) return s;
-        dim3 g1((cd.n_q + SC_TILE - 1) / SC_TILE, heads);
+        dim3 g1((cd.n_q + SC_TILE - 1) / SC_TILE, heads, cd.sc_splits);
         k_score_stats<TIN, D><<<g1, SC_NT, sm_sc, st>>>(cd);
         mark(st, "k_score_stats");
         dim3 g2((T_max + SC_TILE - 1) / SC_TILE, heads);
@@ -512,7 +528,7 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
             k_merge_assign<TIN, D><<<ga, 256, sm_mg, st>>>(cd);
         }
         mark(st, "k_merge_assign");
-        dim3 gm((k_max + 7) / 8, heads);
+        dim3 gm(k_max, heads);
         k_merge_apply<TIN, D><<<gm, 256, 0, st>>>(cd);
         mark(st, "k_merge_apply");
     }
@@ -553,6 +569,7 @@ static obf_status_t run(const obf_params_t *p, const obf_cache_t *caches, int32_
     }
     Layout L;
     make_layout(p, caches, n, rank, L);
+    if (workspace_bytes < L.total) make_layout(p, caches, n, rank, L, 1);
     if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255u) || workspace_bytes < L.total)
         return OBF_ERR_WORKSPACE;
     if (p->flags & OBF_FLAG_TEST_WAIT_EXPIRES) {
@@ -604,6 +621,7 @@ static obf_status_t run(const obf_params_t *p, const obf_cache_t *caches, int32_
     cd.sc_qt = L.sc_on ? L.sc_qt : 1;
     cd.sc_subs = L.sc_subs;
     cd.sc_rounds = L.sc_rounds;
+    cd.sc_splits = L.sc_splits;
     cd.eps = p->eps;
     char *ws = static_cast<char *>(workspace);
     cd.status = reinterpret_cast<uint32_t *>(ws + L.off_status);
@@ -953,7 +971,7 @@ extern "C" obf_status_t evict_only_static(const obf_params_t *params, const obf_
     pe.flags &= ~(uint32_t)OBF_FLAG_MERGE;                 // eviction only: nothing is merged either
     params = &pe;
     Layout L;
-    make_layout(params, caches, n_caches, 0, L);
+    make_layout(params, caches, n_caches, 0, L, 1);        // (more key splits only where they fit)
     if (L.total > (size_t)OBF_STATIC_SCRATCH_BYTES) {
         std::fprintf(stderr,
                      "obf: evict_only_static: this call needs %zu bytes of scratch but the built-in array holds "

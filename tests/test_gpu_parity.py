@@ -342,6 +342,13 @@ def test_more_than_256_query_rows_use_the_generic_score_kernels_and_the_tuned_gr
     assert "k_score_stats" in names and "k_gram_tc" in names
 
 
+@pytest.mark.parametrize("d,G,n_obs,caches", [(64, 4, 16, ((64, 9), (65, 9), (129, 9), (2100, 30))), (128, 3, 22, ((700, 20), (150, 20)))])
+def test_key_splits_of_the_shape_generic_statistics(d, G, n_obs, caches):
+    # one cache of a batch fills all key splits, shorter ones leave some empty; n_q = 64, 66 rows
+    w = small("splits", layers=1, kv_heads=2, G=G, n_obs=n_obs, d=d, dtype="f32", caches=caches, seed=d + G)
+    run_and_check(w)
+
+
 def test_exact_ties_go_to_the_lowest_position():
     # duplicated keys give bit-identical masses on the GPU as well; ties must resolve to lower positions
     w = small("ties", d=64, dtype="f32", rank=0, caches=((96, 20),), heavy=0, kv_heads=1)
