@@ -357,6 +357,7 @@ inline size_t algebra_smem_bytes(int mcap, int rank, int fast_iters)
 template <typename TIN, int D>
 __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant__ CallDev p)
 {
+    pdl_wait();
     typedef AlgShape<D> SH;
     constexpr int RW = SH::RW, NQ = SH::NQ, LD = D + 1;
     extern __shared__ __align__(16) float sm[];
@@ -435,7 +436,18 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
 
         // ---- u (and, for the diagnostics, the plain sum of the deleted values) -------------------
         constexpr int NPART = ALG_NT / D;
-        float sq = 0.f;
+        float sq = 0.f, us[U_LEVELS];                                  // us: what the pass over V added up, per level
+#pragma unroll
+        for (int l = 0; l < U_LEVELS; ++l) us[l] = 0.f;
+        if (tid < D) {
+#pragma unroll 1
+            for (int sp = 0; sp < n_del; ++sp) {
+                const float *uv = p.uvec + ((size_t)g * S + sp) * p.u_levels * D + tid;
+#pragma unroll
+                for (int l = 0; l < U_LEVELS; ++l)
+                    if (l < p.u_levels) us[l] += uv[l * D];
+            }
+        }
         if (p.gram_all) {
             // the retained rows' share of u per mass level, and of the trace of G; a lane fetches one row's mass
             const int col = tid % D, part = tid / D;
@@ -471,15 +483,12 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
         if (tid < D) {
             // per level: what the pass over V added up minus the retained rows' share; smallest masses first
             float s = 0.f;
-            for (int l = 0; l < p.u_levels; ++l) {
-                float sl = 0.f;
-                for (int sp = 0; sp < n_del; ++sp) sl += p.uvec[(((size_t)g * S + sp) * p.u_levels + l) * D + tid];
-                if (p.gram_all) {
-                    float kl = 0.f;
+#pragma unroll
+            for (int l = 0; l < U_LEVELS; ++l) {
+                float kl = 0.f;
+                if (p.gram_all)
                     for (int q = 0; q < NPART; ++q) kl += WS[(q * U_LEVELS + l) * D + tid];
-                    sl -= kl;
-                }
-                s += sl;
+                s += us[l] - kl;
             }
             vu[tid] = s;
             vx[tid] = c.diag ? p.svec[(size_t)g * D + tid] : 0.f;

@@ -96,6 +96,9 @@ struct CallDev {
     uint32_t *hflag;          // [heads_total] HFLAG_*
 };
 
+// Waits until the stream's kernel before this one is over and its writes are visible (see launch() in obf_api.cu).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 __device__ __forceinline__ void locate(const CallDev &p, int g, int &ci, int &lh)
 {
     ci = 0;

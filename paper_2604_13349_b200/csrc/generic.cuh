@@ -23,6 +23,7 @@ constexpr size_t score_smem_bytes() { return 2 * SC_TILE * TD_LD<D> * sizeof(flo
 template <typename TIN, int D>
 __global__ void __launch_bounds__(SC_NT) k_score_stats(const __grid_constant__ CallDev p)
 {
+    pdl_wait();
     extern __shared__ __align__(16) float sm[];
     float *Qs = sm, *Ks = sm + SC_TILE * TD_LD<D>;
     int ci, lh;
@@ -87,6 +88,7 @@ __global__ void __launch_bounds__(SC_NT) k_score_stats(const __grid_constant__ C
 template <typename TIN, int D>
 __global__ void __launch_bounds__(SC_NT) k_score_pool(const __grid_constant__ CallDev p)
 {
+    pdl_wait();
     extern __shared__ __align__(16) float sm[];
     float *Qs = sm, *Ks = sm + SC_TILE * TD_LD<D>;
     float *rm = Ks + SC_TILE * TD_LD<D>, *rz = rm + SC_TILE, *red = rz + SC_TILE;
@@ -155,6 +157,7 @@ constexpr int SEL_NT = 1024;
 
 __global__ void __launch_bounds__(SEL_NT) k_select(const __grid_constant__ CallDev p)
 {
+    pdl_wait();
     __shared__ uint32_t hist[256];
     __shared__ uint32_t s_prefix, s_want;
     __shared__ uint32_t wsum[32];
@@ -271,6 +274,7 @@ constexpr int SEL_SMEM_MAX_T = 16384;
 // added up per position, head 0 first.  grid = (ceil(T_max / 256), layers of all caches).
 __global__ void __launch_bounds__(256) k_layer_sum(const __grid_constant__ CallDev p)
 {
+    pdl_wait();
     int ci, lh;
     locate(p, blockIdx.y * p.kv_heads, ci, lh);
     const CacheDev &c = p.c[ci];
@@ -288,6 +292,7 @@ __global__ void __launch_bounds__(256) k_layer_sum(const __grid_constant__ CallD
 template <int NT, bool LAYER = false>
 __global__ void __launch_bounds__(NT) k_select_smem(const __grid_constant__ CallDev p)
 {
+    pdl_wait();
     extern __shared__ uint32_t sel_keys[];
     __shared__ uint32_t hist[256];
     __shared__ uint32_t s_prefix, s_want;
@@ -494,6 +499,7 @@ constexpr int GATHER_ROWS = 64;
 template <int ROW_BYTES, int WHICH = 3>
 __global__ void __launch_bounds__(256) k_gather(const __grid_constant__ CallDev p)
 {
+    pdl_wait();
     constexpr int CH = ROW_BYTES / 16;             // vectors per row
     constexpr int RPP = 256 / CH;                  // rows per pass of the block
     constexpr int PASSES = GATHER_ROWS / RPP;
@@ -567,6 +573,7 @@ constexpr int qr_block_rows() { return 256 / (D * (int)sizeof(TIN) / 16) * QR_RO
 template <typename TIN, int D>
 __global__ void __launch_bounds__(256) k_quantize_rows(const __grid_constant__ CallDev p)
 {
+    pdl_wait();
     constexpr int CH = D * (int)sizeof(TIN) / 16;                      // threads per row
     constexpr int EPT = 16 / (int)sizeof(TIN);                         // elements per thread
     constexpr int RPP = 256 / CH;                                      // rows per pass of the block
@@ -632,6 +639,7 @@ __global__ void __launch_bounds__(256) k_quantize_rows(const __grid_constant__ C
 template <typename TIN, int D>
 __global__ void __launch_bounds__(256) k_vsum(const __grid_constant__ CallDev p)
 {
+    pdl_wait();
     __shared__ float part[256];
     int ci, lh;
     locate(p, blockIdx.y, ci, lh);
@@ -666,6 +674,7 @@ constexpr int GR_ROWS = 32;
 template <typename TIN, int D>
 __global__ void __launch_bounds__(256) k_gram(const __grid_constant__ CallDev p)
 {
+    pdl_wait();
     constexpr int NV = D / 64;               // float4 groups per thread along each axis
     constexpr int MT = 4 * NV;
     __shared__ __align__(16) float Vs[GR_ROWS * D];

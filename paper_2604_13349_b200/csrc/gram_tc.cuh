@@ -97,6 +97,7 @@ struct TileRun {
 template <int D>
 __global__ void __launch_bounds__(GT_THREADS, 3) k_gram_tc(const __grid_constant__ CallDev p, const __grid_constant__ TcMaps tm)
 {
+    pdl_wait();
     constexpr int GT_STAGES = GramShape<D>::STAGES, GT_TILE_BYTES = GramShape<D>::TILE_BYTES, GT_STAGE_BYTES = GramShape<D>::STAGE_BYTES;
     extern __shared__ uint8_t gt_smem_raw[];
     uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(gt_smem_raw) + 1023) & ~(uintptr_t)1023);

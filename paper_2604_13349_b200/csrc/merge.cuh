@@ -26,6 +26,7 @@ __device__ __forceinline__ void merge_better(float &best, int &best_r, float s, 
 template <typename TIN, int D>
 __global__ void __launch_bounds__(256) k_merge_assign(const __grid_constant__ CallDev p)
 {
+    pdl_wait();
     constexpr int LD = TD_LD<D>;
     extern __shared__ __align__(16) float mg_sm[];
     float *Kj = mg_sm, *Kt = Kj + MG_TILE * LD, *inv_j = Kt + MG_TILE * LD, *inv_t = inv_j + MG_TILE;
@@ -104,6 +105,7 @@ constexpr int MGT_ROWS = 256, MGT_SLOTS = 64, MGT_NT = 128;
 template <int D>
 __global__ void __launch_bounds__(MGT_NT) k_merge_assign_mma(const __grid_constant__ CallDev p)
 {
+    pdl_wait();
     constexpr int CH = D / 8;                                          // 16-byte chunks per row
     constexpr int KS = D / 16;                                         // k-steps of an mma
     __shared__ __align__(16) uint4 Rs[MGT_SLOTS * CH];
@@ -210,36 +212,39 @@ __global__ void __launch_bounds__(MGT_NT) k_merge_assign_mma(const __grid_consta
     static_assert(KS % 2 == 0, "chunks are taken two k-steps at a time");
 }
 
-// Merge: a block per retained slot; each of its warps walks one eighth of the head's routing in ascending position order
-// and the warps' sums are added in that order (a fixed order: the result does not depend on scheduling); the fp32 sum is
-// rounded once to the output type.
+// Merge: WPS warps per retained slot; each walks its share of the head's routing in ascending position order and the
+// warps' sums are added in that order (a fixed order: the result does not depend on scheduling); the fp32 sum is rounded
+// once to the output type.
 // A warp looks at 256 positions at a time (eight loads of the routing in flight), lists the hits in order, and fetches
 // the values of eight of them together before it adds them up.  What bounds the kernel is the slot with the most hits, a
-// heavy hitter's: one row at a time it took 115 us on 36 x 8 heads, T = 1024, 32 slots, a warp per slot with eight rows in
-// flight 44 us, a block per slot MEASURED_APPLY.
-// grid = (k_eff_max, heads_total), 256 threads.
-template <typename TIN, int D>
+// heavy hitter's, and, with many slots, the walks themselves.  36 x 8 heads, T = 1024, 32 slots: one row at a time 115 us,
+// eight rows in flight 44 us, the same with eight warps per slot 48 us, with two 35 us; 6 x 8 heads, T = 1500: one warp per
+// slot 21 us, eight 11 us.
+// grid = (ceil(k_eff_max WPS / 8), heads_total), 256 threads.
+template <typename TIN, int D, int WPS>
 __global__ void __launch_bounds__(256) k_merge_apply(const __grid_constant__ CallDev p)
 {
+    pdl_wait();
     __shared__ int32_t hits_s[8][256];
     __shared__ float sum_s[8][D];
     int ci, lh;
     locate(p, blockIdx.y, ci, lh);
     const CacheDev &c = p.c[ci];
     const int T = c.T, k = c.k_eff, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int r = blockIdx.x;
-    if (r >= k) return;
+    constexpr int SLOTS = 8 / WPS;                                      // slots of a block
+    const int r0 = blockIdx.x * SLOTS, r = r0 + warp / WPS, part = warp % WPS;
+    if (r0 >= k) return;
     constexpr int PER = D / 32;
     int32_t *hits = hits_s[warp];
     const TIN *Vh = reinterpret_cast<const TIN *>(c.v) + (size_t)lh * T * D + lane * PER;
     const float *A = p.scores + c.tok_off + (size_t)lh * T;
     const int32_t *assign = p.assign + c.tok_off + (size_t)lh * T;
-    const float inv_at = 1.f / (A[c.idx_out[(size_t)lh * k + r]] + p.eps);
+    const float inv_at = 1.f / (A[c.idx_out[(size_t)lh * k + min(r, k - 1)]] + p.eps);
     float acc[PER];
 #pragma unroll
     for (int e = 0; e < PER; ++e) acc[e] = 0.f;
-    const int per = (T + 255) / 256 * 32, j_end = min(T, (warp + 1) * per);       // positions of a warp: a multiple of 32
-    for (int jb = warp * per; jb < j_end; jb += 256) {
+    const int per = (T + 32 * WPS - 1) / (32 * WPS) * 32, j_end = r < k ? min(T, (part + 1) * per) : 0;   // positions of a warp: a multiple of 32
+    for (int jb = part * per; jb < j_end; jb += 256) {
         int a[8], n = 0;
 #pragma unroll
         for (int u = 0; u < 8; ++u) a[u] = jb + 32 * u + lane < j_end ? assign[jb + 32 * u + lane] : -1;
@@ -289,11 +294,13 @@ __global__ void __launch_bounds__(256) k_merge_apply(const __grid_constant__ Cal
 #pragma unroll
     for (int e = 0; e < PER; ++e) sum_s[warp][lane * PER + e] = acc[e];
     __syncthreads();
-    if (threadIdx.x < D) {
-        TIN *out = reinterpret_cast<TIN *>(c.v_out) + ((size_t)lh * k + r) * D + threadIdx.x;
+    for (int i = threadIdx.x; i < SLOTS * D; i += 256) {
+        const int sl = i / D, e = i % D;
+        if (r0 + sl >= k) break;
+        TIN *out = reinterpret_cast<TIN *>(c.v_out) + ((size_t)lh * k + r0 + sl) * D + e;
         float sum = 0.f;
 #pragma unroll
-        for (int w = 0; w < 8; ++w) sum += sum_s[w][threadIdx.x];
+        for (int w = 0; w < WPS; ++w) sum += sum_s[sl * WPS + w][e];
         sum += to_f32(*out);
         if constexpr (sizeof(TIN) == 4) *out = sum;
         else *out = __float2bfloat16_rn(sum);

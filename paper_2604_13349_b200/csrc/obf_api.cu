@@ -196,6 +196,12 @@ static void make_layout(const obf_params_t *p, const obf_cache_t *caches, int32_
         const long long want = total < sms ? total : sms;
         L.tc_total_sub = total;
         L.tc_per = (int)((total + want - 1) / want);
+        // Every block leaves a partial Gram matrix per head it touches, which the dense algebra of the head reads one after
+        // the other (about 2000 cycles each, against 700 for a tile in this pass): small calls take runs of about
+        // sqrt(20 / 7 tiles of a head) tiles instead of one tile per block.
+        int nsub_max = 1;
+        for (int i = 0; i < n; ++i) nsub_max = L.nsub_del[i] > nsub_max ? L.nsub_del[i] : nsub_max;
+        while (L.tc_per * L.tc_per * 7 < 20 * nsub_max) ++L.tc_per;
         L.tc_blocks = (int)((total + L.tc_per - 1) / L.tc_per);
         int slots = 1;
         for (int i = 0; i < n; ++i) {
@@ -288,6 +294,31 @@ static obf_status_t set_smem(K kernel, size_t bytes)
     return OBF_OK;
 }
 
+#define OBF_TRY(expr)                        \
+    do {                                     \
+        const obf_status_t s_ = (expr);      \
+        if (s_ != OBF_OK) return s_;         \
+    } while (0)
+
+// Launch that may be set up while the stream's kernel before it still runs: every kernel launched so begins with
+// pdl_wait().  Between two kernels of a call that is about a microsecond less.
+template <typename... P, typename... A>
+static obf_status_t launch(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, const A &...args)
+{
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    OBF_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, args...));
+    return OBF_OK;
+}
+
 // cuTensorMapEncodeTiled, looked up through the runtime so that the library does not link the driver.
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
                                   const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
@@ -343,7 +374,7 @@ static obf_status_t launch_gram_tc(const CallDev &cd, const Layout &L, cudaStrea
     // the whole shared-memory capacity, so that the side stream's blocks find room beside this kernel's
     const obf_status_t sa = set_smem(k_gram_tc<D>, GramShape<D>::SMEM_BYTES);
     if (sa != OBF_OK) return sa;
-    k_gram_tc<D><<<L.tc_blocks, GT_THREADS, GramShape<D>::SMEM_BYTES, st>>>(cd, m);
+    OBF_TRY(launch(k_gram_tc<D>, dim3(L.tc_blocks), GT_THREADS, GramShape<D>::SMEM_BYTES, st, cd, m));
     mark(st, "k_gram_tc");
     return OBF_OK;
 }
@@ -373,7 +404,7 @@ static obf_status_t launch_score_tc(const CallDev &cd, const Layout &L, cudaStre
         int T_max = 1;
         for (int i = 0; i < cd.n_caches; ++i) T_max = cd.c[i].T > T_max ? cd.c[i].T : T_max;
         dim3 gj((T_max + 255) / 256, cd.heads_total);
-        k_score_join<<<gj, 256, 0, st>>>(cd);
+        OBF_TRY(launch(k_score_join, dim3(gj), 256, 0, st, cd));
         mark(st, "k_score_join");
     }
     return OBF_OK;
@@ -391,10 +422,10 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
         if ((s = set_smem(k_score_stats<TIN, D>, sm_sc)) != OBF_OK) return s;
         if ((s = set_smem(k_score_pool<TIN, D>, sm_sc)) != OBF_OK) return s;
         dim3 g1((cd.n_q + SC_TILE - 1) / SC_TILE, heads, cd.sc_splits);
-        k_score_stats<TIN, D><<<g1, SC_NT, sm_sc, st>>>(cd);
+        OBF_TRY(launch(k_score_stats<TIN, D>, dim3(g1), SC_NT, sm_sc, st, cd));
         mark(st, "k_score_stats");
         dim3 g2((T_max + SC_TILE - 1) / SC_TILE, heads);
-        k_score_pool<TIN, D><<<g2, SC_NT, sm_sc, st>>>(cd);
+        OBF_TRY(launch(k_score_pool<TIN, D>, dim3(g2), SC_NT, sm_sc, st, cd));
         mark(st, "k_score_pool");
     }
     // The tuned pass over V needs the masses but not the selection (it sums over all rows, gram_tc.cuh): it runs
@@ -416,15 +447,15 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
         const int n_layers = heads / cd.kv_heads;
         const size_t sm_sel = (size_t)T_max * sizeof(uint32_t);
         dim3 gl((T_max + 255) / 256, n_layers);
-        k_layer_sum<<<gl, 256, 0, sel>>>(cd);
+        OBF_TRY(launch(k_layer_sum, dim3(gl), 256, 0, sel, cd));
         mark(sel, "k_layer_sum");
         const int sms = sm_count();
         if (heads > 2 * sms && heads <= 4 * sms) {
             if ((s = set_smem(k_select_smem<512, true>, sm_sel)) != OBF_OK) return s;
-            k_select_smem<512, true><<<heads, 512, sm_sel, sel>>>(cd);
+            OBF_TRY(launch(k_select_smem<512, true>, dim3(heads), 512, sm_sel, sel, cd));
         } else {
             if ((s = set_smem(k_select_smem<1024, true>, sm_sel)) != OBF_OK) return s;
-            k_select_smem<1024, true><<<heads, 1024, sm_sel, sel>>>(cd);
+            OBF_TRY(launch(k_select_smem<1024, true>, dim3(heads), 1024, sm_sel, sel, cd));
         }
     } else if (T_max <= SEL_SMEM_MAX_T) {
         const size_t sm_sel = (size_t)T_max * sizeof(uint32_t);
@@ -433,19 +464,19 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
         const int sms = sm_count();
         if (heads > 2 * sms && heads <= 4 * sms) {
             if ((s = set_smem(k_select_smem<512>, sm_sel)) != OBF_OK) return s;
-            k_select_smem<512><<<heads, 512, sm_sel, sel>>>(cd);
+            OBF_TRY(launch(k_select_smem<512>, dim3(heads), 512, sm_sel, sel, cd));
         } else {
             if ((s = set_smem(k_select_smem<1024>, sm_sel)) != OBF_OK) return s;
-            k_select_smem<1024><<<heads, 1024, sm_sel, sel>>>(cd);
+            OBF_TRY(launch(k_select_smem<1024>, dim3(heads), 1024, sm_sel, sel, cd));
         }
     } else {
-        k_select<<<heads, SEL_NT, 0, sel>>>(cd);
+        OBF_TRY(launch(k_select, dim3(heads), SEL_NT, 0, sel, cd));
     }
     mark(sel, "k_select");
     dim3 g4((k_max + GATHER_ROWS - 1) / GATHER_ROWS, heads);
     if (side) {
         // the values first: the rest of the call needs them
-        k_gather<D * (int)sizeof(TIN), 1><<<g4, 256, 0, sel>>>(cd);
+        OBF_TRY(launch(k_gather<D * (int)sizeof(TIN), 1>, dim3(g4), 256, 0, sel, cd));
         mark(sel, "k_gather");
         OBF_CUDA_TRY(cudaEventRecord(side->rows_done, side->stream));
         if constexpr (sizeof(TIN) == 2) if (span) {
@@ -453,18 +484,18 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
             // V, whose persistent blocks leave room for one of its blocks per multiprocessor
             const size_t sm_span = span_smem_bytes<D>();
             if ((s = set_smem(k_span_test<D, true>, sm_span)) != OBF_OK) return s;
-            k_span_test<D, true><<<heads, ST_NT, sm_span, sel>>>(cd);
+            OBF_TRY(launch(k_span_test<D, true>, dim3(heads), ST_NT, sm_span, sel, cd));
             mark(sel, "k_span_test");
         }
         OBF_CUDA_TRY(cudaEventRecord(side->join, side->stream));
         // the keys are needed by nothing that follows: they are copied on the caller's stream once the pass over V
         // is over (it is bound by HBM), while the span test finishes on the side stream
         OBF_CUDA_TRY(cudaStreamWaitEvent(st, side->rows_done, 0));
-        k_gather<D * (int)sizeof(TIN), 2><<<g4, 256, 0, st>>>(cd);
+        OBF_TRY(launch(k_gather<D * (int)sizeof(TIN), 2>, dim3(g4), 256, 0, st, cd));
         ++g_last_launches;
         OBF_CUDA_TRY(cudaStreamWaitEvent(st, side->join, 0));
     } else {
-        k_gather<D * (int)sizeof(TIN)><<<g4, 256, 0, sel>>>(cd);
+        OBF_TRY(launch(k_gather<D * (int)sizeof(TIN)>, dim3(g4), 256, 0, sel, cd));
         mark(sel, "k_gather");
     }
     if (cd.rank > 0) {
@@ -476,14 +507,14 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
                     // the span test before the pass over V, which then skips the heads whose retained values span R^d
                     const size_t sm_span0 = span_smem_bytes<D>();
                     if ((s = set_smem(k_span_test<D, true>, sm_span0)) != OBF_OK) return s;
-                    k_span_test<D, true><<<heads, ST_NT, sm_span0, st>>>(cd);
+                    OBF_TRY(launch(k_span_test<D, true>, dim3(heads), ST_NT, sm_span0, st, cd));
                     mark(st, "k_span_test");
                 }
             }
             if (!side && (s = launch_gram_tc<D>(cd, L, st)) != OBF_OK) return s;
         } else {
             dim3 g5(cd.splits, heads);
-            k_gram<TIN, D><<<g5, 256, 0, st>>>(cd);
+            OBF_TRY(launch(k_gram<TIN, D>, dim3(g5), 256, 0, st, cd));
             mark(st, "k_gram");
         }
         bool any_diag = false;
@@ -492,7 +523,7 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
             // the projection cosine of the diagnostics needs the plain sum of the deleted values: one more pass over V
             OBF_CUDA_TRY(cudaMemsetAsync(cd.svec, 0, (size_t)heads * D * sizeof(float), st));
             dim3 gv((T_max + 2047) / 2048, heads);
-            k_vsum<TIN, D><<<gv, 256, 0, st>>>(cd);
+            OBF_TRY(launch(k_vsum<TIN, D>, dim3(gv), 256, 0, st, cd));
             mark(st, "k_vsum");
         }
         const size_t sm_span = span_smem_bytes<D>();
@@ -503,33 +534,39 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
             if (tuned_obf) {
                 // the tuned path forms G_keep inside the span test, from the gathered rows
                 if ((s = set_smem(k_span_test<D, true>, sm_span)) != OBF_OK) return s;
-                k_span_test<D, true><<<heads, ST_NT, sm_span, st>>>(cd);
+                OBF_TRY(launch(k_span_test<D, true>, dim3(heads), ST_NT, sm_span, st, cd));
             } else {
                 if ((s = set_smem(k_span_test<D>, sm_span)) != OBF_OK) return s;
-                k_span_test<D><<<heads, ST_NT, sm_span, st>>>(cd);
+                OBF_TRY(launch(k_span_test<D>, dim3(heads), ST_NT, sm_span, st, cd));
             }
         } else {
             if ((s = set_smem(k_span_test<D>, sm_span)) != OBF_OK) return s;
-            k_span_test<D><<<heads, ST_NT, sm_span, st>>>(cd);
+            OBF_TRY(launch(k_span_test<D>, dim3(heads), ST_NT, sm_span, st, cd));
         }
         if (!side && !cd.skip_full && span) mark(st, "k_span_test");
-        k_obf_algebra<TIN, D><<<heads, ALG_NT, sm_alg, st>>>(cd);
+        OBF_TRY(launch(k_obf_algebra<TIN, D>, dim3(heads), ALG_NT, sm_alg, st, cd));
         mark(st, "k_obf_algebra");
     }
     if (cd.merge) {
         // cache-merging baseline (App. E): route the deleted positions, then add their values into the retained rows
         if constexpr (sizeof(TIN) == 2) {
             dim3 ga((T_max + MGT_ROWS - 1) / MGT_ROWS, heads);
-            k_merge_assign_mma<D><<<ga, MGT_NT, 0, st>>>(cd);
+            OBF_TRY(launch(k_merge_assign_mma<D>, dim3(ga), MGT_NT, 0, st, cd));
         } else {
             const size_t sm_mg = merge_smem_bytes<D>();
             if ((s = set_smem(k_merge_assign<TIN, D>, sm_mg)) != OBF_OK) return s;
             dim3 ga((T_max + MG_TILE - 1) / MG_TILE, heads);
-            k_merge_assign<TIN, D><<<ga, 256, sm_mg, st>>>(cd);
+            OBF_TRY(launch(k_merge_assign<TIN, D>, dim3(ga), 256, sm_mg, st, cd));
         }
         mark(st, "k_merge_assign");
-        dim3 gm(k_max, heads);
-        k_merge_apply<TIN, D><<<gm, 256, 0, st>>>(cd);
+        // warps per slot: as many as keep about two warps on every place the chip has (64 per multiprocessor)
+        const long long slots = (long long)k_max * heads, places = 2ll * 64 * sm_count();
+        const int wps = slots * 8 <= places ? 8 : slots * 4 <= places ? 4 : slots * 2 <= places ? 2 : 1;
+        dim3 gm((k_max * wps + 7) / 8, heads);
+        if (wps == 8) OBF_TRY(launch(k_merge_apply<TIN, D, 8>, dim3(gm), 256, 0, st, cd));
+        else if (wps == 4) OBF_TRY(launch(k_merge_apply<TIN, D, 4>, dim3(gm), 256, 0, st, cd));
+        else if (wps == 2) OBF_TRY(launch(k_merge_apply<TIN, D, 2>, dim3(gm), 256, 0, st, cd));
+        else OBF_TRY(launch(k_merge_apply<TIN, D, 1>, dim3(gm), 256, 0, st, cd));
         mark(st, "k_merge_apply");
     }
     bool any_q8 = false;
@@ -537,7 +574,7 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
     if (any_q8) {
         constexpr int QB = qr_block_rows<TIN, D>();
         dim3 gq((k_max + QB - 1) / QB, heads);
-        k_quantize_rows<TIN, D><<<gq, 256, 0, st>>>(cd);
+        OBF_TRY(launch(k_quantize_rows<TIN, D>, dim3(gq), 256, 0, st, cd));
         mark(st, "k_quantize_rows");
     }
     OBF_CUDA_TRY(cudaGetLastError());

@@ -572,6 +572,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constan
 // grid = (ceil(T_max / 256), heads_total).
 __global__ void __launch_bounds__(256) k_score_join(const __grid_constant__ CallDev p)
 {
+    pdl_wait();
     int ci, lh;
     locate(p, blockIdx.y, ci, lh);
     const CacheDev &c = p.c[ci];

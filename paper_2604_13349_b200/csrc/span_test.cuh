@@ -29,6 +29,7 @@ constexpr size_t span_smem_bytes() { return (size_t)(D * (D + 1) + 32 * 33 + 32 
 template <int D, bool FROM_ROWS = false>
 __global__ void __launch_bounds__(ST_NT, 3) k_span_test(const __grid_constant__ CallDev p)
 {
+    pdl_wait();
     constexpr int LD = D + 1, NB = 32, L11_LD = NB + 1;
     extern __shared__ float st_sm[];
     float *A = st_sm;                  // D x LD, lower triangle is what counts
