@@ -44,7 +44,6 @@
 #include <type_traits>
 
 #include "common.cuh"
-#include "span_test.cuh"
 
 namespace obf {
 
@@ -100,22 +99,22 @@ __device__ __forceinline__ float rsqrt_approx(float x)
 __device__ __forceinline__ float rcp_approx(float x)
 {
     float r;
-    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
 
 // The matrix in registers.  Half-warp g (of ALG_NG) holds rows g, g + ALG_NG, ..; lane c of its sixteen holds of each
 // row the pairs of columns 32 q + 2 c, 32 q + 2 c + 1.  A reflector and the product with it meet the warps in shared
-// memory twice: in order (for the columns) and doubled into pairs with a half-warp's rows next to one another (for its
-// rows).
+// memory twice: in order (for the columns) and with a half-warp's rows next to one another (for its rows; not doubled into
+// the pairs the two-wide FMA takes: a move is cheaper than twice the bytes from shared memory).
 template <int D>
 struct AlgShape {
     static constexpr int RW = D / ALG_NG;        // rows a lane holds
     static constexpr int NQ = D / 32;            // column pairs a lane holds per row
     static constexpr int RPS = 32 / ALG_NG;      // rows a lane holds of 32 consecutive ones
-    static constexpr int GRP = RW + 2;           // pairs per half-warp in the doubled arrays (padded against bank conflicts)
-    static constexpr int DUP = ALG_NG * GRP;     // pairs of one doubled array
-    __device__ static __forceinline__ int dup_index(int i) { return (i % ALG_NG) * GRP + i / ALG_NG; }
+    static constexpr int GRP = RW + 4;           // entries per half-warp in an array by rows (padded against bank conflicts)
+    static constexpr int BYR = ALG_NG * GRP;     // floats of one such array
+    __device__ static __forceinline__ int row_index(int i) { return (i % ALG_NG) * GRP + i / ALG_NG; }
 };
 template <int D>
 using AlgMat = f32x2[AlgShape<D>::RW][AlgShape<D>::NQ];
@@ -139,10 +138,10 @@ __device__ __forceinline__ float alg_dot(const AlgRow<D> &x, const AlgRow<D> &y)
 }
 
 // Stage S serves the reflectors 32 S .. 32 S + 31: their support starts at row and column 32 S or later.
-// p = 2 M v on the rows of the stage; pd may be null.  With vd (the reflector doubled) also this half-warp's share of
+// p = 2 M v on the rows of the stage; pd may be null.  With vd (the reflector by rows) also this half-warp's share of
 // v . p, in kp[grp]: formed from the lanes' partial sums, its reduction runs beside that of p.
 template <int D, int S>
-__device__ __forceinline__ void alg_product(const AlgMat<D> &M, const AlgRow<D> &v2, float *pl, f32x2 *pd, const f32x2 *vd, float *kp,
+__device__ __forceinline__ void alg_product(const AlgMat<D> &M, const AlgRow<D> &v2, float *pl, float *pd, const float *vd, float *kp,
                                             int grp, int c16)
 {
     constexpr int RW = AlgShape<D>::RW, R0 = AlgShape<D>::RPS * S, NR = RW - R0;
@@ -152,15 +151,14 @@ __device__ __forceinline__ void alg_product(const AlgMat<D> &M, const AlgRow<D> 
     for (int r = 0; r < NP; ++r) acc[r] = r < NR ? alg_dot<D, S>(M[R0 + (r < NR ? r : 0)], v2) : 0.f;
     float ka = 0.f, kb = 0.f;
     if (vd) {
-        const f32x2 *vr = vd + grp * AlgShape<D>::GRP + R0;
+        const float *vr = vd + grp * AlgShape<D>::GRP + R0;
 #pragma unroll
-        for (int r = 0; r < NR; r += 2) {
-            const ulonglong2 w = *reinterpret_cast<const ulonglong2 *>(vr + r);
-            float a, b, t;
-            upk(w.x, a, t);
-            upk(w.y, b, t);
-            ka = fmaf(a, acc[r], ka);
-            kb = fmaf(b, acc[r + 1], kb);
+        for (int r = 0; r < NR; r += 4) {
+            const float4 w = *reinterpret_cast<const float4 *>(vr + r);
+            ka = fmaf(w.x, acc[r], ka);
+            kb = fmaf(w.y, acc[r + 1], kb);
+            ka = fmaf(w.z, acc[r + 2], ka);
+            kb = fmaf(w.w, acc[r + 3], kb);
         }
         ka = 2.f * half_sum(ka + kb);
     }
@@ -169,7 +167,7 @@ __device__ __forceinline__ void alg_product(const AlgMat<D> &M, const AlgRow<D> 
     const int r = c16 / LPR;
     if ((c16 % LPR) == 0 && r < NR) {
         pl[grp + ALG_NG * (R0 + r)] = s;
-        if (pd) pd[grp * AlgShape<D>::GRP + R0 + r] = pk(s, s);
+        if (pd) pd[grp * AlgShape<D>::GRP + R0 + r] = s;
     }
     if (vd && c16 == 0) kp[grp] = ka;
 }
@@ -177,7 +175,7 @@ __device__ __forceinline__ void alg_product(const AlgMat<D> &M, const AlgRow<D> 
 // M <- M - v w^T - w v^T with w = p - (v.p) v on the rows and columns of the stage.  x: row `xr` of the stage's first
 // RPS rows as the update leaves it, formed first so that the next reflector need not wait.
 template <int D, int S>
-__device__ __forceinline__ void alg_update(AlgMat<D> &M, const AlgRow<D> &v, const f32x2 *vd, const float *pl, const f32x2 *pd,
+__device__ __forceinline__ void alg_update(AlgMat<D> &M, const AlgRow<D> &v, const float *vd, const float *pl, const float *pd,
                                            const float *kp, int grp, int c16, int xr, AlgRow<D> &x)
 {
     constexpr int RW = AlgShape<D>::RW, NQ = AlgShape<D>::NQ, R0 = AlgShape<D>::RPS * S;
@@ -197,9 +195,10 @@ __device__ __forceinline__ void alg_update(AlgMat<D> &M, const AlgRow<D> &v, con
         w2[q] = mul2(fma2(nk, v[q], w2[q]), neg);
         v2[q] = mul2(v[q], neg);
     }
-    const f32x2 *vr = vd + grp * AlgShape<D>::GRP, *pr = pd + grp * AlgShape<D>::GRP;
+    const float *vr = vd + grp * AlgShape<D>::GRP, *pr = pd + grp * AlgShape<D>::GRP;
     {
-        const f32x2 vx = vr[R0 + xr], wx = fma2(nk, vx, pr[R0 + xr]);
+        const float v1 = vr[R0 + xr], w1 = fmaf(-kk, v1, pr[R0 + xr]);
+        const f32x2 vx = pk(v1, v1), wx = pk(w1, w1);
         const f32x2 odd = mask2(xr & 1), high = mask2(xr & 2);
 #pragma unroll
         for (int q = S; q < NQ; ++q) {
@@ -209,13 +208,14 @@ __device__ __forceinline__ void alg_update(AlgMat<D> &M, const AlgRow<D> &v, con
         }
     }
 #pragma unroll
-    for (int r = R0; r < RW; r += 2) {
-        const ulonglong2 va = *reinterpret_cast<const ulonglong2 *>(vr + r), pa = *reinterpret_cast<const ulonglong2 *>(pr + r);
-        const f32x2 wa = fma2(nk, va.x, pa.x), wb = fma2(nk, va.y, pa.y);
+    for (int r = R0; r < RW; r += 4) {
+        const float4 va = *reinterpret_cast<const float4 *>(vr + r), pa = *reinterpret_cast<const float4 *>(pr + r);
+        const float vv[4] = {va.x, va.y, va.z, va.w}, pp[4] = {pa.x, pa.y, pa.z, pa.w};
 #pragma unroll
-        for (int q = S; q < NQ; ++q) {
-            M[r][q] = fma2(va.x, w2[q], fma2(wa, v2[q], M[r][q]));
-            M[r + 1][q] = fma2(va.y, w2[q], fma2(wb, v2[q], M[r + 1][q]));
+        for (int e = 0; e < 4; ++e) {
+            const float w = fmaf(-kk, vv[e], pp[e]);
+#pragma unroll
+            for (int q = S; q < NQ; ++q) M[r + e][q] = fma2(pk(vv[e], vv[e]), w2[q], fma2(pk(w, w), v2[q], M[r + e][q]));
         }
     }
 }
@@ -251,7 +251,7 @@ __device__ __forceinline__ float alg_tail2(const AlgRow<D> &x, int from, int c16
 
 // Writes the unit reflector of support >= j0 made of x: entry j0 is `first`, the others x, all scaled (a half-warp's lanes).
 template <int D, int FROM = 0>
-__device__ __forceinline__ void alg_store_reflector(const AlgRow<D> &x, int j0, float first, float rs, float *v, f32x2 *vd, int c16)
+__device__ __forceinline__ void alg_store_reflector(const AlgRow<D> &x, int j0, float first, float rs, float *v, float *vd, int c16)
 {
 #pragma unroll
     for (int q = 0; q < AlgShape<D>::NQ; ++q) {
@@ -262,8 +262,8 @@ __device__ __forceinline__ void alg_store_reflector(const AlgRow<D> &x, int j0, 
         b = c + 1 < j0 ? 0.f : (c + 1 == j0 ? first : b) * rs;
         *reinterpret_cast<f32x2 *>(v + c) = pk(a, b);
         if (vd) {
-            vd[AlgShape<D>::dup_index(c)] = pk(a, a);
-            vd[AlgShape<D>::dup_index(c + 1)] = pk(b, b);
+            vd[AlgShape<D>::row_index(c)] = a;
+            vd[AlgShape<D>::row_index(c + 1)] = b;
         }
     }
 }
@@ -271,7 +271,7 @@ __device__ __forceinline__ void alg_store_reflector(const AlgRow<D> &x, int j0, 
 // Reflector j + 1 from row j of the trailing block (entries of x from j on), with the row's diagonal and off-diagonal
 // entry of the tridiagonal form.  Every half-warp computes on its own row; the owner of row j stores.
 template <int D, int FROM>
-__device__ __forceinline__ void alg_row_done(const AlgRow<D> &x, int j, float tiny2, float *Y, f32x2 *vd, float *ta, float *tb,
+__device__ __forceinline__ void alg_row_done(const AlgRow<D> &x, int j, float tiny2, float *Y, float *vd, float *ta, float *tb,
                                              int grp, int lane)
 {
     const int c16 = lane & 15;
@@ -350,7 +350,7 @@ __host__ __device__ constexpr int algebra_eig_floats(int rank, int fast_iters)
 template <int D>
 inline size_t algebra_smem_bytes(int mcap, int rank, int fast_iters)
 {
-    return (size_t)(algebra_y_rows<D>(mcap, rank, fast_iters) * D + 12 * AlgShape<D>::DUP + 2 * D + 6 * D + 96 +
+    return (size_t)(algebra_y_rows<D>(mcap, rank, fast_iters) * D + 6 * AlgShape<D>::BYR + 2 * D + 6 * D + 96 +
                     algebra_eig_floats<D>(rank, fast_iters)) * sizeof(float) + 2 * D * sizeof(int);
 }
 
@@ -362,9 +362,9 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
     constexpr int RW = SH::RW, NQ = SH::NQ, LD = D + 1;
     extern __shared__ __align__(16) float sm[];
     float *Y = sm;                                                    // reflector j in row j, support >= j
-    f32x2 *vdup = reinterpret_cast<f32x2 *>(Y + algebra_y_rows<D>(p.alg_rows, p.rank, p.fast_iters) * D);   // 4 buffers: reflector j in j & 3
-    f32x2 *pdup = vdup + 4 * SH::DUP;                                 // 2 buffers
-    float *pl = reinterpret_cast<float *>(pdup + 2 * SH::DUP);        // 2 buffers of D
+    float *vrows = Y + algebra_y_rows<D>(p.alg_rows, p.rank, p.fast_iters) * D;   // 4 buffers: reflector j in j & 3
+    float *prows = vrows + 4 * SH::BYR;                                 // 2 buffers
+    float *pl = prows + 2 * SH::BYR;        // 2 buffers of D
     float *ta = pl + 2 * D, *tb = ta + D;                             // tridiagonal form
     float *vu = tb + D, *vx = vu + D, *vc = vx + D, *vl = vc + D;     // vectors of d
     float *red = vl + D, *misc = red + 32, *tlam = misc + 32;         // 32 floats each
@@ -606,7 +606,7 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
             auto double_up = [&](int j) __attribute__((always_inline)) {
                 if (tid < D) {
                     const float t = Y[j * D + tid];
-                    vdup[(j & 3) * SH::DUP + SH::dup_index(tid)] = pk(t, t);
+                    vrows[(j & 3) * SH::BYR + SH::row_index(tid)] = t;
                 }
             };
             auto apply_stage = [&](auto stage) __attribute__((always_inline)) {
@@ -617,10 +617,10 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                     const int pb = j & 1;
                     AlgRow<D> v, x;
                     alg_load<D, ST>(v, Y + j * D, c16);
-                    alg_product<D, ST>(M, v, pl + pb * D, pdup + pb * SH::DUP, vdup + (j & 3) * SH::DUP, kpart + pb * ALG_NG, grp, c16);
+                    alg_product<D, ST>(M, v, pl + pb * D, prows + pb * SH::BYR, vrows + (j & 3) * SH::BYR, kpart + pb * ALG_NG, grp, c16);
                     if (j + 1 < m) double_up(j + 1);
                     __syncthreads();                                   // p is there, and the next reflector doubled
-                    alg_update<D, ST>(M, v, vdup + (j & 3) * SH::DUP, pl + pb * D, pdup + pb * SH::DUP, kpart + pb * ALG_NG, grp, c16, 0, x);
+                    alg_update<D, ST>(M, v, vrows + (j & 3) * SH::BYR, pl + pb * D, prows + pb * SH::BYR, kpart + pb * ALG_NG, grp, c16, 0, x);
                 }
             };
             if (m < D) {
@@ -746,7 +746,7 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
 #pragma unroll
                         for (int r = 1; r < RW; ++r) x[q] = sel2(mask2(r == m / ALG_NG), M[r][q], x[q]);
                     }
-                    alg_row_done<D, 0>(x, m, tiny2, Y, vdup + ((m + 1) & 3) * SH::DUP, ta, tb, grp, lane);
+                    alg_row_done<D, 0>(x, m, tiny2, Y, vrows + ((m + 1) & 3) * SH::BYR, ta, tb, grp, lane);
                 }
                 auto reduce_stage = [&](auto stage) __attribute__((always_inline)) {
                     constexpr int ST = decltype(stage)::value;
@@ -757,16 +757,16 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                         AlgRow<D> v, x;
                         __syncthreads();                               // reflector j is there
                         alg_load<D, ST>(v, Y + j * D, c16);
-                        alg_product<D, ST>(M, v, pl + pb * D, pdup + pb * SH::DUP, vdup + (j & 3) * SH::DUP, kpart + pb * ALG_NG, grp, c16);
+                        alg_product<D, ST>(M, v, pl + pb * D, prows + pb * SH::BYR, vrows + (j & 3) * SH::BYR, kpart + pb * ALG_NG, grp, c16);
                         {
                             const float s = -2.f * half_sum(alg_dot<D, ST>(aux, v));
 #pragma unroll
                             for (int q = ST; q < NQ; ++q) aux[q] = fma2(pk(s, s), v[q], aux[q]);
                         }
                         __syncthreads();                               // p is there
-                        alg_update<D, ST>(M, v, vdup + (j & 3) * SH::DUP, pl + pb * D, pdup + pb * SH::DUP, kpart + pb * ALG_NG,
+                        alg_update<D, ST>(M, v, vrows + (j & 3) * SH::BYR, pl + pb * D, prows + pb * SH::BYR, kpart + pb * ALG_NG,
                                           grp, c16, (j / ALG_NG) & (SH::RPS - 1), x);
-                        alg_row_done<D, ST>(x, j, tiny2, Y, vdup + ((j + 1) & 3) * SH::DUP, ta, tb, grp, lane);
+                        alg_row_done<D, ST>(x, j, tiny2, Y, vrows + ((j + 1) & 3) * SH::BYR, ta, tb, grp, lane);
                     }
                 };
                 reduce_stage(std::integral_constant<int, 0>{});

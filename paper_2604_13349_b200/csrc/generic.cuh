@@ -4,7 +4,6 @@
 #pragma once
 
 #include "common.cuh"
-#include "span_test.cuh"
 
 namespace obf {
 

@@ -482,7 +482,7 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
         if constexpr (sizeof(TIN) == 2) if (span) {
             // the span test reads the gathered rows only (it forms G_keep itself): it runs here, beside the pass over
             // V, whose persistent blocks leave room for one of its blocks per multiprocessor
-            const size_t sm_span = span_smem_bytes<D>();
+            const size_t sm_span = span_smem_bytes<D>(true);
             if ((s = set_smem(k_span_test<D, true>, sm_span)) != OBF_OK) return s;
             OBF_TRY(launch(k_span_test<D, true>, dim3(heads), ST_NT, sm_span, sel, cd));
             mark(sel, "k_span_test");
@@ -505,7 +505,7 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
             if constexpr (sizeof(TIN) == 2) {
                 if (cd.skip_full) {
                     // the span test before the pass over V, which then skips the heads whose retained values span R^d
-                    const size_t sm_span0 = span_smem_bytes<D>();
+                    const size_t sm_span0 = span_smem_bytes<D>(tuned_obf);
                     if ((s = set_smem(k_span_test<D, true>, sm_span0)) != OBF_OK) return s;
                     OBF_TRY(launch(k_span_test<D, true>, dim3(heads), ST_NT, sm_span0, st, cd));
                     mark(st, "k_span_test");
@@ -526,7 +526,7 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
             OBF_TRY(launch(k_vsum<TIN, D>, dim3(gv), 256, 0, st, cd));
             mark(st, "k_vsum");
         }
-        const size_t sm_span = span_smem_bytes<D>();
+        const size_t sm_span = span_smem_bytes<D>(tuned_obf);
         if (side || cd.skip_full || !span) {
             // nothing to test, or the span test has been enqueued already: on the side stream (this stream has waited for it) or, with
             // OBF_FLAG_EARLY_OUT, before the pass over V
