@@ -404,36 +404,6 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
         const float *A = p.scores + c.tok_off + (size_t)lh * T;
         const int32_t *idx = c.idx_out + (size_t)lh * k;
 
-        // ---- G into registers, its trace --------------------------------------------
-        AlgMat<D> M;
-        {
-            const float *G = p.gram_d + (size_t)g * S * D * D + grp * D + 2 * c16;
-#pragma unroll
-            for (int r = 0; r < RW; ++r)
-#pragma unroll
-                for (int q = 0; q < NQ; ++q) M[r][q] = *reinterpret_cast<const f32x2 *>(G + r * ALG_NG * D + 32 * q);
-#pragma unroll 1
-            for (int sp = 1; sp < n_del; ++sp) {
-                G += D * D;
-#pragma unroll
-                for (int r = 0; r < RW; ++r)
-#pragma unroll
-                    for (int q = 0; q < NQ; ++q) M[r][q] = add2(M[r][q], *reinterpret_cast<const f32x2 *>(G + r * ALG_NG * D + 32 * q));
-            }
-        }
-        // this thread's share of the diagonal from row `from` on
-        auto diag_part = [&](int from) __attribute__((always_inline)) {
-            float s = 0.f;
-#pragma unroll
-            for (int r = 0; r < RW; ++r) {
-                const int i = grp + ALG_NG * r;
-                float a, b;
-                upk(M[r][r / SH::RPS], a, b);
-                if (i >= from && c16 == (i & 31) >> 1) s += (i & 1) ? b : a;
-            }
-            return s;
-        };
-
         // ---- u (and, for the diagnostics, the plain sum of the deleted values) -------------------
         constexpr int NPART = ALG_NT / D;
         float sq = 0.f, us[U_LEVELS];                                  // us: what the pass over V added up, per level
@@ -479,7 +449,6 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
             for (int l = 0; l < U_LEVELS; ++l) WS[(part * U_LEVELS + l) * D + col] = uk[l];
         }
         const float sq_keep = block_sum<ALG_NT>(sq, red);             // (its barriers also publish WS)
-        const float trAll = block_sum<ALG_NT>(diag_part(0), red);
         if (tid < D) {
             // per level: what the pass over V added up minus the retained rows' share; smallest masses first
             float s = 0.f;
@@ -494,11 +463,6 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
             vx[tid] = c.diag ? p.svec[(size_t)g * D + tid] : 0.f;
         }
         __syncthreads();
-        // squared Frobenius norm of the deleted values (the denominator of RCR).  As a difference of two fp32 traces
-        // it is resolved down to about 1e-6 of the squared norm of all values: below 1e-5 of it the deleted values
-        // count as negligible beside the retained ones and nothing is injected.
-        const float trG = trAll - sq_keep;
-        const bool del_negligible = p.gram_all && !(trG > 1e-5f * trAll);
         // one more vector per half-warp that the reflectors are applied to: u in the first, the sum of the deleted values
         // in the second
         AlgRow<D> aux;
@@ -513,40 +477,52 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
 #pragma unroll
             for (int q = 0; q < NQ; ++q) x[q] = fma2(pk(s, s), v[q], x[q]);
         };
-        // ---- 2. reflectors of the retained rows (Eq. 2), then applied to G from both sides.  Two loops: together their
-        // code outgrows what a multiprocessor fetches at full speed (3500 cycles per row in one loop, 3100 in two) ----
+        // ---- 2. reflectors of the retained rows (Eq. 2).  Two loops, this one and that over G: together their code outgrows
+        // what a multiprocessor fetches at full speed ----
         {
-            // a batch of rows in shared memory: row b0 + grp + ALG_NG s in slot s of the half-warp
+            // a batch of rows in registers (G comes afterwards): row b0 + grp + ALG_NG s in slot s of the half-warp
             constexpr int NS = ALG_BATCH / ALG_NG;
-            float *R = rows_s + grp * D, *n0 = vl;                     // n0: the rows' squared norms
-            // rows of the half-warp from slot s0 on, reflected by v
-            auto reflect_rows = [&](const AlgRow<D> &v, int s0) __attribute__((always_inline)) {
-                AlgRow<D> x[NS];
+            static_assert(NS == 4, "four slots to pick from");
+            AlgRow<D> V[NS];
+            float n0[NS];                                              // the rows' squared norms
+            auto reflect_rows = [&](const AlgRow<D> &v) __attribute__((always_inline)) {
                 float d4[NS];
 #pragma unroll
-                for (int s = 0; s < NS; ++s) alg_load<D>(x[s], R + s * ALG_NG * D, c16);
-#pragma unroll
-                for (int s = 0; s < NS; ++s) d4[s] = alg_dot<D>(x[s], v);
+                for (int s = 0; s < NS; ++s) d4[s] = alg_dot<D>(V[s], v);
                 const float tot = -2.f * transposed_sum<NS, 16>(d4, c16);
 #pragma unroll
                 for (int s = 0; s < NS; ++s) {
                     const float f = __shfl_sync(0xffffffffu, tot, (lane & 16) + (16 / NS) * s);
-                    if (s >= s0) {
 #pragma unroll
-                        for (int q = 0; q < NQ; ++q) *reinterpret_cast<f32x2 *>(R + s * ALG_NG * D + 32 * q + 2 * c16) = fma2(pk(f, f), v[q], x[s][q]);
-                    }
+                    for (int q = 0; q < NQ; ++q) V[s][q] = fma2(pk(f, f), v[q], V[s][q]);
                 }
-                __syncwarp();
             };
             // whether row i of the batch adds a direction to the m there are, and its reflector
             auto candidate = [&](int i) __attribute__((always_inline)) {
                 if (warp != (i % ALG_NG) / 2) return;
                 AlgRow<D> x;
-                alg_load<D>(x, R + (i / ALG_NG) * ALG_NG * D, c16);
-                const float t2 = alg_tail2<D>(x, m, c16), x0 = R[(i / ALG_NG) * ALG_NG * D + (m < D ? m : 0)];
+                float nn = n0[0];
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) x[q] = V[0][q];
+                auto pick = [&](auto slot) __attribute__((always_inline)) {
+                    constexpr int s = decltype(slot)::value;
+                    if (i / ALG_NG == s) {
+                        nn = n0[s];
+#pragma unroll
+                        for (int q = 0; q < NQ; ++q) {
+                            x[q] = V[s][q];
+                            // (keeps the compiler from merging the slots' code into one that addresses the array)
+                            asm volatile("// %1" : "+l"(x[q]) : "n"(s));
+                        }
+                    }
+                };
+                pick(std::integral_constant<int, 1>{});
+                pick(std::integral_constant<int, 2>{});
+                pick(std::integral_constant<int, 3>{});
+                const float t2 = alg_tail2<D>(x, m, c16), x0 = alg_entry<D>(x, m < D ? m : 0, lane);
                 const float nrm = t2 * rsqrt_approx(fmaxf(t2, 1e-37f));
                 if (grp == i % ALG_NG) {
-                    const bool add = m < D && t2 > SPAN_ROW_TOL * SPAN_ROW_TOL * n0[i] && t2 > 1e-37f;
+                    const bool add = m < D && t2 > SPAN_ROW_TOL * SPAN_ROW_TOL * nn && t2 > 1e-37f;
                     if (add) {
                         const float al = x0 >= 0.f ? -nrm : nrm;
                         alg_store_reflector<D>(x, m, x0 - al, rsqrt_approx(2.f * fmaf(nrm, fabsf(x0), t2)), Y + m * D, nullptr, c16);
@@ -556,33 +532,30 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
             };
 #pragma unroll 1
             for (int b0 = 0; b0 < k && m < D; b0 += ALG_BATCH) {
-#pragma unroll 1
+#pragma unroll
                 for (int s = 0; s < NS; ++s) {
-                    const int i = grp + ALG_NG * s;
-                    AlgRow<D> x;
+                    const int i = b0 + grp + ALG_NG * s;
 #pragma unroll
                     for (int q = 0; q < NQ; ++q) {
-                        x[q] = 0ull;
-                        if (b0 + i < k) {
-                            const TIN *src = vk + (size_t)(b0 + i) * D + 32 * q + 2 * c16;
-                            if constexpr (sizeof(TIN) == 4) x[q] = *reinterpret_cast<const f32x2 *>(src);
+                        V[s][q] = 0ull;
+                        if (i < k) {
+                            const TIN *src = vk + (size_t)i * D + 32 * q + 2 * c16;
+                            if constexpr (sizeof(TIN) == 4) V[s][q] = *reinterpret_cast<const f32x2 *>(src);
                             else {
                                 const uint32_t w = *reinterpret_cast<const uint32_t *>(src);
-                                x[q] = pk(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u));
+                                V[s][q] = pk(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u));
                             }
                         }
-                        *reinterpret_cast<f32x2 *>(R + s * ALG_NG * D + 32 * q + 2 * c16) = x[q];
                     }
-                    const float nn = half_sum(alg_dot<D>(x, x));
-                    if (c16 == 0) n0[i] = nn;
                 }
-                __syncwarp();
+#pragma unroll
+                for (int s = 0; s < NS; ++s) n0[s] = half_sum(alg_dot<D>(V[s], V[s]));
                 // (the reflectors that earlier batches found, all published behind a barrier)
 #pragma unroll 1
                 for (int j = 0; j < m; ++j) {
                     AlgRow<D> v;
                     alg_load<D>(v, Y + j * D, c16);
-                    reflect_rows(v, 0);
+                    reflect_rows(v);
                 }
                 const int rows = min(ALG_BATCH, k - b0);
                 candidate(0);
@@ -592,7 +565,7 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                     if (s_flag[i & 1]) {                               // row i has a reflector
                         AlgRow<D> v;
                         alg_load<D>(v, Y + m * D, c16);
-                        reflect_rows(v, (i + ALG_NG - grp) / ALG_NG);
+                        reflect_rows(v);
                         if (++m >= D) break;
                         if (i + 1 < rows) candidate(i + 1);
                         reflect(aux, v);
@@ -603,6 +576,44 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                 // the flag is written again by the next batch
                 __syncthreads();
             }
+        }
+        // ---- G into registers, its trace, and the reflectors applied to it from both sides -----------------------
+        AlgMat<D> M;
+        {
+            const float *G = p.gram_d + (size_t)g * S * D * D + grp * D + 2 * c16;
+#pragma unroll
+            for (int r = 0; r < RW; ++r)
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) M[r][q] = *reinterpret_cast<const f32x2 *>(G + r * ALG_NG * D + 32 * q);
+#pragma unroll 1
+            for (int sp = 1; sp < n_del; ++sp) {
+                G += D * D;
+#pragma unroll
+                for (int r = 0; r < RW; ++r)
+#pragma unroll
+                    for (int q = 0; q < NQ; ++q) M[r][q] = add2(M[r][q], *reinterpret_cast<const f32x2 *>(G + r * ALG_NG * D + 32 * q));
+            }
+        }
+        // this thread's share of the diagonal from row `from` on
+        auto diag_part = [&](int from) __attribute__((always_inline)) {
+            float s = 0.f;
+#pragma unroll
+            for (int r = 0; r < RW; ++r) {
+                const int i = grp + ALG_NG * r;
+                float a, b;
+                upk(M[r][r / SH::RPS], a, b);
+                if (i >= from && c16 == (i & 31) >> 1) s += (i & 1) ? b : a;
+            }
+            return s;
+        };
+
+        const float trAll = block_sum<ALG_NT>(diag_part(0), red);
+        // squared Frobenius norm of the deleted values (the denominator of RCR).  As a difference of two fp32 traces
+        // it is resolved down to about 1e-6 of the squared norm of all values: below 1e-5 of it the deleted values
+        // count as negligible beside the retained ones and nothing is injected.
+        const float trG = trAll - sq_keep;
+        const bool del_negligible = p.gram_all && !(trG > 1e-5f * trAll);
+        {
             auto double_up = [&](int j) __attribute__((always_inline)) {
                 if (tid < D) {
                     const float t = Y[j * D + tid];
