@@ -103,19 +103,19 @@ __device__ __forceinline__ float rcp_approx(float x)
     return r;
 }
 
-// The matrix in registers.  Half-warp g (of ALG_NG) holds rows g, g + ALG_NG, ..; lane c of its sixteen holds of each
-// row the pairs of columns 32 q + 2 c, 32 q + 2 c + 1.  A reflector and the product with it meet the warps in shared
-// memory twice: in order (for the columns) and with a half-warp's rows next to one another (for its rows; not doubled into
-// the pairs the two-wide FMA takes: a move is cheaper than twice the bytes from shared memory).
+// The matrix in registers.  Of every 32 consecutive rows half-warp g (of ALG_NG = 8) holds the four 4 g .. 4 g + 3, lane c
+// of its sixteen of each row the pairs of columns 32 q + 2 c, 32 q + 2 c + 1.  A reflector and the product with it meet the
+// warps in shared memory: a lane reads its columns two by two and its rows four by four from the same array.
 template <int D>
 struct AlgShape {
     static constexpr int RW = D / ALG_NG;        // rows a lane holds
     static constexpr int NQ = D / 32;            // column pairs a lane holds per row
     static constexpr int RPS = 32 / ALG_NG;      // rows a lane holds of 32 consecutive ones
-    static constexpr int GRP = RW + 4;           // entries per half-warp in an array by rows (padded against bank conflicts)
-    static constexpr int BYR = ALG_NG * GRP;     // floats of one such array
-    __device__ static __forceinline__ int row_index(int i) { return (i % ALG_NG) * GRP + i / ALG_NG; }
+    __device__ static __forceinline__ int row(int grp, int r) { return 32 * (r / RPS) + RPS * grp + r % RPS; }
+    __device__ static __forceinline__ int owner(int row) { return (row & 31) / RPS; }                    // its half-warp
+    __device__ static __forceinline__ int slot(int row) { return RPS * (row / 32) + row % RPS; }         // and place there
 };
+static_assert(ALG_NG == 8, "rows are read four at a time");
 template <int D>
 using AlgMat = f32x2[AlgShape<D>::RW][AlgShape<D>::NQ];
 template <int D>
@@ -138,23 +138,21 @@ __device__ __forceinline__ float alg_dot(const AlgRow<D> &x, const AlgRow<D> &y)
 }
 
 // Stage S serves the reflectors 32 S .. 32 S + 31: their support starts at row and column 32 S or later.
-// p = 2 M v on the rows of the stage; pd may be null.  With vd (the reflector by rows) also this half-warp's share of
+// po = 2 M v on the rows of the stage (v in shared memory, its column pairs in v2).  With kp also this half-warp's share of
 // v . p, in kp[grp]: formed from the lanes' partial sums, its reduction runs beside that of p.
 template <int D, int S>
-__device__ __forceinline__ void alg_product(const AlgMat<D> &M, const AlgRow<D> &v2, float *pl, float *pd, const float *vd, float *kp,
-                                            int grp, int c16)
+__device__ __forceinline__ void alg_product(const AlgMat<D> &M, const AlgRow<D> &v2, const float *v, float *po, float *kp, int grp, int c16)
 {
-    constexpr int RW = AlgShape<D>::RW, R0 = AlgShape<D>::RPS * S, NR = RW - R0;
+    constexpr int RW = AlgShape<D>::RW, RPS = AlgShape<D>::RPS, R0 = RPS * S, NR = RW - R0;
     constexpr int NP = NR > 8 ? 16 : NR > 4 ? 8 : NR > 2 ? 4 : 2;
     float acc[NP];
 #pragma unroll
     for (int r = 0; r < NP; ++r) acc[r] = r < NR ? alg_dot<D, S>(M[R0 + (r < NR ? r : 0)], v2) : 0.f;
     float ka = 0.f, kb = 0.f;
-    if (vd) {
-        const float *vr = vd + grp * AlgShape<D>::GRP + R0;
+    if (kp) {
 #pragma unroll
-        for (int r = 0; r < NR; r += 4) {
-            const float4 w = *reinterpret_cast<const float4 *>(vr + r);
+        for (int r = 0; r < NR; r += RPS) {
+            const float4 w = *reinterpret_cast<const float4 *>(v + 32 * (S + r / RPS) + RPS * grp);
             ka = fmaf(w.x, acc[r], ka);
             kb = fmaf(w.y, acc[r + 1], kb);
             ka = fmaf(w.z, acc[r + 2], ka);
@@ -165,22 +163,19 @@ __device__ __forceinline__ void alg_product(const AlgMat<D> &M, const AlgRow<D> 
     const float s = 2.f * transposed_sum<NP, 16>(acc, c16);
     constexpr int LPR = 16 / NP;
     const int r = c16 / LPR;
-    if ((c16 % LPR) == 0 && r < NR) {
-        pl[grp + ALG_NG * (R0 + r)] = s;
-        if (pd) pd[grp * AlgShape<D>::GRP + R0 + r] = s;
-    }
-    if (vd && c16 == 0) kp[grp] = ka;
+    if ((c16 % LPR) == 0 && r < NR) po[AlgShape<D>::row(grp, R0 + r)] = s;
+    if (kp && c16 == 0) kp[grp] = ka;
 }
 
 // M <- M - v w^T - w v^T with w = p - (v.p) v on the rows and columns of the stage.  x: row `xr` of the stage's first
 // RPS rows as the update leaves it, formed first so that the next reflector need not wait.
 template <int D, int S>
-__device__ __forceinline__ void alg_update(AlgMat<D> &M, const AlgRow<D> &v, const float *vd, const float *pl, const float *pd,
-                                           const float *kp, int grp, int c16, int xr, AlgRow<D> &x)
+__device__ __forceinline__ void alg_update(AlgMat<D> &M, const AlgRow<D> &v2, const float *v, const float *p, const float *kp, int grp,
+                                           int c16, int xr, AlgRow<D> &x)
 {
-    constexpr int RW = AlgShape<D>::RW, NQ = AlgShape<D>::NQ, R0 = AlgShape<D>::RPS * S;
-    AlgRow<D> w2, v2;
-    alg_load<D, S>(w2, pl, c16);
+    constexpr int RW = AlgShape<D>::RW, NQ = AlgShape<D>::NQ, RPS = AlgShape<D>::RPS, R0 = RPS * S;
+    AlgRow<D> w2, nv2;
+    alg_load<D, S>(w2, p, c16);
     float kq[ALG_NG / 4], kk = 0.f;
 #pragma unroll
     for (int e = 0; e < ALG_NG / 4; ++e) {
@@ -192,30 +187,30 @@ __device__ __forceinline__ void alg_update(AlgMat<D> &M, const AlgRow<D> &v, con
     const f32x2 nk = pk(-kk, -kk), neg = pk(-1.f, -1.f);
 #pragma unroll
     for (int q = S; q < NQ; ++q) {
-        w2[q] = mul2(fma2(nk, v[q], w2[q]), neg);
-        v2[q] = mul2(v[q], neg);
+        w2[q] = mul2(fma2(nk, v2[q], w2[q]), neg);
+        nv2[q] = mul2(v2[q], neg);
     }
-    const float *vr = vd + grp * AlgShape<D>::GRP, *pr = pd + grp * AlgShape<D>::GRP;
     {
-        const float v1 = vr[R0 + xr], w1 = fmaf(-kk, v1, pr[R0 + xr]);
+        const int row = AlgShape<D>::row(grp, R0) + xr;
+        const float v1 = v[row], w1 = fmaf(-kk, v1, p[row]);
         const f32x2 vx = pk(v1, v1), wx = pk(w1, w1);
         const f32x2 odd = mask2(xr & 1), high = mask2(xr & 2);
 #pragma unroll
         for (int q = S; q < NQ; ++q) {
-            f32x2 m = sel2(odd, M[R0 + 1][q], M[R0][q]);
-            if constexpr (AlgShape<D>::RPS == 4) m = sel2(high, sel2(odd, M[R0 + 3][q], M[R0 + 2][q]), m);
-            x[q] = fma2(vx, w2[q], fma2(wx, v2[q], m));
+            const f32x2 m = sel2(high, sel2(odd, M[R0 + 3][q], M[R0 + 2][q]), sel2(odd, M[R0 + 1][q], M[R0][q]));
+            x[q] = fma2(vx, w2[q], fma2(wx, nv2[q], m));
         }
     }
 #pragma unroll
-    for (int r = R0; r < RW; r += 4) {
-        const float4 va = *reinterpret_cast<const float4 *>(vr + r), pa = *reinterpret_cast<const float4 *>(pr + r);
+    for (int r = R0; r < RW; r += RPS) {
+        const int row = AlgShape<D>::row(grp, r);
+        const float4 va = *reinterpret_cast<const float4 *>(v + row), pa = *reinterpret_cast<const float4 *>(p + row);
         const float vv[4] = {va.x, va.y, va.z, va.w}, pp[4] = {pa.x, pa.y, pa.z, pa.w};
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
+        for (int e = 0; e < RPS; ++e) {
             const float w = fmaf(-kk, vv[e], pp[e]);
 #pragma unroll
-            for (int q = S; q < NQ; ++q) M[r + e][q] = fma2(pk(vv[e], vv[e]), w2[q], fma2(pk(w, w), v2[q], M[r + e][q]));
+            for (int q = S; q < NQ; ++q) M[r + e][q] = fma2(pk(vv[e], vv[e]), w2[q], fma2(pk(w, w), nv2[q], M[r + e][q]));
         }
     }
 }
@@ -251,7 +246,7 @@ __device__ __forceinline__ float alg_tail2(const AlgRow<D> &x, int from, int c16
 
 // Writes the unit reflector of support >= j0 made of x: entry j0 is `first`, the others x, all scaled (a half-warp's lanes).
 template <int D, int FROM = 0>
-__device__ __forceinline__ void alg_store_reflector(const AlgRow<D> &x, int j0, float first, float rs, float *v, float *vd, int c16)
+__device__ __forceinline__ void alg_store_reflector(const AlgRow<D> &x, int j0, float first, float rs, float *v, int c16)
 {
 #pragma unroll
     for (int q = 0; q < AlgShape<D>::NQ; ++q) {
@@ -261,17 +256,13 @@ __device__ __forceinline__ void alg_store_reflector(const AlgRow<D> &x, int j0, 
         a = c < j0 ? 0.f : (c == j0 ? first : a) * rs;
         b = c + 1 < j0 ? 0.f : (c + 1 == j0 ? first : b) * rs;
         *reinterpret_cast<f32x2 *>(v + c) = pk(a, b);
-        if (vd) {
-            vd[AlgShape<D>::row_index(c)] = a;
-            vd[AlgShape<D>::row_index(c + 1)] = b;
-        }
     }
 }
 
 // Reflector j + 1 from row j of the trailing block (entries of x from j on), with the row's diagonal and off-diagonal
 // entry of the tridiagonal form.  Every half-warp computes on its own row; the owner of row j stores.
 template <int D, int FROM>
-__device__ __forceinline__ void alg_row_done(const AlgRow<D> &x, int j, float tiny2, float *Y, float *vd, float *ta, float *tb,
+__device__ __forceinline__ void alg_row_done(const AlgRow<D> &x, int j, float tiny2, float *Y, float *ta, float *tb,
                                              int grp, int lane)
 {
     const int c16 = lane & 15;
@@ -282,8 +273,8 @@ __device__ __forceinline__ void alg_row_done(const AlgRow<D> &x, int j, float ti
     const float vn2 = 2.f * fmaf(nrm, fabsf(x0), n2);                // |x - al e_0|^2
     const bool skip = !(below2 > tiny2) || !(vn2 > 1e-37f);          // nothing beyond the super-diagonal
     const float rs = skip ? 0.f : rsqrt_approx(vn2);
-    if (grp == j % ALG_NG) {
-        alg_store_reflector<D, FROM>(x, j + 1, x0 - al, rs, Y + (j + 1) * D, vd, c16);
+    if (grp == AlgShape<D>::owner(j)) {
+        alg_store_reflector<D, FROM>(x, j + 1, x0 - al, rs, Y + (j + 1) * D, c16);
         if (c16 == 0) {
             ta[j] = dg;
             tb[j] = skip ? x0 : al;
@@ -350,7 +341,7 @@ __host__ __device__ constexpr int algebra_eig_floats(int rank, int fast_iters)
 template <int D>
 inline size_t algebra_smem_bytes(int mcap, int rank, int fast_iters)
 {
-    return (size_t)(algebra_y_rows<D>(mcap, rank, fast_iters) * D + 6 * AlgShape<D>::BYR + 2 * D + 6 * D + 96 +
+    return (size_t)(algebra_y_rows<D>(mcap, rank, fast_iters) * D +  2 * D + 6 * D + 96 +
                     algebra_eig_floats<D>(rank, fast_iters)) * sizeof(float) + 2 * D * sizeof(int);
 }
 
@@ -362,9 +353,7 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
     constexpr int RW = SH::RW, NQ = SH::NQ, LD = D + 1;
     extern __shared__ __align__(16) float sm[];
     float *Y = sm;                                                    // reflector j in row j, support >= j
-    float *vrows = Y + algebra_y_rows<D>(p.alg_rows, p.rank, p.fast_iters) * D;   // 4 buffers: reflector j in j & 3
-    float *prows = vrows + 4 * SH::BYR;                                 // 2 buffers
-    float *pl = prows + 2 * SH::BYR;        // 2 buffers of D
+    float *pl = Y + algebra_y_rows<D>(p.alg_rows, p.rank, p.fast_iters) * D;     // 2 buffers of D: the product with reflector j in j & 1
     float *ta = pl + 2 * D, *tb = ta + D;                             // tridiagonal form
     float *vu = tb + D, *vx = vu + D, *vc = vx + D, *vl = vc + D;     // vectors of d
     float *red = vl + D, *misc = red + 32, *tlam = misc + 32;         // 32 floats each
@@ -525,7 +514,7 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                     const bool add = m < D && t2 > SPAN_ROW_TOL * SPAN_ROW_TOL * nn && t2 > 1e-37f;
                     if (add) {
                         const float al = x0 >= 0.f ? -nrm : nrm;
-                        alg_store_reflector<D>(x, m, x0 - al, rsqrt_approx(2.f * fmaf(nrm, fabsf(x0), t2)), Y + m * D, nullptr, c16);
+                        alg_store_reflector<D>(x, m, x0 - al, rsqrt_approx(2.f * fmaf(nrm, fabsf(x0), t2)), Y + m * D, c16);
                     }
                     if (c16 == 0) s_flag[i & 1] = add ? 1 : 0;
                 }
@@ -580,18 +569,18 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
         // ---- G into registers, its trace, and the reflectors applied to it from both sides -----------------------
         AlgMat<D> M;
         {
-            const float *G = p.gram_d + (size_t)g * S * D * D + grp * D + 2 * c16;
+            const float *G = p.gram_d + (size_t)g * S * D * D + 2 * c16;
 #pragma unroll
             for (int r = 0; r < RW; ++r)
 #pragma unroll
-                for (int q = 0; q < NQ; ++q) M[r][q] = *reinterpret_cast<const f32x2 *>(G + r * ALG_NG * D + 32 * q);
+                for (int q = 0; q < NQ; ++q) M[r][q] = *reinterpret_cast<const f32x2 *>(G + SH::row(grp, r) * D + 32 * q);
 #pragma unroll 1
             for (int sp = 1; sp < n_del; ++sp) {
                 G += D * D;
 #pragma unroll
                 for (int r = 0; r < RW; ++r)
 #pragma unroll
-                    for (int q = 0; q < NQ; ++q) M[r][q] = add2(M[r][q], *reinterpret_cast<const f32x2 *>(G + r * ALG_NG * D + 32 * q));
+                    for (int q = 0; q < NQ; ++q) M[r][q] = add2(M[r][q], *reinterpret_cast<const f32x2 *>(G + SH::row(grp, r) * D + 32 * q));
             }
         }
         // this thread's share of the diagonal from row `from` on
@@ -599,7 +588,7 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
             float s = 0.f;
 #pragma unroll
             for (int r = 0; r < RW; ++r) {
-                const int i = grp + ALG_NG * r;
+                const int i = SH::row(grp, r);
                 float a, b;
                 upk(M[r][r / SH::RPS], a, b);
                 if (i >= from && c16 == (i & 31) >> 1) s += (i & 1) ? b : a;
@@ -614,29 +603,20 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
         const float trG = trAll - sq_keep;
         const bool del_negligible = p.gram_all && !(trG > 1e-5f * trAll);
         {
-            auto double_up = [&](int j) __attribute__((always_inline)) {
-                if (tid < D) {
-                    const float t = Y[j * D + tid];
-                    vrows[(j & 3) * SH::BYR + SH::row_index(tid)] = t;
-                }
-            };
             auto apply_stage = [&](auto stage) __attribute__((always_inline)) {
                 constexpr int ST = decltype(stage)::value;
                 const int j1 = min(32 * ST + 32, m);
 #pragma unroll 1
                 for (int j = 32 * ST; j < j1; ++j) {
-                    const int pb = j & 1;
+                    float *po = pl + (j & 1) * D, *kp = kpart + (j & 1) * ALG_NG;
                     AlgRow<D> v, x;
                     alg_load<D, ST>(v, Y + j * D, c16);
-                    alg_product<D, ST>(M, v, pl + pb * D, prows + pb * SH::BYR, vrows + (j & 3) * SH::BYR, kpart + pb * ALG_NG, grp, c16);
-                    if (j + 1 < m) double_up(j + 1);
-                    __syncthreads();                                   // p is there, and the next reflector doubled
-                    alg_update<D, ST>(M, v, vrows + (j & 3) * SH::BYR, pl + pb * D, prows + pb * SH::BYR, kpart + pb * ALG_NG, grp, c16, 0, x);
+                    alg_product<D, ST>(M, v, Y + j * D, po, kp, grp, c16);
+                    __syncthreads();                                   // p is there
+                    alg_update<D, ST>(M, v, Y + j * D, po, kp, grp, c16, 0, x);
                 }
             };
             if (m < D) {
-                if (m > 0) double_up(0);
-                __syncthreads();
                 apply_stage(std::integral_constant<int, 0>{});
                 apply_stage(std::integral_constant<int, 1>{});
                 if constexpr (D > 64) {
@@ -755,29 +735,28 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                     for (int q = 0; q < NQ; ++q) {
                         x[q] = M[0][q];
 #pragma unroll
-                        for (int r = 1; r < RW; ++r) x[q] = sel2(mask2(r == m / ALG_NG), M[r][q], x[q]);
+                        for (int r = 1; r < RW; ++r) x[q] = sel2(mask2(r == SH::slot(m)), M[r][q], x[q]);
                     }
-                    alg_row_done<D, 0>(x, m, tiny2, Y, vrows + ((m + 1) & 3) * SH::BYR, ta, tb, grp, lane);
+                    alg_row_done<D, 0>(x, m, tiny2, Y, ta, tb, grp, lane);
                 }
                 auto reduce_stage = [&](auto stage) __attribute__((always_inline)) {
                     constexpr int ST = decltype(stage)::value;
                     const int j1 = min(32 * ST + 31, D - 2);
 #pragma unroll 1
                     for (int j = max(m + 1, 32 * ST); j <= j1; ++j) {
-                        const int pb = j & 1;
+                        float *po = pl + (j & 1) * D, *kp = kpart + (j & 1) * ALG_NG;
                         AlgRow<D> v, x;
                         __syncthreads();                               // reflector j is there
                         alg_load<D, ST>(v, Y + j * D, c16);
-                        alg_product<D, ST>(M, v, pl + pb * D, prows + pb * SH::BYR, vrows + (j & 3) * SH::BYR, kpart + pb * ALG_NG, grp, c16);
+                        alg_product<D, ST>(M, v, Y + j * D, po, kp, grp, c16);
                         {
                             const float s = -2.f * half_sum(alg_dot<D, ST>(aux, v));
 #pragma unroll
                             for (int q = ST; q < NQ; ++q) aux[q] = fma2(pk(s, s), v[q], aux[q]);
                         }
                         __syncthreads();                               // p is there
-                        alg_update<D, ST>(M, v, vrows + (j & 3) * SH::BYR, pl + pb * D, prows + pb * SH::BYR, kpart + pb * ALG_NG,
-                                          grp, c16, (j / ALG_NG) & (SH::RPS - 1), x);
-                        alg_row_done<D, ST>(x, j, tiny2, Y, vrows + ((j + 1) & 3) * SH::BYR, ta, tb, grp, lane);
+                        alg_update<D, ST>(M, v, Y + j * D, po, kp, grp, c16, j & (SH::RPS - 1), x);
+                        alg_row_done<D, ST>(x, j, tiny2, Y, ta, tb, grp, lane);
                     }
                 };
                 reduce_stage(std::integral_constant<int, 0>{});
@@ -790,7 +769,7 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                     // the last diagonal entry
                     float a, b;
                     upk(M[RW - 1][NQ - 1], a, b);
-                    if (grp == (D - 1) % ALG_NG && c16 == 15) ta[D - 1] = b;
+                    if (grp == SH::owner(D - 1) && c16 == 15) ta[D - 1] = b;
                 }
                 if (grp == 0) {
 #pragma unroll
@@ -1136,7 +1115,7 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                         AlgRow<D> v;
                         alg_load<D>(v, C + i * D, c16);
                         auto one = [&](auto stage) __attribute__((always_inline)) {
-                            alg_product<D, decltype(stage)::value>(M, v, Yb + i * D, nullptr, nullptr, nullptr, grp, c16);
+                            alg_product<D, decltype(stage)::value>(M, v, nullptr, Yb + i * D, nullptr, grp, c16);
                         };
                         if (D > 64 && m >= 96) one(std::integral_constant<int, D / 32 - 1>{});
                         else if (D > 64 && m >= 64) one(std::integral_constant<int, D / 32 - 2>{});
@@ -1214,7 +1193,7 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                 for (int r = 0; r < RW; ++r)
 #pragma unroll
                     for (int q = 0; q < NQ; ++q) {
-                        const int i = grp + ALG_NG * r, cc = 32 * q + 2 * c16;
+                        const int i = SH::row(grp, r), cc = 32 * q + 2 * c16;
                         float a, b;
                         upk(M[r][q], a, b);
                         B2[i * LD + cc] = (i >= m && cc >= m) ? a : 0.f;

@@ -32,13 +32,12 @@ template <int D>
 struct SpanShape {
     static constexpr int ROWS = 2 * D;             // retained rows that enter G_keep with FROM_ROWS
     static constexpr int LD = D + 2;               // of the matrix on its way from the tensor cores to the registers
-    static constexpr int PG = AlgShape<D>::RW + 4; // a half-warp's entries of the pivot row, next to one another
 };
 
 template <int D>
 constexpr size_t span_smem_bytes(bool from_rows)
 {
-    return (from_rows ? (size_t)D * SpanShape<D>::LD : 0) * sizeof(float) + (size_t)(4 * D + 4 * ALG_NG * SpanShape<D>::PG + D) * sizeof(float);
+    return (from_rows ? (size_t)D * SpanShape<D>::LD : 0) * sizeof(float) + (size_t)(4 * D + D) * sizeof(float);
 }
 
 template <int D, bool FROM_ROWS = false>
@@ -46,11 +45,10 @@ __global__ void __launch_bounds__(ST_NT, 2) k_span_test(const __grid_constant__ 
 {
     pdl_wait();
     typedef AlgShape<D> SH;
-    constexpr int RW = SH::RW, NQ = SH::NQ, LD = SpanShape<D>::LD, PG = SpanShape<D>::PG;
+    constexpr int RW = SH::RW, NQ = SH::NQ, LD = SpanShape<D>::LD;
     extern __shared__ __align__(16) float st_sm[];
-    float *rowo = st_sm;                                   // 2 buffers of 2 pivot rows, in order
-    float *rowp = rowo + 4 * D;                            // the same, half-warp by half-warp
-    float *dg = rowp + 4 * ALG_NG * PG;                    // D original diagonal entries
+    float *rows_s = st_sm;                                 // 2 buffers of 2 pivot rows
+    float *dg = rows_s + 4 * D;                    // D original diagonal entries
     float *A = dg + D;                                     // FROM_ROWS: the rows, then the matrix
 
     const int g = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, grp = tid >> 4, c16 = tid & 15;
@@ -138,44 +136,37 @@ __global__ void __launch_bounds__(ST_NT, 2) k_span_test(const __grid_constant__ 
             }
         __syncthreads();
 #pragma unroll
-        for (int r = 0; r < RW; ++r) alg_load<D>(M[r], A + (grp + ALG_NG * r) * LD, c16);
+        for (int r = 0; r < RW; ++r) alg_load<D>(M[r], A + SH::row(grp, r) * LD, c16);
     } else {
         const int n_part = gram_partial_count(p, c, lh);           // shape-generic path: one per token split
-        const float *G = p.gram_k + (size_t)g * p.gram_slots * D * D + grp * D + 2 * c16;
+        const float *G = p.gram_k + (size_t)g * p.gram_slots * D * D + 2 * c16;
 #pragma unroll
         for (int r = 0; r < RW; ++r)
 #pragma unroll
-            for (int q = 0; q < NQ; ++q) M[r][q] = *reinterpret_cast<const f32x2 *>(G + r * ALG_NG * D + 32 * q);
+            for (int q = 0; q < NQ; ++q) M[r][q] = *reinterpret_cast<const f32x2 *>(G + SH::row(grp, r) * D + 32 * q);
 #pragma unroll 1
         for (int sp = 1; sp < n_part; ++sp) {
             G += D * D;
 #pragma unroll
             for (int r = 0; r < RW; ++r)
 #pragma unroll
-                for (int q = 0; q < NQ; ++q) M[r][q] = add2(M[r][q], *reinterpret_cast<const f32x2 *>(G + r * ALG_NG * D + 32 * q));
+                for (int q = 0; q < NQ; ++q) M[r][q] = add2(M[r][q], *reinterpret_cast<const f32x2 *>(G + SH::row(grp, r) * D + 32 * q));
         }
     }
 #pragma unroll
     for (int r = 0; r < RW; ++r) {
-        const int i = grp + ALG_NG * r;
+        const int i = SH::row(grp, r);
         float a, b;
         upk(M[r][r / SH::RPS], a, b);
         if (c16 == (i & 31) >> 1) dg[i] = (i & 1) ? b : a;
     }
     // row `row`, one of the two of buffer `buf`, for everybody (a half-warp's lanes)
     auto publish = [&](int buf, int row, const AlgRow<D> &x) __attribute__((always_inline)) {
-        float *ro = rowo + (2 * buf + row) * D + 2 * c16;
-        float *rp = rowp + ((2 * buf + row) * ALG_NG + (2 * c16) % ALG_NG) * PG + 2 * c16 / ALG_NG;
+        float *ro = rows_s + (2 * buf + row) * D + 2 * c16;
 #pragma unroll
-        for (int q = 0; q < NQ; ++q) {
-            float a, b;
-            upk(x[q], a, b);
-            *reinterpret_cast<f32x2 *>(ro + 32 * q) = x[q];
-            rp[32 * q / ALG_NG] = a;
-            rp[32 * q / ALG_NG + PG] = b;
-        }
+        for (int q = 0; q < NQ; ++q) *reinterpret_cast<f32x2 *>(ro + 32 * q) = x[q];
     };
-    if (grp < 2) publish(0, grp, M[0]);
+    if (grp == 0) { publish(0, 0, M[0]); publish(0, 1, M[1]); }
     bool ok = true;
     // the pivots 32 S .. 32 S + 31, two at a time: rows and columns before 32 S are finished
     auto pivots = [&](auto stage) __attribute__((always_inline)) {
@@ -183,7 +174,7 @@ __global__ void __launch_bounds__(ST_NT, 2) k_span_test(const __grid_constant__ 
 #pragma unroll 1
         for (int j = 32 * S; ok && j < 32 * S + 32; j += 2) {
             const int buf = (j >> 1) & 1;
-            const float *ra = rowo + 2 * buf * D, *rb = ra + D;
+            const float *ra = rows_s + 2 * buf * D, *rb = ra + D;
             __syncthreads();                               // rows j and j + 1 are there, as the pivots before j have left them
             const float p0 = ra[j], e = ra[j + 1], i0 = -rcp_approx(p0), l = e * i0, p1 = fmaf(l, e, rb[j + 1]), i1 = -rcp_approx(p1);
             ok = p0 > CHOL_PIVOT_TOL * dg[j] && p0 > 0.f && p1 > CHOL_PIVOT_TOL * dg[j + 1] && p1 > 0.f;   // the same in every thread
@@ -195,34 +186,35 @@ __global__ void __launch_bounds__(ST_NT, 2) k_span_test(const __grid_constant__ 
                 v1[q] = mul2(fma2(pk(l, l), v0[q], v1[q]), pk(i1, i1));        // row j + 1 without pivot j, over its pivot
                 v0[q] = mul2(v0[q], pk(i0, i0));
             }
-            if (j + 2 < D && warp == ((j + 2) % ALG_NG) / 2) {
-                // rows j + 2 and j + 3, one per half-warp, before the others
-                const int i = j + 2 + (grp & 1), r2 = (j + 2) / ALG_NG;
-                const float w0 = ra[i], w1 = fmaf(l, w0, rb[i]);
+            if (j + 2 < D && grp == SH::owner(j + 2)) {
+                // rows j + 2 and j + 3 before the others
+                const float2 ea = *reinterpret_cast<const float2 *>(ra + j + 2), eb = *reinterpret_cast<const float2 *>(rb + j + 2);
+                const float w0[2] = {ea.x, ea.y}, w1[2] = {fmaf(l, ea.x, eb.x), fmaf(l, ea.y, eb.y)};
                 auto take = [&](auto cand) __attribute__((always_inline)) {
                     constexpr int R = decltype(cand)::value;
-                    if (R < RW && r2 == R) {
-                        AlgRow<D> x;
+                    if (R < RW && SH::slot(j + 2) == R) {
 #pragma unroll
-                        for (int q = 0; q < NQ; ++q) {
-                            x[q] = M[R < RW ? R : 0][q];
-                            if (q >= S) x[q] = fma2(pk(w1, w1), v1[q], fma2(pk(w0, w0), v0[q], x[q]));
-                            // (keeps the compiler from merging the candidates' code into one that addresses the array)
-                            asm volatile("// %1" : "+l"(x[q]) : "n"(R));
+                        for (int e = 0; e < 2; ++e) {
+                            AlgRow<D> x;
+#pragma unroll
+                            for (int q = 0; q < NQ; ++q) {
+                                x[q] = M[R + e < RW ? R + e : 0][q];
+                                if (q >= S) x[q] = fma2(pk(w1[e], w1[e]), v1[q], fma2(pk(w0[e], w0[e]), v0[q], x[q]));
+                                // (keeps the compiler from merging the candidates' code into one that addresses the array)
+                                asm volatile("// %1" : "+l"(x[q]) : "n"(R));
+                            }
+                            publish(buf ^ 1, e, x);
                         }
-                        publish(buf ^ 1, grp & 1, x);
                     }
                 };
                 take(std::integral_constant<int, R0>{});
-                take(std::integral_constant<int, R0 + 1>{});
                 take(std::integral_constant<int, R0 + 2>{});
-                take(std::integral_constant<int, R0 + 3>{});
                 take(std::integral_constant<int, R0 + 4>{});
             }
-            const float *pa = rowp + (2 * buf * ALG_NG + grp) * PG, *pb = pa + ALG_NG * PG;
 #pragma unroll
             for (int r = R0; r < RW; r += 4) {
-                const float4 a4 = *reinterpret_cast<const float4 *>(pa + r), b4 = *reinterpret_cast<const float4 *>(pb + r);
+                const int row = SH::row(grp, r);
+                const float4 a4 = *reinterpret_cast<const float4 *>(ra + row), b4 = *reinterpret_cast<const float4 *>(rb + row);
                 const float aa[4] = {a4.x, a4.y, a4.z, a4.w}, bb[4] = {b4.x, b4.y, b4.z, b4.w};
 #pragma unroll
                 for (int x = 0; x < 4; ++x) {
@@ -233,7 +225,7 @@ __global__ void __launch_bounds__(ST_NT, 2) k_span_test(const __grid_constant__ 
             }
         }
     };
-    static_assert(SH::RPS == 4, "five candidates for the next rows");
+    static_assert(SH::RPS == 4, "three places for the next rows");
     pivots(std::integral_constant<int, 0>{});
     pivots(std::integral_constant<int, 1>{});
     if constexpr (D > 64) {
