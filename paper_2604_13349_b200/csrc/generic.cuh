@@ -148,6 +148,22 @@ __global__ void __launch_bounds__(SC_NT) k_score_pool(const __grid_constant__ Ca
     }
 }
 
+// What a selection leaves for its head: the demand sums and, where asked for, a fresh diagnostics record.
+__device__ __forceinline__ void store_selection(const CallDev &p, const CacheDev &c, int g, int lh, float a_keep, float a_del, float next, uint32_t tau)
+{
+    float *sm = p.sums + (size_t)g * 4;
+    const float kth = tau == 0xFFFFFFFFu ? INFINITY : key_score(tau);
+    sm[0] = a_keep; sm[1] = a_del; sm[2] = kth; sm[3] = next;
+    if (c.diag) {
+        obf_diag_t dg;
+        dg.a_keep = a_keep; dg.a_del = a_del; dg.alpha = a_del / (a_keep + p.eps);
+        dg.rcr = 0.f; dg.delta_norm = 0.f; dg.kth_score = kth; dg.next_score = next;
+        dg.lam_1 = dg.lam_rho = dg.lam_next = 0.f;
+        dg.span_rank = -1; dg.rho_eff = 0; dg.status = OBF_DEV_SKIPPED; dg.revr = 0.f; dg.pc = 0.f;
+        c.diag[lh] = dg;
+    }
+}
+
 // Step a2: radix select of the k_eff largest masses on their order-preserving
 // 32-bit keys (4 passes of 8 bits), then one ordered pass that emits the
 // retained positions in ascending order; among masses equal to the k_eff-th
@@ -249,18 +265,13 @@ __global__ void __launch_bounds__(SEL_NT) k_select(const __grid_constant__ CallD
     const float a_del = block_sum<SEL_NT>(sd, red);
     const float next = block_max<SEL_NT>(nx, red);
     if (tid == 0) {
-        float *s = p.sums + (size_t)blockIdx.x * 4;
-        s[0] = a_keep; s[1] = a_del; s[2] = tau == 0xFFFFFFFFu ? INFINITY : key_score(tau); s[3] = next;
-        if (c.diag) {
-            obf_diag_t dg;
-            dg.a_keep = a_keep; dg.a_del = a_del; dg.alpha = a_del / (a_keep + p.eps);
-            dg.rcr = 0.f; dg.delta_norm = 0.f; dg.kth_score = tau == 0xFFFFFFFFu ? INFINITY : key_score(tau); dg.next_score = next;
-            dg.lam_1 = dg.lam_rho = dg.lam_next = 0.f;
-            dg.span_rank = -1; dg.rho_eff = 0; dg.status = OBF_DEV_SKIPPED; dg.revr = 0.f; dg.pc = 0.f;
-            c.diag[lh] = dg;
-        }
+        store_selection(p, c, blockIdx.x, lh, a_keep, a_del, next, tau);
     }
 }
+
+// Retained rows that the selection copies itself (k_select_smem): with this few a copy of its own costs a launch, 2 us, for
+// what the head's block has in hand a moment after the positions; the block's threads fetch all of them at once.
+constexpr int SEL_GATHER_MAX = 64;
 
 // Step a2 for heads whose T keys fit in shared memory (the usual case): same result as
 // k_select, bit for bit, but the order-preserving keys are read from global memory
@@ -288,8 +299,10 @@ __global__ void __launch_bounds__(256) k_layer_sum(const __grid_constant__ CallD
 // With LAYER every head's block selects on its layer's summed masses (the layer's heads repeat the same
 // selection side by side rather than one block writing all of them in turn) and then writes the shared
 // positions, the keep flags and the demand sums of the head's own masses.
+// gather_vecs > 0: every budget is at most SEL_GATHER_MAX and the block copies its head's retained rows of K and V too, that
+// many 16-byte vectors each.
 template <int NT, bool LAYER = false>
-__global__ void __launch_bounds__(NT) k_select_smem(const __grid_constant__ CallDev p)
+__global__ void __launch_bounds__(NT) k_select_smem(const __grid_constant__ CallDev p, int gather_vecs)
 {
     pdl_wait();
     extern __shared__ uint32_t sel_keys[];
@@ -297,7 +310,8 @@ __global__ void __launch_bounds__(NT) k_select_smem(const __grid_constant__ Call
     __shared__ uint32_t s_prefix, s_want;
     constexpr int NW = NT / 32;
     __shared__ uint32_t wtot[32];
-    __shared__ float red[32];
+    __shared__ float red[3][32];
+    __shared__ int s_idx[SEL_GATHER_MAX];
     int ci, lh;
     locate(p, blockIdx.x, ci, lh);
     const CacheDev &c = p.c[ci];
@@ -399,6 +413,36 @@ __global__ void __launch_bounds__(NT) k_select_smem(const __grid_constant__ Call
         wtot[lane] = inc - w;              // positions before this warp's run: greater (low half), equal (high half)
     }
     __syncthreads();
+    // retained rows, once their positions are in s_idx
+    auto copy_rows = [&]() {
+        __syncthreads();
+        const size_t to = (size_t)lh * k * gather_vecs;
+        const uint4 *ks = reinterpret_cast<const uint4 *>(c.k) + (size_t)lh * T * gather_vecs, *vs = reinterpret_cast<const uint4 *>(c.v) + (size_t)lh * T * gather_vecs;
+        for (int e = tid; e < k * gather_vecs; e += NT) {
+            const int r = e / gather_vecs, ch = e - r * gather_vecs;
+            const int j = s_idx[r];
+            if ((unsigned)j >= (unsigned)T) {             // never dereference a position outside the cache
+                atomicOr(p.status, OBF_DEV_INTERNAL);
+                continue;
+            }
+            const size_t from = (size_t)j * gather_vecs + ch;
+            const uint4 a = ks[from], b = vs[from];
+            reinterpret_cast<uint4 *>(c.k_out)[to + e] = a;
+            reinterpret_cast<uint4 *>(c.v_out)[to + e] = b;
+        }
+    };
+    // block totals of the retained and the deleted mass and the largest deleted one
+    auto finish = [&](float sk, float sd, float nx) {
+        sk = warp_sum(sk); sd = warp_sum(sd); nx = warp_max(nx);
+        if (lane == 0) { red[0][warp] = sk; red[1][warp] = sd; red[2][warp] = nx; }
+        __syncthreads();
+        if (warp == 0) {
+            sk = warp_sum(lane < NW ? red[0][lane] : 0.f);
+            sd = warp_sum(lane < NW ? red[1][lane] : 0.f);
+            nx = warp_max(lane < NW ? red[2][lane] : -1.0f);
+            if (lane == 0) store_selection(p, c, blockIdx.x, lh, sk, sd, nx, tau);
+        }
+    };
     uint32_t run_gt = wtot[warp] & 0xFFFFu, run_eq = wtot[warp] >> 16;
     float sk = 0.f, sd = 0.f, nx = -1.0f;
     const uint32_t lt_mask = (1u << lane) - 1u;
@@ -422,7 +466,10 @@ __global__ void __launch_bounds__(NT) k_select_smem(const __grid_constant__ Call
             keep[j] = kp ? 1 : 0;
             if (kp) {
                 const uint32_t pos = gt_before + min(eq_before, want);
-                if (pos < (uint32_t)k) idx[pos] = j;
+                if (pos < (uint32_t)k) {
+                    idx[pos] = j;
+                    if (gather_vecs) s_idx[pos] = j;
+                }
                 else atomicOr(p.status, OBF_DEV_INTERNAL);
                 sk += a;
             } else { sd += a; nx = fmaxf(nx, a); }
@@ -435,56 +482,23 @@ __global__ void __launch_bounds__(NT) k_select_smem(const __grid_constant__ Call
         // the largest summed mass among the deleted positions, for the diagnostics
         for (int j = tid; j < T; j += NT)
             if (sel_keys[j] == 0xFFFFFFFFu) nx = fmaxf(nx, __uint_as_float(A[j]));
-        const float next = block_max<NT>(nx, red);
-        {
-            float *Ah = Af;
-            uint8_t *keep_h = keep;
-            int32_t *idx_h = idx;
-            sk = 0.f; sd = 0.f;
-            for (int j = tid; j < T; j += NT) {
-                const uint32_t pos = sel_keys[j];
-                const float a = Ah[j];
-                const bool kp = pos != 0xFFFFFFFFu;
-                keep_h[j] = kp ? 1 : 0;
-                if (kp) {
-                    idx_h[pos] = j;
-                    sk += a;
-                } else {
-                    sd += a;
-                }
-            }
-            const float a_keep = block_sum<NT>(sk, red);
-            const float a_del = block_sum<NT>(sd, red);
-            if (tid == 0) {
-                float *sm = p.sums + (size_t)blockIdx.x * 4;
-                sm[0] = a_keep; sm[1] = a_del; sm[2] = tau == 0xFFFFFFFFu ? INFINITY : key_score(tau); sm[3] = next;
-                if (c.diag) {
-                    obf_diag_t dg;
-                    dg.a_keep = a_keep; dg.a_del = a_del; dg.alpha = a_del / (a_keep + p.eps);
-                    dg.rcr = 0.f; dg.delta_norm = 0.f; dg.kth_score = tau == 0xFFFFFFFFu ? INFINITY : key_score(tau); dg.next_score = next;
-                    dg.lam_1 = dg.lam_rho = dg.lam_next = 0.f;
-                    dg.span_rank = -1; dg.rho_eff = 0; dg.status = OBF_DEV_SKIPPED; dg.revr = 0.f; dg.pc = 0.f;
-                    c.diag[lh] = dg;
-                }
+        sk = 0.f; sd = 0.f;
+        for (int j = tid; j < T; j += NT) {
+            const uint32_t pos = sel_keys[j];
+            const float a = Af[j];
+            const bool kp = pos != 0xFFFFFFFFu;
+            keep[j] = kp ? 1 : 0;
+            if (kp) {
+                idx[pos] = j;
+                if (gather_vecs) s_idx[pos] = j;
+                sk += a;
+            } else {
+                sd += a;
             }
         }
-        return;
     }
-    const float a_keep = block_sum<NT>(sk, red);
-    const float a_del = block_sum<NT>(sd, red);
-    const float next = block_max<NT>(nx, red);
-    if (tid == 0) {
-        float *sm = p.sums + (size_t)blockIdx.x * 4;
-        sm[0] = a_keep; sm[1] = a_del; sm[2] = tau == 0xFFFFFFFFu ? INFINITY : key_score(tau); sm[3] = next;
-        if (c.diag) {
-            obf_diag_t dg;
-            dg.a_keep = a_keep; dg.a_del = a_del; dg.alpha = a_del / (a_keep + p.eps);
-            dg.rcr = 0.f; dg.delta_norm = 0.f; dg.kth_score = tau == 0xFFFFFFFFu ? INFINITY : key_score(tau); dg.next_score = next;
-            dg.lam_1 = dg.lam_rho = dg.lam_next = 0.f;
-            dg.span_rank = -1; dg.rho_eff = 0; dg.status = OBF_DEV_SKIPPED; dg.revr = 0.f; dg.pc = 0.f;
-            c.diag[lh] = dg;
-        }
-    }
+    if (gather_vecs) copy_rows();
+    finish(sk, sd, nx);
 }
 
 // Step a3: K_out = K[idx], V_out = V[idx] as 16-byte vectors.  A block copies GATHER_ROWS

@@ -442,6 +442,8 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
         OBF_CUDA_TRY(cudaStreamWaitEvent(side->stream, side->fork, 0));
         if ((s = launch_gram_tc<D>(cd, L, st)) != OBF_OK) return s;
     }
+    // few retained rows and no span test that waits for them beside the pass over V: the selection copies them itself
+    const int gather_vecs = T_max <= SEL_SMEM_MAX_T && k_max <= SEL_GATHER_MAX && !span ? D * (int)sizeof(TIN) / 16 : 0;
     if (cd.layerwise) {
         // masses of a layer's KV heads added up, then every head's block selects on its layer's sums
         const int n_layers = heads / cd.kv_heads;
@@ -452,10 +454,10 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
         const int sms = sm_count();
         if (heads > 2 * sms && heads <= 4 * sms) {
             if ((s = set_smem(k_select_smem<512, true>, sm_sel)) != OBF_OK) return s;
-            OBF_TRY(launch(k_select_smem<512, true>, dim3(heads), 512, sm_sel, sel, cd));
+            OBF_TRY(launch(k_select_smem<512, true>, dim3(heads), 512, sm_sel, sel, cd, gather_vecs));
         } else {
             if ((s = set_smem(k_select_smem<1024, true>, sm_sel)) != OBF_OK) return s;
-            OBF_TRY(launch(k_select_smem<1024, true>, dim3(heads), 1024, sm_sel, sel, cd));
+            OBF_TRY(launch(k_select_smem<1024, true>, dim3(heads), 1024, sm_sel, sel, cd, gather_vecs));
         }
     } else if (T_max <= SEL_SMEM_MAX_T) {
         const size_t sm_sel = (size_t)T_max * sizeof(uint32_t);
@@ -464,17 +466,22 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
         const int sms = sm_count();
         if (heads > 2 * sms && heads <= 4 * sms) {
             if ((s = set_smem(k_select_smem<512>, sm_sel)) != OBF_OK) return s;
-            OBF_TRY(launch(k_select_smem<512>, dim3(heads), 512, sm_sel, sel, cd));
+            OBF_TRY(launch(k_select_smem<512>, dim3(heads), 512, sm_sel, sel, cd, gather_vecs));
         } else {
             if ((s = set_smem(k_select_smem<1024>, sm_sel)) != OBF_OK) return s;
-            OBF_TRY(launch(k_select_smem<1024>, dim3(heads), 1024, sm_sel, sel, cd));
+            OBF_TRY(launch(k_select_smem<1024>, dim3(heads), 1024, sm_sel, sel, cd, gather_vecs));
         }
     } else {
         OBF_TRY(launch(k_select, dim3(heads), SEL_NT, 0, sel, cd));
     }
     mark(sel, "k_select");
     dim3 g4((k_max + GATHER_ROWS - 1) / GATHER_ROWS, heads);
-    if (side) {
+    if (gather_vecs) {
+        if (side) {
+            OBF_CUDA_TRY(cudaEventRecord(side->join, side->stream));
+            OBF_CUDA_TRY(cudaStreamWaitEvent(st, side->join, 0));
+        }
+    } else if (side) {
         // the values first: the rest of the call needs them
         OBF_TRY(launch(k_gather<D * (int)sizeof(TIN), 1>, dim3(g4), 256, 0, sel, cd));
         mark(sel, "k_gather");

@@ -922,3 +922,24 @@ def test_fast_path_matches_the_oracles_same_iteration(dtype, d, rank, caches):
                 tol = (2e-3 * scale + 1e-4) if dtype == "f32" else (2e-2 * np.abs(ref["V_out"]) + 2e-3 * scale + 1e-3)
                 assert np.all(np.abs(gv - ref["V_out"]) <= tol)
     print("\n[fast path] worst relative delta error %.3g" % worst)
+
+
+# ---------------------------------------------------------------------------
+# few retained rows: the selection copies them itself, with more of them a kernel of its own does
+# ---------------------------------------------------------------------------
+@pytest.mark.parametrize("dtype,d,flags", [("f32", 32, 0), ("f32", 128, 0), ("bf16", 64, 0), ("bf16", 128, 0),
+                                           ("bf16", 128, P.binding.OBF_FLAG_LAYERWISE)])
+@pytest.mark.parametrize("caches", [((300, 1),), ((64, 64), (701, 63)), ((1500, 64),), ((300, 65), (90, 7))])
+def test_retained_rows_are_copied_whoever_copies_them(dtype, d, flags, caches):
+    w = small("copies", layers=2, d=d, dtype=dtype, rank=1, caches=caches, seed=71)
+    arrays = [synth.gen_cache(w, ci) for ci in range(len(w.caches))]
+    for evict in (True, False):
+        outs, _, st = par.run_gpu(w, arrays, evict=evict, flags=flags)
+        assert st & 0xFF == 0
+        for a, o in zip(arrays, outs):
+            idx = o["idx"].cpu().numpy()
+            assert np.all(np.diff(idx, axis=-1) > 0)
+            for l, h in all_heads(w):
+                assert np.array_equal(o["K_out"][l, h].float().cpu().numpy(), par.f32_view(a["K"][l, h], dtype)[idx[l, h]])
+                if evict:
+                    assert np.array_equal(o["V_out"][l, h].float().cpu().numpy(), par.f32_view(a["V"][l, h], dtype)[idx[l, h]])
