@@ -720,6 +720,10 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                         }
                         *reinterpret_cast<uint4 *>(rows + e0) = raw;
                     }
+                    // the int8 copy that was made with the gather is of the rows before; every thread reads back what it wrote
+                    if (c.v_q8)
+                        for (int e0 = tid * EPT; e0 < k * D; e0 += ALG_NT * EPT)
+                            quantize16<TIN, D>(*reinterpret_cast<const uint4 *>(rows + e0), c.v_q8, c.v_scale, (size_t)lh * k + e0 / D, e0 % D / EPT);
                 }
             };
             const float inv_del = 1.f / (a_del + p.eps);

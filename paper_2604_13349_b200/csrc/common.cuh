@@ -314,4 +314,56 @@ __device__ __forceinline__ float key_score(uint32_t k)
     return __uint_as_float((k & 0x80000000u) ? (k & 0x7FFFFFFFu) : ~k);
 }
 
+// 16 bytes of a row as floats: 8 bf16 or 4 fp32 values.
+template <typename TIN>
+__device__ __forceinline__ void unpack16(const uint4 &v, float (&x)[16 / sizeof(TIN)])
+{
+    if constexpr (sizeof(TIN) == 4) {
+        x[0] = __uint_as_float(v.x); x[1] = __uint_as_float(v.y); x[2] = __uint_as_float(v.z); x[3] = __uint_as_float(v.w);
+    } else {
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) { x[2 * e] = __uint_as_float(w[e] << 16); x[2 * e + 1] = __uint_as_float(w[e] & 0xFFFF0000u); }
+    }
+}
+
+// Post-hoc int8 quantisation of a row of the compacted relay (App. E): symmetric, one fp32 scale per row, scale =
+// max|x| / 127, code = round-half-even(x / scale).  The row lies in 16-byte vectors on CH neighbouring lanes of a warp
+// (they find its maximum in log2 CH shuffle steps), lane ch of them holds `raw`; all of them call.
+template <typename TIN, int D>
+__device__ __forceinline__ void quantize16(const uint4 &raw, int8_t *q8, float *scales, size_t row, int ch)
+{
+    constexpr int CH = D * (int)sizeof(TIN) / 16, EPT = 16 / (int)sizeof(TIN);
+    static_assert(CH >= 1 && CH <= 32 && (CH & (CH - 1)) == 0, "a row's threads are a power-of-two run of lanes");
+    const uint32_t lanes = (uint32_t)((1ull << CH) - 1ull) << (threadIdx.x & 31 & ~(CH - 1));
+    float x[EPT];
+    unpack16<TIN>(raw, x);
+    float amax = 0.f;
+#pragma unroll
+    for (int e = 0; e < EPT; ++e) amax = fmaxf(amax, fabsf(x[e]));
+#pragma unroll
+    for (int o = CH / 2; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(lanes, amax, o));
+    const float scale = amax / 127.0f;
+    // code = rint(x / scale) with the quotient rounded to fp32 first.  x * (1 / scale) is within 2.3e-5 of that
+    // quotient (|x / scale| <= 127), so both round to the same integer unless the product is that close to a
+    // half-integer: only then (a few elements in ten thousand) the quotient itself is formed.
+    const float rcp = scale > 0.f ? 1.0f / scale : 0.f;
+    uint32_t packed[EPT / 4];
+#pragma unroll
+    for (int w = 0; w < EPT / 4; ++w) packed[w] = 0u;
+#pragma unroll
+    for (int e = 0; e < EPT; ++e) {
+        const float pr = x[e] * rcp;
+        float v = rintf(pr);
+        if (fabsf(fabsf(pr - v) - 0.5f) < 2.44140625e-4f && scale > 0.f) v = rintf(x[e] / scale);
+        v = fminf(fmaxf(v, -127.f), 127.f);
+        packed[e / 4] |= (uint32_t)(uint8_t)(int8_t)v << (8 * (e % 4));
+    }
+    // EPT bytes per thread (the arrays are 8-byte aligned: validated on the host)
+    int8_t *dst = q8 + row * D + ch * EPT;
+    if constexpr (EPT == 8) *reinterpret_cast<uint2 *>(dst) = make_uint2(packed[0], packed[1]);
+    else *reinterpret_cast<uint32_t *>(dst) = packed[0];
+    if (ch == 0) scales[row] = scale;
+}
+
 }  // namespace obf

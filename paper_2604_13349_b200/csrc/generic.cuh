@@ -509,10 +509,15 @@ constexpr int GATHER_ROWS = 64;
 
 // WHICH: 3 = keys and values, 1 = values only, 2 = keys only (the keys are needed by nothing that follows in
 // the call, so their copy can run beside the later kernels).
-template <int ROW_BYTES, int WHICH = 3>
+// Where a cache wants the int8 copy of its relay, a row is quantised while it is in registers (an injection quantises its
+// rows again, k_obf_algebra; values that are merged are quantised afterwards).  40 layers x 8 heads, 811 of 8192 rows: 511 us
+// with a pass of its own over the compacted rows, 477 so (498 when the copy of the keys, which runs beside the span test,
+// quantises the values too: the span test fills the register files).
+template <typename TIN, int D, int WHICH = 3>
 __global__ void __launch_bounds__(256) k_gather(const __grid_constant__ CallDev p)
 {
     pdl_wait();
+    constexpr int ROW_BYTES = D * (int)sizeof(TIN);
     constexpr int CH = ROW_BYTES / 16;             // vectors per row
     constexpr int RPP = 256 / CH;                  // rows per pass of the block
     constexpr int PASSES = GATHER_ROWS / RPP;
@@ -557,94 +562,37 @@ __global__ void __launch_bounds__(256) k_gather(const __grid_constant__ CallDev 
                 if (WHICH & 1) *reinterpret_cast<uint4 *>(vo + (size_t)r[u] * ROW_BYTES + ch * 16) = vv[u];
             }
         }
-    }
-}
-
-// Post-hoc int8 quantisation of the compacted relay (App. E): symmetric, one fp32 scale per row of K_out and of
-// V_out, scale = max|x| / 127, code = round-half-even(x / scale).
-// A row is read as 16-byte vectors, one per thread, so a row of ROW_BYTES takes ROW_BYTES / 16 neighbouring lanes
-// (they find the row's maximum with that many shuffle steps); a thread has QR_ROWS rows of both arrays in flight.
-// grid = (ceil(k_eff_max / QR_BLOCK_ROWS), heads_total), 256 threads.
-constexpr int QR_ROWS = 4;
-
-// 16 bytes of a row as floats: 8 bf16 or 4 fp32 values.
-template <typename TIN>
-__device__ __forceinline__ void unpack16(const uint4 &v, float (&x)[16 / sizeof(TIN)])
-{
-    if constexpr (sizeof(TIN) == 4) {
-        x[0] = __uint_as_float(v.x); x[1] = __uint_as_float(v.y); x[2] = __uint_as_float(v.z); x[3] = __uint_as_float(v.w);
-    } else {
-        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+        if (c.k_q8) {
+            const size_t head = (size_t)lh * c.k_eff;
 #pragma unroll
-        for (int e = 0; e < 4; ++e) { x[2 * e] = __uint_as_float(w[e] << 16); x[2 * e + 1] = __uint_as_float(w[e] & 0xFFFF0000u); }
+            for (int u = 0; u < 4; ++u) {
+                if (j[u] < 0) continue;                            // (the lanes of a row agree)
+                if (WHICH & 2) quantize16<TIN, D>(kv[u], c.k_q8, c.k_scale, head + r[u], ch);
+                if ((WHICH & 1) && !p.merge) quantize16<TIN, D>(vv[u], c.v_q8, c.v_scale, head + r[u], ch);
+            }
+        }
     }
 }
 
-template <typename TIN, int D>
-constexpr int qr_block_rows() { return 256 / (D * (int)sizeof(TIN) / 16) * QR_ROWS; }
+// The int8 copy of the values of a merged cache, whose rows are final only then (quantize16 does the work).
+// grid = (ceil(k_eff_max / QR_ROWS), heads_total), 256 threads.
+constexpr int QR_ROWS = 64;
 
 template <typename TIN, int D>
-__global__ void __launch_bounds__(256) k_quantize_rows(const __grid_constant__ CallDev p)
+__global__ void __launch_bounds__(256) k_quantize_values(const __grid_constant__ CallDev p)
 {
     pdl_wait();
-    constexpr int CH = D * (int)sizeof(TIN) / 16;                      // threads per row
-    constexpr int EPT = 16 / (int)sizeof(TIN);                         // elements per thread
-    constexpr int RPP = 256 / CH;                                      // rows per pass of the block
-    static_assert(CH >= 1 && CH <= 32 && (CH & (CH - 1)) == 0, "a row's threads are a power-of-two run of lanes");
+    constexpr int CH = D * (int)sizeof(TIN) / 16;
     int ci, lh;
     locate(p, blockIdx.y, ci, lh);
     const CacheDev &c = p.c[ci];
-    if (!c.k_q8) return;
-    const int ch = threadIdx.x % CH, rr = threadIdx.x / CH;
-    const int r0 = blockIdx.x * (RPP * QR_ROWS) + rr;                  // this thread's rows: r0 + i RPP
-    if (blockIdx.x * (RPP * QR_ROWS) >= c.k_eff) return;
-    const size_t row0 = (size_t)lh * c.k_eff;
-    uint4 raw[2][QR_ROWS];
-#pragma unroll
-    for (int which = 0; which < 2; ++which)
-#pragma unroll
-        for (int i = 0; i < QR_ROWS; ++i) {
-            const int r = r0 + i * RPP;
-            const TIN *src = reinterpret_cast<const TIN *>(which ? c.v_out : c.k_out) + (row0 + r) * D + ch * EPT;
-            raw[which][i] = r < c.k_eff ? *reinterpret_cast<const uint4 *>(src) : make_uint4(0u, 0u, 0u, 0u);
-        }
-#pragma unroll
-    for (int which = 0; which < 2; ++which)
-#pragma unroll
-        for (int i = 0; i < QR_ROWS; ++i) {
-            const int r = r0 + i * RPP;
-            float x[EPT];
-            unpack16<TIN>(raw[which][i], x);
-            float amax = 0.f;
-#pragma unroll
-            for (int e = 0; e < EPT; ++e) amax = fmaxf(amax, fabsf(x[e]));
-            // (every lane takes part: rows past the end hold zeros)
-#pragma unroll
-            for (int o = CH / 2; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-            const float scale = amax / 127.0f;
-            // code = rint(x / scale) with the quotient rounded to fp32 first.  x * (1 / scale) is within 2.3e-5 of that
-            // quotient (|x / scale| <= 127), so both round to the same integer unless the product is that close to a
-            // half-integer: only then (a few elements in ten thousand) the quotient itself is formed.
-            const float rcp = scale > 0.f ? 1.0f / scale : 0.f;
-            uint32_t packed[EPT / 4];
-#pragma unroll
-            for (int w = 0; w < EPT / 4; ++w) packed[w] = 0u;
-#pragma unroll
-            for (int e = 0; e < EPT; ++e) {
-                const float pr = x[e] * rcp;
-                float v = rintf(pr);
-                if (fabsf(fabsf(pr - v) - 0.5f) < 2.44140625e-4f && scale > 0.f) v = rintf(x[e] / scale);
-                v = fminf(fmaxf(v, -127.f), 127.f);
-                packed[e / 4] |= (uint32_t)(uint8_t)(int8_t)v << (8 * (e % 4));
-            }
-            if (r < c.k_eff) {
-                // EPT bytes per thread (the arrays are 8-byte aligned: validated on the host)
-                int8_t *dst = (which ? c.v_q8 : c.k_q8) + (row0 + r) * D + ch * EPT;
-                if constexpr (EPT == 8) *reinterpret_cast<uint2 *>(dst) = make_uint2(packed[0], packed[1]);
-                else *reinterpret_cast<uint32_t *>(dst) = packed[0];
-                if (ch == 0) (which ? c.v_scale : c.k_scale)[row0 + r] = scale;
-            }
-        }
+    const int r0 = blockIdx.x * QR_ROWS;
+    if (!c.v_q8 || r0 >= c.k_eff) return;
+    const size_t head = (size_t)lh * c.k_eff;
+    for (int r = r0 + threadIdx.x / CH; r < min(r0 + QR_ROWS, c.k_eff); r += 256 / CH) {
+        const uint4 raw = reinterpret_cast<const uint4 *>(c.v_out)[(head + r) * CH + threadIdx.x % CH];
+        quantize16<TIN, D>(raw, c.v_q8, c.v_scale, head + r, threadIdx.x % CH);
+    }
 }
 
 // Diagnostics only (projection cosine): s = sum of the deleted value rows of a head, for heads with a

@@ -442,8 +442,10 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
         OBF_CUDA_TRY(cudaStreamWaitEvent(side->stream, side->fork, 0));
         if ((s = launch_gram_tc<D>(cd, L, st)) != OBF_OK) return s;
     }
-    // few retained rows and no span test that waits for them beside the pass over V: the selection copies them itself
-    const int gather_vecs = T_max <= SEL_SMEM_MAX_T && k_max <= SEL_GATHER_MAX && !span ? D * (int)sizeof(TIN) / 16 : 0;
+    bool any_q8 = false;
+    for (int i = 0; i < cd.n_caches; ++i) any_q8 = any_q8 || cd.c[i].k_q8 != nullptr;
+    // few retained rows, no int8 copy of them and no span test that waits for them beside the pass over V: the selection copies them itself
+    const int gather_vecs = T_max <= SEL_SMEM_MAX_T && k_max <= SEL_GATHER_MAX && !span && !any_q8 ? D * (int)sizeof(TIN) / 16 : 0;
     if (cd.layerwise) {
         // masses of a layer's KV heads added up, then every head's block selects on its layer's sums
         const int n_layers = heads / cd.kv_heads;
@@ -483,7 +485,7 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
         }
     } else if (side) {
         // the values first: the rest of the call needs them
-        OBF_TRY(launch(k_gather<D * (int)sizeof(TIN), 1>, dim3(g4), 256, 0, sel, cd));
+        OBF_TRY(launch(k_gather<TIN, D, 1>, dim3(g4), 256, 0, sel, cd));
         mark(sel, "k_gather");
         OBF_CUDA_TRY(cudaEventRecord(side->rows_done, side->stream));
         if constexpr (sizeof(TIN) == 2) if (span) {
@@ -498,11 +500,11 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
         // the keys are needed by nothing that follows: they are copied on the caller's stream once the pass over V
         // is over (it is bound by HBM), while the span test finishes on the side stream
         OBF_CUDA_TRY(cudaStreamWaitEvent(st, side->rows_done, 0));
-        OBF_TRY(launch(k_gather<D * (int)sizeof(TIN), 2>, dim3(g4), 256, 0, st, cd));
+        OBF_TRY(launch(k_gather<TIN, D, 2>, dim3(g4), 256, 0, st, cd));
         ++g_last_launches;
         OBF_CUDA_TRY(cudaStreamWaitEvent(st, side->join, 0));
     } else {
-        OBF_TRY(launch(k_gather<D * (int)sizeof(TIN)>, dim3(g4), 256, 0, sel, cd));
+        OBF_TRY(launch(k_gather<TIN, D>, dim3(g4), 256, 0, sel, cd));
         mark(sel, "k_gather");
     }
     if (cd.rank > 0) {
@@ -576,13 +578,10 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
         else OBF_TRY(launch(k_merge_apply<TIN, D, 1>, dim3(gm), 256, 0, st, cd));
         mark(st, "k_merge_apply");
     }
-    bool any_q8 = false;
-    for (int i = 0; i < cd.n_caches; ++i) any_q8 = any_q8 || cd.c[i].k_q8 != nullptr;
-    if (any_q8) {
-        constexpr int QB = qr_block_rows<TIN, D>();
-        dim3 gq((k_max + QB - 1) / QB, heads);
-        OBF_TRY(launch(k_quantize_rows<TIN, D>, dim3(gq), 256, 0, st, cd));
-        mark(st, "k_quantize_rows");
+    if (any_q8 && cd.merge) {
+        dim3 gq((k_max + QR_ROWS - 1) / QR_ROWS, heads);
+        OBF_TRY(launch(k_quantize_values<TIN, D>, dim3(gq), 256, 0, st, cd));
+        mark(st, "k_quantize_values");
     }
     OBF_CUDA_TRY(cudaGetLastError());
     return OBF_OK;

@@ -927,7 +927,7 @@ def test_fast_path_matches_the_oracles_same_iteration(dtype, d, rank, caches):
 # ---------------------------------------------------------------------------
 # few retained rows: the selection copies them itself, with more of them a kernel of its own does
 # ---------------------------------------------------------------------------
-@pytest.mark.parametrize("dtype,d,flags", [("f32", 32, 0), ("f32", 128, 0), ("bf16", 64, 0), ("bf16", 128, 0),
+@pytest.mark.parametrize("dtype,d,flags", [("f32", 64, 0), ("f32", 128, 0), ("bf16", 64, 0), ("bf16", 128, 0),
                                            ("bf16", 128, P.binding.OBF_FLAG_LAYERWISE)])
 @pytest.mark.parametrize("caches", [((300, 1),), ((64, 64), (701, 63)), ((1500, 64),), ((300, 65), (90, 7))])
 def test_retained_rows_are_copied_whoever_copies_them(dtype, d, flags, caches):
