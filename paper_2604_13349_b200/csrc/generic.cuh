@@ -273,12 +273,7 @@ __global__ void __launch_bounds__(SEL_NT) k_select(const __grid_constant__ CallD
 // what the head's block has in hand a moment after the positions; the block's threads fetch all of them at once.
 constexpr int SEL_GATHER_MAX = 64;
 
-// Step a2 for heads whose T keys fit in shared memory (the usual case): same result as
-// k_select, bit for bit, but the order-preserving keys are read from global memory
-// once.  The radix histogram is built with one shared-memory atomic per distinct digit
-// and warp; the ordered pass gives every warp a contiguous run of positions, so two
-// block-wide barriers suffice.
-constexpr int SEL_SMEM_MAX_T = 16384;
+constexpr int SEL_SMEM_MAX_T = 16384;               // keys of a head that fit in shared memory (k_select_smem)
 
 // Layerwise selector, first half (Section 3.2, retention rule, second form): the masses of a layer's KV heads
 // added up per position, head 0 first.  grid = (ceil(T_max / 256), layers of all caches).
@@ -296,19 +291,32 @@ __global__ void __launch_bounds__(256) k_layer_sum(const __grid_constant__ CallD
     p.lscores[c.tok_off / p.kv_heads + (size_t)(lh / p.kv_heads) * c.T + j] = s;
 }
 
+// Step a2 for heads whose T keys fit in shared memory (the usual case): same result as k_select, bit for bit.
+// What bounds it is the chain of barriers and serial steps, not the keys: four passes of 8 bits with their searches were
+// 1500 cycles each before a key was looked at.  So the keys are counted by their upper 11 bits while they are loaded (four
+// bins per octave: few equal ones in a warp), one search finds the bin of the k-th largest, and as it holds few keys as a
+// rule (at most SEL_CAND_MAX) those are listed and ranked against one another, which ends the search; a fuller bin (many
+// masses within a quarter of an octave, or equal) is split by the next 11 and the last 10 bits first.  Every warp has a
+// contiguous run of positions for the listing and the ordered pass.
+// Counters are 16 bits wide (T < 65536) so that, at T = 8192, two blocks find room beside a block of the pass over V.
+// 8 heads, T = 2048: 8.5 -> 6.7 us; 288 heads, T = 4096: 16 -> 11.6; 320 heads, T = 8192, beside the pass over V: 56 -> 40.
 // With LAYER every head's block selects on its layer's summed masses (the layer's heads repeat the same
-// selection side by side rather than one block writing all of them in turn) and then writes the shared
-// positions, the keep flags and the demand sums of the head's own masses.
+// selection side by side rather than one block writing all of them in turn) and writes the demand sums of the head's own.
 // gather_vecs > 0: every budget is at most SEL_GATHER_MAX and the block copies its head's retained rows of K and V too, that
 // many 16-byte vectors each.
+constexpr int SEL_CAND_MAX = 256, SEL_BINS = 2048;
+
 template <int NT, bool LAYER = false>
-__global__ void __launch_bounds__(NT) k_select_smem(const __grid_constant__ CallDev p, int gather_vecs)
+__global__ void __launch_bounds__(NT, 2048 / NT) k_select_smem(const __grid_constant__ CallDev p, int gather_vecs)
 {
     pdl_wait();
     extern __shared__ uint32_t sel_keys[];
-    __shared__ uint32_t hist[256];
-    __shared__ uint32_t s_prefix, s_want;
-    constexpr int NW = NT / 32;
+    constexpr int NW = NT / 32, WPT = SEL_BINS / 2 / NT;                // words of two bins per thread
+    static_assert(WPT >= 1 && SEL_BINS / 2 % NT == 0, "whole words per thread");
+    __shared__ uint32_t hist[SEL_BINS / 2];
+    __shared__ __align__(16) uint32_t cand[SEL_CAND_MAX];               // listed keys
+    __shared__ uint8_t cand_warp[SEL_CAND_MAX];                         // the warp whose run a listed key lies in
+    __shared__ uint32_t s_bin, s_want, s_count, s_listed, s_tau;
     __shared__ uint32_t wtot[32];
     __shared__ float red[3][32];
     __shared__ int s_idx[SEL_GATHER_MAX];
@@ -316,106 +324,192 @@ __global__ void __launch_bounds__(NT) k_select_smem(const __grid_constant__ Call
     locate(p, blockIdx.x, ci, lh);
     const CacheDev &c = p.c[ci];
     const int T = c.T, k = c.k_eff;
-    float *Af = p.scores + c.tok_off + (size_t)lh * T;
+    const float *Af = p.scores + c.tok_off + (size_t)lh * T;
     const uint32_t *A = LAYER ? reinterpret_cast<const uint32_t *>(p.lscores + c.tok_off / p.kv_heads + (size_t)(lh / p.kv_heads) * T)
                               : reinterpret_cast<const uint32_t *>(Af);
     uint8_t *keep = p.keep + c.tok_off + (size_t)lh * T;
     int32_t *idx = c.idx_out + (size_t)lh * k;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
-    for (int j = tid; j < T; j += NT) sel_keys[j] = select_key(p, j, A[j]);
-    if (tid == 0) { s_prefix = 0u; s_want = (uint32_t)k; }
-    uint32_t mask = 0u;
-    const int T_pad = (T + NT - 1) / NT * NT;
-    for (int shift = 24; shift >= 0; shift -= 8) {
-        if (tid < 256) hist[tid] = 0u;
+    // adds the warp's keys to the bins; `in`: this lane's key counts
+    auto count = [&](uint32_t digit, bool in) {
+        const uint32_t ins = __ballot_sync(0xffffffffu, in);
+        if (ins == 0u) return;
+        // one digit for the whole warp (equal masses) is counted once
+        const int first = __ffs(ins) - 1;
+        const uint32_t d0 = __shfl_sync(0xffffffffu, digit, first);
+        if (__all_sync(0xffffffffu, !in || digit == d0)) {
+            if (lane == first) atomicAdd(&hist[d0 >> 1], (uint32_t)__popc(ins) << (16 * (d0 & 1u)));
+        } else if (in) {
+            atomicAdd(&hist[digit >> 1], 1u << (16 * (digit & 1u)));
+        }
+    };
+    // the bin that holds the want-th largest key counted -> s_bin, s_count; what is still wanted of it -> s_want.  Thread 0
+    // owns the highest bins.
+    auto search = [&](uint32_t want) {
         __syncthreads();
-        const uint32_t prefix = s_prefix;
+        uint32_t h[WPT], own = 0u;
+#pragma unroll
+        for (int w = 0; w < WPT; ++w) {
+            h[w] = hist[(NT - 1 - tid) * WPT + WPT - 1 - w];
+            own += (h[w] >> 16) + (h[w] & 0xFFFFu);
+        }
+        uint32_t upto = own;                            // inclusive sum over the warp's lanes <= this one
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t n = __shfl_up_sync(0xffffffffu, upto, o);
+            if (lane >= o) upto += n;
+        }
+        if (lane == 31) wtot[warp] = upto;
+        __syncthreads();
+        upto += __reduce_add_sync(0xffffffffu, lane < warp ? wtot[lane] : 0u);
+        uint32_t above = upto - own;
+        if (above < want && want <= upto) {
+#pragma unroll
+            for (int b = 0; b < 2 * WPT; ++b) {
+                const uint32_t n = (b & 1) ? h[b / 2] & 0xFFFFu : h[b / 2] >> 16;
+                if (above < want && want <= above + n) {
+                    s_bin = (uint32_t)(((NT - 1 - tid) * WPT + WPT - 1 - b / 2) * 2 + 1 - (b & 1));
+                    s_count = n;
+                    s_want = want - above;
+                }
+                above += n;
+            }
+        }
+        __syncthreads();
+    };
+
+    // keys into shared memory, counted by their upper 11 bits on the way; four loads in flight
+    const int T_pad = (T + NT - 1) / NT * NT;
+    bool clear = true;
+    for (int j0 = tid; j0 < T_pad; j0 += 4 * NT) {
+        uint32_t a[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) a[u] = j0 + u * NT < T ? A[j0 + u * NT] : 0u;
+        if (clear) {
+            // (while the first loads are on their way)
+#pragma unroll
+            for (int w = 0; w < WPT; ++w) hist[tid + w * NT] = 0u;
+            if (tid == 0) { s_bin = 0u; s_count = 0u; s_want = 1u; s_listed = 0u; s_tau = 0u; }
+            __syncthreads();
+            clear = false;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int j = j0 + u * NT;
+            const uint32_t key = select_key(p, j, a[u]);
+            if (j < T) sel_keys[j] = key;
+            count(key >> 21, j < T);
+        }
+    }
+    search((uint32_t)k);
+    uint32_t prefix = s_bin << 21, mask = 0xFFE00000u, want = s_want, n_in = s_count;
+    // a full bin: the next 11 bits, then the last 10
+    for (int shift = 10; shift >= 0 && n_in > (uint32_t)SEL_CAND_MAX; shift -= 10) {
+#pragma unroll
+        for (int w = 0; w < WPT; ++w) hist[tid + w * NT] = 0u;
+        __syncthreads();
         for (int j = tid; j < T_pad; j += NT) {
             const uint32_t u = j < T ? sel_keys[j] : 0u;
-            const bool cand = j < T && (u & mask) == prefix;
-            const uint32_t digit = (u >> shift) & 255u;
-            // after the first passes few keys are still candidates: most warps have none and skip the counting
-            const uint32_t cands = __ballot_sync(0xffffffffu, cand);
-            if (cands == 0u) continue;
-            if (shift == 24) {
-                // top byte (sign and exponent): a handful of values per warp.  Lanes with the same digit add up among
-                // themselves first; lanes that are no candidates form one group of their own, which adds nothing
-                const uint32_t peers = __match_any_sync(0xffffffffu, cand ? digit : 256u);
-                if (cand && lane == __ffs(peers) - 1) atomicAdd(&hist[digit], (uint32_t)__popc(peers));
-            } else {
-                // mantissa bytes: spread over the bins, so every candidate counts itself (matching 32 different digits
-                // costs far more than 32 atomics on different banks); one digit for the whole warp is counted once
-                const uint32_t d0 = __shfl_sync(0xffffffffu, digit, __ffs(cands) - 1);
-                if (__all_sync(0xffffffffu, !cand || digit == d0)) {
-                    if (lane == __ffs(cands) - 1) atomicAdd(&hist[d0], (uint32_t)__popc(cands));
-                } else if (cand) {
-                    atomicAdd(&hist[digit], 1u);
-                }
-            }
+            count((u >> shift) & (shift ? 0x7FFu : 0x3FFu), j < T && (u & mask) == prefix);
         }
-        __syncthreads();
-        if (warp == 0) {
-            // lane l owns bins [8l, 8l+8); walk down from the top bin
-            uint32_t own = 0u;
-#pragma unroll
-            for (int b = 0; b < 8; ++b) own += hist[lane * 8 + b];
-            uint32_t above = own;                       // inclusive sum over lanes >= this one
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t n = __shfl_down_sync(0xffffffffu, above, o);
-                if (lane + o < 32) above += n;
-            }
-            const uint32_t want = s_want;
-            const uint32_t excl = above - own;          // keys in bins above this lane's
-            const bool mine = excl < want && want <= above;
-            const uint32_t who = __ballot_sync(0xffffffffu, mine);
-            // total < want cannot happen (want <= candidates); guard anyway: lowest bin
-            const int sel_lane = who ? 31 - __clz(who) : 0;
-            if (lane == sel_lane) {
-                uint32_t cum = who ? excl : 0u;
-                int b = 7;
-                for (; b > 0; --b) {
-                    const uint32_t h = hist[lane * 8 + b];
-                    if (cum + h >= want) break;
-                    cum += h;
-                }
-                s_want = want - cum;
-                s_prefix = prefix | ((uint32_t)(lane * 8 + b) << shift);
-            }
-        }
-        mask |= 255u << shift;
-        __syncthreads();
+        search(want);
+        prefix |= s_bin << shift;
+        mask |= (shift ? 0x7FFu : 0x3FFu) << shift;
+        want = s_want;
+        n_in = s_count;
     }
-    const uint32_t tau = s_prefix;       // key of the k-th largest mass
-    const uint32_t want = s_want;        // how many positions with key == tau are retained (>= 1)
 
-    // ordered pass: warp w owns positions [w * seg, (w + 1) * seg)
+    // warp w owns positions [w * seg, (w + 1) * seg): its keys above the bin are counted, those in it listed
     const int seg = ((T + NW - 1) / NW + 31) / 32 * 32;
     const int j_begin = warp * seg, j_end = min(T, j_begin + seg);
+    const uint32_t lt_mask = (1u << lane) - 1u;
+    const bool listing = n_in <= (uint32_t)SEL_CAND_MAX;                // otherwise the bin is one value, all of its bits known
     uint32_t n_gt = 0u, n_eq = 0u;
+#pragma unroll 4
     for (int j0 = j_begin; j0 < j_end; j0 += 32) {
         const int j = j0 + lane;
         const uint32_t u = j < j_end ? sel_keys[j] : 0u;
-        n_gt += __popc(__ballot_sync(0xffffffffu, j < j_end && u > tau));
-        n_eq += __popc(__ballot_sync(0xffffffffu, j < j_end && u == tau));
-    }
-    if (lane == 0) wtot[warp] = n_gt | (n_eq << 16);
-    __syncthreads();
-    if (warp == 0) {
-        const uint32_t w = lane < NW ? wtot[lane] : 0u;
-        uint32_t inc = w;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t n = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o) inc += n;
+        const bool in = j < j_end && (u & mask) == prefix;
+        const uint32_t m_in = __ballot_sync(0xffffffffu, in);
+        n_gt += __popc(__ballot_sync(0xffffffffu, j < j_end && (u & mask) > prefix));
+        n_eq += __popc(m_in);
+        if (listing && in) {
+            const uint32_t at = atomicAdd(&s_listed, 1u);
+            if (at < (uint32_t)SEL_CAND_MAX) { cand[at] = u; cand_warp[at] = (uint8_t)warp; }
         }
-        wtot[lane] = inc - w;              // positions before this warp's run: greater (low half), equal (high half)
     }
+    if (lane == 0) wtot[warp] = n_gt | (listing ? 0u : n_eq << 16);
     __syncthreads();
-    // retained rows, once their positions are in s_idx
-    auto copy_rows = [&]() {
+    if (listing) {
+        // every listed key against all of them (slots past the end, up to the next multiple of four, count as lower)
+        const int n = (int)min(n_in, (uint32_t)SEL_CAND_MAX);
+        const uint32_t mine = tid < n ? cand[tid] : 0u;
+        uint32_t gt = 0u, eq = 0u;
+        if (tid < n) {
+            for (int i = 0; i < n; i += 4) {
+                const uint4 q = *reinterpret_cast<const uint4 *>(cand + i);
+                const uint32_t v[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const bool there = i + e < n;
+                    gt += there && v[e] > mine;
+                    eq += there && v[e] == mine;
+                }
+            }
+            if (gt < want && want <= gt + eq) { s_tau = mine; s_want = want - gt; }     // (equal keys write the same)
+        }
         __syncthreads();
+        if (tid < n && mine >= s_tau) atomicAdd(&wtot[cand_warp[tid]], mine > s_tau ? 1u : 0x10000u);
+        __syncthreads();
+    }
+    const uint32_t tau = listing ? s_tau : prefix;       // key of the k-th largest mass
+    want = listing ? s_want : want;                      // how many positions with key == tau are retained (>= 1)
+
+    // positions before this warp's run: greater (low half), equal (high half).  (No half carries over: T < 65536.)
+    const uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? wtot[lane] : 0u);
+    uint32_t run_gt = before & 0xFFFFu, run_eq = before >> 16;
+    float sk = 0.f, sd = 0.f, nx = -1.0f;
+    for (int j0 = j_begin; j0 < j_end; j0 += 128) {
+        uint32_t key[4];
+        float own[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int j = j0 + 32 * u + lane;
+            key[u] = j < j_end ? sel_keys[j] : 0u;
+            // a protected position's key is not its mass; a layer's is not its heads'
+            own[u] = j < j_end && (LAYER || j < p.n_sink) ? Af[j] : key_score(key[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int j = j0 + 32 * u + lane;
+            const bool valid = j < j_end, gt = valid && key[u] > tau, eq = valid && key[u] == tau;
+            const uint32_t m_gt = __ballot_sync(0xffffffffu, gt), m_eq = __ballot_sync(0xffffffffu, eq);
+            const uint32_t gt_before = run_gt + __popc(m_gt & lt_mask), eq_before = run_eq + __popc(m_eq & lt_mask);
+            const bool kp = gt || (eq && eq_before < want);
+            if (valid) {
+                keep[j] = kp ? 1 : 0;
+                if (kp) {
+                    const uint32_t pos = gt_before + min(eq_before, want);
+                    if (pos < (uint32_t)k) {
+                        idx[pos] = j;
+                        if (gather_vecs) s_idx[pos] = j;
+                    }
+                    else atomicOr(p.status, OBF_DEV_INTERNAL);
+                    sk += own[u];
+                } else { sd += own[u]; nx = fmaxf(nx, key_score(key[u])); }
+            }
+            run_gt += __popc(m_gt);
+            run_eq += __popc(m_eq);
+        }
+    }
+
+    // block totals of the retained and the deleted mass and the largest deleted one: the last warp, which has the least to
+    // copy, adds up the warps' shares
+    sk = warp_sum(sk); sd = warp_sum(sd); nx = warp_max(nx);
+    if (lane == 0) { red[0][warp] = sk; red[1][warp] = sd; red[2][warp] = nx; }
+    __syncthreads();
+    if (gather_vecs) {
         const size_t to = (size_t)lh * k * gather_vecs;
         const uint4 *ks = reinterpret_cast<const uint4 *>(c.k) + (size_t)lh * T * gather_vecs, *vs = reinterpret_cast<const uint4 *>(c.v) + (size_t)lh * T * gather_vecs;
         for (int e = tid; e < k * gather_vecs; e += NT) {
@@ -430,75 +524,13 @@ __global__ void __launch_bounds__(NT) k_select_smem(const __grid_constant__ Call
             reinterpret_cast<uint4 *>(c.k_out)[to + e] = a;
             reinterpret_cast<uint4 *>(c.v_out)[to + e] = b;
         }
-    };
-    // block totals of the retained and the deleted mass and the largest deleted one
-    auto finish = [&](float sk, float sd, float nx) {
-        sk = warp_sum(sk); sd = warp_sum(sd); nx = warp_max(nx);
-        if (lane == 0) { red[0][warp] = sk; red[1][warp] = sd; red[2][warp] = nx; }
-        __syncthreads();
-        if (warp == 0) {
-            sk = warp_sum(lane < NW ? red[0][lane] : 0.f);
-            sd = warp_sum(lane < NW ? red[1][lane] : 0.f);
-            nx = warp_max(lane < NW ? red[2][lane] : -1.0f);
-            if (lane == 0) store_selection(p, c, blockIdx.x, lh, sk, sd, nx, tau);
-        }
-    };
-    uint32_t run_gt = wtot[warp] & 0xFFFFu, run_eq = wtot[warp] >> 16;
-    float sk = 0.f, sd = 0.f, nx = -1.0f;
-    const uint32_t lt_mask = (1u << lane) - 1u;
-    for (int j0 = j_begin; j0 < j_end; j0 += 32) {
-        const int j = j0 + lane;
-        const bool valid = j < j_end;
-        const uint32_t u = valid ? sel_keys[j] : 0u;
-        const bool gt = valid && u > tau, eq = valid && u == tau;
-        const uint32_t m_gt = __ballot_sync(0xffffffffu, gt), m_eq = __ballot_sync(0xffffffffu, eq);
-        const uint32_t gt_before = run_gt + __popc(m_gt & lt_mask), eq_before = run_eq + __popc(m_eq & lt_mask);
-        const bool kp = gt || (eq && eq_before < want);
-        if (LAYER) {
-            // what was decided for a position, kept for the per-head sweep below: its output slot, or "deleted"
-            if (valid) {
-                const uint32_t pos = gt_before + min(eq_before, want);
-                if (kp && pos >= (uint32_t)k) atomicOr(p.status, OBF_DEV_INTERNAL);
-                sel_keys[j] = (kp && pos < (uint32_t)k) ? pos : 0xFFFFFFFFu;
-            }
-        } else if (valid) {
-            const float a = j < p.n_sink ? __uint_as_float(A[j]) : key_score(u);     // a protected position's key is not its mass
-            keep[j] = kp ? 1 : 0;
-            if (kp) {
-                const uint32_t pos = gt_before + min(eq_before, want);
-                if (pos < (uint32_t)k) {
-                    idx[pos] = j;
-                    if (gather_vecs) s_idx[pos] = j;
-                }
-                else atomicOr(p.status, OBF_DEV_INTERNAL);
-                sk += a;
-            } else { sd += a; nx = fmaxf(nx, a); }
-        }
-        run_gt += __popc(m_gt);
-        run_eq += __popc(m_eq);
     }
-    if (LAYER) {
-        __syncthreads();
-        // the largest summed mass among the deleted positions, for the diagnostics
-        for (int j = tid; j < T; j += NT)
-            if (sel_keys[j] == 0xFFFFFFFFu) nx = fmaxf(nx, __uint_as_float(A[j]));
-        sk = 0.f; sd = 0.f;
-        for (int j = tid; j < T; j += NT) {
-            const uint32_t pos = sel_keys[j];
-            const float a = Af[j];
-            const bool kp = pos != 0xFFFFFFFFu;
-            keep[j] = kp ? 1 : 0;
-            if (kp) {
-                idx[pos] = j;
-                if (gather_vecs) s_idx[pos] = j;
-                sk += a;
-            } else {
-                sd += a;
-            }
-        }
+    if (warp == NW - 1) {
+        sk = warp_sum(lane < NW ? red[0][lane] : 0.f);
+        sd = warp_sum(lane < NW ? red[1][lane] : 0.f);
+        nx = warp_max(lane < NW ? red[2][lane] : -1.0f);
+        if (lane == 0) store_selection(p, c, blockIdx.x, lh, sk, sd, nx, tau);
     }
-    if (gather_vecs) copy_rows();
-    finish(sk, sd, nx);
 }
 
 // Step a3: K_out = K[idx], V_out = V[idx] as 16-byte vectors.  A block copies GATHER_ROWS

@@ -943,3 +943,41 @@ def test_retained_rows_are_copied_whoever_copies_them(dtype, d, flags, caches):
                 assert np.array_equal(o["K_out"][l, h].float().cpu().numpy(), par.f32_view(a["K"][l, h], dtype)[idx[l, h]])
                 if evict:
                     assert np.array_equal(o["V_out"][l, h].float().cpu().numpy(), par.f32_view(a["V"][l, h], dtype)[idx[l, h]])
+
+
+# ---------------------------------------------------------------------------
+# selection: masses so close together that one bin of the first count holds most of them (further counts), or spread
+# (the bin's keys are ranked at once)
+# ---------------------------------------------------------------------------
+@pytest.mark.parametrize("flags", [0, P.binding.OBF_FLAG_LAYERWISE, P.binding.OBF_FLAG_SINK(4)])
+@pytest.mark.parametrize("T,budget", [(257, 100), (3001, 500), (16384, 1700)])
+@pytest.mark.parametrize("spread", [0.0, 1e-5, 1e-3, 0.3])
+def test_selection_of_close_masses(flags, T, budget, spread):
+    w = small("close", dtype="bf16", d=128, caches=((T, budget),), heavy=0, seed=73)
+    a = synth.gen_cache(w, 0)
+    a["K"] = synth.to_bf16_bits(synth.bf16_bits_to_f32(a["K"]) * np.float32(spread))
+    out = par.run_gpu(w, [a], evict=True, flags=flags)[0][0]
+    scores = out["scores"].float().cpu().numpy().reshape(w.kv_heads, T)
+    sink = 4 if flags == P.binding.OBF_FLAG_SINK(4) else 0
+    for h in range(w.kv_heads):
+        s = scores[h].copy()
+        if flags == P.binding.OBF_FLAG_LAYERWISE:
+            s = scores[0].copy()
+            for g in range(1, w.kv_heads):
+                s = s + scores[g]
+        s[:sink] = np.inf
+        idx = out["idx"][0, h].cpu().numpy()
+        # the largest masses, the lowest positions among equals
+        assert np.array_equal(idx, np.sort(np.lexsort((np.arange(T), -s))[:len(idx)])), (h, spread)
+
+
+@pytest.mark.parametrize("dtype,d", [("f32", 64), ("bf16", 128)])
+def test_int8_copy_of_merged_values(dtype, d):
+    w = small("q8m", layers=2, d=d, dtype=dtype, caches=((300, 63), (200, 65), (90, 1)), seed=87)
+    arrays = [synth.gen_cache(w, ci) for ci in range(len(w.caches))]
+    outs, _, st = par.run_gpu(w, arrays, flags=P.binding.OBF_FLAG_MERGE, want_int8=True)
+    assert st & 0xFF == 0
+    for o in outs:
+        for name in ("K", "V"):
+            codes, scales = oracle.quantize_rows(o[name + "_out"].float().cpu().numpy())
+            assert np.array_equal(o[name + "_q8"].cpu().numpy(), codes) and np.array_equal(o[name + "_scale"].cpu().numpy(), scales)
