@@ -454,7 +454,7 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
         OBF_TRY(launch(k_layer_sum, dim3(gl), 256, 0, sel, cd));
         mark(sel, "k_layer_sum");
         const int sms = sm_count();
-        if (heads > 2 * sms && heads <= 4 * sms) {
+        if (heads > sms) {
             if ((s = set_smem(k_select_smem<512, true>, sm_sel)) != OBF_OK) return s;
             OBF_TRY(launch(k_select_smem<512, true>, dim3(heads), 512, sm_sel, sel, cd, gather_vecs));
         } else {
@@ -463,10 +463,11 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
         }
     } else if (T_max <= SEL_SMEM_MAX_T) {
         const size_t sm_sel = (size_t)T_max * sizeof(uint32_t);
-        // blocks of 1024 threads fit twice on an SM; when the heads then need a second, nearly empty wave,
-        // blocks of 512 threads (four per SM) finish sooner
+        // up to a head per SM: the most threads a block can have; with more heads, blocks of 512 threads: four of them fit
+        // on an SM and two beside a block of the pass over V, where only one of 1024 does (36 x 8 heads, T = 1024: 233 ->
+        // 229 us a call; eviction at T = 4096 167.6 -> 166.8)
         const int sms = sm_count();
-        if (heads > 2 * sms && heads <= 4 * sms) {
+        if (heads > sms) {
             if ((s = set_smem(k_select_smem<512>, sm_sel)) != OBF_OK) return s;
             OBF_TRY(launch(k_select_smem<512>, dim3(heads), 512, sm_sel, sel, cd, gather_vecs));
         } else {
