@@ -26,19 +26,17 @@
 //      delta = A_del / (A_keep + eps) * Delta (Eq. 6), V_out = V_keep + delta on the head's retained rows (Eq. 7).
 //
 // What bounds it: the chain of d - 2 dependent reflectors, each a matrix-vector product, a reduction, a rank-two
-// update and the norm of the next row.  The matrix therefore lives in REGISTERS (half-warp g of 8 holds rows g, g + 8, ..,
+// update and the norm of the next row.  The matrix therefore lives in REGISTERS (of every 32 rows half-warp g of 8 holds four,
 // a lane pairs of columns for the two-wide FMA); only the reflector and the product cross warps, through shared memory,
 // at one block barrier per reflector of a retained row and two per reflector of the tridiagonal form.  Steps run in
 // stages of 32 so that finished rows and column pairs cost nothing and every register index is static.  128 threads of
 // 255 registers and less than 113 KB per block: two blocks share a multiprocessor.  What is run once per head is written
 // as small loops: a section's first pass costs about 130 cycles per 128 bytes of its code, more than its arithmetic.
-// Measured on 36 x 8 heads, budget 32, rank 2, head_dim 128 (every head back-filled): 0.178 ms against 0.534 ms for the
-// same algebra on a matrix in shared memory (Gram-Schmidt basis, M = P G P, then the reduction); cycles of one block with
-// its neighbour on the multiprocessor: load 16 k, retained rows 49 k, their reflectors on G 51 k, tridiagonal form 146 k
-// (1550 per reflector; a product and an update of the first stage take 467 and 558 by themselves), eigenvalues 11 k,
-// eigenvectors 15 k, way back 18 k.  Slower were: eight warps with half the registers (0.21), the chain of reflectors in a
-// warp of its own beside the matrix warps (0.20 to 0.26: the registers it takes cost the others more), one copy of the
-// step's code for all stages (0.26), retained rows and G in one loop (0.186).
+// Measured on 36 x 8 heads, budget 32, rank 2, head_dim 128 (every head back-filled): 0.139 ms against 0.534 ms for the
+// same algebra on a matrix in shared memory (Gram-Schmidt basis, M = P G P, then the reduction).  Slower were: eight warps
+// with half the registers, the chain of reflectors in a warp of its own beside the matrix warps (the registers it takes cost
+// the others more), one copy of the step's code for all stages, the reflectors on G sixteen at a time in compact form (code
+// that runs twice costs more to fetch than it saves), the auxiliary vector or the next row's norm in one warp only.
 #pragma once
 
 #include <type_traits>

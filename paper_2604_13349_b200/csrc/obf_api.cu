@@ -341,13 +341,13 @@ static EncodeTiledFn tensor_map_encoder()
 
 // Tensor map of a bf16 array [heads, rows, d] as [heads][64-column blocks][rows][64]: a box is GT_TILE rows of all
 // blocks with the 128-byte swizzle, block after block; rows past `rows` read as zero.
-static obf_status_t encode_rows_map(CUtensorMap *m, const void *ptr, uint64_t d, uint64_t rows, uint64_t heads)
+static obf_status_t encode_rows_map(CUtensorMap *m, const void *ptr, uint64_t d, uint64_t rows, uint64_t heads, uint32_t box_rows, uint32_t box_blocks)
 {
     EncodeTiledFn enc = tensor_map_encoder();
     if (!enc) return OBF_ERR_CUDA;
     cuuint64_t dims[4] = {64, rows, d / 64, heads};
     cuuint64_t strides[3] = {d * 2, 128, rows * d * 2};
-    cuuint32_t box[4] = {64, (cuuint32_t)GT_TILE, (cuuint32_t)(d / 64), 1};
+    cuuint32_t box[4] = {64, box_rows, box_blocks, 1};
     cuuint32_t es[4] = {1, 1, 1, 1};
     const CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(ptr), dims, strides, box, es,
                            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -368,7 +368,7 @@ static obf_status_t launch_gram_tc(const CallDev &cd, const Layout &L, cudaStrea
     if (L.tc_blocks == 0) return OBF_OK;
     const uint64_t hpc = (uint64_t)cd.heads_per_cache;
     for (int i = 0; i < cd.n_caches; ++i) {
-        const obf_status_t s = encode_rows_map(&m.a[i], cd.c[i].v, D, (uint64_t)cd.c[i].T, hpc);
+        const obf_status_t s = encode_rows_map(&m.a[i], cd.c[i].v, D, (uint64_t)cd.c[i].T, hpc, GT_TILE, D / 64);
         if (s != OBF_OK) return s;
     }
     // the whole shared-memory capacity, so that the side stream's blocks find room beside this kernel's
@@ -386,9 +386,11 @@ static obf_status_t launch_score_tc(const CallDev &cd, const Layout &L, cudaStre
     static thread_local TcMaps maps;
     const uint64_t hpc = (uint64_t)cd.heads_per_cache;
     for (int i = 0; i < cd.n_caches; ++i) {
-        obf_status_t s = encode_rows_map(&maps.a[i], cd.c[i].k, D, (uint64_t)cd.c[i].T, hpc);
+        obf_status_t s = encode_rows_map(&maps.a[i], cd.c[i].k, D, (uint64_t)cd.c[i].T, hpc, 128, D / 64);
         if (s != OBF_OK) return s;
-        if ((s = encode_rows_map(&maps.b[i], cd.c[i].q, D, (uint64_t)cd.n_q, hpc)) != OBF_OK) return s;
+        if ((s = encode_rows_map(&maps.b[i], cd.c[i].q, D, (uint64_t)cd.n_q, hpc, 128, D / 64)) != OBF_OK) return s;
+        // the queries again, in boxes of 32 rows of one column block
+        if (cd.n_caches <= ST_PART_MAP && (s = encode_rows_map(&maps.b[ST_PART_MAP + i], cd.c[i].q, D, (uint64_t)cd.n_q, hpc, 32, 1)) != OBF_OK) return s;
     }
     const size_t smem = score_tc_smem_bytes<D>();
     OBF_CUDA_TRY(cudaFuncSetAttribute(k_score_tc<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));

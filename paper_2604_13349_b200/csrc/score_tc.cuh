@@ -64,10 +64,18 @@ template <int D>
 constexpr size_t score_tc_smem_bytes() { return 1024 + (size_t)(2 + ST_STAGES) * 128 * D * 2 + (2 * 2 * ST_GROUPS * 128 + 2 * 128) * sizeof(float) + 64; }
 static_assert(ST_STAGES == ST_TBUF, "a ring stage is released by the accumulator barrier of the same index");
 
+// An item with up to 32 (64) queries, the second one of a head with 160 for instance, would leave three (two) schedulers of
+// four without work in a statistics pass, as a group's warps own 32 rows of its operand each: the item's queries are loaded
+// four times (twice), and the copies share the columns of a tile.  The tensor maps for that sit behind those of the first
+// ST_PART_MAP caches (a third array of maps made every launch 1 to 2 us slower); calls with more caches go without.
+// 36 x 8 heads of 160 queries, T = 2048: 105 -> 97 us; 2 x 4 heads of 64 queries, T = 400: 10.2 -> 9.2.
+constexpr int ST_PART_MAP = OBF_MAX_CACHES / 2;
+
 struct ScoreItem {
     int r, cache, lh, chunk, nt;   // r: round; lh: KV head in the cache; nt: tiles of the chunk that hold at least one key
     int lv, qt;                    // lv = lh * query tiles + qt: the (head, query tile) pair; qt: which 128 query rows
     int nq;                        // query rows of the item (at most 128)
+    int copies;                    // of them in the operand of its statistics pass: 1, 2 or 4
 };
 
 // What a block needs of a cache to find its work of a round (kept in shared memory).
@@ -92,8 +100,11 @@ __device__ __forceinline__ bool score_item(const CallDev &p, const ScoreTab *tab
     it.cache = ci;
     it.lv = lv;
     it.lh = p.sc_qt == 2 ? lv >> 1 : lv;
-    it.qt = p.sc_qt == 2 ? lv & 1 : 0;
+    // (a block that meets an even number of items a round would always get the same tile of a head, half of the blocks the
+    // larger one: the two change places from round to round; T = 1024, teams of two blocks: 62 -> 54 us)
+    it.qt = p.sc_qt == 2 ? (lv ^ ((c.hpr & 1) ? 0 : r - c.round_base)) & 1 : 0;
     it.nq = min(128, p.n_q - 128 * it.qt);
+    it.copies = p.n_caches > ST_PART_MAP || it.nq > 64 ? 1 : it.nq > 32 ? 2 : 4;
     it.chunk = c.chunk;
     const int tiles = (c.T - c.chunk * ST_CHUNK + 127) >> 7;
     it.nt = tiles < ST_TILES ? tiles : ST_TILES;
@@ -269,7 +280,14 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constan
                 if (nq[kind] > 0 && !tc::mbar_wait(&bar_q_free[kind], (nq[kind] - 1) & 1u, wc, 64)) return false;
                 const uint32_t qdst = tc::smem_u32(q_s + kind * ST_TILE_BYTES);
                 tc::mbar_expect_tx(&bar_q_full[kind], ST_TILE_BYTES);
-                tc::tma_load_rows(qdst, &tm.b[item.cache], &bar_q_full[kind], item.qt * 128, item.lh);      // rows past n_q read as zero
+                if (kind == 0 && item.copies > 1) {
+                    for (int r = 0; r < 4; ++r)
+                        for (int b = 0; b < D / 64; ++b)
+                            tc::tma_load_block(qdst + r * 32 * 128 + b * ST_BOX_BYTES, &tm.b[ST_PART_MAP + item.cache], &bar_q_full[kind],
+                                               item.qt * 128 + 32 * (r % (4 / item.copies)), b, item.lh);
+                } else {
+                    tc::tma_load_rows(qdst, &tm.b[item.cache], &bar_q_full[kind], item.qt * 128, item.lh);      // rows past n_q read as zero
+                }
                 ++nq[kind];
                 return true;
             };
@@ -375,23 +393,23 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constan
         const float sc = ST_LOG2E * rsqrtf((float)D);
         uint32_t it = 0, n_b[2] = {0u, 0u};
 
-        // The first `pieces` 32-column pieces of an accumulator tile (at most four), `work(half piece, registers)` on each 16
+        // `pieces` 32-column pieces of an accumulator tile from piece `first` on, `work(half piece, registers)` on each 16
         // columns while the next 16 are on their way; the tile is handed back as soon as its last columns are in
         // registers.  An item with fewer than 128 query rows (the second one of a head with, say, 160) costs by what it
         // has: a warp whose lanes hold no query walks no piece of a statistics pass, and a pooling pass walks the columns
         // that hold queries.
-        auto walk_tile = [&](uint32_t ti, int pieces, auto &&work) {
+        auto walk_tile = [&](uint32_t ti, int first, int pieces, auto &&work) {
             const uint32_t tb = ti % ST_TBUF;
             tc::mbar_wait(&bar_t_full[tb], (ti / ST_TBUF) & 1u, wc, 20);
             tc::tc_fence_after();
-            const uint32_t ta = tlane + tb * 128u;
+            const uint32_t ta = tlane + tb * 128u + 32u * first;
             uint32_t ra[16], rb[16];
             if (pieces > 0) tc::tmem_ld16(ta, ra);
 #pragma unroll 1
             for (int pc = 0; pc < pieces; ++pc) {
                 tc::tmem_ld_wait16(ra);
                 tc::tmem_ld16(ta + 32u * pc + 16u, rb);
-                work(2 * pc, ra);
+                work(2 * (first + pc), ra);
                 tc::tmem_ld_wait16(rb);
                 if (pc + 1 < pieces) {
                     tc::tmem_ld16(ta + 32u * pc + 32u, ra);
@@ -400,7 +418,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constan
                     __syncwarp();
                     if (lane == 0) tc::mbar_arrive(&bar_t_empty[tb]);
                 }
-                work(2 * pc + 1, rb);
+                work(2 * (first + pc) + 1, rb);
             }
             if (pieces == 0) {
                 __syncwarp();
@@ -424,7 +442,8 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constan
                 float m = -INFINITY, z = 0.f;
                 if (my_t < item.nt) {
                     const int key0 = item.chunk * ST_CHUNK + my_t * 128;                  // key of column 0 of the tile
-                    walk_tile(it + my_t, 32 * q < item.nq ? 4 : 0, [&](int hp, uint32_t (&rr)[16]) {
+                    const int share = 4 / item.copies;           // pieces of 32 columns per copy
+                    walk_tile(it + my_t, q / share * share, item.copies > 1 || 32 * q < item.nq ? share : 0, [&](int hp, uint32_t (&rr)[16]) {
                         // two copies of the update: the one that masks missing keys runs for a head's ragged last tile only
                         const int k0 = key0 + 16 * hp;
                         if (k0 + 16 > T) stats_update<true>(rr, T - k0, sc, m, z);
@@ -450,7 +469,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constan
                 const int my_t = (int)((uint32_t)(grp - (int)it) % ST_GROUPS);
                 if (my_t < prev.nt) {
                     f32x2 a0 = 0ull, a1 = 0ull;
-                    walk_tile(it + my_t, (prev.nq + 31) >> 5, [&](int hp, uint32_t (&rr)[16]) { pool_piece(rr, mp + 16 * hp, sc, a0, a1); });
+                    walk_tile(it + my_t, 0, (prev.nq + 31) >> 5, [&](int hp, uint32_t (&rr)[16]) { pool_piece(rr, mp + 16 * hp, sc, a0, a1); });
                     const float a = sum2(add2(a0, a1));
                     const int j = prev.chunk * ST_CHUNK + my_t * 128 + row;
                     if (j < T) {
@@ -490,18 +509,25 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constan
             tc::mbar_wait(&bar_st_ready[buf], n_a[buf] & 1u, wc, 20);
             float M = -INFINITY, Z = 0.f;
             {
-                float m[ST_TILES], z[ST_TILES];
+                // tile by tile, and copy by copy of the queries in a tile
+                const int rows = 128 / item.copies;
+#pragma unroll 1
+                for (int r = t; r < 128 && mine; r += rows) {
+                    float m[ST_TILES], z[ST_TILES], Mn = M;
 #pragma unroll
-                for (int e = 0; e < ST_TILES; ++e) {
-                    const int at = (buf * ST_TILES + e) * 128 + t;
-                    m[e] = e < item.nt ? s_m[at] : -INFINITY;
-                    z[e] = e < item.nt ? s_z[at] : 0.f;
-                    M = fmaxf(M, m[e]);
+                    for (int e = 0; e < ST_TILES; ++e) {
+                        const int at = (buf * ST_TILES + e) * 128 + r;
+                        m[e] = e < item.nt ? s_m[at] : -INFINITY;
+                        z[e] = e < item.nt ? s_z[at] : 0.f;
+                        Mn = fmaxf(Mn, m[e]);
+                    }
+                    const float Mf = fmaxf(Mn, -3e38f);                        // (-inf - -inf would be a NaN)
+                    Z *= ex2_approx(M - Mf);
+#pragma unroll
+                    for (int e = 0; e < ST_TILES; ++e) Z += z[e] * ex2_approx(m[e] - Mf);
+                    M = Mn;
                 }
                 ++n_a[buf];
-                const float Mf = fmaxf(M, -3e38f);                             // (-inf - -inf would be a NaN)
-#pragma unroll
-                for (int e = 0; e < ST_TILES; ++e) Z += z[e] * ex2_approx(m[e] - Mf);
                 if (mine && !p.debug_drop_publish)
                     st_relaxed_gpu_u64(words + (size_t)item.chunk * 128, ((unsigned long long)__float_as_uint(Z) << 32) | __float_as_uint(M));
             }

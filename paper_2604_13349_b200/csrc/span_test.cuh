@@ -16,9 +16,9 @@
 // for every 128 bytes of instructions it touches for the first time.  Hence the plainest form: the matrix in registers,
 // laid out as in the dense algebra, and one rank-two update per pair of pivots, a small loop body with one block
 // barrier: the owners of the next two rows update and publish them before the rest of their rows.  A blocked
-// form (32-wide panels, the diagonal block in one warp's registers, 8 x 4 tiles behind it) took 33 us for eight heads and
-// 54 us for 320; this one 27 us and 57 us (pairs of pivots; one pivot per barrier 36, entries doubled into pairs in shared
-// memory 30).
+// form (32-wide panels, the diagonal block in one warp's registers, 8 x 4 tiles behind it) took 33 us for eight heads; this
+// one takes 26 (one pivot per barrier 36, entries doubled into pairs in shared memory 30, four pivots per barrier with the
+// owners freeing their four rows of one another by shuffles 30).
 #pragma once
 
 #include "algebra.cuh"

@@ -109,6 +109,13 @@ __device__ __forceinline__ void tma_load_rows(uint32_t dst, const CUtensorMap *m
                  ::"r"(dst), "l"(map), "r"(smem_u32(bar)), "r"(0), "r"(row), "r"(head) : "memory");
 }
 
+// The same for one 64-column block of the map's box of rows.
+__device__ __forceinline__ void tma_load_block(uint32_t dst, const CUtensorMap *map, uint64_t *bar, int row, int block, int head)
+{
+    asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
+                 ::"r"(dst), "l"(map), "r"(smem_u32(bar)), "r"(0), "r"(row), "r"(block), "r"(head) : "memory");
+}
+
 // Asks for the tile to be brought into the L2 cache; nothing lands in shared memory.
 __device__ __forceinline__ void tma_prefetch_rows(const CUtensorMap *map, int row, int head)
 {

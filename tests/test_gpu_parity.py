@@ -981,3 +981,12 @@ def test_int8_copy_of_merged_values(dtype, d):
         for name in ("K", "V"):
             codes, scales = oracle.quantize_rows(o[name + "_out"].float().cpu().numpy())
             assert np.array_equal(o[name + "_q8"].cpu().numpy(), codes) and np.array_equal(o[name + "_scale"].cpu().numpy(), scales)
+
+
+# ---------------------------------------------------------------------------
+# query rows of a head: up to 32 (64) of a tile are worked on as four (two) copies, each on its share of the keys
+# ---------------------------------------------------------------------------
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("n_obs", [1, 16, 17, 32, 33, 64, 65, 80, 81, 96, 97, 128])
+def test_query_rows(d, n_obs):
+    run_and_check(small("rows", G=2, n_obs=n_obs, d=d, dtype="bf16", caches=((700, 40), (129, 20)) * (9 if n_obs == 80 else 1), seed=91))
