@@ -536,7 +536,17 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                     }
                 }
 #pragma unroll
-                for (int s = 0; s < NS; ++s) n0[s] = half_sum(alg_dot<D>(V[s], V[s]));
+                for (int s = 0; s < NS; ++s) {
+                    n0[s] = half_sum(alg_dot<D>(V[s], V[s]));
+                    // a reflector depends on its row's direction alone: rows whose squares leave the range of fp32's normal numbers
+                    // are brought back by a power of two
+                    if (n0[s] > 0.f && !(n0[s] > 1e-24f && n0[s] < 1e24f)) {
+                        const float f = n0[s] < 1.f ? 1.8446744e19f : 5.421011e-20f;            // 2^64, 2^-64
+#pragma unroll
+                        for (int q = 0; q < NQ; ++q) V[s][q] = mul2(V[s][q], pk(f, f));
+                        n0[s] = half_sum(alg_dot<D>(V[s], V[s]));
+                    }
+                }
                 // (the reflectors that earlier batches found, all published behind a barrier)
 #pragma unroll 1
                 for (int j = 0; j < m; ++j) {
@@ -634,9 +644,22 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                 __syncthreads();
                 pc = misc[8];
             }
-            const float trM = block_sum<ALG_NT>(diag_part(m), red);
+            float trM = block_sum<ALG_NT>(diag_part(m), red);
             rcr = del_negligible ? 0.f : trM / (trG + p.eps);
             if (!(rcr >= RCR_SKIP_TOL)) { done = true; status |= OBF_DEV_SKIPPED; }
+            // What follows squares the block's entries, so a trace far from one (values of 1e-11 or 1e9, say) is brought there by a
+            // power of two: exact, and C does not depend on it.  misc[10]: what one stands for from here on (read behind barriers).
+            if (tid == 0) misc[10] = 1.f;
+            if (!done && !(trM > 1e-6f && trM < 1e6f)) {
+                const uint32_t e = min(max(__float_as_uint(trM) >> 23, 1u), 253u);
+                const float f = __uint_as_float((254u - e) << 23);
+#pragma unroll
+                for (int r = 0; r < RW; ++r)
+#pragma unroll
+                    for (int q = 0; q < NQ; ++q) M[r][q] = mul2(M[r][q], pk(f, f));
+                trM *= f;
+                if (tid == 0) misc[10] = __uint_as_float(e << 23);
+            }
 
             // Delta in the rotated coordinates (vx, all d of them, zero below m) -> delta, published and injected (Eq. 6-7).
             // hi: the reflectors hi .. m + 1 and m - 1 .. 0 lead back.
@@ -814,11 +837,12 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                 __syncthreads();
                 const float l1 = tlam[0];
                 while (rho < rmax && tlam[rho] > EIG_RANK_TOL * l1 && tlam[rho] > 0.f) ++rho;
-                lam1 = l1 * bound;
-                lam_rho = rho > 0 ? tlam[rho - 1] * bound : 0.f;
-                lam_next = rho < ne ? fmaxf(tlam[rho] * bound, 0.f) : 0.f;
+                const float unit = misc[10];
+                lam1 = l1 * bound * unit;
+                lam_rho = rho > 0 ? tlam[rho - 1] * bound * unit : 0.f;
+                lam_next = rho < ne ? fmaxf(tlam[rho] * bound, 0.f) * unit : 0.f;
                 for (int t = 0; t < rho; ++t) revr += tlam[t];
-                revr *= bound / (trM + p.eps);                         // trace of R^T R = sum of all its eigenvalues
+                revr *= bound * unit / (trM * unit + p.eps);                         // trace of R^T R = sum of all its eigenvalues
                 bool clustered = false;
                 for (int t = 1; t < rho; ++t) clustered = clustered || tlam[t - 1] - tlam[t] <= EIG_CLUSTER_TOL * fabsf(l1);
                 // Close neighbours: inverse iteration on the scaled T: factor T - lambda I once (LU with row interchanges), three solves; the operands of four steps are fetched together, ahead of the chain that needs them
@@ -1177,8 +1201,9 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                 }
                 __syncthreads();
                 for (int t = 0; t < rho; ++t) revr += vl[t];
-                revr /= trM + p.eps;
-                lam1 = rho > 0 ? vl[0] : 0.f; lam_rho = rho > 0 ? vl[rho - 1] : 0.f; lam_next = 0.f;
+                const float unit = misc[10];
+                revr *= unit / (trM * unit + p.eps);
+                lam1 = rho > 0 ? vl[0] * unit : 0.f; lam_rho = rho > 0 ? vl[rho - 1] * unit : 0.f; lam_next = 0.f;
                 if (tid < D) {
                     float sacc = 0.f;
                     for (int t = 0; t < rho; ++t) sacc = fmaf(vc[t], C[t * D + tid], sacc);
@@ -1297,8 +1322,9 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                     misc[1] = l1; misc[2] = last; misc[3] = nxt; misc[4] = (float)n; misc[5] = kept;
                 }
                 __syncthreads();
-                lam1 = misc[1]; lam_rho = misc[2]; lam_next = misc[3]; rho = (int)misc[4];
-                revr = misc[5] / (trM + p.eps);
+                const float unit = misc[10];
+                lam1 = misc[1] * unit; lam_rho = misc[2] * unit; lam_next = misc[3] * unit; rho = (int)misc[4];
+                revr = misc[5] * unit / (trM * unit + p.eps);
                 if (tid < rho) {
                     const int col = isel[tid];
                     float s = 0.f;

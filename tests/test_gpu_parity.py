@@ -990,3 +990,54 @@ def test_int8_copy_of_merged_values(dtype, d):
 @pytest.mark.parametrize("n_obs", [1, 16, 17, 32, 33, 64, 65, 80, 81, 96, 97, 128])
 def test_query_rows(d, n_obs):
     run_and_check(small("rows", G=2, n_obs=n_obs, d=d, dtype="bf16", caches=((700, 40), (129, 20)) * (9 if n_obs == 80 else 1), seed=91))
+
+
+# ---------------------------------------------------------------------------
+# scale of the values: delta is linear in them, and Eq. 2 and Eq. 5 depend on directions only
+# ---------------------------------------------------------------------------
+def _scaled(a, dtype, factor):
+    if dtype == "f32":
+        return a * np.float32(factor)
+    return synth.to_bf16_bits(synth.bf16_bits_to_f32(a) * np.float32(factor))
+
+
+def _falling_values(w, seed):
+    """Values whose channels fall off by 0.7 each (eigenvalues of the residual a factor of two apart), down to 1e-2."""
+    d, rng = w.head.head_dim, np.random.default_rng(seed)
+    v = rng.standard_normal((w.layers, w.kv_heads, w.caches[0].T, d)) * np.maximum(0.7 ** np.arange(d), 1e-2)
+    return v.astype(np.float32) if w.dtype == "f32" else synth.to_bf16_bits(v.astype(np.float32))
+
+
+@pytest.mark.parametrize("dtype,d", [("f32", 64), ("f32", 128), ("bf16", 64), ("bf16", 128)])
+@pytest.mark.parametrize("rank,flags", [(2, 0), (9, 0), (2, P.binding.OBF_FLAG_FAST_PATH)])
+def test_scale_of_the_values_scales_the_backfill(dtype, d, rank, flags):
+    w = small("scale", d=d, dtype=dtype, rank=rank, caches=((700, 20),), seed=101)
+    a = synth.gen_cache(w, 0)
+    a["V"] = _falling_values(w, 102)
+    params = par.params_for(w, None, flags)
+    params.eps = 0.0                                                 # (the epsilon of Eq. 4 and Eq. 6 has a scale of its own)
+
+    def run(arrays):
+        dev = {name: par.to_device(arrays[name], dtype) for name in "KVQ"}
+        out = P.compress_caches(params, [dict(dev, budget=w.caches[0].budget)])[0]
+        torch.cuda.synchronize()
+        assert P.obf_last_device_status(out["workspace"]) & 0xFF == 0
+        return out["idx"].cpu().numpy(), out["delta"].cpu().numpy().astype(np.float64)
+
+    idx, want = run(a)
+    assert np.all(np.linalg.norm(want, axis=-1) > 0)
+    runs = [(2.0 ** e, dict(a, V=_scaled(a["V"], dtype, 2.0 ** e))) for e in (-45, 32)]
+    tiny = a["V"].copy()                                             # the retained rows alone: the same span
+    for h in range(w.kv_heads):
+        tiny[0, h, idx[0, h]] = _scaled(a["V"][0, h, idx[0, h]], dtype, 2.0 ** -66)
+    runs.append((1.0, dict(a, V=tiny)))
+    for factor, b in runs:
+        got = run(b)[1] / factor
+        # fp32 rounding against eigenvalues that lie apart by a tenth of the largest or more down to the second, and by
+        # 0.5^9 of it at the ninth: 2^-24 / 0.002 = 3e-5, times three for the roundings of G and of the solve
+        err = np.linalg.norm(got - want, axis=-1)
+        tol = 1e-4 * np.linalg.norm(want, axis=-1)
+        if dtype == "bf16":
+            # the retained rows' share is taken out of fp32 sums over all rows: a few ulps of the largest retained value
+            tol += 2.0 ** -22 * np.array([np.linalg.norm(par.f32_view(a["V"][0, h], dtype)[idx[0, h]], axis=-1).max() for h in range(w.kv_heads)])
+        assert np.all(err <= tol), (factor, err, tol)
