@@ -540,8 +540,9 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                     n0[s] = half_sum(alg_dot<D>(V[s], V[s]));
                     // a reflector depends on its row's direction alone: rows whose squares leave the range of fp32's normal numbers
                     // are brought back by a power of two
-                    if (n0[s] > 0.f && !(n0[s] > 1e-24f && n0[s] < 1e24f)) {
-                        const float f = n0[s] < 1.f ? 1.8446744e19f : 5.421011e-20f;            // 2^64, 2^-64
+                    const bool far = n0[s] > 0.f && !(n0[s] > 1e-24f && n0[s] < 1e24f);
+                    if (__any_sync(0xffffffffu, far)) {                // (the sum below takes the whole warp)
+                        const float f = !far ? 1.f : n0[s] < 1.f ? 1.8446744e19f : 5.421011e-20f;   // 2^64, 2^-64
 #pragma unroll
                         for (int q = 0; q < NQ; ++q) V[s][q] = mul2(V[s][q], pk(f, f));
                         n0[s] = half_sum(alg_dot<D>(V[s], V[s]));

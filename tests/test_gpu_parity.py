@@ -1026,7 +1026,10 @@ def test_scale_of_the_values_scales_the_backfill(dtype, d, rank, flags):
 
     idx, want = run(a)
     assert np.all(np.linalg.norm(want, axis=-1) > 0)
-    runs = [(2.0 ** e, dict(a, V=_scaled(a["V"], dtype, 2.0 ** e))) for e in (-45, 32)]
+    rows = np.median(np.linalg.norm(par.f32_view(a["V"], dtype), axis=-1))
+    # (the last two: retained rows on both sides of the norms 1e-12 and 1e12, where the kernel begins to rescale rows)
+    exps = (-45, 32, round(np.log2(1e-12 / rows)), round(np.log2(1e12 / rows)))
+    runs = [(2.0 ** e, dict(a, V=_scaled(a["V"], dtype, 2.0 ** e))) for e in exps]
     tiny = a["V"].copy()                                             # the retained rows alone: the same span
     for h in range(w.kv_heads):
         tiny[0, h, idx[0, h]] = _scaled(a["V"][0, h, idx[0, h]], dtype, 2.0 ** -66)
