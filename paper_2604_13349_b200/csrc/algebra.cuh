@@ -54,7 +54,8 @@ constexpr float RCR_SKIP_TOL = 1e-6f;
 constexpr float EIG_RANK_TOL = 1e-5f;
 constexpr int JACOBI_MAX_SWEEPS = 30;
 constexpr int ALG_TRI_MAX_RANK = 8;     // up to this rank only rank + 1 eigenvalues and rank eigenvectors are computed
-constexpr float EIG_CLUSTER_TOL = 1e-3f; // eigenvalues closer than this (relative to the largest) are orthogonalised explicitly
+constexpr float EIG_CLUSTER_TOL = 1e-3f; // eigenvalues closer than this (relative to the largest): inverse iteration, kept orthogonal during it
+constexpr float EIG_NEAR_TOL = 5e-2f;    // closer than this: one more step of inverse iteration on the twisted factors, then made orthogonal
 
 // a where the mask is all ones, b where it is zero.  (A conditional between array elements would be a conditional
 // address, and the array would have to live in memory.)
@@ -846,6 +847,27 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                 revr *= bound * unit / (trM * unit + p.eps);                         // trace of R^T R = sum of all its eigenvalues
                 bool clustered = false;
                 for (int t = 1; t < rho; ++t) clustered = clustered || tlam[t - 1] - tlam[t] <= EIG_CLUSTER_TOL * fabsf(l1);
+                // one warp, in order of the eigenvalues: orthogonal to the neighbours before it that are closer than tol, unit length
+                auto orthogonal = [&](float tol) __attribute__((always_inline)) {
+                    for (int j = 1; j < rho; ++j) {
+                        float *y = vec + (j * 6 + 5) * D;
+                        for (int i2 = 0; i2 < j; ++i2) {
+                            if (fabsf(tlam[i2] - tlam[j]) > tol * fabsf(l1)) continue;
+                            const float *z = vec + (i2 * 6 + 5) * D;
+                            float dsum = 0.f;
+                            for (int cc = lane; cc < n; cc += 32) dsum = fmaf(y[cc], z[cc], dsum);
+                            dsum = warp_sum(dsum);
+                            for (int cc = lane; cc < n; cc += 32) y[cc] -= dsum * z[cc];
+                            __syncwarp();
+                        }
+                        float n2 = 0.f;
+                        for (int cc = lane; cc < n; cc += 32) n2 = fmaf(y[cc], y[cc], n2);
+                        n2 = warp_sum(n2);
+                        const float inv = n2 > 0.f ? rsqrtf(n2) : 0.f;
+                        for (int cc = lane; cc < n; cc += 32) y[cc] *= inv;
+                        __syncwarp();
+                    }
+                };
                 // Close neighbours: inverse iteration on the scaled T: factor T - lambda I once (LU with row interchanges), three solves; the operands of four steps are fetched together, ahead of the chain that needs them
                 constexpr float PERT = 4e-7f;
                 if (!clustered) {
@@ -853,7 +875,11 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                     // the same time; where the two meet with the smallest remainder gamma the eigenvector has its largest
                     // entry, and its other entries follow outwards by multiplication alone (Fernando's method).  The residual
                     // is gamma over the vector's length; should it exceed 2e-7 of the spectrum's bound the inverse iteration
-                    // below takes over.  Each lane's operands lie in the order it needs them, four to a load.
+                    // below takes over.  gamma is about the shift's error, a few 1e-8 of the bound, and a neighbour's share of the
+                    // vector is that over its distance (2e-5 of delta for one at 2e-3): with a neighbour, wanted or not, within
+                    // EIG_NEAR_TOL one step of inverse iteration with the same factors squares that away, down to what T's own
+                    // rounding leaves, at two multiply-adds per entry and no division, and wanted neighbours are made orthogonal.
+                    // Farther ones leave less than 1e-6.  Each lane's operands lie in the order it needs them, four to a load.
                     constexpr float PIV = 1e-10f;
                     if (tid == 0) misc[7] = 0.f;
                     __syncthreads();
@@ -902,38 +928,96 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                             const int oa = __shfl_xor_sync(0xffffffffu, at, o);
                             if (ob < best || (ob == best && oa < at)) { best = ob; at = oa; }
                         }
-                        // the multipliers along both arms, from the twist outwards
-                        for (int i = lane; i < 4 * n4; i += 32) {
-                            const int u = at - 1 - i, w = at + 1 + i;
-                            pb[i] = u >= 0 ? -db[u] * scl * rcp_approx(pa[u]) : 0.f;
-                            qb[i] = w < n ? -db[w - 1] * scl * rcp_approx(qa[n - 1 - w]) : 0.f;
+                        // the multipliers along both arms and the pivots' reciprocals, from the twist outwards
+                        const float gam = pa[at] + qa[n - 1 - at] - (sa[at] - lam);
+                        constexpr int PL = D / 32;                     // entries a lane holds
+                        float rt[PL], rb[PL];
+#pragma unroll
+                        for (int q = 0; q < PL; ++q) {
+                            const int i = lane + 32 * q, u = at - 1 - i, w = at + 1 + i;
+                            rt[q] = u >= 0 ? rcp_approx(pa[u]) : 0.f;
+                            rb[q] = w < n ? rcp_approx(qa[n - 1 - w]) : 0.f;
                         }
                         __syncwarp();
-                        if (lane < 2) {
-                            float *mu = lane ? qb : pb;
-                            float x = 1.f;
+#pragma unroll
+                        for (int q = 0; q < PL; ++q) {
+                            const int i = lane + 32 * q, u = at - 1 - i, w = at + 1 + i;
+                            pa[i] = rt[q];
+                            qa[i] = rb[q];
+                            pb[i] = u >= 0 ? -db[u] * scl * rt[q] : 0.f;
+                            qb[i] = w < n ? -db[w - 1] * scl * rb[q] : 0.f;
+                        }
+                        __syncwarp();
+                        // lanes 0 and 1 take an arm each (what they learn of one another passes through the whole warp)
+                        const float *mu = lane ? qb : pb, *rc = lane ? qa : pa;
+                        float *x = lane ? y : pa + 4 * D;
+                        const int len = lane > 1 ? 0 : lane ? n - 1 - at : at;
+                        float n1 = 0.f, z = 1.f;                       // n1: squares of the first vector's entries; z: the entry at the twist
+                        {
+                            float c = 1.f;
 #pragma unroll 1
-                            for (int t = (lane ? n - 1 - at : at); t > 0; t -= 4, mu += 4) {
-                                const float4 mv = *reinterpret_cast<const float4 *>(mu);
+                            for (int t = 0; t < len; t += 4) {
+                                const float4 mv = *reinterpret_cast<const float4 *>(mu + t);
                                 float4 o;
-                                o.x = mv.x * x; o.y = mv.y * o.x; o.z = mv.z * o.y; x = o.w = mv.w * o.z;
-                                *reinterpret_cast<float4 *>(mu) = o;
+                                o.x = mv.x * c; o.y = mv.y * o.x; o.z = mv.z * o.y; c = o.w = mv.w * o.z;
+                                n1 = fmaf(o.x, o.x, fmaf(o.y, o.y, fmaf(o.z, o.z, fmaf(o.w, o.w, n1))));
+                                *reinterpret_cast<float4 *>(x + t) = o;
+                            }
+                        }
+                        const bool close = (e > 0 && tlam[e - 1] - lam < EIG_NEAR_TOL * l1) || (e + 1 < ne && lam - tlam[e + 1] < EIG_NEAR_TOL * l1);
+                        if (close) {                                   // (the same in every lane)
+                            // the step of inverse iteration: along both arms to the twist ..
+                            float g = 0.f, mn = 0.f;
+#pragma unroll 1
+                            for (int t = (len + 3) / 4 * 4 - 4; t >= 0; t -= 4) {
+                                const float4 xv = *reinterpret_cast<const float4 *>(x + t), mv = *reinterpret_cast<const float4 *>(mu + t);
+                                float4 o;
+                                o.w = fmaf(mn, g, xv.w); o.z = fmaf(mv.w, o.w, xv.z); o.y = fmaf(mv.z, o.z, xv.y); g = o.x = fmaf(mv.y, o.y, xv.x);
+                                mn = mv.x;
+                                *reinterpret_cast<float4 *>(x + t) = o;
+                            }
+                            g *= mn;
+                            __syncwarp();
+                            // .. across it and back
+                            z = (1.f + __shfl_sync(0xffffffffu, g, 0) + __shfl_sync(0xffffffffu, g, 1)) * rcp_approx(copysignf(fmaxf(fabsf(gam), PIV), gam));
+                            float c = z;
+#pragma unroll 1
+                            for (int t = 0; t < len; t += 4) {
+                                const float4 xv = *reinterpret_cast<const float4 *>(x + t), mv = *reinterpret_cast<const float4 *>(mu + t);
+                                const float4 rv = *reinterpret_cast<const float4 *>(rc + t);
+                                float4 o;
+                                o.x = fmaf(mv.x, c, xv.x * rv.x); o.y = fmaf(mv.y, o.x, xv.y * rv.y);
+                                o.z = fmaf(mv.z, o.y, xv.z * rv.z); c = o.w = fmaf(mv.w, o.z, xv.w * rv.w);
+                                *reinterpret_cast<float4 *>(x + t) = o;
                             }
                         }
                         __syncwarp();
-                        float n2 = 0.f;
-                        for (int i = lane; i < n; i += 32) {
-                            const float t = i == at ? 1.f : i < at ? pb[at - 1 - i] : qb[i - at - 1];
-                            y[i] = t;
-                            n2 = fmaf(t, t, n2);
+                        n1 = 1.f + __shfl_sync(0xffffffffu, n1, 0) + __shfl_sync(0xffffffffu, n1, 1);
+                        float yv[PL], n2 = 0.f;
+                        // (z is about 1 / gamma: the entries are brought to the first vector's scale before they are squared)
+                        const float zr = rcp_approx(z);
+#pragma unroll
+                        for (int q = 0; q < PL; ++q) {
+                            const int i = lane + 32 * q;
+                            yv[q] = i < n ? zr * (i == at ? z : i < at ? pa[4 * D + at - 1 - i] : y[i - at - 1]) : 0.f;
+                            n2 = fmaf(yv[q], yv[q], n2);
                         }
                         n2 = warp_sum(n2);
                         const float inv = rsqrtf(n2);
-                        for (int i = lane; i < n; i += 32) y[i] *= inv;
-                        if (lane == 0 && !(best * inv <= 2e-7f)) misc[7] = 1.f;
+                        __syncwarp();
+#pragma unroll
+                        for (int q = 0; q < PL; ++q)
+                            if (lane + 32 * q < n) y[lane + 32 * q] = yv[q] * inv;
+                        if (lane == 0 && !(best * rsqrtf(n1) <= 2e-7f)) misc[7] = 1.f;
                     }
                     __syncthreads();
                     clustered = misc[7] != 0.f;
+                    bool near = false;
+                    for (int t = 1; t < rho; ++t) near = near || tlam[t - 1] - tlam[t] < EIG_NEAR_TOL * l1;
+                    if (near && !clustered) {
+                        if (warp == 0) orthogonal(EIG_NEAR_TOL);
+                        __syncthreads();
+                    }
                 }
                 for (int e = warp; clustered && e < rho; e += ALG_NW) {
                     float *dd = vec + e * 6 * D, *dl = dd + D, *du = dl + D, *du2 = du + D, *pv = du2 + D, *y = pv + D;
@@ -1055,27 +1139,7 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                     }
                     if (clustered) {
                         __syncthreads();
-                        if (warp == 0) {
-                            // in order of the eigenvalues: orthogonal to the close neighbours before it, unit length
-                            for (int j = 1; j < rho; ++j) {
-                                float *y = vec + (j * 6 + 5) * D;
-                                for (int i2 = 0; i2 < j; ++i2) {
-                                    if (fabsf(tlam[i2] - tlam[j]) > EIG_CLUSTER_TOL * fabsf(l1)) continue;
-                                    const float *z = vec + (i2 * 6 + 5) * D;
-                                    float dsum = 0.f;
-                                    for (int cc = lane; cc < n; cc += 32) dsum = fmaf(y[cc], z[cc], dsum);
-                                    dsum = warp_sum(dsum);
-                                    for (int cc = lane; cc < n; cc += 32) y[cc] -= dsum * z[cc];
-                                    __syncwarp();
-                                }
-                                float n2 = 0.f;
-                                for (int cc = lane; cc < n; cc += 32) n2 = fmaf(y[cc], y[cc], n2);
-                                n2 = warp_sum(n2);
-                                const float inv = n2 > 0.f ? rsqrtf(n2) : 0.f;
-                                for (int cc = lane; cc < n; cc += 32) y[cc] *= inv;
-                                __syncwarp();
-                            }
-                        }
+                        if (warp == 0) orthogonal(EIG_CLUSTER_TOL);
                         __syncthreads();
                     }
                 }

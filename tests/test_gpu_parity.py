@@ -610,6 +610,37 @@ def test_residual_with_two_equal_leading_singular_values(rank):
         assert np.all(np.linalg.norm(d, axis=-1) > 1e-4)
 
 
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("rank", [2, 4])
+@pytest.mark.parametrize("gap", [1e-2, 2e-3, 1.2e-3])
+def test_close_eigenvalues_inside_the_principal_subspace(d, rank, gap):
+    # The last two of the wanted eigenvalues lie a small gap apart and a fifth from the next one: the vectors of the two are
+    # sensitive to the gap, the subspace (Eq. 5) is not, so delta must not be either.  No part of the deleted values lies in the
+    # retained span, whose coordinates are separate.
+    T, k, n = 600, 24, d - 24
+    w = small("close", d=d, dtype="f32", rank=rank, kv_heads=1, caches=((T, k),), seed=103)
+    for seed in range(4):
+        a = synth.gen_cache(w, 0)
+        rng = np.random.default_rng(seed)
+        idx = oracle.topk(oracle.scores(a["K"][0, 0], a["Q"].reshape(1, 1, w.n_q, d)[0, 0]), k)[0]
+        lam = 0.8 ** np.arange(n)
+        lam[rank - 1] = lam[rank - 2] - gap * lam[0]
+        lam[rank:] = lam[rank - 1] * 0.8 ** np.arange(1, n - rank + 1)
+        U = np.linalg.qr(rng.standard_normal((T - k, n)))[0]
+        W = np.linalg.qr(rng.standard_normal((n, n)))[0]
+        V = np.zeros((T, d))
+        dele = np.setdiff1d(np.arange(T), idx)
+        V[idx, :k] = rng.standard_normal((k, k))
+        V[dele, k:] = (U * np.sqrt(lam)) @ W * np.sqrt(T)
+        a["V"] = (V @ np.linalg.qr(rng.standard_normal((d, d)))[0]).astype(np.float32)[None, None]
+        out = par.run_gpu(w, [a])[0][0]
+        g_idx = out["idx"][0, 0].cpu().numpy()
+        ref = oracle.backfill(a["K"][0, 0], a["V"][0, 0], out["scores"][0, 0].cpu().numpy().astype(np.float64), g_idx, rank)["delta"]
+        got = out["delta"][0, 0].cpu().numpy().astype(np.float64)
+        # some 32 roundings of 2^-24 on the way to the subspace, over its distance of 0.2 (0.8^rank of it at most) from the rest
+        assert np.linalg.norm(got - ref) <= 32 * par.U32 / (0.2 * 0.8 ** (rank - 2)) * np.linalg.norm(ref), (seed, np.linalg.norm(got - ref) / np.linalg.norm(ref))
+
+
 # ---------------------------------------------------------------------------
 # protected sink prefix: the first s positions are retained besides the budget
 # ---------------------------------------------------------------------------
