@@ -9,6 +9,10 @@
 // retained rows are taken out of u (and out of the trace of G) by the dense algebra, which reads them anyway.
 // It can thus run beside the selection and the gather instead of after them.
 //
+// Heads of 64 channels are different: what the subtraction leaves behind is a few fp32 ulps of the largest retained value, and
+// those heads were computed without it.  Their pass runs after the selection (12 us of a call with 288 heads) and over the
+// deleted rows only: a retained token's mass counts as zero, and its row is cleared in shared memory before the MMA.
+//
 // (Whether span(V_keep) = R^d, Eq. 2, is decided by k_span_test from the gathered rows themselves.)
 //
 // Work decomposition.  Every head owns ceil(T / 128) tiles of 128 tokens of V.  All tiles of a launch form one sequence, cut into
@@ -43,6 +47,7 @@ struct GramShape {
     static constexpr int TILE_BYTES = GT_TILE * D * 2;
     static constexpr int STAGE_BYTES = TILE_BYTES + GT_BLOCK_BYTES;
     static constexpr size_t SMEM_BYTES = 1024 + (size_t)STAGES * STAGE_BYTES + 64;
+    static constexpr bool DELETED = D == 64;       // over the deleted rows only, after the selection; else over all rows, beside it
 };
 constexpr int GT_NU = 16;                          // columns of the mass block that enter the MMA
 static_assert(3 * U_LEVELS <= GT_NU, "the mass columns must fit the MMA's extra columns");
@@ -98,6 +103,7 @@ template <int D>
 __global__ void __launch_bounds__(GT_THREADS, 3) k_gram_tc(const __grid_constant__ CallDev p, const __grid_constant__ TcMaps tm)
 {
     pdl_wait();
+    constexpr bool DELETED = GramShape<D>::DELETED;
     constexpr int GT_STAGES = GramShape<D>::STAGES, GT_TILE_BYTES = GramShape<D>::TILE_BYTES, GT_STAGE_BYTES = GramShape<D>::STAGE_BYTES;
     extern __shared__ uint8_t gt_smem_raw[];
     uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(gt_smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -207,8 +213,8 @@ __global__ void __launch_bounds__(GT_THREADS, 3) k_gram_tc(const __grid_constant
             auto seek = [&]() {
                 while (have && (it % GT_STAGES) != (uint32_t)mw) step();
             };
-            // masses of tokens lane, lane + 32, .. of the tile the walk stands on
-            auto fetch = [&](float (&a)[4]) {
+            // masses of tokens lane, lane + 32, .. of the tile the walk stands on; kept: which of them are retained (a bit each)
+            auto fetch = [&](float (&a)[4], uint32_t &kept) {
                 const CacheDev &c = p.c[cache];
                 const float *A = p.scores + c.tok_off + (size_t)lh * c.T;
 #pragma unroll
@@ -216,21 +222,33 @@ __global__ void __launch_bounds__(GT_THREADS, 3) k_gram_tc(const __grid_constant
                     const int j = (sub0 + t) * GT_TILE + lane + 32 * e;
                     a[e] = j < c.T ? __ldg(A + j) : 0.f;
                 }
+                kept = 0u;
+                if (DELETED) {
+                    const uint8_t *keep = p.keep + c.tok_off + (size_t)lh * c.T;
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const int j = (sub0 + t) * GT_TILE + lane + 32 * e;
+                        kept |= (j < c.T && __ldg(keep + j) != 0 ? 1u : 0u) << e;
+                    }
+                }
             };
             seek();
             float a_next[4] = {0.f, 0.f, 0.f, 0.f};
-            if (have) fetch(a_next);
+            uint32_t kept_next = 0u;
+            if (have) fetch(a_next, kept_next);
             uint8_t *ab = tiles + mw * GT_STAGE_BYTES + GT_TILE_BYTES;     // this stage's mass block
             while (have) {
                 float a[4];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) a[e] = a_next[e];
+                for (int e = 0; e < 4; ++e) a[e] = DELETED && (kept_next >> e & 1u) ? 0.f : a_next[e];
+                const uint32_t kept = kept_next;
                 const uint32_t ph = (it / GT_STAGES) & 1u;
                 // this warp's next tile: its masses are in flight while the current ones are written
                 step();
                 seek();
-                if (have) fetch(a_next);
-                if (!tc::mbar_wait(&bar_empty[mw], ph ^ 1u, wc)) break;   // the stage's last user is done with its mass block
+                if (have) fetch(a_next, kept_next);
+                // the stage's last user is done with its mass block (the warp leaves as one when a wait runs out)
+                if (!__all_sync(0xffffffffu, tc::mbar_wait(&bar_empty[mw], ph ^ 1u, wc))) break;
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     const int k = lane + 32 * e;
@@ -255,6 +273,21 @@ __global__ void __launch_bounds__(GT_THREADS, 3) k_gram_tc(const __grid_constant
                     *reinterpret_cast<uint4 *>(rowp + ((0 ^ (k & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
                     *reinterpret_cast<uint4 *>(rowp + ((1 ^ (k & 7)) << 4)) = make_uint4(w[4], w[5], w[6], w[7]);
                 }
+                if (DELETED) {
+                    // the rows of retained tokens, once the tile is there (a token's row is 128 bytes per column block): eight lanes
+                    // clear a row
+                    if (!__all_sync(0xffffffffu, tc::mbar_wait(&bar_full[mw], ph, wc))) break;
+                    uint8_t *tile = ab - GT_TILE_BYTES;
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        uint32_t rows = __ballot_sync(0xffffffffu, kept >> e & 1u);
+                        while (rows) {
+                            const int k = 32 * e + __ffs(rows) - 1;
+                            rows &= rows - 1;
+                            if (lane < D / 8) *reinterpret_cast<uint4 *>(tile + (lane >> 3) * GT_BLOCK_BYTES + k * 128 + 16 * (lane & 7)) = make_uint4(0u, 0u, 0u, 0u);
+                        }
+                    }
+                }
                 tc::fence_async_smem();
                 __syncwarp();
                 if (lane == 0) tc::mbar_arrive(&bar_ready[mw]);
@@ -271,7 +304,7 @@ __global__ void __launch_bounds__(GT_THREADS, 3) k_gram_tc(const __grid_constant
         while (run.next(p, cache, lh, sub0, nsub, slot)) {
             const int g = p.c[cache].head_base + lh;
             const uint32_t buf = seg & 1u;
-            if (!tc::mbar_wait(&bar_acc_full[buf], (seg >> 1) & 1u, wc)) break;
+            if (!__all_sync(0xffffffffu, tc::mbar_wait(&bar_acc_full[buf], (seg >> 1) & 1u, wc))) break;
             tc::tc_fence_after();
             const uint32_t tl = tmem + ((uint32_t)(q * 32) << 16);
             float *dst = p.gram_d + ((size_t)g * p.gram_slots + slot) * D * D + (size_t)row * D;

@@ -437,7 +437,8 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
     // retained values can only span R^d where there are d of them: with smaller budgets there is nothing to test
     const bool span = cd.rank > 0 && k_max >= D;
     // With OBF_FLAG_EARLY_OUT the span test comes first and the pass over V skips what it found full: one stream.
-    SideStream *side = (tuned_obf && !g_prof.active && !cd.skip_full) ? side_stream() : nullptr;
+    // (A pass over the deleted rows only needs the selection: one stream as well.)
+    SideStream *side = (tuned_obf && !GramShape<D>::DELETED && !g_prof.active && !cd.skip_full) ? side_stream() : nullptr;
     cudaStream_t sel = side ? side->stream : st;       // stream of selection and gather
     if (side) {
         OBF_CUDA_TRY(cudaEventRecord(side->fork, st));
@@ -660,7 +661,7 @@ static obf_status_t run(const obf_params_t *p, const obf_cache_t *caches, int32_
     cd.splits = L.splits;
     cd.gram_slots = L.gram_slots;
     cd.tc_per = L.tc_per;
-    cd.gram_all = L.tc_per ? 1 : 0;
+    cd.gram_all = L.tc_per && !(p->head_dim == 64 ? GramShape<64>::DELETED : GramShape<128>::DELETED) ? 1 : 0;
     cd.u_levels = L.tc_per ? U_LEVELS : 1;
     cd.tc_total_sub = L.tc_total_sub;
     cd.sc_nq = L.sc_on ? L.sc_nq : 0;

@@ -1075,3 +1075,35 @@ def test_scale_of_the_values_scales_the_backfill(dtype, d, rank, flags):
             # the retained rows' share is taken out of fp32 sums over all rows: a few ulps of the largest retained value
             tol += 2.0 ** -22 * np.array([np.linalg.norm(par.f32_view(a["V"][0, h], dtype)[idx[0, h]], axis=-1).max() for h in range(w.kv_heads)])
         assert np.all(err <= tol), (factor, err, tol)
+
+
+@pytest.mark.parametrize("large", [10.0, 1000.0])
+@pytest.mark.parametrize("flags", [0, P.binding.OBF_FLAG_EARLY_OUT])
+def test_heads_of_64_channels_keep_their_precision_beside_large_retained_values(large, flags):
+    # the sums of Eq. 3 and Eq. 4 run over the deleted rows alone: retained values a thousand times as large leave no trace in
+    # them.  Retained tokens lie anywhere in the tiles of 128, the last tile is ragged, and budgets on both sides of 64 take
+    # both copies of the retained rows
+    w = small("large64", layers=2, d=64, dtype="bf16", rank=2, caches=((700, 20), (129, 33), (128, 9), (1500, 64)), seed=107)
+    arrays = [synth.gen_cache(w, ci) for ci in range(len(w.caches))]
+    for ci, a in enumerate(arrays):
+        T, rng = w.caches[ci].T, np.random.default_rng(ci)
+        # (eigenvalues about 16 : 4 : 0.25 and no small ones, so that the retained rows' span is well conditioned)
+        V = rng.standard_normal((w.layers, w.kv_heads, T, 64)) * np.array([4.0, 2.0] + 62 * [0.5])
+        Qv = a["Q"].reshape(w.layers, w.kv_heads, w.n_q, 64)
+        for l, h in all_heads(w):
+            A = oracle.scores(par.f32_view(a["K"][l, h], "bf16"), par.f32_view(Qv[l, h], "bf16"))
+            # (of the cache with a budget of head_dim all retained rows are multiples of one another)
+            idx = oracle.topk(A, w.caches[ci].budget)[0]
+            V[l, h, idx] = large * (V[l, h, idx] if w.caches[ci].budget < 64 else V[l, h, idx[:1]])
+        a["V"] = synth.to_bf16_bits(V.astype(np.float32))
+    outs, _, st = par.run_gpu(w, arrays, flags=flags)
+    assert st & 0xFF == 0
+    for a, o in zip(arrays, outs):
+        for l, h in all_heads(w):
+            ref = oracle.backfill(par.f32_view(a["K"][l, h], "bf16"), par.f32_view(a["V"][l, h], "bf16"),
+                                  o["scores"][l, h].cpu().numpy().astype(np.float64), o["idx"][l, h].cpu().numpy(), w.rank)
+            gap = (ref["diag"]["lam_rho"] - ref["diag"]["lam_next"]) / ref["diag"]["lam_1"]
+            err = np.linalg.norm(o["delta"][l, h].cpu().numpy().astype(np.float64) - ref["delta"]) / np.linalg.norm(ref["delta"])
+            # 64 fp32 roundings over the distance of the subspace from the rest (measured before the tensor cores took
+            # these heads over: 1e-6)
+            assert err <= 64 * par.U32 / gap, (l, h, err, gap)
