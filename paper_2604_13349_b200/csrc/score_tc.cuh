@@ -60,8 +60,15 @@ constexpr int ST_MESSENGERS = 4;                    // messenger warps, a query 
 constexpr int ST_THREADS = 64 + ST_CONSUMERS + 32 * ST_MESSENGERS + 32;
 constexpr int ST_MAX_NQ = 256;                      // two query tiles of 128 rows
 constexpr float ST_LOG2E = 1.4426950408889634f;
+// M' has the magnitude of the logits and its rounding, up to 2^-18 of a weight, is common to all keys of a query.  Heads of 64
+// channels were computed without it and keep that precision: their references stay within 1 of the maximum (64 otherwise), and
+// a weight is exp2(s c - M) times 1 / Z.  Sum of a row's weights at logits of 100: off by up to 4e-6 with M', 3e-7 so; masses
+// against 64 bits, T = 1024, 160 queries, small logits: 2.1e-7 and 1.3e-7 (at large ones 4e-7 either way, from the tensor cores'
+// sums).
 template <int D>
-constexpr size_t score_tc_smem_bytes() { return 1024 + (size_t)(2 + ST_STAGES) * 128 * D * 2 + (2 * 2 * ST_GROUPS * 128 + 2 * 128) * sizeof(float) + 64; }
+constexpr bool ST_FINE = D == 64;
+template <int D>
+constexpr size_t score_tc_smem_bytes() { return 1024 + (size_t)(2 + ST_STAGES) * 128 * D * 2 + (2 * 2 * ST_GROUPS * 128 + (ST_FINE<D> ? 4 : 2) * 128) * sizeof(float) + 64; }
 static_assert(ST_STAGES == ST_TBUF, "a ring stage is released by the accumulator barrier of the same index");
 
 // An item with up to 32 (64) queries, the second one of a head with 160 for instance, would leave three (two) schedulers of
@@ -172,11 +179,20 @@ __device__ __forceinline__ void exp2_add(f32x2 &acc, uint32_t s0, uint32_t s1, f
     acc = add2(acc, pk(ex2_approx(a), ex2_approx(b)));
 }
 
+// Two logits at a time: exp2(s c + o) w, added to an accumulator pair.
+__device__ __forceinline__ void exp2_fma(f32x2 &acc, uint32_t s0, uint32_t s1, f32x2 sc, f32x2 o, f32x2 w)
+{
+    float a, b;
+    upk(fma2(pk(__uint_as_float(s0), __uint_as_float(s1)), sc, o), a, b);
+    acc = fma2(pk(ex2_approx(a), ex2_approx(b)), w, acc);
+}
+
 // Pass A on one thread's 16 logits of a piece: reference m (log2 domain) and sum z of exp2(s c - m) of one query.  The
-// reference is the largest logit up to the last piece that exceeded it by 64: no more is needed for a sum that neither
-// overflows nor loses its small terms, and the step that changes it is then a branch hardly ever taken.  z >= 1 wherever a
-// finite logit was met.  With MASKED only the first n_valid columns are keys.
-template <bool MASKED>
+// reference is the largest logit up to the last piece that exceeded it by MARGIN = 64: no more is needed for a sum that neither
+// overflows nor loses its small terms, and the step that changes it is then a branch hardly ever taken.  (With 1 the terms that
+// count lose no bits to the distance from the reference.)  z >= 1 wherever a finite logit was met.  With MASKED only the first
+// n_valid columns are keys.
+template <bool MASKED, int MARGIN>
 __device__ __forceinline__ void stats_update(uint32_t (&rr)[16], int n_valid, float sc, float &m, float &z)
 {
     if (MASKED) {
@@ -191,7 +207,7 @@ __device__ __forceinline__ void stats_update(uint32_t (&rr)[16], int n_valid, fl
         t1 = max3(t1, __uint_as_float(rr[e + 2]), __uint_as_float(rr[e + 3]));
     }
     const float t = fmaxf(t0, t1) * sc;
-    if (t > m + 64.f) {
+    if (t > m + (float)MARGIN) {
         z *= ex2_approx(m - t);                                                        // (0 * exp2(-inf) at first)
         m = t;
     }
@@ -207,15 +223,22 @@ __device__ __forceinline__ void stats_update(uint32_t (&rr)[16], int n_valid, fl
 }
 
 // Pass B on one thread's 16 logits of a piece: the softmax weights of one key under 16 queries, added to a0, a1.
-// mp: -M'_t of those queries (shared memory, the same address for every lane).
-__device__ __forceinline__ void pool_piece(const uint32_t (&rr)[16], const float *mp, float sc, f32x2 &a0, f32x2 &a1)
+// mp: -M'_t of those queries (shared memory, the same address for every lane); with FINE -M_t, and 1 / Z_t behind it at rz.
+template <bool FINE>
+__device__ __forceinline__ void pool_piece(const uint32_t (&rr)[16], const float *mp, const float *rz, float sc, f32x2 &a0, f32x2 &a1)
 {
     const f32x2 sc2 = pk(sc, sc);
 #pragma unroll
     for (int e = 0; e < 16; e += 4) {
         const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(mp + e);
-        exp2_add(a0, rr[e], rr[e + 1], sc2, v.x);
-        exp2_add(a1, rr[e + 2], rr[e + 3], sc2, v.y);
+        if constexpr (FINE) {
+            const ulonglong2 w = *reinterpret_cast<const ulonglong2 *>(rz + e);
+            exp2_fma(a0, rr[e], rr[e + 1], sc2, v.x, w.x);
+            exp2_fma(a1, rr[e + 2], rr[e + 3], sc2, v.y, w.y);
+        } else {
+            exp2_add(a0, rr[e], rr[e + 1], sc2, v.x);
+            exp2_add(a1, rr[e + 2], rr[e + 3], sc2, v.y);
+        }
     }
 }
 
@@ -229,7 +252,9 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constan
     uint8_t *ring = q_s + 2 * ST_TILE_BYTES;                       // ST_STAGES x 32 KiB
     float *s_m = reinterpret_cast<float *>(ring + ST_STAGES * ST_TILE_BYTES);   // [2][tile of the chunk][128 queries] tile maxima
     float *s_z = s_m + 2 * ST_GROUPS * 128;                        // [2][tile of the chunk][128 queries] tile sums
+    constexpr bool FINE = ST_FINE<D>;
     float *s_mp = s_z + 2 * ST_GROUPS * 128;                       // [2][128] -M'_t of the head being pooled
+    float *s_rz = s_mp + 2 * 128;                                  // with FINE: -M_t there, [2][128] 1 / Z_t here
     __shared__ uint64_t bar_q_full[2], bar_q_free[2], bar_full[ST_STAGES];
     __shared__ uint64_t bar_t_full[ST_TBUF], bar_t_empty[ST_TBUF];
     __shared__ uint64_t bar_st_ready[2], bar_mp_ready[2];
@@ -446,8 +471,8 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constan
                     walk_tile(it + my_t, q / share * share, item.copies > 1 || 32 * q < item.nq ? share : 0, [&](int hp, uint32_t (&rr)[16]) {
                         // two copies of the update: the one that masks missing keys runs for a head's ragged last tile only
                         const int k0 = key0 + 16 * hp;
-                        if (k0 + 16 > T) stats_update<true>(rr, T - k0, sc, m, z);
-                        else stats_update<false>(rr, 16, sc, m, z);
+                        if (k0 + 16 > T) stats_update<true, FINE ? 1 : 64>(rr, T - k0, sc, m, z);
+                        else stats_update<false, FINE ? 1 : 64>(rr, 16, sc, m, z);
                     });
                     // hand (m, z) of the tile to the messengers, filed under the tile's place in the chunk: they merge a
                     // chunk's tiles in that order whichever groups worked on them.  (The buffer is free: what the
@@ -465,11 +490,11 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constan
                 const int T = s_tab[prev.cache].T, buf = (i - 1) & 1;
                 tc::mbar_wait(&bar_mp_ready[buf], n_b[buf] & 1u, wc, 20);
                 ++n_b[buf];
-                const float *mp = s_mp + buf * 128;
+                const float *mp = s_mp + buf * 128, *rz = s_rz + buf * 128;
                 const int my_t = (int)((uint32_t)(grp - (int)it) % ST_GROUPS);
                 if (my_t < prev.nt) {
                     f32x2 a0 = 0ull, a1 = 0ull;
-                    walk_tile(it + my_t, 0, (prev.nq + 31) >> 5, [&](int hp, uint32_t (&rr)[16]) { pool_piece(rr, mp + 16 * hp, sc, a0, a1); });
+                    walk_tile(it + my_t, 0, (prev.nq + 31) >> 5, [&](int hp, uint32_t (&rr)[16]) { pool_piece<FINE>(rr, mp + 16 * hp, rz + 16 * hp, sc, a0, a1); });
                     const float a = sum2(add2(a0, a1));
                     const int j = prev.chunk * ST_CHUNK + my_t * 128 + row;
                     if (j < T) {
@@ -572,18 +597,20 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constan
                 M = Mn;
             }
             // (the buffer is free: every consumer has pooled with its last contents before it handed in this round's statistics)
-            float mp = INFINITY;                                               // exp2(-inf) = 0 for padding columns
+            float mp = INFINITY, rz = 0.f;                                     // exp2(-inf) = 0 for padding columns
             if (mine) {
                 // the keys outside the prompt take their share of the normaliser
                 fold_lse_extra(extra, M, Z);
-                mp = M + lg2_approx(Z);
-                if (gave_up) mp = 0.f;
-                else if (!(Z > 0.f) || !isfinite(mp)) {
+                mp = FINE ? M : M + lg2_approx(Z);
+                rz = FINE ? 1.f / Z : 1.f;
+                if (gave_up) { mp = 0.f; rz = 1.f; }
+                else if (!(Z > 0.f) || !isfinite(mp) || !isfinite(rz)) {
                     if (item.chunk == 0) atomicOr(p.status, OBF_DEV_NONFINITE);
                     mp = __int_as_float(0x7fc00000);
                 }
             }
             s_mp[buf * 128 + t] = -mp;
+            if (FINE) s_rz[buf * 128 + t] = rz;
             __syncwarp();
             if (lane == 0) tc::mbar_arrive(&bar_mp_ready[buf]);
         }

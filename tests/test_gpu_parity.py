@@ -1107,3 +1107,18 @@ def test_heads_of_64_channels_keep_their_precision_beside_large_retained_values(
             # 64 fp32 roundings over the distance of the subspace from the rest (measured before the tensor cores took
             # these heads over: 1e-6)
             assert err <= 64 * par.U32 / gap, (l, h, err, gap)
+
+
+@pytest.mark.parametrize("T,n_obs", [(128, 1), (700, 1), (2049, 1), (700, 2)])
+def test_softmax_rows_of_heads_of_64_channels_add_up_to_one(T, n_obs):
+    # with logits of 100 (base 2) a normaliser kept as a logarithm would be rounded to 2^-18: the same error in every weight of
+    # the row.  What is left is the exponential's own 2^-22.5, once in the sum and once in a weight that may be most of the row,
+    # and three roundings
+    w = small("rows64", d=64, dtype="bf16", rank=0, kv_heads=8, G=1, n_obs=n_obs, caches=((T, 20),), seed=109)
+    a = synth.gen_cache(w, 0)
+    K, Q = par.f32_view(a["K"], "bf16")[0], par.f32_view(a["Q"], "bf16")[0]
+    top = np.abs(np.einsum("htd,hqd->hqt", K, Q)).max(axis=(1, 2)) / 8.0 * np.log2(np.e)
+    a["Q"] = synth.to_bf16_bits((Q * (100.0 / top)[:, None, None]).astype(np.float32))[None]
+    out = par.run_gpu(w, [a], evict=True)[0][0]
+    rows = out["scores"].cpu().numpy().astype(np.float64)[0].sum(axis=-1)
+    assert np.all(np.abs(rows / n_obs - 1.0) <= 2 * 2.0 ** -22.5 + 3 * par.U32), rows - n_obs
