@@ -9,18 +9,47 @@ namespace obf {
 
 constexpr int SC_TILE = 64;           // queries x keys per score tile
 constexpr int SC_NT = 256;
-constexpr int SC_MAX_SPLITS = 32;     // key splits of the statistics kernel
 constexpr float LOG2E = 1.4426950408889634f;
 
+// A row's statistics are folded over its keys in an order that T alone decides, whatever else is in the call: the key tiles are
+// cut into up to 32 leaves of at least two tiles, the leaves are padded to a power of two, and neighbours are folded pair by
+// pair.  The statistics kernel gives a block one aligned run of leaves, a power of two of them; the pooling kernel folds the
+// runs' results.  However many blocks share a row, it is the same tree, so that a head's masses do not depend on the other
+// heads of the call or on the scratch it was given.  (80 registers, three blocks on a multiprocessor.)
+constexpr int SC_LEAVES = 32;
+constexpr int SC_MAX_SPLITS = SC_LEAVES;
+__host__ __device__ constexpr int sc_leaf_tiles(int T)
+{
+    const int tiles = (T + SC_TILE - 1) / SC_TILE, per = (tiles + SC_LEAVES - 1) / SC_LEAVES;
+    return per < 2 ? 2 : per;
+}
+__host__ __device__ constexpr int sc_leaves(int T)
+{
+    const int n = ((T + SC_TILE - 1) / SC_TILE + sc_leaf_tiles(T) - 1) / sc_leaf_tiles(T);
+    int p = 1;
+    while (p < n) p *= 2;
+    return p;
+}
+
+// (m, z) <- the fold of (m, z) and (m2, z2); (-inf, 0) is the empty one and changes nothing.
+__device__ __forceinline__ void sc_fold(float &m, float &z, float m2, float z2)
+{
+    const float M = fmaxf(m, m2), Mf = fmaxf(M, -3e38f);                       // (-inf - -inf would be a NaN)
+    z = fmaf(z2, exp2f(m2 - Mf), z * exp2f(m - Mf));
+    m = M;
+}
+
+constexpr int SC_STACK = 5;                     // levels of a block's run of leaves (k_score_stats)
+static_assert(1 << SC_STACK == SC_LEAVES && 2 * SC_STACK <= 18, "they lie where the pooling kernel has its 18 rows of 64");
 template <int D>
 constexpr size_t score_smem_bytes() { return 2 * SC_TILE * TD_LD<D> * sizeof(float) + 2 * SC_TILE * sizeof(float)
                                              + 16 * SC_TILE * sizeof(float); }
 
 // Step a1, first pass (Eq. 1): for every query row the running maximum of the
-// scaled logits (log2 domain) and the softmax normaliser over the keys of a split (the pooling kernel folds the splits).
-// grid = (ceil(n_q/64), heads_total, key splits).
+// scaled logits (log2 domain) and the softmax normaliser over the keys of a split, an aligned run of leaves (above).
+// grid = (ceil(n_q/64), heads_total, key splits); blocks beyond a cache's leaves exit.
 template <typename TIN, int D>
-__global__ void __launch_bounds__(SC_NT) k_score_stats(const __grid_constant__ CallDev p)
+__global__ void __launch_bounds__(SC_NT, 3) k_score_stats(const __grid_constant__ CallDev p)
 {
     pdl_wait();
     extern __shared__ __align__(16) float sm[];
@@ -35,48 +64,64 @@ __global__ void __launch_bounds__(SC_NT) k_score_stats(const __grid_constant__ C
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
     const float sc = LOG2E * rsqrtf((float)D);
 
+    const int leaves = sc_leaves(T), splits = min(p.sc_splits, leaves), run = leaves / splits;     // all powers of two
+    if ((int)blockIdx.z >= splits) return;
     load_rows_f32<TIN, D, SC_NT>(Qs, TD_LD<D>, Qh, q0, n_q, SC_TILE);
-    float m[4], Z[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) { m[i] = -INFINITY; Z[i] = 0.f; }
+    const int leaf_keys = sc_leaf_tiles(T) * SC_TILE;
+    // finished subtrees that wait for their right neighbour, one per level and row
+    float *wait_m = Ks + SC_TILE * TD_LD<D>, *wait_z = wait_m + SC_STACK * SC_TILE;
 
-    const int per = ((T + SC_TILE - 1) / SC_TILE + p.sc_splits - 1) / p.sc_splits * SC_TILE;
-    const int j_end = min(T, ((int)blockIdx.z + 1) * per);
-    for (int j0 = blockIdx.z * per; j0 < j_end; j0 += SC_TILE) {
-        __syncthreads();
-        load_rows_f32<TIN, D, SC_NT>(Ks, TD_LD<D>, Kh, j0, T, SC_TILE);
-        __syncthreads();
-        float acc[4][4];
-        tile_dots<D>(Qs, Ks, ty, tx, acc);
+    for (int leaf = 0; leaf < run; ++leaf) {
+        const int j_begin = (blockIdx.z * run + leaf) * leaf_keys, j_end = min(T, j_begin + leaf_keys);
+        float m[4], Z[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            float tm = -INFINITY;
+        for (int i = 0; i < 4; ++i) { m[i] = -INFINITY; Z[i] = 0.f; }
+        for (int j0 = j_begin; j0 < j_end; j0 += SC_TILE) {
+            __syncthreads();
+            load_rows_f32<TIN, D, SC_NT>(Ks, TD_LD<D>, Kh, j0, T, SC_TILE);
+            __syncthreads();
+            float acc[4][4];
+            tile_dots<D>(Qs, Ks, ty, tx, acc);
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                acc[i][j] = (j0 + tx + 16 * j < T) ? acc[i][j] * sc : -INFINITY;
-                tm = fmaxf(tm, acc[i][j]);
+            for (int i = 0; i < 4; ++i) {
+                float tm = -INFINITY;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    acc[i][j] = (j0 + tx + 16 * j < T) ? acc[i][j] * sc : -INFINITY;
+                    tm = fmaxf(tm, acc[i][j]);
+                }
+#pragma unroll
+                for (int o = 8; o > 0; o >>= 1) tm = fmaxf(tm, __shfl_xor_sync(0xffffffffu, tm, o));
+                const float nm = fmaxf(m[i], tm);
+                float s = 0.f;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) s += exp2f(acc[i][j] - nm);
+#pragma unroll
+                for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+                Z[i] = Z[i] * exp2f(m[i] - nm) + s;
+                m[i] = nm;
             }
-#pragma unroll
-            for (int o = 8; o > 0; o >>= 1) tm = fmaxf(tm, __shfl_xor_sync(0xffffffffu, tm, o));
-            const float nm = fmaxf(m[i], tm);
-            float s = 0.f;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) s += exp2f(acc[i][j] - nm);
-#pragma unroll
-            for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            Z[i] = Z[i] * exp2f(m[i] - nm) + s;
-            m[i] = nm;
         }
-    }
-    if (tx == 0) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int row = q0 + ty + 16 * i;
-            if (row < n_q) {
-                if (c.lse_extra && blockIdx.z == 0) fold_lse_extra(c.lse_extra[(size_t)lh * n_q + row], m[i], Z[i]);
-                float *st = p.stats + (((size_t)blockIdx.y * p.sc_splits + blockIdx.z) * n_q + row) * 2;
-                st[0] = m[i];
-                st[1] = Z[i];
+        // the sixteen lanes of a row hold the same: the first four fold and store a row each
+        const int slot = ty + 16 * tx, row = q0 + slot;
+        if (tx < 4 && row < n_q) {
+            float mi = tx == 0 ? m[0] : tx == 1 ? m[1] : tx == 2 ? m[2] : m[3];
+            float zi = tx == 0 ? Z[0] : tx == 1 ? Z[1] : tx == 2 ? Z[2] : Z[3];
+            // the keys outside the prompt go with the first leaf
+            if (c.lse_extra && blockIdx.z == 0 && leaf == 0) fold_lse_extra(c.lse_extra[(size_t)lh * n_q + row], mi, zi);
+            int level = 0;
+#pragma unroll 1
+            for (; (leaf >> level) & 1; ++level) {
+                float M = wait_m[level * SC_TILE + slot], S = wait_z[level * SC_TILE + slot];
+                sc_fold(M, S, mi, zi);
+                mi = M;
+                zi = S;
+            }
+            if (leaf + 1 < run) {
+                wait_m[level * SC_TILE + slot] = mi;
+                wait_z[level * SC_TILE + slot] = zi;
+            } else {
+                reinterpret_cast<float2 *>(p.stats)[((size_t)blockIdx.y * p.sc_splits + blockIdx.z) * n_q + row] = make_float2(mi, zi);
             }
         }
     }
@@ -85,7 +130,7 @@ __global__ void __launch_bounds__(SC_NT) k_score_stats(const __grid_constant__ C
 // Step a1, second pass (Eq. 1): A_j = sum_t exp(s_tj - m_t) / Z_t for a tile of 64 keys.
 // grid = (ceil(T_max/64), heads_total); blocks beyond a cache's T exit.
 template <typename TIN, int D>
-__global__ void __launch_bounds__(SC_NT) k_score_pool(const __grid_constant__ CallDev p)
+__global__ void __launch_bounds__(SC_NT, 3) k_score_pool(const __grid_constant__ CallDev p)
 {
     pdl_wait();
     extern __shared__ __align__(16) float sm[];
@@ -107,23 +152,36 @@ __global__ void __launch_bounds__(SC_NT) k_score_pool(const __grid_constant__ Ca
     for (int q0 = 0; q0 < n_q; q0 += SC_TILE) {
         __syncthreads();
         load_rows_f32<TIN, D, SC_NT>(Qs, TD_LD<D>, Qh, q0, n_q, SC_TILE);
-        if (threadIdx.x < SC_TILE) {
-            // the row's statistics over all keys, from the splits' (an empty split has the maximum -inf and the sum 0)
-            const int row = q0 + threadIdx.x;
-            const float2 *st = reinterpret_cast<const float2 *>(p.stats) + (size_t)blockIdx.y * p.sc_splits * n_q + min(row, n_q - 1);
-            float M = -INFINITY, Z = 0.f;
-            for (int s0 = 0; s0 < p.sc_splits; s0 += 4) {
-                float2 v[4];
+        {
+            // a row's statistics over all keys, the upper levels of the tree: four threads per row, a run of splits each
+            constexpr int PER = SC_MAX_SPLITS / 4;
+            static_assert(SC_NT == 4 * SC_TILE && PER >= 1, "four threads per row");
+            const int slot = threadIdx.x >> 2, part = threadIdx.x & 3, row = q0 + slot, splits = min(p.sc_splits, sc_leaves(T));
+            const float2 *st = reinterpret_cast<const float2 *>(p.stats) + ((size_t)blockIdx.y * p.sc_splits + part * PER) * n_q + min(row, n_q - 1);
+            float2 v[PER];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) v[e] = s0 + e < p.sc_splits ? st[(size_t)(s0 + e) * n_q] : make_float2(-INFINITY, 0.f);
-                const float Mn = fmaxf(fmaxf(fmaxf(v[0].x, v[1].x), fmaxf(v[2].x, v[3].x)), M), Mf = fmaxf(Mn, -3e38f);
-                Z *= exp2f(M - Mf);
+            for (int e = 0; e < PER; ++e) v[e] = part * PER + e < splits ? st[(size_t)e * n_q] : make_float2(-INFINITY, 0.f);
 #pragma unroll
-                for (int e = 0; e < 4; ++e) Z = fmaf(v[e].y, exp2f(v[e].x - Mf), Z);
-                M = Mn;
+            for (int w = 1; w < PER; w *= 2)
+                if (w < splits) {
+#pragma unroll
+                    for (int e = 0; e < PER; e += 2 * w) sc_fold(v[e].x, v[e].y, v[e + w].x, v[e + w].y);
+                }
+            float M = v[0].x, Z = v[0].y;
+            if (splits > PER) {
+#pragma unroll
+                for (int o = 1; o < 4; o *= 2) {
+                    const float m2 = __shfl_xor_sync(0xffffffffu, M, o), z2 = __shfl_xor_sync(0xffffffffu, Z, o);
+                    float ml = part & o ? m2 : M, zl = part & o ? z2 : Z;
+                    sc_fold(ml, zl, part & o ? M : m2, part & o ? Z : z2);
+                    M = ml;
+                    Z = zl;
+                }
             }
-            rm[threadIdx.x] = row < n_q ? M : 0.f;
-            rz[threadIdx.x] = row < n_q ? 1.0f / Z : 0.f;
+            if (part == 0) {
+                rm[slot] = row < n_q ? M : 0.f;
+                rz[slot] = row < n_q ? 1.0f / Z : 0.f;
+            }
         }
         __syncthreads();
         float acc[4][4];

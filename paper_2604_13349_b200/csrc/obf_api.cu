@@ -127,15 +127,13 @@ static int choose_splits(int heads_total, int T_max)
 
 // Key splits of the shape-generic statistics kernel: its grid of (64 queries, head) tiles leaves most of the chip idle on
 // small calls, and a block walks all of a split's keys one tile after the other.  About four blocks per multiprocessor
-// (two or three are resident), at least two tiles of keys each.
+// (two or three are resident), a power of two of splits (generic.cuh: the masses do not depend on how many).
 static int score_splits(int heads_total, int n_q, int T_max)
 {
     const long long tiles = (long long)((n_q + SC_TILE - 1) / SC_TILE) * heads_total;
-    const int key_tiles = (T_max + SC_TILE - 1) / SC_TILE;
-    long long s = (4 * 148 + tiles - 1) / tiles;
-    if (s > key_tiles / 2) s = key_tiles / 2;
-    if (s > SC_MAX_SPLITS) s = SC_MAX_SPLITS;
-    return s < 1 ? 1 : (int)s;
+    int s = 1;
+    while (s < sc_leaves(T_max) && 2 * s * tiles <= 6 * 148) s *= 2;
+    return s;
 }
 
 // Retained positions of a cache: the protected prefix plus at most `budget` of the other positions.
@@ -166,7 +164,7 @@ static obf_status_t validate_shapes(const obf_params_t *p, const obf_cache_t *ca
     return OBF_OK;
 }
 
-// key_splits: at most this many for the shape-generic statistics kernel (a caller's scratch may not hold more).
+// key_splits: at most this many for the shape-generic statistics kernel (the library's own scratch may not hold more).
 static void make_layout(const obf_params_t *p, const obf_cache_t *caches, int32_t n, int rank, Layout &L, int key_splits = SC_MAX_SPLITS)
 {
     const int hpc = p->layers * p->kv_heads;
@@ -592,7 +590,7 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
 }
 
 static obf_status_t run(const obf_params_t *p, const obf_cache_t *caches, int32_t n, int rank,
-                        void *workspace, size_t workspace_bytes, void *stream)
+                        void *workspace, size_t workspace_bytes, void *stream, int key_splits = SC_MAX_SPLITS)
 {
     g_last_launches = 0;
     obf_status_t s = validate_shapes(p, caches, n, rank);
@@ -615,8 +613,7 @@ static obf_status_t run(const obf_params_t *p, const obf_cache_t *caches, int32_
             return OBF_ERR_INVALID_ARG;
     }
     Layout L;
-    make_layout(p, caches, n, rank, L);
-    if (workspace_bytes < L.total) make_layout(p, caches, n, rank, L, 1);
+    make_layout(p, caches, n, rank, L, key_splits);
     if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255u) || workspace_bytes < L.total)
         return OBF_ERR_WORKSPACE;
     if (p->flags & OBF_FLAG_TEST_WAIT_EXPIRES) {
@@ -1018,7 +1015,9 @@ extern "C" obf_status_t evict_only_static(const obf_params_t *params, const obf_
     pe.flags &= ~(uint32_t)OBF_FLAG_MERGE;                 // eviction only: nothing is merged either
     params = &pe;
     Layout L;
-    make_layout(params, caches, n_caches, 0, L, 1);        // (more key splits only where they fit)
+    int key_splits = SC_MAX_SPLITS;                        // (fewer where that many do not fit: the masses are the same)
+    make_layout(params, caches, n_caches, 0, L, key_splits);
+    while (L.total > (size_t)OBF_STATIC_SCRATCH_BYTES && L.sc_splits > 1) make_layout(params, caches, n_caches, 0, L, key_splits = L.sc_splits / 2);
     if (L.total > (size_t)OBF_STATIC_SCRATCH_BYTES) {
         std::fprintf(stderr,
                      "obf: evict_only_static: this call needs %zu bytes of scratch but the built-in array holds "
@@ -1030,7 +1029,7 @@ extern "C" obf_status_t evict_only_static(const obf_params_t *params, const obf_
     if ((s = static_scratch_ptr(&scratch)) != OBF_OK) return s;
     // run() clears the status word at the head of the scratch; every other region is
     // written by an earlier kernel of the same call before a later one reads it.
-    return run(params, caches, n_caches, 0, scratch, (size_t)OBF_STATIC_SCRATCH_BYTES, stream);
+    return run(params, caches, n_caches, 0, scratch, (size_t)OBF_STATIC_SCRATCH_BYTES, stream, key_splits);
 }
 
 extern "C" obf_status_t obf_static_scratch_status(void *stream, uint32_t *device_status)

@@ -108,6 +108,19 @@ def test_compress_rejects_before_any_launch(lib):
     assert lib.obf_last_launch_count() == 0
 
 
+@pytest.mark.parametrize("dtype", [P.OBF_F32, P.OBF_BF16])
+@pytest.mark.parametrize("T", [300, 4000])
+def test_a_workspace_smaller_than_reported_is_refused(lib, dtype, T):
+    # also where the shape-generic kernels could make do with less
+    params, caches = _params(dtype=dtype, flags=binding.OBF_FLAG_GENERIC_PATH), [_cache(T=T)]
+    need = P.obf_workspace_bytes(params, caches)
+    for call in (P.obf_compress, P.evict_only):
+        if call is P.evict_only:
+            params.rank = 0
+            need = P.obf_workspace_bytes(params, caches)
+        assert call(params, caches, 0x1000, need - 1, stream=0, check=False) == binding.OBF_ERR_WORKSPACE
+
+
 def test_missing_library_fails_loudly(monkeypatch, tmp_path):
     monkeypatch.setattr(binding, "_lib", None)
     monkeypatch.setattr(build, "LIB_PATH", str(tmp_path / "nope.so"))

@@ -1122,3 +1122,37 @@ def test_softmax_rows_of_heads_of_64_channels_add_up_to_one(T, n_obs):
     out = par.run_gpu(w, [a], evict=True)[0][0]
     rows = out["scores"].cpu().numpy().astype(np.float64)[0].sum(axis=-1)
     assert np.all(np.abs(rows / n_obs - 1.0) <= 2 * 2.0 ** -22.5 + 3 * par.U32), rows - n_obs
+
+
+# ---------------------------------------------------------------------------
+# the masses of a head depend on the head alone: not on the other heads of the call, the slabs it is cut into or the scratch
+# ---------------------------------------------------------------------------
+def _random_caches(layers, kv_heads, G, n_obs, d, Ts, dtype, seed):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    tdt = torch.float32 if dtype == "f32" else torch.bfloat16
+    return [{"K": torch.randn((layers, kv_heads, T, d), generator=g, device="cuda").mul_(2.0).to(tdt),
+             "V": torch.randn((layers, kv_heads, T, d), generator=g, device="cuda").to(tdt),
+             "Q": torch.randn((layers, kv_heads * G, n_obs, d), generator=g, device="cuda").mul_(2.0).to(tdt)} for T in Ts]
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("Ts", [(64, 129), (300, 2100), (1024, 5000), (257,)])
+def test_masses_do_not_depend_on_the_other_heads_of_the_call(dtype, Ts):
+    # fp32, and bf16 on the shape-generic kernels: 40 layers x 4 heads against their last layer alone
+    flags = 0 if dtype == "f32" else P.binding.OBF_FLAG_GENERIC_PATH
+    dt = P.OBF_F32 if dtype == "f32" else P.OBF_BF16
+    dev = _random_caches(40, 4, 2, 33, 64, Ts, dtype, 113)
+    lse = [torch.randn((40, 8, 33), device="cuda") for _ in Ts]
+    whole = P.compress_caches(P.make_params(40, 4, 8, 64, 33, 0, dt, flags=flags),
+                              [dict(x, budget=20, lse_extra=e) for x, e in zip(dev, lse)], evict=True, want_scores=True)
+    for ci, (x, e) in enumerate(zip(dev, lse)):
+        part = {name: t[-1:].contiguous() for name, t in x.items()}
+        for heads in (slice(0, 4), slice(2, 3)):
+            one = {"K": part["K"][:, heads].contiguous(), "V": part["V"][:, heads].contiguous(),
+                   "Q": part["Q"][:, 2 * heads.start:2 * heads.stop].contiguous(),
+                   "lse_extra": e[-1:, 2 * heads.start:2 * heads.stop].contiguous()}
+            n = heads.stop - heads.start
+            out = P.compress_caches(P.make_params(1, n, 2 * n, 64, 33, 0, dt, flags=flags), [dict(one, budget=20)],
+                                    evict=True, want_scores=True)[0]
+            assert torch.equal(out["scores"], whole[ci]["scores"][-1:, heads])
+            assert torch.equal(out["idx"], whole[ci]["idx"][-1:, heads])

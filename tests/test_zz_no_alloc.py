@@ -84,3 +84,20 @@ def test_static_scratch_entry_point_rejects_shapes_beyond_its_array(capfd):
     assert rc == binding.OBF_ERR_WORKSPACE
     err = capfd.readouterr().err
     assert str(need) in err and str(binding.OBF_STATIC_SCRATCH_BYTES) in err
+
+
+def test_static_scratch_with_fewer_key_splits_computes_the_same():
+    # fp32, long prompts: the statistics of all the key splits that the workspace form uses do not fit the array, those of one do
+    T, n_obs = 205000, 448
+    g = torch.Generator(device="cuda").manual_seed(5)
+    K, V = (torch.randn((1, 8, T, 64), generator=g, device="cuda") for _ in range(2))
+    Q = torch.randn((1, 8, n_obs, 64), generator=g, device="cuda")
+    params = P.make_params(1, 8, 8, 64, n_obs, 0, P.OBF_F32)
+    ref = P.compress_caches(params, [dict(K=K, V=V, Q=Q, budget=50)], evict=True, want_scores=True)[0]
+    assert P.obf_workspace_bytes(params, ref["cache_structs"]) > binding.OBF_STATIC_SCRATCH_BYTES
+    o = {n: torch.zeros_like(ref[n]) for n in ("K_out", "V_out", "idx", "scores")}
+    P.evict_only_static(params, [P.make_cache(K, V, Q, T, 50, o["K_out"], o["V_out"], o["idx"], None, o["scores"])])
+    torch.cuda.synchronize()
+    assert P.obf_static_scratch_status() & 0xFF == 0
+    for n in o:
+        assert torch.equal(o[n], ref[n]), n
