@@ -754,6 +754,10 @@ struct HostArena {
     size_t ws, ws_bytes, total;
 };
 
+// The host-staged call works on slabs of layers.
+static int host_slabs(int layers) { return layers < 4 ? layers : 4; }
+static int host_slab_begin(int layers, int n_slabs, int sl) { return (int)((long long)layers * sl / n_slabs); }
+
 static void host_arena_layout(const obf_params_t *p, const obf_cache_t *caches, int32_t n, HostArena &H)
 {
     const size_t e = p->dtype == OBF_F32 ? 4 : 2;
@@ -772,10 +776,19 @@ static void host_arena_layout(const obf_params_t *p, const obf_cache_t *caches, 
         H.delta[i] = o; o = align_up(o + hpc * d * 4, 256);
         H.lse[i] = o; if (caches[i].lse_extra) o = align_up(o + (size_t)p->layers * p->q_heads * p->n_obs * 4, 256);
     }
-    Layout L;
-    make_layout(p, caches, n, effective_rank(p), L);
-    H.ws = o; H.ws_bytes = L.total; o += L.total;
-    H.total = o;
+    // the workspace serves one slab of layers after the other, and a slab can need more of it than the whole call would: fewer
+    // heads share the chip with more token splits each
+    H.ws = o;
+    H.ws_bytes = 0;
+    obf_params_t ps = *p;
+    const int n_slabs = host_slabs(p->layers);
+    for (int sl = -1; sl < n_slabs; ++sl) {
+        ps.layers = sl < 0 ? p->layers : host_slab_begin(p->layers, n_slabs, sl + 1) - host_slab_begin(p->layers, n_slabs, sl);
+        Layout L;
+        make_layout(&ps, caches, n, effective_rank(p), L);
+        if (L.total > H.ws_bytes) H.ws_bytes = L.total;
+    }
+    H.total = o + H.ws_bytes;
 }
 
 obf_status_t obf_host_arena_bytes(const obf_params_t *params, const obf_cache_t *caches, int32_t n_caches,
@@ -842,13 +855,13 @@ obf_status_t obf_compress_host(const obf_params_t *params, const obf_cache_t *ca
     const size_t H_kv = (size_t)params->kv_heads, d = params->head_dim;
     HostPipe *hp = host_pipe();
     if (!hp) return OBF_ERR_CUDA;
-    const int n_slabs = params->layers < 4 ? params->layers : 4;
+    const int n_slabs = host_slabs(params->layers);
     // nothing of this call may start before what the caller's stream already holds (an earlier call on the arena)
     OBF_CUDA_TRY(cudaEventRecord(hp->start, st));
     OBF_CUDA_TRY(cudaStreamWaitEvent(hp->cin, hp->start, 0));
     OBF_CUDA_TRY(cudaStreamWaitEvent(hp->cout, hp->start, 0));
     for (int sl = 0; sl < n_slabs; ++sl) {
-        const size_t l0 = (size_t)params->layers * sl / n_slabs, l1 = (size_t)params->layers * (sl + 1) / n_slabs;
+        const size_t l0 = host_slab_begin(params->layers, n_slabs, sl), l1 = host_slab_begin(params->layers, n_slabs, sl + 1);
         const size_t nl = l1 - l0;
         obf_params_t ps = *params;
         ps.layers = (int32_t)nl;

@@ -121,6 +121,29 @@ def test_a_workspace_smaller_than_reported_is_refused(lib, dtype, T):
         assert call(params, caches, 0x1000, need - 1, stream=0, check=False) == binding.OBF_ERR_WORKSPACE
 
 
+@pytest.mark.parametrize("dtype", [P.OBF_F32, P.OBF_BF16])
+def test_the_host_arena_holds_the_workspace_of_every_slab_of_layers(lib, dtype):
+    # the host-staged call works on four slabs of layers; a slab's heads can be split more finely than the whole call's
+    e = 4 if dtype == P.OBF_F32 else 2
+
+    def up(x):
+        return (x + 255) // 256 * 256
+
+    for kv_heads, d, n_obs in ((8, 64, 8), (8, 128, 16), (3, 128, 48), (1, 64, 40)):
+        for layers in list(range(1, 41)) + [99]:
+            for T in (129, 400, 1024, 3000):
+                params = _params(layers=layers, kv_heads=kv_heads, q_heads=4 * kv_heads, head_dim=d, n_obs=n_obs, rank=2, dtype=dtype)
+                cache = _cache(T=T, budget=20)
+                rows = layers * kv_heads
+                data = (2 * up(rows * T * d * e) + up(rows * 4 * n_obs * d * e) + 2 * up(rows * 20 * d * e) + up(rows * 20 * 4)
+                        + up(rows * binding.DIAG_BYTES) + up(rows * d * 4))
+                room = P.obf_host_arena_bytes(params, [cache]) - data
+                n = min(layers, 4)
+                for sl in range(n):
+                    params.layers = layers * (sl + 1) // n - layers * sl // n
+                    assert P.obf_workspace_bytes(params, [cache]) <= room, (kv_heads, d, layers, T, sl)
+
+
 def test_missing_library_fails_loudly(monkeypatch, tmp_path):
     monkeypatch.setattr(binding, "_lib", None)
     monkeypatch.setattr(build, "LIB_PATH", str(tmp_path / "nope.so"))

@@ -1156,3 +1156,18 @@ def test_masses_do_not_depend_on_the_other_heads_of_the_call(dtype, Ts):
                                     evict=True, want_scores=True)[0]
             assert torch.equal(out["scores"], whole[ci]["scores"][-1:, heads])
             assert torch.equal(out["idx"], whole[ci]["idx"][-1:, heads])
+
+
+def test_host_entry_point_on_fp32_layers_matches_the_device_entry_point():
+    # 37 layers: slabs of 9 and 10, whose heads share the chip differently from those of the whole call
+    dev = _random_caches(37, 8, 1, 8, 64, (700,), "f32", 117)[0]
+    params = P.make_params(37, 8, 8, 64, 8, 2, P.OBF_F32)
+    ref = P.compress_caches(params, [dict(dev, budget=12)], want_scores=True)[0]
+    h = {n: t.cpu().pin_memory() for n, t in dev.items()}
+    oK, oV = torch.empty((37, 8, 12, 64)).pin_memory(), torch.empty((37, 8, 12, 64)).pin_memory()
+    oI, oS = torch.empty((37, 8, 12), dtype=torch.int32).pin_memory(), torch.empty((37, 8, 700)).pin_memory()
+    c = P.make_cache(h["K"], h["V"], h["Q"], 700, 12, oK, oV, oI, None, oS)
+    arena = torch.empty(P.obf_host_arena_bytes(params, [c]), dtype=torch.uint8, device="cuda")
+    P.obf_compress_host(params, [c], arena)
+    assert torch.equal(oS, ref["scores"].cpu()) and torch.equal(oI, ref["idx"].cpu()) and torch.equal(oK, ref["K_out"].cpu())
+    assert torch.allclose(oV, ref["V_out"].cpu(), rtol=1e-4, atol=4e-6)
