@@ -338,11 +338,17 @@ __host__ __device__ constexpr int algebra_eig_floats(int rank, int fast_iters)
 }
 
 template <int D>
-inline size_t algebra_smem_bytes(int mcap, int rank, int fast_iters)
+constexpr size_t algebra_smem_bytes(int mcap, int rank, int fast_iters)
 {
     return (size_t)(algebra_y_rows<D>(mcap, rank, fast_iters) * D +  2 * D + 6 * D + 96 +
                     algebra_eig_floats<D>(rank, fast_iters)) * sizeof(float) + 2 * D * sizeof(int);
 }
+// The most any call needs: the Jacobi route with d basis rows.
+template <int D>
+constexpr size_t ALG_SMEM_MAX = algebra_smem_bytes<D>(D, D, 0);
+static_assert(ALG_SMEM_MAX<128> >= algebra_smem_bytes<128>(128, 128, 1) && ALG_SMEM_MAX<128> >= algebra_smem_bytes<128>(128, ALG_TRI_MAX_RANK, 0) &&
+              ALG_SMEM_MAX<64> >= algebra_smem_bytes<64>(64, 64, 1) && ALG_SMEM_MAX<64> >= algebra_smem_bytes<64>(64, ALG_TRI_MAX_RANK, 0), "no route needs more");
+static_assert(ALG_SMEM_MAX<128> <= 227 * 1024 - 1024, "a block has 227 KB, some of it static");
 
 template <typename TIN, int D>
 __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant__ CallDev p)

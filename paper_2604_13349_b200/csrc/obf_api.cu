@@ -284,6 +284,8 @@ static bool misaligned(const void *p) { return (reinterpret_cast<uintptr_t>(p) &
         }                                                                         \
     } while (0)
 
+// The limit belongs to the kernel, not to the launch, and host threads share it: a kernel whose use of shared memory varies
+// is given the most it can ever need, the same in every call, so that no call lowers it between another's limit and launch.
 template <typename K>
 static obf_status_t set_smem(K kernel, size_t bytes)
 {
@@ -456,10 +458,10 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
         mark(sel, "k_layer_sum");
         const int sms = sm_count();
         if (heads > sms) {
-            if ((s = set_smem(k_select_smem<512, true>, sm_sel)) != OBF_OK) return s;
+            if ((s = set_smem(k_select_smem<512, true>, SEL_SMEM_MAX_T * sizeof(uint32_t))) != OBF_OK) return s;
             OBF_TRY(launch(k_select_smem<512, true>, dim3(heads), 512, sm_sel, sel, cd, gather_vecs));
         } else {
-            if ((s = set_smem(k_select_smem<1024, true>, sm_sel)) != OBF_OK) return s;
+            if ((s = set_smem(k_select_smem<1024, true>, SEL_SMEM_MAX_T * sizeof(uint32_t))) != OBF_OK) return s;
             OBF_TRY(launch(k_select_smem<1024, true>, dim3(heads), 1024, sm_sel, sel, cd, gather_vecs));
         }
     } else if (T_max <= SEL_SMEM_MAX_T) {
@@ -469,10 +471,10 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
         // 229 us a call; eviction at T = 4096 167.6 -> 166.8)
         const int sms = sm_count();
         if (heads > sms) {
-            if ((s = set_smem(k_select_smem<512>, sm_sel)) != OBF_OK) return s;
+            if ((s = set_smem(k_select_smem<512>, SEL_SMEM_MAX_T * sizeof(uint32_t))) != OBF_OK) return s;
             OBF_TRY(launch(k_select_smem<512>, dim3(heads), 512, sm_sel, sel, cd, gather_vecs));
         } else {
-            if ((s = set_smem(k_select_smem<1024>, sm_sel)) != OBF_OK) return s;
+            if ((s = set_smem(k_select_smem<1024>, SEL_SMEM_MAX_T * sizeof(uint32_t))) != OBF_OK) return s;
             OBF_TRY(launch(k_select_smem<1024>, dim3(heads), 1024, sm_sel, sel, cd, gather_vecs));
         }
     } else {
@@ -511,7 +513,7 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
     }
     if (cd.rank > 0) {
         const size_t sm_alg = algebra_smem_bytes<D>(cd.alg_rows, cd.rank, cd.fast_iters);
-        if ((s = set_smem(k_obf_algebra<TIN, D>, sm_alg)) != OBF_OK) return s;
+        if ((s = set_smem(k_obf_algebra<TIN, D>, ALG_SMEM_MAX<D>)) != OBF_OK) return s;
         if (tuned_obf) {
             if constexpr (sizeof(TIN) == 2) {
                 if (cd.skip_full) {

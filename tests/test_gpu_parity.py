@@ -1171,3 +1171,37 @@ def test_host_entry_point_on_fp32_layers_matches_the_device_entry_point():
     P.obf_compress_host(params, [c], arena)
     assert torch.equal(oS, ref["scores"].cpu()) and torch.equal(oI, ref["idx"].cpu()) and torch.equal(oK, ref["K_out"].cpu())
     assert torch.allclose(oV, ref["V_out"].cpu(), rtol=1e-4, atol=4e-6)
+
+
+# ---------------------------------------------------------------------------
+# calls of different shapes from several host threads: a kernel's shared-memory limit is one for all of them
+# ---------------------------------------------------------------------------
+@pytest.mark.parametrize("what", ["selection", "algebra"])
+def test_threads_with_different_shared_memory_needs(what):
+    # long against short prompts (64 KB of selection keys or 1 KB); full eigen-decompositions against a single vector (200 KB or
+    # 60 KB of the dense algebra).  Every call has to be accepted
+    import threading
+    shapes = [(16384, 20, 0, 64), (256, 20, 0, 64)] if what == "selection" else [(200, 20, 9, 128), (200, 2, 1, 128)]
+    failures, start = [], threading.Barrier(len(shapes))
+
+    def worker(T, budget, rank, d):
+        stream = torch.cuda.Stream()
+        with torch.cuda.stream(stream):
+            x = _random_caches(1, 1, 1, 1, d, (T,), "f32", 127)[0]
+            params = P.make_params(1, 1, 1, d, 1, rank, P.OBF_F32)
+            out = P.compress_caches(params, [dict(x, budget=budget)], stream=stream)[0]
+            stream.synchronize()
+            start.wait()
+            for i in range(600 if what == "selection" else 100):
+                rc = P.obf_compress(params, out["cache_structs"], out["workspace"], stream=stream, check=False)
+                if rc != P.binding.OBF_OK:
+                    failures.append((T, rank, i, rc))
+                    break
+            stream.synchronize()
+
+    threads = [threading.Thread(target=worker, args=s) for s in shapes]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failures, failures
