@@ -55,6 +55,22 @@ static SideStream *side_stream()
     return &s;
 }
 
+// While the side stream holds work of a call: should the call end early, on an error, the caller's stream waits for that work
+// all the same, which uses the caller's outputs and workspace.
+struct SideWork {
+    SideStream *side = nullptr;
+    cudaStream_t st = nullptr;
+    obf_status_t join()
+    {
+        SideStream *s = side;
+        side = nullptr;
+        if (!s) return OBF_OK;
+        const cudaError_t a = cudaEventRecord(s->join, s->stream), b = cudaStreamWaitEvent(st, s->join, 0);
+        return a == cudaSuccess && b == cudaSuccess ? OBF_OK : OBF_ERR_CUDA;
+    }
+    ~SideWork() { (void)join(); }
+};
+
 static inline void mark(cudaStream_t st, const char *name)
 {
     ++g_last_launches;
@@ -280,6 +296,7 @@ static bool misaligned(const void *p) { return (reinterpret_cast<uintptr_t>(p) &
         cudaError_t e_ = (expr);                                                  \
         if (e_ != cudaSuccess) {                                                  \
             std::fprintf(stderr, "obf: %s failed: %s\n", #expr, cudaGetErrorString(e_)); \
+            (void)cudaGetLastError();      /* reported here: not the next call's */       \
             return OBF_ERR_CUDA;                                                  \
         }                                                                         \
     } while (0)
@@ -440,9 +457,12 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
     // (A pass over the deleted rows only needs the selection: one stream as well.)
     SideStream *side = (tuned_obf && !GramShape<D>::DELETED && !g_prof.active && !cd.skip_full) ? side_stream() : nullptr;
     cudaStream_t sel = side ? side->stream : st;       // stream of selection and gather
+    SideWork side_work;
     if (side) {
         OBF_CUDA_TRY(cudaEventRecord(side->fork, st));
         OBF_CUDA_TRY(cudaStreamWaitEvent(side->stream, side->fork, 0));
+        side_work.side = side;
+        side_work.st = st;
         if ((s = launch_gram_tc<D>(cd, L, st)) != OBF_OK) return s;
     }
     bool any_q8 = false;
@@ -483,10 +503,7 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
     mark(sel, "k_select");
     dim3 g4((k_max + GATHER_ROWS - 1) / GATHER_ROWS, heads);
     if (gather_vecs) {
-        if (side) {
-            OBF_CUDA_TRY(cudaEventRecord(side->join, side->stream));
-            OBF_CUDA_TRY(cudaStreamWaitEvent(st, side->join, 0));
-        }
+        OBF_TRY(side_work.join());
     } else if (side) {
         // the values first: the rest of the call needs them
         OBF_TRY(launch(k_gather<TIN, D, 1>, dim3(g4), 256, 0, sel, cd));
@@ -500,13 +517,12 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
             OBF_TRY(launch(k_span_test<D, true>, dim3(heads), ST_NT, sm_span, sel, cd));
             mark(sel, "k_span_test");
         }
-        OBF_CUDA_TRY(cudaEventRecord(side->join, side->stream));
         // the keys are needed by nothing that follows: they are copied on the caller's stream once the pass over V
         // is over (it is bound by HBM), while the span test finishes on the side stream
         OBF_CUDA_TRY(cudaStreamWaitEvent(st, side->rows_done, 0));
         OBF_TRY(launch(k_gather<TIN, D, 2>, dim3(g4), 256, 0, st, cd));
         ++g_last_launches;
-        OBF_CUDA_TRY(cudaStreamWaitEvent(st, side->join, 0));
+        OBF_TRY(side_work.join());
     } else {
         OBF_TRY(launch(k_gather<TIN, D>, dim3(g4), 256, 0, sel, cd));
         mark(sel, "k_gather");

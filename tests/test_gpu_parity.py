@@ -1205,3 +1205,25 @@ def test_threads_with_different_shared_memory_needs(what):
     for t in threads:
         t.join()
     assert not failures, failures
+
+
+def test_a_call_that_fails_halfway_leaves_no_work_unjoined():
+    # More heads than a grid has rows: the copy of the retained rows is refused at its launch, after the call has forked to the
+    # library's stream.  The call is captured and the graph never launched, so nothing runs; a fork that is not joined again
+    # would make the end of the capture fail.
+    n = 65536
+    params = P.make_params(n, 1, 1, 128, 1, 1, P.OBF_BF16)
+    buf = torch.zeros(4096, dtype=torch.uint8, device="cuda")
+    ptr = (buf.data_ptr() + 255) // 256 * 256
+    cache = P.make_cache(ptr, ptr, ptr, 256, 130, ptr, ptr, ptr)
+    warm = small("warm", d=128, dtype="bf16", caches=((256, 130),))       # (streams and events exist before the capture)
+    par.run_gpu(warm, [synth.gen_cache(warm, 0)])
+    stream = torch.cuda.Stream()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)                         # (never instantiated)
+    rc = None
+    with torch.cuda.graph(graph, stream=stream):
+        rc = P.obf_compress(params, [cache], ptr, P.obf_workspace_bytes(params, [cache]), stream=stream, check=False)
+    assert rc == P.binding.OBF_ERR_CUDA
+    del graph
+    ok = par.run_gpu(warm, [synth.gen_cache(warm, 0)])                    # the next call is accepted
+    assert ok[2] & 0xFF == 0
