@@ -279,7 +279,12 @@ const char *obf_phase_name(int32_t phase);
  *   ignored) and returns the same codes, plus OBF_ERR_WORKSPACE - with a
  *   message on stderr naming both sizes - when the call shape needs more
  *   scratch than OBF_STATIC_SCRATCH_BYTES (obf_workspace_bytes with rank 0
- *   tells how much a shape needs).
+ *   tells how much a shape needs; for bf16 heads of 64 channels the size with
+ *   OBF_FLAG_GENERIC_PATH, less its key splits, decides: a call that only the
+ *   tensor-core kernel's statistics make too large is enqueued as groups of
+ *   heads, or of layers with OBF_FLAG_LAYERWISE, one after the other.  Where
+ *   not even one such head or layer of every cache fits, the shape-generic
+ *   kernels run, whose masses differ in the last fp32 digits).
  * - Calls no cudaMalloc, cudaFree or any other allocating routine.
  * - The first call on each device resolves the array's device address
  *   (cudaGetSymbolAddress, with that device current); make that first call

@@ -1037,6 +1037,67 @@ obf_status_t static_scratch_ptr(void **out)
 
 }  // namespace
 
+namespace {
+
+// A shape whose tuned layout does not fit the array although the shape-generic one does: groups of heads (of layers, with the
+// layerwise selector) one after the other on the same scratch.  A head's result does not depend on the others of the call,
+// so that this is what evict_only computes.  OBF_ERR_WORKSPACE when not even one of them fits.
+obf_status_t run_in_groups(const obf_params_t *p, const obf_cache_t *caches, int32_t n, void *scratch, void *stream)
+{
+    obf_params_t pg = *p;
+    int units = p->layers;
+    if (!(p->flags & OBF_FLAG_LAYERWISE)) {
+        // heads one by one: every array is [layers x kv_heads][..]
+        units = p->layers * p->kv_heads;
+        pg.q_heads = p->q_heads / p->kv_heads;
+        pg.kv_heads = 1;
+    }
+    int per = units;
+    for (int n_groups = 2;; ++n_groups) {
+        if (per == 1) return OBF_ERR_WORKSPACE;
+        pg.layers = per = (units + n_groups - 1) / n_groups;
+        Layout L;
+        make_layout(&pg, caches, n, 0, L);
+        if (L.total <= (size_t)OBF_STATIC_SCRATCH_BYTES) break;
+    }
+    const size_t e = p->dtype == OBF_F32 ? 4 : 2, d = p->head_dim, n_q = (size_t)(p->q_heads / p->kv_heads) * p->n_obs;
+    int32_t launches = 0;
+    for (int u = 0; u < units; u += per) {
+        const size_t h = (size_t)u * pg.kv_heads;                          // heads before this group's
+        pg.layers = per < units - u ? per : units - u;
+        obf_cache_t c[OBF_MAX_CACHES];
+        for (int i = 0; i < n; ++i) {
+            const size_t T = caches[i].T, ke = (size_t)k_eff_of(p, caches[i]);
+            auto at = [](auto *base, size_t elements) { return base ? base + elements : nullptr; };
+            c[i] = caches[i];
+            c[i].k = at(static_cast<const char *>(c[i].k), h * T * d * e);
+            c[i].v = at(static_cast<const char *>(c[i].v), h * T * d * e);
+            c[i].q_obs = at(static_cast<const char *>(c[i].q_obs), h * n_q * d * e);
+            c[i].k_out = at(static_cast<char *>(c[i].k_out), h * ke * d * e);
+            c[i].v_out = at(static_cast<char *>(c[i].v_out), h * ke * d * e);
+            c[i].idx_out = at(c[i].idx_out, h * ke);
+            c[i].diag_out = at(c[i].diag_out, h);
+            c[i].scores_out = at(c[i].scores_out, h * T);
+            c[i].delta_out = at(c[i].delta_out, h * d);
+            c[i].lse_extra = at(c[i].lse_extra, h * n_q);
+            c[i].k_q8_out = at(c[i].k_q8_out, h * ke * d);
+            c[i].v_q8_out = at(c[i].v_q8_out, h * ke * d);
+            c[i].k_scale_out = at(c[i].k_scale_out, h * ke);
+            c[i].v_scale_out = at(c[i].v_scale_out, h * ke);
+            c[i].assign_out = at(c[i].assign_out, h * T);
+        }
+        g_keep_status = u > 0;
+        const obf_status_t s = run(&pg, c, n, 0, scratch, (size_t)OBF_STATIC_SCRATCH_BYTES, stream);
+        g_keep_status = false;
+        if (s != OBF_OK) return s;
+        launches += g_last_launches;
+    }
+    g_last_launches = launches;
+    return OBF_OK;
+}
+
+}  // namespace
+
 extern "C" obf_status_t evict_only_static(const obf_params_t *params, const obf_cache_t *caches,
                                           int32_t n_caches, void *stream)
 {
@@ -1049,7 +1110,16 @@ extern "C" obf_status_t evict_only_static(const obf_params_t *params, const obf_
     int key_splits = SC_MAX_SPLITS;                        // (fewer where that many do not fit: the masses are the same)
     make_layout(params, caches, n_caches, 0, L, key_splits);
     while (L.total > (size_t)OBF_STATIC_SCRATCH_BYTES && L.sc_splits > 1) make_layout(params, caches, n_caches, 0, L, key_splits = L.sc_splits / 2);
-    if (L.total > (size_t)OBF_STATIC_SCRATCH_BYTES) {
+    bool groups = false;
+    if (L.total > (size_t)OBF_STATIC_SCRATCH_BYTES && L.sc_on && params->head_dim == 64) {
+        // heads of 64 channels: the tensor-core kernel's chunk statistics, two bytes and more per position, do not count
+        obf_params_t pg = pe;
+        pg.flags |= OBF_FLAG_GENERIC_PATH;
+        Layout G;
+        make_layout(&pg, caches, n_caches, 0, G, 1);
+        groups = G.total <= (size_t)OBF_STATIC_SCRATCH_BYTES;
+    }
+    if (!groups && L.total > (size_t)OBF_STATIC_SCRATCH_BYTES) {
         std::fprintf(stderr,
                      "obf: evict_only_static: this call needs %zu bytes of scratch but the built-in array holds "
                      "%zu; use evict_only with a caller-provided workspace\n",
@@ -1058,8 +1128,16 @@ extern "C" obf_status_t evict_only_static(const obf_params_t *params, const obf_
     }
     void *scratch = nullptr;
     if ((s = static_scratch_ptr(&scratch)) != OBF_OK) return s;
-    // run() clears the status word at the head of the scratch; every other region is
-    // written by an earlier kernel of the same call before a later one reads it.
+    // run() clears the status word at the head of the scratch, the tuned score kernel's chunk statistics and, where two query
+    // tiles add theirs up, the masses; every other region is written by an earlier kernel of the same call before a later one
+    // reads it.
+    if (groups) {
+        if ((s = run_in_groups(params, caches, n_caches, scratch, stream)) != OBF_ERR_WORKSPACE) return s;
+        // one head of every cache (a layer of every cache, with the layerwise selector) is too much for it: the shape-generic
+        // kernels
+        pe.flags |= OBF_FLAG_GENERIC_PATH;
+        key_splits = 1;
+    }
     return run(params, caches, n_caches, 0, scratch, (size_t)OBF_STATIC_SCRATCH_BYTES, stream, key_splits);
 }
 
