@@ -61,11 +61,9 @@ struct CallDev {
     int32_t tc_per;           // tuned path: tiles per block of the pass over V (0: shape-generic path)
     int32_t pad1_;
     long long tc_total_sub;   // tuned path: tiles in the tile sequence of the pass over V
-    int32_t gram_all;         // 1: gram_d and uvec run over all rows of V (tuned path), 0: over the deleted rows only
-    int32_t u_levels;         // partial u vectors per partial Gram matrix: U_LEVELS with gram_all, else 1
+    int32_t gram_all;         // 1: gram_d and uvec run over all rows of V (tuned path, heads of 128 channels), 0: over the deleted rows only
+    int32_t u_levels;         // partial u vectors per partial Gram matrix: U_LEVELS on the tuned path, else 1
     int32_t alg_rows;         // dense algebra: basis rows any head of the call can have, min(largest k_eff, d)
-    int32_t sc_nq;            // tuned score kernel: query rows of its tiles (0: shape-generic score kernels)
-    int32_t sc_subs;          // 128-key tiles per chunk
     int32_t sc_rounds;        // rounds of the persistent score kernel
     int32_t sc_qt;            // tuned score kernel: 128-row query tiles per head (1 or 2)
     float *sc_part;           // per (head, chunk, query of 128): chunk maximum and normaliser as one 64-bit word, zero until published

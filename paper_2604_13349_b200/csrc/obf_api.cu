@@ -90,7 +90,7 @@ struct Layout {
     int heads_total;
     size_t tok_total;
     size_t tok_off[OBF_MAX_CACHES];
-    // tuned bf16 / head_dim 128 path
+    // tuned bf16 path
     bool tuned;
     int gram_slots;                 // partial Gram matrices stored per head
     int tc_per, tc_blocks;          // tiles per block and blocks of the tensor-core pass over V
@@ -99,7 +99,7 @@ struct Layout {
     long long sub_base[OBF_MAX_CACHES];
     // tensor-core score kernel
     bool sc_on;
-    int sc_nq, sc_subs, sc_blocks, sc_rounds, sc_qt;
+    int sc_blocks, sc_rounds, sc_qt;
     int sc_team[OBF_MAX_CACHES], sc_hpr[OBF_MAX_CACHES], sc_round_base[OBF_MAX_CACHES];
     size_t sc_part_off[OBF_MAX_CACHES], sc_part_pairs;
     size_t off_sc_part;
@@ -225,7 +225,7 @@ static void make_layout(const obf_params_t *p, const obf_cache_t *caches, int32_
         L.gram_slots = slots;
     }
     L.sc_on = false;
-    L.sc_nq = L.sc_subs = L.sc_blocks = L.sc_rounds = 0;
+    L.sc_blocks = L.sc_rounds = 0;
     L.sc_qt = 1;
     L.sc_part_pairs = 0;
     if (L.tuned && n_q <= ST_MAX_NQ) {
@@ -234,8 +234,6 @@ static void make_layout(const obf_params_t *p, const obf_cache_t *caches, int32_
         const int hpc_real = hpc;
         const int hpc = hpc_real * L.sc_qt;
         // chunks of ST_TILES 128-key tiles, one per block and round; a head's team must fit in one round
-        L.sc_nq = 128;
-        L.sc_subs = ST_TILES;
         long long blocks_wanted = 0;
         for (int i = 0; i < n; ++i) {
             L.sc_team[i] = (caches[i].T + ST_CHUNK - 1) / ST_CHUNK;
@@ -679,9 +677,7 @@ static obf_status_t run(const obf_params_t *p, const obf_cache_t *caches, int32_
     cd.gram_all = L.tc_per && !(p->head_dim == 64 ? GramShape<64>::DELETED : GramShape<128>::DELETED) ? 1 : 0;
     cd.u_levels = L.tc_per ? U_LEVELS : 1;
     cd.tc_total_sub = L.tc_total_sub;
-    cd.sc_nq = L.sc_on ? L.sc_nq : 0;
     cd.sc_qt = L.sc_on ? L.sc_qt : 1;
-    cd.sc_subs = L.sc_subs;
     cd.sc_rounds = L.sc_rounds;
     cd.sc_splits = L.sc_splits;
     cd.eps = p->eps;

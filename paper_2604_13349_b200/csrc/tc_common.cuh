@@ -123,11 +123,6 @@ __device__ __forceinline__ void tma_prefetch_rows(const CUtensorMap *map, int ro
                  ::"l"(map), "r"(0), "r"(row), "r"(head) : "memory");
 }
 
-__device__ __forceinline__ void prefetch_tensormap(const CUtensorMap *map)
-{
-    asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
-}
-
 // Generic-proxy writes to shared memory become visible to the tensor core / TMA.
 __device__ __forceinline__ void fence_async_smem()
 {
@@ -218,11 +213,6 @@ __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t a_desc, uint
 __device__ __forceinline__ void umma_commit(uint64_t *bar)
 {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-
-__device__ __forceinline__ void named_barrier(int id, int threads)
-{
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 
 }  // namespace tc
