@@ -47,6 +47,15 @@ def load_peaks():
     return 6650.0, "fallback"
 
 
+def load_tensor_peak():
+    """TFLOP/s of bf16 products on the tensor cores, as a burst (the kernel is timed by itself)."""
+    path = os.path.join(ROOT, "MEASURED_PEAKS.json")
+    if os.path.exists(path):
+        with open(path) as f:
+            return float(json.load(f)["bf16_tflops"]), "measured"
+    return 1590.0, "fallback"
+
+
 class ClockSampler:
     """Samples SM clocks and throttle reasons with nvidia-smi while the timed region runs."""
     FIELDS = ("clocks.sm,clocks.max.sm,power.draw,clocks_event_reasons.hw_slowdown,"
@@ -167,16 +176,17 @@ def run_reference(args):
 
 
 # fp32 work of the dense algebra per (layer, KV head) whose retained values do not span R^d, as the kernel
-# formulates it (Eq. 2-6): twice-iterated Gram-Schmidt over the k retained rows, P = I - Q^T Q, the two products of
-# M = P G P, the Householder reduction of M to tridiagonal form and the way back for rank + 1 vectors.
-def algebra_flops(d: int, k: int, rank: int) -> float:
+# formulates it (Eq. 2-6): a reflector per retained row, taken to the rows after it; every reflector to the Gram matrix from both
+# sides (a product and a rank-two update of the block it reaches, both triangles); on the exact route the trailing block's further
+# reflectors to tridiagonal form; on the fixed-iteration route three products with the block instead; one vector back through the
+# reflectors.  (What the eigenpairs of the tridiagonal form cost is of order rank * d.)
+def algebra_flops(d: int, k: int, rank: int, fast: bool = False) -> float:
     m = min(k, d)
-    gram_schmidt = 2 * 2 * (2.0 * d) * sum(min(i, d) for i in range(k))     # two passes of dot + update against i rows
-    projector = 2.0 * m * d * d
-    products = 2 * 2.0 * d ** 3
-    tridiagonal = 4.0 / 3.0 * d ** 3 * 2                                     # both triangles are updated
-    back = (rank + 1) * 2 * 2.0 * d * d
-    return gram_schmidt + projector + products + tridiagonal + back
+    rows = 4.0 * d * sum(min(i, m) for i in range(k))
+    last = m if fast else d - 1
+    two_sided = sum(6.0 * (d - j) ** 2 for j in range(last))
+    iterations = 3 * min(rank, d - m) * 2.0 * (d - m) ** 2 if fast else 0.0
+    return rows + two_sided + iterations + 4.0 * d * last
 
 
 # The source files a kernel's DRAM traffic depends on: its own file, what it includes, and the host file that sizes
@@ -314,23 +324,30 @@ class Bench:
         kernel_bytes = {"k_score_stats": kv + q, "k_score_pool": kv + q + sc,
                         "k_score_tc": kv + q + sc,                          # K and Q read once, A written
                         "k_gram": kv, "k_gram_tc": kv + sc,                 # V and A read once
-                        "k_gather": 2 * ob, "k_select": sc}.get(dom)
+                        "k_gather": 2 * ob, "k_select": sc,
+                        "k_merge_apply": kv + 2 * sc + ob // 2}.get(dom)   # V, A and the routing read, rows written
         common = {"kernel": dom, "kernel_ms": phase_acc[dom],
                   "whole_step_frac": (step_bytes / (ms_per_step * 1e-3) / 1e9) / peak,
                   "whole_step_peak": peak, "whole_step_peak_kind": peak_kind,
                   "phases_ms": {k: round(v, 4) for k, v in phase_acc.items()}}
         if kernel_bytes is None:
-            # the dense algebra (and the span test): no HBM traffic to speak of, fp32 arithmetic in shared memory.
+            # the dense algebra (and the span test): no HBM traffic to speak of, fp32 arithmetic in registers.
             # Peak: 148 SMs x 128 FMA lanes x 2 flop x SM clock.
             hpc = w.layers * w.kv_heads
-            if dom.startswith("k_merge"):
-                # cache-merging baseline: the similarities of every position with every retained key
-                flops = sum(hpc * 2.0 * c.T * min(c.budget, c.T) * w.head.head_dim for c in w.caches)
-            else:
-                flops = sum(hpc * algebra_flops(w.head.head_dim, min(c.budget, c.T), w.rank)
-                            for c in w.caches if min(c.budget, c.T) < w.head.head_dim)
             clock = sm_mhz or 1965.0
             alu_peak = 148 * 128 * 2 * clock * 1e6 / 1e12
+            if dom.startswith("k_merge"):
+                # cache-merging baseline: the similarities of every position with every retained key; bf16 keys are multiplied
+                # on the tensor cores
+                flops = sum(hpc * 2.0 * c.T * min(c.budget, c.T) * w.head.head_dim for c in w.caches)
+                if w.dtype == "bf16":
+                    tensor_peak, kind = load_tensor_peak()
+                    ach = flops / (phase_acc[dom] * 1e-3) / 1e12
+                    return dict(common, bound="tensor", achieved=ach, peak=tensor_peak, unit="TFLOP/s", frac=ach / tensor_peak,
+                                peak_kind=kind, traffic=None, algorithmic_flops_per_launch=flops)
+            else:
+                flops = sum(hpc * algebra_flops(w.head.head_dim, min(c.budget, c.T), w.rank, w.fast_path)
+                            for c in w.caches if min(c.budget, c.T) < w.head.head_dim)
             ach = flops / (phase_acc[dom] * 1e-3) / 1e12
             return dict(common, bound="alu", achieved=ach, peak=alu_peak, unit="TFLOP/s", frac=ach / alu_peak,
                         peak_kind="derived: 148 SMs x 128 fp32 FMA lanes x 2 x %.0f MHz" % clock, traffic=None,
