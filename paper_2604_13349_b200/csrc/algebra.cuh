@@ -32,7 +32,7 @@
 // stages of 32 so that finished rows and column pairs cost nothing and every register index is static.  128 threads of
 // 255 registers and less than 113 KB per block: two blocks share a multiprocessor.  What is run once per head is written
 // as small loops: a section's first pass costs about 130 cycles per 128 bytes of its code, more than its arithmetic.
-// Measured on 36 x 8 heads, budget 32, rank 2, head_dim 128 (every head back-filled): 0.139 ms against 0.534 ms for the
+// Measured on 36 x 8 heads, budget 32, rank 2, head_dim 128 (every head back-filled): 0.141 ms against 0.534 ms for the
 // same algebra on a matrix in shared memory (Gram-Schmidt basis, M = P G P, then the reduction).  Slower were: eight warps
 // with half the registers, the chain of reflectors in a warp of its own beside the matrix warps (the registers it takes cost
 // the others more), one copy of the step's code for all stages, the reflectors on G sixteen at a time in compact form (code
