@@ -356,9 +356,9 @@ class Bench:
         r = dict(common, bound="hbm", achieved=achieved, peak=peak, unit="GB/s", frac=achieved / peak,
                  peak_kind=peak_kind, traffic=measured_traffic(dom, w.name), algorithmic_bytes_per_launch=kernel_bytes)
         if dom == "k_score_tc":
-            # the attention-mass kernel evaluates 2 exponentials per (query, key): a second ceiling beside HBM is
+            # the attention-mass kernel evaluates an exponential per (query, key): a second ceiling beside HBM is
             # the special-function unit (16 results per clock and SM)
-            n_exp = 2.0 * sum(w.layers * w.kv_heads * c.T * w.n_q for c in w.caches)
+            n_exp = 1.0 * sum(w.layers * w.kv_heads * c.T * w.n_q for c in w.caches)
             sfu_peak = 16 * 148 * (sm_mhz or 1965.0) * 1e6 / 1e9
             r["sfu"] = {"unit": "Gexp/s", "achieved": n_exp / (phase_acc[dom] * 1e-3) / 1e9, "peak": sfu_peak,
                         "frac": n_exp / (phase_acc[dom] * 1e-3) / 1e9 / sfu_peak}

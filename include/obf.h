@@ -281,8 +281,10 @@ const char *obf_phase_name(int32_t phase);
  *   message on stderr naming both sizes - when the call shape needs more
  *   scratch than OBF_STATIC_SCRATCH_BYTES (obf_workspace_bytes with rank 0
  *   tells how much a shape needs; for bf16 heads of 64 channels the size with
- *   OBF_FLAG_GENERIC_PATH, less its key splits, decides: a call that only the
- *   tensor-core kernel's statistics make too large is enqueued as groups of
+ *   OBF_FLAG_GENERIC_PATH, less its key splits, decides, for bf16 heads of 128
+ *   channels that with the tensor-core kernel's statistics, 1 KB a head and 128
+ *   query rows, per 512 positions instead of 256: a call that only those
+ *   statistics make too large is enqueued as groups of
  *   heads, or of layers with OBF_FLAG_LAYERWISE, one after the other.  Where
  *   not even one such head or layer of every cache fits, the shape-generic
  *   kernels run, whose masses differ in the last fp32 digits).

@@ -32,11 +32,8 @@ struct CacheDev {
     int32_t pad_;
     size_t tok_off;           // offset of this cache in the per-token workspace arrays (elements)
     long long sub_base;       // tuned path: index of this cache's first tile in the tile sequence of the pass over V
-    // tuned score kernel: a head's chunks are worked on by a team of slots, heads are dealt in rounds
-    int32_t sc_team;          // chunks (= blocks) per head
-    int32_t sc_hpr;           // heads per round
-    int32_t sc_round_base;    // first round of this cache
-    int32_t pad2_;
+    int32_t sc_team;          // tuned score kernel: chunks per head
+    int32_t sc_item_base;     // and the cache's first (head, chunk) pair in the call's sequence of them
     size_t sc_part_off;       // offset of this cache in sc_part, in (max, sum) pairs
 };
 
@@ -64,9 +61,9 @@ struct CallDev {
     int32_t gram_all;         // 1: gram_d and uvec run over all rows of V (tuned path, heads of 128 channels), 0: over the deleted rows only
     int32_t u_levels;         // partial u vectors per partial Gram matrix: U_LEVELS on the tuned path, else 1
     int32_t alg_rows;         // dense algebra: basis rows any head of the call can have, min(largest k_eff, d)
-    int32_t sc_rounds;        // rounds of the persistent score kernel
+    int32_t sc_items;         // (head, chunk) pairs of the persistent score kernel
     int32_t sc_qt;            // tuned score kernel: 128-row query tiles per head (1 or 2)
-    float *sc_part;           // per (head, chunk, query of 128): chunk maximum and normaliser as one 64-bit word, zero until published
+    float *sc_part;           // per (head, query tile, chunk, query of 128): chunk reference and normaliser as one 64-bit word, zero until published
     int32_t sc_splits;        // shape-generic statistics kernel: key splits per (head, 64 queries)
     float eps;
     int32_t kv_heads;         // KV heads per layer

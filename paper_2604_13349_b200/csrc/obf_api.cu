@@ -99,9 +99,10 @@ struct Layout {
     long long sub_base[OBF_MAX_CACHES];
     // tensor-core score kernel
     bool sc_on;
-    int sc_blocks, sc_rounds, sc_qt;
-    int sc_team[OBF_MAX_CACHES], sc_hpr[OBF_MAX_CACHES], sc_round_base[OBF_MAX_CACHES];
+    int sc_blocks, sc_items, sc_qt;
+    int sc_team[OBF_MAX_CACHES], sc_item_base[OBF_MAX_CACHES];
     size_t sc_part_off[OBF_MAX_CACHES], sc_part_pairs;
+    size_t sc_part_512;             // as many pairs as chunks of 512 keys would have (evict_only_static)
     size_t off_sc_part;
 };
 
@@ -225,46 +226,38 @@ static void make_layout(const obf_params_t *p, const obf_cache_t *caches, int32_
         L.gram_slots = slots;
     }
     L.sc_on = false;
-    L.sc_blocks = L.sc_rounds = 0;
+    L.sc_blocks = L.sc_items = 0;
     L.sc_qt = 1;
-    L.sc_part_pairs = 0;
+    L.sc_part_pairs = L.sc_part_512 = 0;
     if (L.tuned && n_q <= ST_MAX_NQ) {
-        // more than 128 query rows per head: two work items per head, one per 128 rows
+        // more than 128 query rows per head: two query tiles, worked on by the same slots
         L.sc_qt = (n_q + 127) / 128;
-        const int hpc_real = hpc;
-        const int hpc = hpc_real * L.sc_qt;
-        // chunks of ST_TILES 128-key tiles, one per block and round; a head's team must fit in one round
-        long long blocks_wanted = 0;
+        // chunks of ST_CHUNK keys, dealt to the slots of the grid; a head's chunks wait for one another, so that there must be a
+        // slot for each of them
+        long long items = 0;
+        size_t pairs = 0;
+        int team_max = 1;
         for (int i = 0; i < n; ++i) {
             L.sc_team[i] = (caches[i].T + ST_CHUNK - 1) / ST_CHUNK;
-            blocks_wanted += (long long)hpc * L.sc_team[i];
+            if (L.sc_team[i] > team_max) team_max = L.sc_team[i];
+            L.sc_item_base[i] = (int)items;
+            items += (long long)hpc * L.sc_team[i];
+            L.sc_part_off[i] = pairs;
+            pairs += (size_t)hpc * L.sc_qt * L.sc_team[i] * 128;
+            L.sc_part_512 += (size_t)hpc * L.sc_qt * ((caches[i].T + 511) / 512) * 128;
         }
         const long long sms = sm_count();
-        L.sc_blocks = (int)(blocks_wanted < sms ? blocks_wanted : sms);
-        bool fits = true;
-        int rounds = 0;
-        size_t pairs = 0;
-        for (int i = 0; i < n; ++i) {
-            if (L.sc_team[i] > L.sc_blocks) { fits = false; break; }
-            L.sc_hpr[i] = L.sc_blocks / L.sc_team[i];
-            if (L.sc_hpr[i] > hpc) L.sc_hpr[i] = hpc;
-            L.sc_round_base[i] = rounds;
-            rounds += (hpc + L.sc_hpr[i] - 1) / L.sc_hpr[i];
-            L.sc_part_off[i] = pairs;
-            pairs += (size_t)hpc * L.sc_team[i] * 128;
-        }
-        L.sc_on = fits;
-        L.sc_rounds = rounds;
+        L.sc_blocks = (int)(items < sms ? items : sms);
+        L.sc_on = team_max <= ST_SLOTS * L.sc_blocks && items < (1ll << 30);
+        L.sc_items = (int)items;
         L.sc_part_pairs = pairs;
     }
     size_t o = 0;
-    // cleared before every call, in this order: the status word, the score kernel's chunk statistics and, where two query
-    // tiles add their masses up, the masses
+    // cleared before every call: the status word and the score kernel's chunk statistics
     L.off_status = o; o += 256;
     L.off_sc_part = o; if (L.sc_on) o = align_up(o + L.sc_part_pairs * 2 * sizeof(float), 256);
-    L.off_scores = o; L.clear_end = o;
-    o = align_up(o + tok * sizeof(float), 256);
-    if (L.sc_on && L.sc_qt == 2) L.clear_end = o;
+    L.clear_end = o;
+    L.off_scores = o; o = align_up(o + tok * sizeof(float), 256);
     L.off_keep = o;   o = align_up(o + tok, 256);
     L.sc_splits = score_splits(L.heads_total, n_q, T_max);
     if (L.sc_splits > key_splits) L.sc_splits = key_splits;
@@ -401,7 +394,7 @@ static obf_status_t launch_score_tc(const CallDev &cd, const Layout &L, cudaStre
     static thread_local TcMaps maps;
     const uint64_t hpc = (uint64_t)cd.heads_per_cache;
     for (int i = 0; i < cd.n_caches; ++i) {
-        obf_status_t s = encode_rows_map(&maps.a[i], cd.c[i].k, D, (uint64_t)cd.c[i].T, hpc, 128, D / 64);
+        obf_status_t s = encode_rows_map(&maps.a[i], cd.c[i].k, D, (uint64_t)cd.c[i].T, hpc, ST_CHUNK, D / 64);
         if (s != OBF_OK) return s;
         if ((s = encode_rows_map(&maps.b[i], cd.c[i].q, D, (uint64_t)cd.n_q, hpc, 128, D / 64)) != OBF_OK) return s;
         // the queries again, in boxes of 32 rows of one column block
@@ -670,8 +663,7 @@ static obf_status_t run(const obf_params_t *p, const obf_cache_t *caches, int32_
         c.nsub_del = L.tc_per ? L.nsub_del[i] : 0;
         c.sub_base = L.tc_per ? L.sub_base[i] : 0;
         c.sc_team = L.sc_on ? L.sc_team[i] : 0;
-        c.sc_hpr = L.sc_on ? L.sc_hpr[i] : 0;
-        c.sc_round_base = L.sc_on ? L.sc_round_base[i] : 0;
+        c.sc_item_base = L.sc_on ? L.sc_item_base[i] : 0;
         c.sc_part_off = L.sc_on ? L.sc_part_off[i] : 0;
         if (c.T > T_max) T_max = c.T;
         if (c.k_eff > k_max) k_max = c.k_eff;
@@ -689,7 +681,7 @@ static obf_status_t run(const obf_params_t *p, const obf_cache_t *caches, int32_
     cd.u_levels = L.tc_per ? U_LEVELS : 1;
     cd.tc_total_sub = L.tc_total_sub;
     cd.sc_qt = L.sc_on ? L.sc_qt : 1;
-    cd.sc_rounds = L.sc_rounds;
+    cd.sc_items = L.sc_items;
     cd.sc_splits = L.sc_splits;
     cd.eps = p->eps;
     char *ws = static_cast<char *>(workspace);
@@ -1118,13 +1110,18 @@ extern "C" obf_status_t evict_only_static(const obf_params_t *params, const obf_
     make_layout(params, caches, n_caches, 0, L, key_splits);
     while (L.total > (size_t)OBF_STATIC_SCRATCH_BYTES && L.sc_splits > 1) make_layout(params, caches, n_caches, 0, L, key_splits = L.sc_splits / 2);
     bool groups = false;
-    if (L.total > (size_t)OBF_STATIC_SCRATCH_BYTES && L.sc_on && params->head_dim == 64) {
-        // heads of 64 channels: the tensor-core kernel's chunk statistics, two bytes and more per position, do not count
-        obf_params_t pg = pe;
-        pg.flags |= OBF_FLAG_GENERIC_PATH;
-        Layout G;
-        make_layout(&pg, caches, n_caches, 0, G, 1);
-        groups = G.total <= (size_t)OBF_STATIC_SCRATCH_BYTES;
+    if (L.total > (size_t)OBF_STATIC_SCRATCH_BYTES && L.sc_on) {
+        // Shapes that the array always took stay accepted though the tensor-core kernel's statistics have grown: heads of 64 channels
+        // once had none, those of 128 channels one per 512 positions.
+        size_t need = L.total - (L.sc_part_pairs - L.sc_part_512) * 2 * sizeof(float);
+        if (params->head_dim == 64) {
+            obf_params_t pg = pe;
+            pg.flags |= OBF_FLAG_GENERIC_PATH;
+            Layout G;
+            make_layout(&pg, caches, n_caches, 0, G, 1);
+            need = G.total;
+        }
+        groups = need <= (size_t)OBF_STATIC_SCRATCH_BYTES;
     }
     if (!groups && L.total > (size_t)OBF_STATIC_SCRATCH_BYTES) {
         std::fprintf(stderr,
@@ -1135,8 +1132,7 @@ extern "C" obf_status_t evict_only_static(const obf_params_t *params, const obf_
     }
     void *scratch = nullptr;
     if ((s = static_scratch_ptr(&scratch)) != OBF_OK) return s;
-    // run() clears the status word at the head of the scratch, the tuned score kernel's chunk statistics and, where two query
-    // tiles add theirs up, the masses; every other region is written by an earlier kernel of the same call before a later one
+    // run() clears the status word at the head of the scratch and the tuned score kernel's chunk statistics; every other region is written by an earlier kernel of the same call before a later one
     // reads it.
     if (groups) {
         if ((s = run_in_groups(params, caches, n_caches, scratch, stream)) != OBF_ERR_WORKSPACE) return s;

@@ -1227,3 +1227,34 @@ def test_a_call_that_fails_halfway_leaves_no_work_unjoined():
     del graph
     ok = par.run_gpu(warm, [synth.gen_cache(warm, 0)])                    # the next call is accepted
     assert ok[2] & 0xFF == 0
+
+
+@pytest.mark.parametrize("d,G,n_obs,caches", [
+    (128, 1, 1, ((128, 9), (256, 9), (257, 9), (385, 9))),          # one query, whole and barely begun chunks of 256 keys and halves
+    (128, 2, 16, ((129, 9), (160, 9), (1025, 9))),                  # 32 queries: four copies, a piece of 32 keys with one key
+    (128, 3, 11, ((255, 9), (300, 9))),                             # 33: two copies
+    (64, 8, 8, ((383, 9), (512, 9))),                               # 64
+    (64, 5, 13, ((287, 9),)),                                       # 65: one copy, an odd number of queries
+    (128, 8, 16, ((4100, 9), (140, 9))),                            # 128, more than sixteen chunks of a head
+    (64, 3, 43, ((200, 9), (4400, 9))),                             # 129: a second tile of one query
+    (128, 8, 32, ((8500, 9),)),                                     # 256, chunks fetched in two sweeps
+])
+def test_score_kernel_at_the_edges_of_its_chunks_pieces_and_copies(d, G, n_obs, caches):
+    # masses, positions and outputs against the oracle (run_and_check: 2e-7 + 1e-5 of the mass, fp32 sums and exponentials)
+    w = small("chunks", layers=1, kv_heads=3, G=G, n_obs=n_obs, d=d, dtype="bf16", rank=1, caches=caches, n_outlier=3, n_sink=4,
+              heavy=5, seed=900 + G * n_obs)
+    a, _, _ = run_and_check(w)
+    assert "k_score_tc" in [n for n, _ in P.obf_compress_profiled(par.params_for(w), a[0]["cache_structs"], a[0]["workspace"])]
+
+
+def test_masses_of_a_head_do_not_depend_on_the_rest_of_the_call():
+    # chunks are dealt over the whole call: the order in which a row's statistics are added is the head's alone
+    g = torch.Generator(device="cuda").manual_seed(3)
+    K, V, Q = (torch.randn((5, 4, rows, 128), generator=g, device="cuda", dtype=torch.bfloat16) for rows in (2900, 2900, 40))
+    params = P.make_params(5, 4, 4, 128, 40, 0, P.OBF_BF16)
+    whole = P.compress_caches(params, [dict(K=K, V=V, Q=Q, budget=30)], evict=True, want_scores=True)[0]
+    for l in range(5):
+        one = [x[l:l + 1].contiguous() for x in (K, V, Q)]
+        part = P.compress_caches(P.make_params(1, 4, 4, 128, 40, 0, P.OBF_BF16), [dict(K=one[0], V=one[1], Q=one[2], budget=30)],
+                                 evict=True, want_scores=True)[0]
+        assert torch.equal(part["scores"][0], whole["scores"][l]) and torch.equal(part["idx"][0], whole["idx"][l])

@@ -124,3 +124,26 @@ def test_static_scratch_takes_heads_of_64_channels_in_groups(layers, kv_heads, T
     for o, r in zip(outs, ref):
         for n in o:
             assert torch.equal(o[n], r[n]), n
+
+
+@pytest.mark.parametrize("layers,kv_heads,Ts,flags", [(9, 8, (16000,), 0), (9, 8, (9000, 7000), binding.OBF_FLAG_SINK(4)),
+                                                      (9, 8, (14500,), binding.OBF_FLAG_LAYERWISE)])
+def test_static_scratch_takes_heads_of_128_channels_in_groups(layers, kv_heads, Ts, flags):
+    # seven bytes a position fit the array (masses, flags and statistics per 512 positions), nine (per 256) do not
+    g = torch.Generator(device="cuda").manual_seed(8)
+    dev = [{n: torch.randn((layers, kv_heads, rows, 128), generator=g, device="cuda", dtype=torch.bfloat16)
+            for n, rows in (("K", T), ("V", T), ("Q", 5))} for T in Ts]
+    params = P.make_params(layers, kv_heads, kv_heads, 128, 5, 0, P.OBF_BF16, flags=flags)
+    ref = P.compress_caches(params, [dict(x, budget=70) for x in dev], evict=True, want_scores=True)
+    assert P.obf_workspace_bytes(params, ref[0]["cache_structs"]) > binding.OBF_STATIC_SCRATCH_BYTES
+    outs, cs = [], []
+    for x, r, T in zip(dev, ref, Ts):
+        o = {n: torch.zeros_like(r[n]) for n in ("K_out", "V_out", "idx", "scores")}
+        outs.append(o)
+        cs.append(P.make_cache(x["K"], x["V"], x["Q"], T, 70, o["K_out"], o["V_out"], o["idx"], None, o["scores"]))
+    P.evict_only_static(params, cs)
+    torch.cuda.synchronize()
+    assert P.obf_static_scratch_status() & 0xFF == 0
+    for o, r in zip(outs, ref):
+        for n in o:
+            assert torch.equal(o[n], r[n]), n
