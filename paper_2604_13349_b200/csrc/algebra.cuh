@@ -350,6 +350,145 @@ static_assert(ALG_SMEM_MAX<128> >= algebra_smem_bytes<128>(128, 128, 1) && ALG_S
               ALG_SMEM_MAX<64> >= algebra_smem_bytes<64>(64, 64, 1) && ALG_SMEM_MAX<64> >= algebra_smem_bytes<64>(64, ALG_TRI_MAX_RANK, 0), "no route needs more");
 static_assert(ALG_SMEM_MAX<128> <= 227 * 1024 - 1024, "a block has 227 KB, some of it static");
 
+// 2. Reflectors of a head's k retained rows (Eq. 2), into Y (shared memory): how many there are.  A loop of its own and not one with
+// that over G: together their code outgrows what a multiprocessor fetches at full speed.
+template <typename TIN, int D>
+__device__ __forceinline__ int alg_reflectors(const TIN *vk, int k, float *Y, int *s_flag)
+{
+    constexpr int NQ = AlgShape<D>::NQ;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, grp = tid >> 4, c16 = tid & 15;
+    int m = 0;
+    // a batch of rows in registers (G comes afterwards): row b0 + grp + ALG_NG s in slot s of the half-warp
+    constexpr int NS = ALG_BATCH / ALG_NG;
+    static_assert(NS == 4, "four slots to pick from");
+    AlgRow<D> V[NS];
+    float n0[NS];                                              // the rows' squared norms
+    auto reflect_rows = [&](const AlgRow<D> &v) __attribute__((always_inline)) {
+        float d4[NS];
+#pragma unroll
+        for (int s = 0; s < NS; ++s) d4[s] = alg_dot<D>(V[s], v);
+        const float tot = -2.f * transposed_sum<NS, 16>(d4, c16);
+#pragma unroll
+        for (int s = 0; s < NS; ++s) {
+            const float f = __shfl_sync(0xffffffffu, tot, (lane & 16) + (16 / NS) * s);
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) V[s][q] = fma2(pk(f, f), v[q], V[s][q]);
+        }
+    };
+    // whether row i of the batch adds a direction to the m there are, and its reflector
+    auto candidate = [&](int i) __attribute__((always_inline)) {
+        if (warp != (i % ALG_NG) / 2) return;
+        AlgRow<D> x;
+        float nn = n0[0];
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) x[q] = V[0][q];
+        auto pick = [&](auto slot) __attribute__((always_inline)) {
+            constexpr int s = decltype(slot)::value;
+            if (i / ALG_NG == s) {
+                nn = n0[s];
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) {
+                    x[q] = V[s][q];
+                    // (keeps the compiler from merging the slots' code into one that addresses the array)
+                    asm volatile("// %1" : "+l"(x[q]) : "n"(s));
+                }
+            }
+        };
+        pick(std::integral_constant<int, 1>{});
+        pick(std::integral_constant<int, 2>{});
+        pick(std::integral_constant<int, 3>{});
+        const float t2 = alg_tail2<D>(x, m, c16), x0 = alg_entry<D>(x, m < D ? m : 0, lane);
+        const float nrm = t2 * rsqrt_approx(fmaxf(t2, 1e-37f));
+        if (grp == i % ALG_NG) {
+            const bool add = m < D && t2 > SPAN_ROW_TOL * SPAN_ROW_TOL * nn && t2 > 1e-37f;
+            if (add) {
+                const float al = x0 >= 0.f ? -nrm : nrm;
+                alg_store_reflector<D>(x, m, x0 - al, rsqrt_approx(2.f * fmaf(nrm, fabsf(x0), t2)), Y + m * D, c16);
+            }
+            if (c16 == 0) s_flag[i & 1] = add ? 1 : 0;
+        }
+    };
+#pragma unroll 1
+    for (int b0 = 0; b0 < k && m < D; b0 += ALG_BATCH) {
+#pragma unroll
+        for (int s = 0; s < NS; ++s) {
+            const int i = b0 + grp + ALG_NG * s;
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) {
+                V[s][q] = 0ull;
+                if (i < k) {
+                    const TIN *src = vk + (size_t)i * D + 32 * q + 2 * c16;
+                    if constexpr (sizeof(TIN) == 4) V[s][q] = *reinterpret_cast<const f32x2 *>(src);
+                    else {
+                        const uint32_t w = *reinterpret_cast<const uint32_t *>(src);
+                        V[s][q] = pk(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u));
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int s = 0; s < NS; ++s) {
+            n0[s] = half_sum(alg_dot<D>(V[s], V[s]));
+            // a reflector depends on its row's direction alone: rows whose squares leave the range of fp32's normal numbers
+            // are brought back by a power of two
+            const bool far = n0[s] > 0.f && !(n0[s] > 1e-24f && n0[s] < 1e24f);
+            if (__any_sync(0xffffffffu, far)) {                // (the sum below takes the whole warp)
+                const float f = !far ? 1.f : n0[s] < 1.f ? 1.8446744e19f : 5.421011e-20f;   // 2^64, 2^-64
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) V[s][q] = mul2(V[s][q], pk(f, f));
+                n0[s] = half_sum(alg_dot<D>(V[s], V[s]));
+            }
+        }
+        // (the reflectors that earlier batches found, all published behind a barrier)
+#pragma unroll 1
+        for (int j = 0; j < m; ++j) {
+            AlgRow<D> v;
+            alg_load<D>(v, Y + j * D, c16);
+            reflect_rows(v);
+        }
+        const int rows = min(ALG_BATCH, k - b0);
+        candidate(0);
+#pragma unroll 1
+        for (int i = 0; i < rows; ++i) {
+            __syncthreads();
+            if (s_flag[i & 1]) {                               // row i has a reflector
+                AlgRow<D> v;
+                alg_load<D>(v, Y + m * D, c16);
+                reflect_rows(v);
+                if (++m >= D) break;
+                if (i + 1 < rows) candidate(i + 1);
+            } else if (i + 1 < rows) {
+                candidate(i + 1);
+            }
+        }
+        // the flag is written again by the next batch
+        __syncthreads();
+    }
+    return m;
+}
+
+// The reflectors of every head's retained rows, beside the pass over V where that waits for the selection (bf16 heads of 64 channels)
+// and no budget reaches head_dim.  16 x 8 heads of 64 channels, 32 of 3001 rows: 126 -> 120 us a call.  Heads of 128 channels find
+// theirs in k_obf_algebra: two of them share a multiprocessor there and hide it, and their call got slower (36 x 8 heads, 1024
+// positions: 229 -> 233).
+template <typename TIN, int D>
+__global__ void __launch_bounds__(ALG_NT) k_obf_rows(const __grid_constant__ CallDev p)
+{
+    pdl_wait();
+    extern __shared__ __align__(16) float sm[];
+    __shared__ int s_flag[2];
+    const int g = blockIdx.x;
+    int ci, lh;
+    locate(p, g, ci, lh);
+    const CacheDev &c = p.c[ci];
+    const int k = c.k_eff;
+    if (c.T <= k) return;
+    const int m = alg_reflectors<TIN, D>(reinterpret_cast<const TIN *>(c.v_out) + (size_t)lh * k * D, k, sm, s_flag);
+    float4 *dst = reinterpret_cast<float4 *>(p.rows_y + (size_t)g * p.alg_rows * D);
+    for (int e = threadIdx.x; e < m * (D / 4); e += ALG_NT) dst[e] = reinterpret_cast<const float4 *>(sm)[e];
+    if (threadIdx.x == 0) p.rows_m[g] = m;
+}
+
 template <typename TIN, int D>
 __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant__ CallDev p)
 {
@@ -471,116 +610,14 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
 #pragma unroll
             for (int q = 0; q < NQ; ++q) x[q] = fma2(pk(s, s), v[q], x[q]);
         };
-        // ---- 2. reflectors of the retained rows (Eq. 2).  Two loops, this one and that over G: together their code outgrows
-        // what a multiprocessor fetches at full speed ----
-        {
-            // a batch of rows in registers (G comes afterwards): row b0 + grp + ALG_NG s in slot s of the half-warp
-            constexpr int NS = ALG_BATCH / ALG_NG;
-            static_assert(NS == 4, "four slots to pick from");
-            AlgRow<D> V[NS];
-            float n0[NS];                                              // the rows' squared norms
-            auto reflect_rows = [&](const AlgRow<D> &v) __attribute__((always_inline)) {
-                float d4[NS];
-#pragma unroll
-                for (int s = 0; s < NS; ++s) d4[s] = alg_dot<D>(V[s], v);
-                const float tot = -2.f * transposed_sum<NS, 16>(d4, c16);
-#pragma unroll
-                for (int s = 0; s < NS; ++s) {
-                    const float f = __shfl_sync(0xffffffffu, tot, (lane & 16) + (16 / NS) * s);
-#pragma unroll
-                    for (int q = 0; q < NQ; ++q) V[s][q] = fma2(pk(f, f), v[q], V[s][q]);
-                }
-            };
-            // whether row i of the batch adds a direction to the m there are, and its reflector
-            auto candidate = [&](int i) __attribute__((always_inline)) {
-                if (warp != (i % ALG_NG) / 2) return;
-                AlgRow<D> x;
-                float nn = n0[0];
-#pragma unroll
-                for (int q = 0; q < NQ; ++q) x[q] = V[0][q];
-                auto pick = [&](auto slot) __attribute__((always_inline)) {
-                    constexpr int s = decltype(slot)::value;
-                    if (i / ALG_NG == s) {
-                        nn = n0[s];
-#pragma unroll
-                        for (int q = 0; q < NQ; ++q) {
-                            x[q] = V[s][q];
-                            // (keeps the compiler from merging the slots' code into one that addresses the array)
-                            asm volatile("// %1" : "+l"(x[q]) : "n"(s));
-                        }
-                    }
-                };
-                pick(std::integral_constant<int, 1>{});
-                pick(std::integral_constant<int, 2>{});
-                pick(std::integral_constant<int, 3>{});
-                const float t2 = alg_tail2<D>(x, m, c16), x0 = alg_entry<D>(x, m < D ? m : 0, lane);
-                const float nrm = t2 * rsqrt_approx(fmaxf(t2, 1e-37f));
-                if (grp == i % ALG_NG) {
-                    const bool add = m < D && t2 > SPAN_ROW_TOL * SPAN_ROW_TOL * nn && t2 > 1e-37f;
-                    if (add) {
-                        const float al = x0 >= 0.f ? -nrm : nrm;
-                        alg_store_reflector<D>(x, m, x0 - al, rsqrt_approx(2.f * fmaf(nrm, fabsf(x0), t2)), Y + m * D, c16);
-                    }
-                    if (c16 == 0) s_flag[i & 1] = add ? 1 : 0;
-                }
-            };
-#pragma unroll 1
-            for (int b0 = 0; b0 < k && m < D; b0 += ALG_BATCH) {
-#pragma unroll
-                for (int s = 0; s < NS; ++s) {
-                    const int i = b0 + grp + ALG_NG * s;
-#pragma unroll
-                    for (int q = 0; q < NQ; ++q) {
-                        V[s][q] = 0ull;
-                        if (i < k) {
-                            const TIN *src = vk + (size_t)i * D + 32 * q + 2 * c16;
-                            if constexpr (sizeof(TIN) == 4) V[s][q] = *reinterpret_cast<const f32x2 *>(src);
-                            else {
-                                const uint32_t w = *reinterpret_cast<const uint32_t *>(src);
-                                V[s][q] = pk(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u));
-                            }
-                        }
-                    }
-                }
-#pragma unroll
-                for (int s = 0; s < NS; ++s) {
-                    n0[s] = half_sum(alg_dot<D>(V[s], V[s]));
-                    // a reflector depends on its row's direction alone: rows whose squares leave the range of fp32's normal numbers
-                    // are brought back by a power of two
-                    const bool far = n0[s] > 0.f && !(n0[s] > 1e-24f && n0[s] < 1e24f);
-                    if (__any_sync(0xffffffffu, far)) {                // (the sum below takes the whole warp)
-                        const float f = !far ? 1.f : n0[s] < 1.f ? 1.8446744e19f : 5.421011e-20f;   // 2^64, 2^-64
-#pragma unroll
-                        for (int q = 0; q < NQ; ++q) V[s][q] = mul2(V[s][q], pk(f, f));
-                        n0[s] = half_sum(alg_dot<D>(V[s], V[s]));
-                    }
-                }
-                // (the reflectors that earlier batches found, all published behind a barrier)
-#pragma unroll 1
-                for (int j = 0; j < m; ++j) {
-                    AlgRow<D> v;
-                    alg_load<D>(v, Y + j * D, c16);
-                    reflect_rows(v);
-                }
-                const int rows = min(ALG_BATCH, k - b0);
-                candidate(0);
-#pragma unroll 1
-                for (int i = 0; i < rows; ++i) {
-                    __syncthreads();
-                    if (s_flag[i & 1]) {                               // row i has a reflector
-                        AlgRow<D> v;
-                        alg_load<D>(v, Y + m * D, c16);
-                        reflect_rows(v);
-                        if (++m >= D) break;
-                        if (i + 1 < rows) candidate(i + 1);
-                        reflect(aux, v);
-                    } else if (i + 1 < rows) {
-                        candidate(i + 1);
-                    }
-                }
-                // the flag is written again by the next batch
-                __syncthreads();
-            }
+        // ---- 2. reflectors of the retained rows, unless k_obf_rows has found them ----
+        if (p.rows_y) {
+            m = p.rows_m[g];
+            const float4 *src = reinterpret_cast<const float4 *>(p.rows_y + (size_t)g * p.alg_rows * D);
+            for (int e = tid; e < m * (D / 4); e += ALG_NT) reinterpret_cast<float4 *>(Y)[e] = src[e];
+            __syncthreads();
+        } else {
+            m = alg_reflectors<TIN, D>(vk, k, Y, s_flag);
         }
         // ---- G into registers, its trace, and the reflectors applied to it from both sides -----------------------
         AlgMat<D> M;
@@ -628,6 +665,11 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                     AlgRow<D> v, x;
                     alg_load<D, ST>(v, Y + j * D, c16);
                     alg_product<D, ST>(M, v, Y + j * D, po, kp, grp, c16);
+                    {
+                        const float s = -2.f * half_sum(alg_dot<D, ST>(aux, v));
+#pragma unroll
+                        for (int q = ST; q < NQ; ++q) aux[q] = fma2(pk(s, s), v[q], aux[q]);
+                    }
                     __syncthreads();                                   // p is there
                     alg_update<D, ST>(M, v, Y + j * D, po, kp, grp, c16, 0, x);
                 }

@@ -89,6 +89,8 @@ struct CallDev {
     float *delta;             // [heads_total, d]
     float *svec;              // [heads_total, d] sum of the deleted value rows (only filled when diagnostics are asked for)
     uint32_t *hflag;          // [heads_total] HFLAG_*
+    float *rows_y;            // [heads_total, alg_rows, d] reflectors of the retained rows (k_obf_rows), or null: the dense algebra finds them itself
+    int32_t *rows_m;          // [heads_total] how many
 };
 
 // Waits until the stream's kernel before this one is over and its writes are visible (see launch() in obf_api.cu).

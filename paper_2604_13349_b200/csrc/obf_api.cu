@@ -84,7 +84,8 @@ static inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; 
 
 struct Layout {
     size_t off_status, off_scores, off_keep, off_stats, off_sums, off_lscores, clear_end;
-    size_t off_gram_d, off_gram_k, off_uvec, off_delta, off_hflag, off_svec, off_assign;
+    size_t off_gram_d, off_gram_k, off_uvec, off_delta, off_hflag, off_svec, off_assign, off_rows_y, off_rows_m;
+    bool rows;                      // the retained rows' reflectors come from a kernel of their own
     size_t total;
     int splits, sc_splits;
     int heads_total;
@@ -265,6 +266,7 @@ static void make_layout(const obf_params_t *p, const obf_cache_t *caches, int32_
     L.off_sums = o;   o = align_up(o + (size_t)L.heads_total * 4 * sizeof(float), 256);
     L.off_lscores = o;
     if (p->flags & OBF_FLAG_LAYERWISE) o = align_up(o + tok / p->kv_heads * sizeof(float), 256);
+    L.rows = false;
     L.off_gram_d = L.off_gram_k = L.off_uvec = L.off_delta = L.off_hflag = L.off_svec = o;
     if (rank > 0) {
         const size_t gsz = (size_t)L.heads_total * L.gram_slots * d * d * sizeof(float);
@@ -274,6 +276,13 @@ static void make_layout(const obf_params_t *p, const obf_cache_t *caches, int32_
         L.off_delta = o;  o = align_up(o + (size_t)L.heads_total * d * sizeof(float), 256);
         L.off_hflag = o;  o = align_up(o + (size_t)L.heads_total * sizeof(uint32_t), 256);
         L.off_svec = o;   o = align_up(o + (size_t)L.heads_total * d * sizeof(float), 256);
+        int k_max = 1;
+        for (int i = 0; i < n; ++i) k_max = k_eff_of(p, caches[i]) > k_max ? k_eff_of(p, caches[i]) : k_max;
+        L.rows = L.tc_per && d == 64 && GramShape<64>::DELETED && k_max < d;
+        if (L.rows) {
+            L.off_rows_y = o; o = align_up(o + (size_t)L.heads_total * k_max * d * sizeof(float), 256);
+            L.off_rows_m = o; o = align_up(o + (size_t)L.heads_total * sizeof(int32_t), 256);
+        }
     }
     L.off_assign = o;
     if (p->flags & OBF_FLAG_MERGE) o = align_up(o + tok * sizeof(int32_t), 256);
@@ -496,16 +505,26 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
     }
     mark(sel, "k_select");
     if (side && FORK_LATE) {
-        if (gather_vecs) {
+        if (gather_vecs && !L.rows) {
             side = nullptr;                                            // nothing to run beside the pass
         } else {
             OBF_TRY(fork_and_pass());
             sel = side->stream;
         }
     }
+    auto launch_rows = [&](cudaStream_t on) -> obf_status_t {
+        if (!L.rows) return OBF_OK;
+        OBF_TRY(set_smem(k_obf_rows<TIN, D>, (size_t)D * D * sizeof(float)));
+        OBF_TRY(launch(k_obf_rows<TIN, D>, dim3(heads), ALG_NT, (size_t)cd.alg_rows * D * sizeof(float), on, cd));
+        mark(on, "k_obf_rows");
+        return OBF_OK;
+    };
     dim3 g4((k_max + GATHER_ROWS - 1) / GATHER_ROWS, heads);
     if (gather_vecs) {
-        OBF_TRY(side_work.join());
+        if (side) {
+            OBF_TRY(launch_rows(sel));
+            OBF_TRY(side_work.join());
+        }
     } else if (side) {
         // the values first: the rest of the call needs them
         OBF_TRY(launch(k_gather<TIN, D, 1>, dim3(g4), 256, 0, sel, cd));
@@ -519,6 +538,7 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
             OBF_TRY(launch(k_span_test<D, true>, dim3(heads), ST_NT, sm_span, sel, cd));
             mark(sel, "k_span_test");
         }
+        OBF_TRY(launch_rows(sel));
         // the keys are needed by nothing that follows: they are copied on the caller's stream once the pass over V
         // is over (it is bound by HBM), while the span test finishes on the side stream
         OBF_CUDA_TRY(cudaStreamWaitEvent(st, side->rows_done, 0));
@@ -542,7 +562,10 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
                     mark(st, "k_span_test");
                 }
             }
-            if (!side && (s = launch_gram_tc<D>(cd, L, st)) != OBF_OK) return s;
+            if (!side) {
+                OBF_TRY(launch_rows(st));
+                OBF_TRY(launch_gram_tc<D>(cd, L, st));
+            }
         } else {
             dim3 g5(cd.splits, heads);
             OBF_TRY(launch(k_gram<TIN, D>, dim3(g5), 256, 0, st, cd));
@@ -711,6 +734,10 @@ static obf_status_t run(const obf_params_t *p, const obf_cache_t *caches, int32_
     cd.delta = reinterpret_cast<float *>(ws + L.off_delta);
     cd.hflag = reinterpret_cast<uint32_t *>(ws + L.off_hflag);
     cd.svec = reinterpret_cast<float *>(ws + L.off_svec);
+    if (L.rows) {
+        cd.rows_y = reinterpret_cast<float *>(ws + L.off_rows_y);
+        cd.rows_m = reinterpret_cast<int32_t *>(ws + L.off_rows_m);
+    }
     cd.assign = reinterpret_cast<int32_t *>(ws + L.off_assign);
     cd.merge = (p->flags & OBF_FLAG_MERGE) ? 1 : 0;
 

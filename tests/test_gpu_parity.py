@@ -1258,3 +1258,14 @@ def test_masses_of_a_head_do_not_depend_on_the_rest_of_the_call():
         part = P.compress_caches(P.make_params(1, 4, 4, 128, 40, 0, P.OBF_BF16), [dict(K=one[0], V=one[1], Q=one[2], budget=30)],
                                  evict=True, want_scores=True)[0]
         assert torch.equal(part["scores"][0], whole["scores"][l]) and torch.equal(part["idx"][0], whole["idx"][l])
+
+
+@pytest.mark.parametrize("caches", [((300, 1), (200, 31)), ((700, 32), (161, 33)), ((400, 63),), ((130, 130), (500, 40))])
+@pytest.mark.parametrize("rank", [2, 9])
+def test_reflectors_found_beside_the_pass_over_values(caches, rank):
+    # bf16 heads of 64 channels, every budget below 64 (but in the last case, whose first cache is kept whole): batches of 32 rows
+    # with remainders, the tridiagonal and the Jacobi route of the dense algebra behind them
+    w = small("rows", layers=2, kv_heads=3, G=4, n_obs=4, d=64, dtype="bf16", rank=rank, caches=caches, seed=61 + rank)
+    a, _, _ = run_and_check(w)
+    names = [n for n, _ in P.obf_compress_profiled(par.params_for(w), a[0]["cache_structs"], a[0]["workspace"])]
+    assert ("k_obf_rows" in names) == all(min(b, T) < 64 for T, b in caches)
