@@ -405,9 +405,11 @@ static obf_status_t launch_score_tc(const CallDev &cd, const Layout &L, cudaStre
     for (int i = 0; i < cd.n_caches; ++i) {
         obf_status_t s = encode_rows_map(&maps.a[i], cd.c[i].k, D, (uint64_t)cd.c[i].T, hpc, ST_CHUNK, D / 64);
         if (s != OBF_OK) return s;
-        if ((s = encode_rows_map(&maps.b[i], cd.c[i].q, D, (uint64_t)cd.n_q, hpc, 128, D / 64)) != OBF_OK) return s;
-        // the queries again, in boxes of 32 rows of one column block
-        if (cd.n_caches <= ST_PART_MAP && (s = encode_rows_map(&maps.b[ST_PART_MAP + i], cd.c[i].q, D, (uint64_t)cd.n_q, hpc, 32, 1)) != OBF_OK) return s;
+        // the queries of a tile at once and, for copies of them, in boxes of 32 rows of one column block (above ST_PART_MAP caches
+        // the boxes only)
+        const bool many = cd.n_caches > ST_PART_MAP;
+        if (!many && (s = encode_rows_map(&maps.b[i], cd.c[i].q, D, (uint64_t)cd.n_q, hpc, 128, D / 64)) != OBF_OK) return s;
+        if ((s = encode_rows_map(&maps.b[many ? i : ST_PART_MAP + i], cd.c[i].q, D, (uint64_t)cd.n_q, hpc, 32, 1)) != OBF_OK) return s;
     }
     const size_t smem = score_tc_smem_bytes<D>();
     OBF_CUDA_TRY(cudaFuncSetAttribute(k_score_tc<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));

@@ -54,8 +54,10 @@ constexpr size_t score_tc_smem_bytes()
 
 // An item with up to 32 (64) queries, the second one of a head with 160 for instance, would leave three (two) schedulers of
 // four without work, as a group's warps own 32 rows of its operand each: the item's queries are loaded
-// four times (twice), and the copies share the columns of a tile.  The tensor maps for that sit behind those of the first
-// ST_PART_MAP caches (a third array of maps made every launch 1 to 2 us slower); calls with more caches go without.
+// four times (twice), and the copies share the columns of a tile.  The tensor maps for that, of boxes of 32 rows and one column
+// block, sit behind those of the first ST_PART_MAP caches (a third array of maps made every launch 1 to 2 us slower).  Calls with
+// more caches have these maps only and load all their queries through them: a head's copies, and with them the order in which
+// its statistics are added, never depend on how many caches a call has.
 constexpr int ST_PART_MAP = OBF_MAX_CACHES / 2;
 
 struct ScoreItem {
@@ -84,7 +86,7 @@ __device__ __forceinline__ void score_item(const CallDev &p, const ScoreTab *tab
     it.chunk = rel - it.lh * c.team;
     it.keys = min(ST_CHUNK, c.T - it.chunk * ST_CHUNK);
     it.nq = min(128, p.n_q - 128 * qt);
-    it.copies = p.n_caches > ST_PART_MAP || it.nq > 64 ? 1 : it.nq > 32 ? 2 : 4;
+    it.copies = it.nq > 64 ? 1 : it.nq > 32 ? 2 : 4;
 }
 
 __device__ __forceinline__ float ex2_approx(float x)
@@ -258,10 +260,11 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constan
             auto load = [&](const ScoreItem &it, int qt, bool keys) {
                 tc::mbar_expect_tx(full, Q_BYTES + (keys ? K_BYTES : 0));
                 if (keys) tc::tma_load_rows(k_addr, &tm.a[it.cache], full, it.chunk * ST_CHUNK, it.lh);
-                if (it.copies > 1) {
+                if (it.copies > 1 || p.n_caches > ST_PART_MAP) {
+                    const CUtensorMap *boxes = &tm.b[(p.n_caches > ST_PART_MAP ? 0 : ST_PART_MAP) + it.cache];
                     for (int r = 0; r < 4; ++r)
                         for (int b = 0; b < D / 64; ++b)
-                            tc::tma_load_block(q_addr + r * 32 * 128 + b * ST_BOX_BYTES, &tm.b[ST_PART_MAP + it.cache], full,
+                            tc::tma_load_block(q_addr + r * 32 * 128 + b * ST_BOX_BYTES, boxes, full,
                                                qt * 128 + 32 * (r % (4 / it.copies)), b, it.lh);
                 } else {
                     tc::tma_load_rows(q_addr, &tm.b[it.cache], full, qt * 128, it.lh);          // rows past n_q read as zero

@@ -1269,3 +1269,16 @@ def test_reflectors_found_beside_the_pass_over_values(caches, rank):
     a, _, _ = run_and_check(w)
     names = [n for n, _ in P.obf_compress_profiled(par.params_for(w), a[0]["cache_structs"], a[0]["workspace"])]
     assert ("k_obf_rows" in names) == all(min(b, T) < 64 for T, b in caches)
+
+
+@pytest.mark.parametrize("G,n_obs,d", [(1, 20, 128), (2, 25, 64), (4, 25, 128), (3, 50, 64)])      # four copies, two, one, a second tile
+def test_masses_of_a_head_do_not_depend_on_the_number_of_caches(G, n_obs, d):
+    # seventeen caches: more than the score kernel has two tensor maps of the queries for
+    caches = tuple((129 + 71 * i, 9) for i in range(17))
+    w = small("many", layers=1, kv_heads=2, G=G, n_obs=n_obs, d=d, dtype="bf16", rank=1, caches=caches, heavy=5, seed=300 + n_obs)
+    a, _, arrays = run_and_check(w)
+    for ci in range(17):
+        one = dataclasses.replace(w, caches=(w.caches[ci],))
+        b, _, st = par.run_gpu(one, [arrays[ci]])
+        assert st & 0xFF == 0
+        assert torch.equal(a[ci]["scores"], b[0]["scores"]) and torch.equal(a[ci]["idx"], b[0]["idx"]), ci
