@@ -63,6 +63,7 @@ struct CallDev {
     int32_t alg_rows;         // dense algebra: basis rows any head of the call can have, min(largest k_eff, d)
     int32_t sc_items;         // (head, chunk) pairs of the persistent score kernel
     int32_t sc_qt;            // tuned score kernel: 128-row query tiles per head (1 or 2)
+    int32_t sc_single;        // and whether every one of them has too many queries for copies (score_tc.cuh)
     float *sc_part;           // per (head, query tile, chunk, query of 128): chunk reference and normaliser as one 64-bit word, zero until published
     int32_t sc_splits;        // shape-generic statistics kernel: key splits per (head, 64 queries)
     float eps;

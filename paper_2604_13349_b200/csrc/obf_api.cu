@@ -707,6 +707,7 @@ static obf_status_t run(const obf_params_t *p, const obf_cache_t *caches, int32_
     cd.tc_total_sub = L.tc_total_sub;
     cd.sc_qt = L.sc_on ? L.sc_qt : 1;
     cd.sc_items = L.sc_items;
+    cd.sc_single = cd.n_q - 128 * (cd.sc_qt - 1) > 64 ? 1 : 0;
     cd.sc_splits = L.sc_splits;
     cd.eps = p->eps;
     char *ws = static_cast<char *>(workspace);

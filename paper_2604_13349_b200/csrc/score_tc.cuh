@@ -86,7 +86,9 @@ __device__ __forceinline__ void score_item(const CallDev &p, const ScoreTab *tab
     it.chunk = rel - it.lh * c.team;
     it.keys = min(ST_CHUNK, c.T - it.chunk * ST_CHUNK);
     it.nq = min(128, p.n_q - 128 * qt);
-    it.copies = it.nq > 64 ? 1 : it.nq > 32 ? 2 : 4;
+    // (the first term says no more than the second, but for the whole call: without it the consumers' code came out 1 to 3 % slower,
+    // 36 x 8 heads of 4096 positions, 128 queries: 133.3 -> 136.7 us, 256 queries: 240 -> 247)
+    it.copies = p.sc_single || it.nq > 64 ? 1 : it.nq > 32 ? 2 : 4;
 }
 
 __device__ __forceinline__ float ex2_approx(float x)
