@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(GT_THREADS, 3) k_gram_tc(const __grid_constant
             // nothing this thread started may still be in flight when the block exits
             const uint32_t issued = it;
             for (uint32_t j = issued > (uint32_t)GT_STAGES ? issued - GT_STAGES : 0u; j < issued; ++j)
-                tc::mbar_wait(&bar_full[j % GT_STAGES], (j / GT_STAGES) & 1u, wc);
+                tc::mbar_drain(&bar_full[j % GT_STAGES], (j / GT_STAGES) & 1u, wc);
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
@@ -190,6 +190,9 @@ __global__ void __launch_bounds__(GT_THREADS, 3) k_gram_tc(const __grid_constant
                 ++seg;
                 if (s_abort) break;
             }
+            // nor may an instruction (a stage is handed back when its tile's are done)
+            for (uint32_t j = it > (uint32_t)GT_STAGES ? it - GT_STAGES : 0u; j < it; ++j)
+                tc::mbar_drain(&bar_empty[j % GT_STAGES], (j / GT_STAGES) & 1u, wc);
         }
     } else if (warp < 6) {
         // ---------------- masses: three bf16 columns per level and tile ----------------

@@ -273,7 +273,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constan
                 }
             };
             int n = slot * (int)gridDim.x + (int)blockIdx.x, qt = 0;
-            uint32_t u = 0, used[2] = {0u, 0u};                    // items of this slot so far, and of them those with keys in a half
+            uint32_t u = 0, used[2] = {0u, 0u};                    // items of this slot so far, and the tiles handed to the tensor cores
             ScoreItem item;
             bool have = n < n_items;
             if (have) {
@@ -299,6 +299,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constan
                         tc::umma_bf16(tmem + g * ST_HALF, dq + (uint64_t)((kk >> 2) * (ST_BOX_BYTES >> 4) + (kk & 3) * 2),
                                       dk + (uint64_t)((kk >> 2) * (ST_CHUNK * 128 >> 4) + (kk & 3) * 2), idesc, kk > 0 ? 1u : 0u);
                     tc::umma_commit(&bar_t_full[g]);
+                    ++used[h];
                 }
                 if (dead) break;
                 // the next item's operands once the instructions have read this one's
@@ -311,13 +312,15 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constan
                 have = n < n_items;
                 if (have) score_item(p, s_tab, n, qt, item);
                 ++u;
-                for (int h = 0; h < halves && !dead; ++h) dead = !tc::mbar_wait(&bar_t_full[2 * slot + h], used[h]++ & 1u, wc, 20);
-                if (dead) break;
+                for (int h = 0; h < halves && !dead; ++h) dead = !tc::mbar_wait(&bar_t_full[2 * slot + h], (used[h] - 1) & 1u, wc, 20);
+                if (dead) { have = false; break; }                 // (nothing more has been loaded)
                 if (have) load(item, qt, !same);
             }
-            // nothing this thread started may still be in flight when the block exits (u, u - 1: the last load, waited for or not)
-            if (u > 0) tc::mbar_wait(full, (u - 1) & 1u, wc, 20);
-            if (have) tc::mbar_wait(full, u & 1u, wc, 20);
+            // nothing this thread started may still be in flight when the block exits, also where a wait ran out
+            const uint32_t loads = u + (have ? 1u : 0u);
+            if (loads > 0) tc::mbar_drain(full, (loads - 1) & 1u, wc);
+            for (int h = 0; h < 2; ++h)
+                if (used[h] > 0) tc::mbar_drain(&bar_t_full[2 * slot + h], (used[h] - 1) & 1u, wc);
         }
     } else {
         // ---------------- consumers ----------------

@@ -99,6 +99,21 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, const 
     }
 }
 
+// Waits until the phase has completed whatever has become of the block, at most for the wait limit: a thread that gives up, or
+// is done, lets the copies and tensor-core instructions it started come to their end before the block's memory is given back.
+__device__ __forceinline__ void mbar_drain(uint64_t *bar, uint32_t parity, const WaitCtx &w)
+{
+    if (mbar_try(bar, parity)) return;
+    const uint64_t t0 = global_ns();
+    while (!mbar_try(bar, parity)) {
+        if (global_ns() - t0 > w.limit_ns) {
+            *w.abort_flag = 1u;
+            atomicOr(w.status, OBF_DEV_TIMEOUT);
+            return;
+        }
+    }
+}
+
 // ---- TMA -----------------------------------------------------------------------
 // Load of a tile of rows, all its 64-column blocks at once, through a tensor map over [heads][blocks][rows][64]
 // (obf_api.cu: encode_rows_map) into shared memory; completion is signalled on `bar` as transaction bytes.  One

@@ -1282,3 +1282,18 @@ def test_masses_of_a_head_do_not_depend_on_the_number_of_caches(G, n_obs, d):
         b, _, st = par.run_gpu(one, [arrays[ci]])
         assert st & 0xFF == 0
         assert torch.equal(a[ci]["scores"], b[0]["scores"]) and torch.equal(a[ci]["idx"], b[0]["idx"]), ci
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_a_wait_that_runs_out_between_two_query_tiles(d):
+    # every slot has a second tile of queries to load and multiply when the wait of the first one runs out (20 ms): the block lets
+    # what it started come to its end, and the call after it finds everything as it should be
+    w = small("expire2", layers=1, kv_heads=4, G=8, n_obs=32, d=d, dtype="bf16", rank=1, caches=((2000, 40),), heavy=5, seed=17)
+    arrays = [synth.gen_cache(w, 0)]
+    outs, dev, st = par.run_gpu(w, arrays, flags=P.binding.OBF_FLAG_TEST_WAIT_EXPIRES)
+    assert st & P.binding.OBF_DEV_TIMEOUT
+    ws = outs[0]["workspace"]
+    good = P.compress_caches(par.params_for(w), dev, want_scores=True, workspace=ws)
+    torch.cuda.synchronize()
+    assert P.obf_last_device_status(ws) & 0xFF == 0
+    par.check_cache(w, 0, arrays[0], good[0], all_heads(w))
