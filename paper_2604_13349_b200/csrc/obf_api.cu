@@ -412,12 +412,14 @@ static obf_status_t launch_score_tc(const CallDev &cd, const Layout &L, cudaStre
         if ((s = encode_rows_map(&maps.b[many ? i : ST_PART_MAP + i], cd.c[i].q, D, (uint64_t)cd.n_q, hpc, 32, 1)) != OBF_OK) return s;
     }
     const size_t smem = score_tc_smem_bytes<D>();
-    OBF_CUDA_TRY(cudaFuncSetAttribute(k_score_tc<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    bool longest = false;
+    for (int i = 0; i < cd.n_caches; ++i) longest = longest || cd.c[i].sc_team > ST_FLAT;
+    const void *kernel = longest ? reinterpret_cast<const void *>(k_score_tc<D, true>) : reinterpret_cast<const void *>(k_score_tc<D, false>);
+    OBF_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     // The blocks of a head's team wait for one another, so the whole grid has to be resident at once: a
     // cooperative launch starts only when it is (the grid never exceeds one block per multiprocessor).
     void *args[2] = {const_cast<CallDev *>(&cd), &maps};
-    OBF_CUDA_TRY(cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(k_score_tc<D>), dim3(L.sc_blocks), dim3(ST_THREADS),
-                                             args, smem, st));
+    OBF_CUDA_TRY(cudaLaunchCooperativeKernel(kernel, dim3(L.sc_blocks), dim3(ST_THREADS), args, smem, st));
     mark(st, "k_score_tc");
     bool any_out = false;
     for (int i = 0; i < cd.n_caches; ++i) any_out = any_out || cd.c[i].scores_out != nullptr;

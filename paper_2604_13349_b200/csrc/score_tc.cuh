@@ -45,6 +45,7 @@ constexpr int ST_PIECES = ST_HALF / 32;             // of 32 columns, each with 
 constexpr int ST_BOX_BYTES = 128 * 128;              // a 64-channel column block of the queries: 128 rows of 128 bytes
 constexpr int ST_THREADS = 32 * ST_SLOTS + 128 * ST_GROUPS;
 constexpr int ST_MAX_NQ = 256;                      // two query tiles of 128 rows
+constexpr int ST_FLAT = 32;                         // chunks of a head whose statistics are folded in one step: sixteen words a group, all in flight at once
 constexpr float ST_LOG2E = 1.4426950408889634f;
 template <int D>
 constexpr size_t score_tc_smem_bytes()
@@ -207,7 +208,10 @@ __device__ __forceinline__ void pool64(const uint32_t (&lo)[32], const uint32_t 
 // Lane bit 4: piece, bits 3, 2: block of eight columns in it, bits 1, 0: pair of columns.
 __device__ __forceinline__ int score_col(int lane) { return 8 * (lane >> 2) + 2 * (lane & 3); }
 
-template <int D>
+// LONG: some head of the call has more than ST_FLAT chunks (an instantiation of its own: with both ways of folding in one, heads of up
+// to ST_FLAT chunks were 1 to 3 % slower).  Folding all chunks of a long head in every slot, sixteen words a sweep, cost 8 heads of 75000
+// positions 165 us, this way 77 (the kernel that visited every tile twice: 91); 8 heads of 16384: 27.3, 25.4, 23.9; 128 heads of 12000: 189, 180, 157.
+template <int D, bool LONG>
 __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constant__ CallDev p, const __grid_constant__ TcMaps tm)
 {
     constexpr int Q_BYTES = 128 * D * 2, K_BYTES = ST_CHUNK * D * 2;
@@ -382,61 +386,73 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constan
                 // until it is published, never zero afterwards (the sum of a finite maximum's own weight is above a half; the sum
                 // of a chunk without a finite logit is written as -0).  A word vouches for itself, so nothing is counted and
                 // nothing fenced.  The two groups of the slot fold half of the head's chunks each, in ascending order.
-                if (half == 0 && row < it.nq) {
-                    float M = -INFINITY, Z = 0.f;
-#pragma unroll 1
-                    for (int r = row; r < 128; r += rows) {
-                        score_fold(M, Z, s_m[group * 128 + r], s_z[group * 128 + r]);
-                        score_fold(M, Z, s_m[(group + 1) * 128 + r], s_z[(group + 1) * 128 + r]);
-                    }
-                    const uint32_t zb = Z == 0.f ? 0x80000000u : __float_as_uint(Z);
-                    if (!p.debug_drop_publish)
-                        st_relaxed_gpu_u64(words + (size_t)it.chunk * 128 + row, ((unsigned long long)zb << 32) | __float_as_uint(M));
-                }
+                // In a head of more than ST_FLAT chunks every sixteenth chunk first folds the fifteen after it into its own (hop 0) and
+                // publishes the sum of the sixteen; these sums come first among the head's words and are what everybody folds (hop 1).
+                // Which way a head goes, and so the order of its sums, depends on its own length alone.
                 {
                     float M = -INFINITY, Z = 0.f;
-                    bool gave_up = false;
-                    const int per = (c.sc_team + 1) >> 1, c_end = min(c.sc_team, per * (half + 1));
-                    // sixteen chunks in flight per sweep; a warp without queries has nothing to fetch
+                    if (half == 0 && row < it.nq) {
 #pragma unroll 1
-                    for (int c0 = per * half; c0 < c_end && 32 * q < it.nq && !gave_up; c0 += 16) {
-                        unsigned long long w[16];
-                        const unsigned long long *from = words + (size_t)c0 * 128 + row;
-#pragma unroll
-                        for (int e = 0; e < 16; ++e) w[e] = (c0 + e < c_end && row < it.nq) ? 0ull : 0x80000000ff800000ull;   // (-inf, -0)
-                        // (many chunks are never there at once, and polls in vain hold up those who publish: T = 8192 273 -> 267 us; with few
-                        // chunks the pause would be longer than the wait)
-                        if (c.sc_team >= 16) __nanosleep(600);
-                        uint64_t t0 = 0ull;
-                        for (;;) {
-#pragma unroll
-                            for (int e = 0; e < 16; ++e)
-                                if ((uint32_t)(w[e] >> 32) == 0u) w[e] = ld_relaxed_gpu_u64(from + e * 128);
-                            uint32_t least = 0xFFFFFFFFu;
-#pragma unroll
-                            for (int e = 0; e < 16; ++e) least = min(least, (uint32_t)(w[e] >> 32));
-                            // the warp leaves the loop as one: votes, not per-lane exits
-                            if (__all_sync(0xffffffffu, least != 0u)) break;
-                            const uint64_t now = tc::global_ns();
-                            if (t0 == 0ull) t0 = now;
-                            if (__any_sync(0xffffffffu, *(volatile uint32_t *)&s_abort != 0u || now - t0 > p.wait_limit_ns)) {
-                                if (lane == 0) {
-                                    s_abort = 1u;
-                                    atomicOr(p.status, OBF_DEV_TIMEOUT);
-                                }
-                                gave_up = true;
-                                break;
-                            }
-                            __nanosleep(32);
+                        for (int r = row; r < 128; r += rows) {
+                            score_fold(M, Z, s_m[group * 128 + r], s_z[group * 128 + r]);
+                            score_fold(M, Z, s_m[(group + 1) * 128 + r], s_z[(group + 1) * 128 + r]);
                         }
-                        float Mn = M;
+                    }
+                    const bool flat = !LONG || c.sc_team <= ST_FLAT;
+                    const int n_words = flat ? c.sc_team : (c.sc_team + 15) >> 4, per = (n_words + 1) >> 1;
+                    const int behind = n_words + 15 * (it.chunk >> 4);             // where the fifteen words are
+                    const int at = flat ? it.chunk : it.chunk & 15 ? behind + (it.chunk & 15) - 1 : it.chunk >> 4;
+#pragma unroll 1
+                    for (int hop = !flat && half == 0 && !(it.chunk & 15) ? 0 : 1; hop < 2; ++hop) {
+                        if (hop == 1) {
+                            if (half == 0 && row < it.nq && !p.debug_drop_publish) {
+                                const uint32_t zb = Z == 0.f ? 0x80000000u : __float_as_uint(Z);
+                                st_relaxed_gpu_u64(words + (size_t)at * 128 + row, ((unsigned long long)zb << 32) | __float_as_uint(M));
+                            }
+                            M = -INFINITY;
+                            Z = 0.f;
+                        }
+                        const int c0 = hop == 0 ? behind : per * half;
+                        const int c_end = hop == 0 ? min(behind + 15, c.sc_team) : min(n_words, per * (half + 1));
+                        if (c0 < c_end && 32 * q < it.nq) {
+                            // at most sixteen words, in flight together; a warp without queries has nothing to fetch
+                            unsigned long long w[16];
+                            const unsigned long long *from = words + (size_t)c0 * 128 + row;
 #pragma unroll
-                        for (int e = 0; e < 16; e += 2) Mn = max3(Mn, __uint_as_float((uint32_t)w[e]), __uint_as_float((uint32_t)w[e + 1]));
-                        const float Mf = fmaxf(Mn, -3e38f);
-                        Z *= exp2_whole(M - Mf);
+                            for (int e = 0; e < 16; ++e) w[e] = (c0 + e < c_end && row < it.nq) ? 0ull : 0x80000000ff800000ull;   // (-inf, -0)
+                            // (many chunks are never there at once, and polls in vain hold up those who publish: T = 8192 273 -> 267 us; with few
+                            // chunks the pause would be longer than the wait)
+                            if (hop == 1 && c.sc_team >= 16) __nanosleep(600);
+                            uint64_t t0 = 0ull;
+                            for (;;) {
 #pragma unroll
-                        for (int e = 0; e < 16; ++e) Z = fmaf(__uint_as_float((uint32_t)(w[e] >> 32)), exp2_whole(__uint_as_float((uint32_t)w[e]) - Mf), Z);
-                        M = Mn;
+                                for (int e = 0; e < 16; ++e)
+                                    if ((uint32_t)(w[e] >> 32) == 0u) w[e] = ld_relaxed_gpu_u64(from + e * 128);
+                                uint32_t least = 0xFFFFFFFFu;
+#pragma unroll
+                                for (int e = 0; e < 16; ++e) least = min(least, (uint32_t)(w[e] >> 32));
+                                // the warp leaves the loop as one: votes, not per-lane exits
+                                if (__all_sync(0xffffffffu, least != 0u)) break;
+                                const uint64_t now = tc::global_ns();
+                                if (t0 == 0ull) t0 = now;
+                                if (__any_sync(0xffffffffu, *(volatile uint32_t *)&s_abort != 0u || now - t0 > p.wait_limit_ns)) {
+                                    if (lane == 0) {
+                                        s_abort = 1u;
+                                        atomicOr(p.status, OBF_DEV_TIMEOUT);
+                                    }
+                                    break;
+                                }
+                                __nanosleep(32);
+                            }
+                            float Mn = M;
+#pragma unroll
+                            for (int e = 0; e < 16; e += 2) Mn = max3(Mn, __uint_as_float((uint32_t)w[e]), __uint_as_float((uint32_t)w[e + 1]));
+                            const float Mf = fmaxf(Mn, -3e38f);
+                            Z *= exp2_whole(M - Mf);
+#pragma unroll
+                            for (int e = 0; e < 16; ++e) Z = fmaf(__uint_as_float((uint32_t)(w[e] >> 32)), exp2_whole(__uint_as_float((uint32_t)w[e]) - Mf), Z);
+                            M = Mn;
+                        }
                     }
                     s_fm[group * 128 + row] = M;
                     s_fz[group * 128 + row] = Z;

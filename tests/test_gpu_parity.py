@@ -1297,3 +1297,19 @@ def test_a_wait_that_runs_out_between_two_query_tiles(d):
     torch.cuda.synchronize()
     assert P.obf_last_device_status(ws) & 0xFF == 0
     par.check_cache(w, 0, arrays[0], good[0], all_heads(w))
+
+
+@pytest.mark.parametrize("d,G,n_obs,caches", [
+    (128, 2, 16, ((8192, 9), (8193, 9), (300, 9))),                # 32 chunks: folded in one step; 33: a last sixteen of one; a short one
+    (64, 4, 32, ((12288, 9),)),                                    # three whole sixteens
+    (128, 4, 40, ((12289, 9),)),                                   # and a chunk more, with two tiles of queries
+    (64, 1, 50, ((75776, 9),)),                                    # as many as there are slots on 148 multiprocessors
+])
+def test_score_kernel_folds_long_heads_in_two_steps(d, G, n_obs, caches):
+    w = small("longer", layers=1, kv_heads=2, G=G, n_obs=n_obs, d=d, dtype="bf16", rank=1, caches=caches, n_outlier=3, n_sink=4,
+              heavy=5, seed=700 + n_obs)
+    a, _, arrays = run_and_check(w)
+    assert "k_score_tc" in [n for n, _ in P.obf_compress_profiled(par.params_for(w), a[0]["cache_structs"], a[0]["workspace"])]
+    for ci, c in enumerate(w.caches):                              # the masses of a head do not depend on the length of the others
+        b, _, _ = par.run_gpu(dataclasses.replace(w, caches=(c,)), [arrays[ci]])
+        assert torch.equal(a[ci]["scores"], b[0]["scores"]) and torch.equal(a[ci]["idx"], b[0]["idx"])
