@@ -509,18 +509,17 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
     }
     mark(sel, "k_select");
     if (side && FORK_LATE) {
-        if (gather_vecs && !L.rows) {
-            side = nullptr;                                            // nothing to run beside the pass
-        } else {
-            OBF_TRY(fork_and_pass());
-            sel = side->stream;
-        }
+        OBF_TRY(fork_and_pass());
+        sel = side->stream;
     }
     auto launch_rows = [&](cudaStream_t on) -> obf_status_t {
-        if (!L.rows) return OBF_OK;
-        OBF_TRY(set_smem(k_obf_rows<TIN, D>, (size_t)D * D * sizeof(float)));
-        OBF_TRY(launch(k_obf_rows<TIN, D>, dim3(heads), ALG_NT, (size_t)cd.alg_rows * D * sizeof(float), on, cd));
-        mark(on, "k_obf_rows");
+        // (bf16 heads of 64 channels only: make_layout)
+        if constexpr (sizeof(TIN) == 2 && GramShape<D>::DELETED) {
+            if (!L.rows) return OBF_OK;
+            OBF_TRY(set_smem(k_obf_rows<TIN, D>, (size_t)D * D * sizeof(float)));
+            OBF_TRY(launch(k_obf_rows<TIN, D>, dim3(heads), ALG_NT, (size_t)cd.alg_rows * D * sizeof(float), on, cd));
+            mark(on, "k_obf_rows");
+        }
         return OBF_OK;
     };
     dim3 g4((k_max + GATHER_ROWS - 1) / GATHER_ROWS, heads);

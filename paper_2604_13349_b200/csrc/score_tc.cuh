@@ -25,12 +25,14 @@
 // lowest unfinished head always makes progress.  Every wait is bounded (tc_common.cuh).
 //
 // What bounds it is the latency of a slot's chain, 14000 cycles per 256 keys at T = 8192 (logits 1500, statistics 4200, the
-// exchange 4500, pooling 2900, last sum 1000), of which tensor memory allows two at a time; special-function unit 30 % busy, issue
-// slots 46 %, DRAM 29 %.  Against the form before it (every tile visited twice, for the statistics and for the pooling: two
-// exponentials, two MMAs and two trips from L2) it is slower in a burst, 253 -> 267 us for 40 x 8 heads of 8192 positions, and
-// faster back to back, where the power limit counts what is done: that call 515 -> 482 us, 36 x 8 heads of 4096, eviction, 186 -> 171,
-// four caches 1016 -> 958; one layer of 2048 positions 57 -> 52.5, 16 x 8 heads of 64 channels 134.5 -> 126.  Chunks of 512 keys shared by
-// clusters of two blocks, four slots of 128 keys, and warps that pool three tiles behind the one they compute were no faster.
+// exchange 4500, pooling 2900, last sum 1000), of which tensor memory allows two at a time; the special-function unit is a third
+// busy, the issue slots half, DRAM a third.  Against the form before it (every tile visited twice, for the statistics and for the
+// pooling: two exponentials, two MMAs and two trips from L2), calls in bursts of 10 ms and back to back for seconds, where the power
+// limit counts what is done: 40 x 8 heads of 8192 positions 459 -> 464 us and 513 -> 481, 36 x 8 of 4096, eviction, 169 -> 169.5 and
+// 185 -> 168; one layer of 2048 positions 57.4 -> 53.4, 16 x 8 heads of 64 channels 136 -> 120.  Slower in a burst: 36 x 8 heads of 4096
+// with 160 queries 194 -> 214, 128 heads of 12000 171 -> 193 and of 16384 237 -> 268, 8 heads of up to 300 positions with 256
+// queries 19 -> 20.5.  Chunks of 512 keys shared by clusters of two blocks, four slots of 128 keys, warps that pool three tiles behind
+// the one they compute, and rounds of whole heads (each rank of slots its own, or one head across the ranks) were no faster.
 #pragma once
 
 #include "tc_common.cuh"
@@ -420,8 +422,11 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constan
                             const unsigned long long *from = words + (size_t)c0 * 128 + row;
 #pragma unroll
                             for (int e = 0; e < 16; ++e) w[e] = (c0 + e < c_end && row < it.nq) ? 0ull : 0x80000000ff800000ull;   // (-inf, -0)
-                            // (many chunks are never there at once, and polls in vain hold up those who publish: T = 8192 273 -> 267 us; with few
-                            // chunks the pause would be longer than the wait)
+                            // From sixteen chunks on they are never there at once, and polls in vain hold up those who publish; with fewer
+                            // the pause would be longer than the wait (36 x 8 heads of 3500 positions, 64 channels: 106.7 us without, 109.9
+                            // with one of 400 ns).  600, 400 and no ns: 32 x 8 heads of 8192 positions with 32 queries 188.1, 190.6, 195.3 us,
+                            // with 128 231.3, 229.0, 235.1, with 160 377.6, 370.2, 372.0, with 128 of 64 channels 220.0, 212.8, 211.0;
+                            // 36 x 8 of 4096 with 128 131.4, 130.5, 133.6.
                             if (hop == 1 && c.sc_team >= 16) __nanosleep(600);
                             uint64_t t0 = 0ull;
                             for (;;) {

@@ -56,16 +56,6 @@ __device__ __forceinline__ bool mbar_try(uint64_t *bar, uint32_t parity, uint32_
     return ok != 0;
 }
 
-// Non-blocking test of the phase with the given parity.  Two of these issued back to back overlap
-// their latency, which a pair of parked tests does not.
-__device__ __forceinline__ bool mbar_test(uint64_t *bar, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile("{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-                 : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
-    return ok != 0;
-}
-
 // What a block shares to give up cleanly: the abort flag lives in shared memory,
 // the status word in the workspace.
 struct WaitCtx {
@@ -129,13 +119,6 @@ __device__ __forceinline__ void tma_load_block(uint32_t dst, const CUtensorMap *
 {
     asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
                  ::"r"(dst), "l"(map), "r"(smem_u32(bar)), "r"(0), "r"(row), "r"(block), "r"(head) : "memory");
-}
-
-// Asks for the tile to be brought into the L2 cache; nothing lands in shared memory.
-__device__ __forceinline__ void tma_prefetch_rows(const CUtensorMap *map, int row, int head)
-{
-    asm volatile("cp.async.bulk.prefetch.tensor.4d.L2.global.tile [%0, {%1, %2, %1, %3}];"
-                 ::"l"(map), "r"(0), "r"(row), "r"(head) : "memory");
 }
 
 // Generic-proxy writes to shared memory become visible to the tensor core / TMA.
