@@ -308,8 +308,8 @@ def test_retained_rows_with_a_dominant_common_component():
 
 @pytest.mark.parametrize("T,budget", [(20000, 300), (70000, 250), (80000, 200)])
 def test_long_prompts_take_the_fallback_kernels(T, budget):
-    # 20000 keys: more than the select kernel keeps in shared memory; 70000 keys: one head's team is 137 blocks,
-    # nearly the whole grid of the persistent score kernel; 80000 keys: more chunks than that kernel has blocks,
+    # 20000 keys: more than the select kernel keeps in shared memory; 70000 keys: one head is 274 chunks,
+    # nearly all slots of the persistent score kernel, two a block; 80000 keys: more chunks than that kernel has slots,
     # so the shape-generic score kernels run (the Gram pass stays tuned)
     w = small("long", layers=1, kv_heads=1, G=4, n_obs=8, d=128, dtype="bf16", rank=1, caches=((T, budget),),
               n_outlier=3, n_sink=4, heavy=8, seed=T % 97)
@@ -1313,3 +1313,27 @@ def test_score_kernel_folds_long_heads_in_two_steps(d, G, n_obs, caches):
     for ci, c in enumerate(w.caches):                              # the masses of a head do not depend on the length of the others
         b, _, _ = par.run_gpu(dataclasses.replace(w, caches=(c,)), [arrays[ci]])
         assert torch.equal(a[ci]["scores"], b[0]["scores"]) and torch.equal(a[ci]["idx"], b[0]["idx"])
+
+
+@pytest.mark.parametrize("d,G,n_obs", [(64, 4, 7), (128, 4, 8), (64, 4, 15), (128, 4, 16), (64, 4, 32), (128, 4, 32), (64, 4, 40), (128, 8, 32)])
+def test_score_kernel_reuses_its_slots(d, G, n_obs):
+    # 48 heads of (2 + 3 + 6) + 8 chunks are 912, three for every slot: both slots of a block, their buffers and barriers met again by
+    # last chunks of one half (300 = 256 + 44, 1380 = 5 * 256 + 100) and of two (700 = 2 * 256 + 188, 1950 = 7 * 256 + 158); four, two
+    # and one copies, two tiles
+    caches = ((300, 9), (700, 9), (1380, 9), (1950, 9))
+    w = small("slots", layers=6, kv_heads=8, G=G, n_obs=n_obs, d=d, dtype="bf16", rank=1, caches=caches, heavy=3, n_outlier=3,
+              seed=40 + n_obs + d)
+    _, reps, _ = run_and_check(w, evict=True, heads=[(l, (3 * l + 1) % 8) for l in range(6)] + [(5, 7)])
+    assert len(reps) == 7 * len(caches)
+
+
+def test_masses_of_a_head_do_not_depend_on_the_other_heads_of_its_slots():
+    # 800 chunks of ten a head: slots are used again, and by which chunk follows from all that comes before
+    g = torch.Generator(device="cuda").manual_seed(4)
+    K, V, Q = (torch.randn((10, 8, rows, 64), generator=g, device="cuda", dtype=torch.bfloat16) for rows in (2500, 2500, 70))
+    whole = P.compress_caches(P.make_params(10, 8, 8, 64, 70, 0, P.OBF_BF16), [dict(K=K, V=V, Q=Q, budget=30)], evict=True, want_scores=True)[0]
+    for l in range(10):
+        one = [x[l:l + 1].contiguous() for x in (K, V, Q)]
+        part = P.compress_caches(P.make_params(1, 8, 8, 64, 70, 0, P.OBF_BF16), [dict(K=one[0], V=one[1], Q=one[2], budget=30)],
+                                 evict=True, want_scores=True)[0]
+        assert torch.equal(part["scores"][0], whole["scores"][l]) and torch.equal(part["idx"][0], whole["idx"][l])

@@ -147,3 +147,25 @@ def test_static_scratch_takes_heads_of_128_channels_in_groups(layers, kv_heads, 
     for o, r in zip(outs, ref):
         for n in o:
             assert torch.equal(o[n], r[n]), n
+
+
+def test_static_scratch_falls_back_to_the_generic_kernels_where_a_head_of_every_cache_does_not_fit():
+    # 32 caches of one head: seven bytes a position fit the array, nine do not, and there is nothing to make groups of
+    T, flags = 33000, binding.OBF_FLAG_GENERIC_PATH
+    g = torch.Generator(device="cuda").manual_seed(9)
+    dev = [{n: torch.randn((1, 1, rows, 128), generator=g, device="cuda", dtype=torch.bfloat16) for n, rows in (("K", T), ("V", T), ("Q", 5))}
+           for _ in range(32)]
+    ref = P.compress_caches(P.make_params(1, 1, 1, 128, 5, 0, P.OBF_BF16, flags=flags), [dict(x, budget=70) for x in dev], evict=True, want_scores=True)
+    params = P.make_params(1, 1, 1, 128, 5, 0, P.OBF_BF16)
+    assert P.obf_workspace_bytes(params, ref[0]["cache_structs"]) > binding.OBF_STATIC_SCRATCH_BYTES
+    outs, cs = [], []
+    for x, r in zip(dev, ref):
+        o = {n: torch.zeros_like(r[n]) for n in ("K_out", "V_out", "idx", "scores")}
+        outs.append(o)
+        cs.append(P.make_cache(x["K"], x["V"], x["Q"], T, 70, o["K_out"], o["V_out"], o["idx"], None, o["scores"]))
+    P.evict_only_static(params, cs)
+    torch.cuda.synchronize()
+    assert P.obf_static_scratch_status() & 0xFF == 0
+    for o, r in zip(outs, ref):
+        for n in o:
+            assert torch.equal(o[n], r[n]), n
