@@ -535,7 +535,7 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
         OBF_CUDA_TRY(cudaEventRecord(side->rows_done, side->stream));
         if constexpr (sizeof(TIN) == 2) if (span) {
             // the span test reads the gathered rows only (it forms G_keep itself): it runs here, beside the pass over
-            // V, whose persistent blocks leave room for one of its blocks per multiprocessor
+            // V, whose persistent blocks leave room for two of its blocks per multiprocessor
             const size_t sm_span = span_smem_bytes<D>(true);
             if ((s = set_smem(k_span_test<D, true>, sm_span)) != OBF_OK) return s;
             OBF_TRY(launch(k_span_test<D, true>, dim3(heads), ST_NT, sm_span, sel, cd));

@@ -140,6 +140,31 @@ def test_span_test_at_budgets_around_head_dim_and_its_row_limit(dtype, d, budget
         assert all(dg["span_rank"] == min(b, d) for dg in P.parse_diag(o["diag"]))
 
 
+@pytest.mark.parametrize("dtype,d", [("bf16", 128), ("bf16", 64), ("f32", 128), ("f32", 64)])
+@pytest.mark.parametrize("channel", [1, 15, 16, 33, -1])
+def test_span_test_finds_one_channel_that_depends_on_another(dtype, d, channel):
+    # one channel repeats the first of its panel or of all (first and last pivots of a panel, first and last panel) on every row that can
+    # be retained: the span lacks one dimension, which a few unselectable tokens carry
+    channel %= d
+    w = small("dep", d=d, dtype=dtype, rank=1, caches=((600, d + 40),), heavy=0, kv_heads=2, seed=60 + channel)
+    arrays = [synth.gen_cache(w, 0)]
+    a = arrays[0]
+    K = par.f32_view(a["K"], dtype).copy(); V = par.f32_view(a["V"], dtype).copy()
+    Qv = par.f32_view(a["Q"], dtype).reshape(1, 2, w.n_q, d)
+    g = np.random.default_rng(channel)
+    kept_apart = V[..., channel].copy()
+    V[..., channel] = V[..., 0 if channel % 2 else 16 * (channel // 16) - 1]
+    for h in range(2):
+        qm = Qv[0, h].mean(axis=0)
+        odd = g.choice(600, 15, replace=False)
+        K[0, h, odd] = -1.5 * qm / np.linalg.norm(qm) * np.linalg.norm(K[0, h, odd], axis=1, keepdims=True)
+        V[0, h, odd, channel] = kept_apart[0, h, odd]
+    a["K"], a["V"] = (synth.to_bf16_bits(K), synth.to_bf16_bits(V)) if dtype == "bf16" else (K, V)
+    outs, reps, _ = run_and_check(w, arrays=arrays)
+    assert all(dg["span_rank"] == d - 1 for dg in P.parse_diag(outs[0]["diag"]))
+    assert all(not r.oracle_skipped for r in reps)
+
+
 def test_budget_above_head_dim_full_rank_is_bit_exact_eviction():
     w = small("full", d=64, dtype="bf16", rank=3, caches=((400, 90),))
     outs, reps, _ = run_and_check(w)
