@@ -281,6 +281,39 @@ __device__ __forceinline__ void alg_row_done(const AlgRow<D> &x, int j, float ti
     }
 }
 
+// x with its entries before `from` zero.
+template <int D, int FROM = 0>
+__device__ __forceinline__ void alg_masked(AlgRow<D> &m, const AlgRow<D> &x, int from, int c16)
+{
+#pragma unroll
+    for (int q = FROM; q < AlgShape<D>::NQ; ++q) {
+        float a, b;
+        upk(x[q], a, b);
+        const int c = 32 * q + 2 * c16;
+        m[q] = pk(c >= from ? a : 0.f, c + 1 >= from ? b : 0.f);
+    }
+}
+// w: x from entry j0 + 1 on as it is (m, masked), entry j0 `first`, zeros before.
+template <int D, int FROM = 0>
+__device__ __forceinline__ void alg_with_first(AlgRow<D> &w, const AlgRow<D> &m, int j0, float first, int c16)
+{
+#pragma unroll
+    for (int q = FROM; q < AlgShape<D>::NQ; ++q) {
+        float a, b;
+        upk(m[q], a, b);
+        const int c = 32 * q + 2 * c16;
+        w[q] = pk(c == j0 ? first : a, c + 1 == j0 ? first : b);
+    }
+}
+// Half of |w|^2 and w's first entry, for a row of first entry x0 whose other squares sum to `below2`: w = x + sign(x0) |x| e_0.
+__device__ __forceinline__ float alg_first(float x0, float below2, float &first, float &al)
+{
+    const float n2 = fmaf(x0, x0, below2), nrm = n2 * rsqrt_approx(fmaxf(n2, 1e-37f));
+    al = x0 >= 0.f ? -nrm : nrm;
+    first = x0 - al;
+    return fmaf(nrm, fabsf(x0), n2);
+}
+
 // Sturm counts of the tridiagonal matrix (diagonal a, squared off-diagonals b2, scaled to a spectrum within [-1, 1]) at
 // two shifts: the number of eigenvalues below each, as the sign changes of the leading principal minors'
 // three-term recurrence p_i = (a_i - x) p_{i-1} - b2_{i-1} p_{i-2} (Givens' bisection).  No division: a step of the chain
@@ -352,17 +385,21 @@ static_assert(ALG_SMEM_MAX<128> <= 227 * 1024 - 1024, "a block has 227 KB, some 
 
 // 2. Reflectors of a head's k retained rows (Eq. 2), into Y (shared memory): how many there are.  A loop of its own and not one with
 // that over G: together their code outgrows what a multiprocessor fetches at full speed.
+// The next row passes through `next` (2 buffers of D + 4 floats) one reflector early, and every half-warp finds every reflector for
+// itself; and as a reflector is its row but for one entry, which the row's norm decides, all products with it are formed while the
+// norm is still being added up: one reduction and one barrier a row.  With the owner's reflector sent to the others, then their
+// products, 1010 cycles a row of 128 channels, this way 660 (two heads on a multiprocessor 1070 and 900).
 template <typename TIN, int D>
-__device__ __forceinline__ int alg_reflectors(const TIN *vk, int k, float *Y, int *s_flag)
+__device__ __forceinline__ int alg_reflectors(const TIN *vk, int k, float *Y, float *next)
 {
     constexpr int NQ = AlgShape<D>::NQ;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, grp = tid >> 4, c16 = tid & 15;
+    const int tid = threadIdx.x, lane = tid & 31, warp = warp_uniform(tid >> 5), grp = tid >> 4, c16 = tid & 15;
     int m = 0;
     // a batch of rows in registers (G comes afterwards): row b0 + grp + ALG_NG s in slot s of the half-warp
     constexpr int NS = ALG_BATCH / ALG_NG;
     static_assert(NS == 4, "four slots to pick from");
     AlgRow<D> V[NS];
-    float n0[NS];                                              // the rows' squared norms
+    float n0[NS] = {0.f, 0.f, 0.f, 0.f};                       // the rows' squared norms
     auto reflect_rows = [&](const AlgRow<D> &v) __attribute__((always_inline)) {
         float d4[NS];
 #pragma unroll
@@ -375,38 +412,17 @@ __device__ __forceinline__ int alg_reflectors(const TIN *vk, int k, float *Y, in
             for (int q = 0; q < NQ; ++q) V[s][q] = fma2(pk(f, f), v[q], V[s][q]);
         }
     };
-    // whether row i of the batch adds a direction to the m there are, and its reflector
-    auto candidate = [&](int i) __attribute__((always_inline)) {
+    // row i of the batch, as the reflectors so far leave it, for everybody, with its squared norm
+    auto publish = [&](int i) __attribute__((always_inline)) {
         if (warp != (i % ALG_NG) / 2) return;
-        AlgRow<D> x;
-        float nn = n0[0];
+        const f32x2 odd = mask2(i / ALG_NG & 1), high = mask2(i / ALG_NG & 2);
+        const float nn = i / ALG_NG & 2 ? (i / ALG_NG & 1 ? n0[3] : n0[2]) : (i / ALG_NG & 1 ? n0[1] : n0[0]);
+        float *to = next + (i & 1) * (D + 4);
+        if (grp != i % ALG_NG) return;
 #pragma unroll
-        for (int q = 0; q < NQ; ++q) x[q] = V[0][q];
-        auto pick = [&](auto slot) __attribute__((always_inline)) {
-            constexpr int s = decltype(slot)::value;
-            if (i / ALG_NG == s) {
-                nn = n0[s];
-#pragma unroll
-                for (int q = 0; q < NQ; ++q) {
-                    x[q] = V[s][q];
-                    // (keeps the compiler from merging the slots' code into one that addresses the array)
-                    asm volatile("// %1" : "+l"(x[q]) : "n"(s));
-                }
-            }
-        };
-        pick(std::integral_constant<int, 1>{});
-        pick(std::integral_constant<int, 2>{});
-        pick(std::integral_constant<int, 3>{});
-        const float t2 = alg_tail2<D>(x, m, c16), x0 = alg_entry<D>(x, m < D ? m : 0, lane);
-        const float nrm = t2 * rsqrt_approx(fmaxf(t2, 1e-37f));
-        if (grp == i % ALG_NG) {
-            const bool add = m < D && t2 > SPAN_ROW_TOL * SPAN_ROW_TOL * nn && t2 > 1e-37f;
-            if (add) {
-                const float al = x0 >= 0.f ? -nrm : nrm;
-                alg_store_reflector<D>(x, m, x0 - al, rsqrt_approx(2.f * fmaf(nrm, fabsf(x0), t2)), Y + m * D, c16);
-            }
-            if (c16 == 0) s_flag[i & 1] = add ? 1 : 0;
-        }
+        for (int q = 0; q < NQ; ++q)
+            *reinterpret_cast<f32x2 *>(to + 32 * q + 2 * c16) = sel2(high, sel2(odd, V[3][q], V[2][q]), sel2(odd, V[1][q], V[0][q]));
+        if (c16 == 0) to[D] = nn;
     };
 #pragma unroll 1
     for (int b0 = 0; b0 < k && m < D; b0 += ALG_BATCH) {
@@ -432,7 +448,7 @@ __device__ __forceinline__ int alg_reflectors(const TIN *vk, int k, float *Y, in
             // a reflector depends on its row's direction alone: rows whose squares leave the range of fp32's normal numbers
             // are brought back by a power of two
             const bool far = n0[s] > 0.f && !(n0[s] > 1e-24f && n0[s] < 1e24f);
-            if (__any_sync(0xffffffffu, far)) {                // (the sum below takes the whole warp)
+            if (warp_uniform(far)) {                           // (any of them: the sum below takes the whole warp)
                 const float f = !far ? 1.f : n0[s] < 1.f ? 1.8446744e19f : 5.421011e-20f;   // 2^64, 2^-64
 #pragma unroll
                 for (int q = 0; q < NQ; ++q) V[s][q] = mul2(V[s][q], pk(f, f));
@@ -447,21 +463,52 @@ __device__ __forceinline__ int alg_reflectors(const TIN *vk, int k, float *Y, in
             reflect_rows(v);
         }
         const int rows = min(ALG_BATCH, k - b0);
-        candidate(0);
+        publish(0);
+        if (rows > 1) publish(1);
+        __syncthreads();
+        AlgRow<D> x;                                           // row i as all reflectors before it leave it (the same in every half-warp)
+        alg_load<D>(x, next, c16);
+        float nn = next[D];
 #pragma unroll 1
         for (int i = 0; i < rows; ++i) {
-            __syncthreads();
-            if (s_flag[i & 1]) {                               // row i has a reflector
-                AlgRow<D> v;
-                alg_load<D>(v, Y + m * D, c16);
-                reflect_rows(v);
-                if (++m >= D) break;
-                if (i + 1 < rows) candidate(i + 1);
-            } else if (i + 1 < rows) {
-                candidate(i + 1);
+            AlgRow<D> r;
+            const float *from = next + ((i + 1) & 1) * (D + 4);
+            alg_load<D>(r, from, c16);
+            const float nr = from[D];
+            // The reflector of row i (zero unless the row adds a direction to the m there are) is the row but for its entry m: every product
+            // with it is formed with the row's rest while the row's norm, which decides about that entry, is still being added up.
+            AlgRow<D> w;
+            alg_masked<D>(w, x, m + 1, c16);
+            float d8[8] = {alg_dot<D>(w, w), alg_dot<D>(r, w), 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, f[NS];
+#pragma unroll
+            for (int s = 0; s < NS; ++s) d8[2 + s] = alg_dot<D>(V[s], w);
+            const float tot = transposed_sum<8, 16>(d8, c16), below2 = __shfl_sync(0xffffffffu, tot, lane & 16);
+            const float x0 = alg_entry<D>(x, m, lane);
+            float first, al;
+            const float h = alg_first(x0, below2, first, al), t2 = fmaf(x0, x0, below2);
+            const bool add = warp_uniform(t2 > SPAN_ROW_TOL * SPAN_ROW_TOL * nn && t2 > 1e-37f);
+            const float b = add ? -rcp_approx(h) : 0.f;
+            alg_with_first<D>(w, w, m, first, c16);
+            const float fr = b * fmaf(alg_entry<D>(r, m, lane), first, __shfl_sync(0xffffffffu, tot, (lane & 16) + 2));
+#pragma unroll
+            for (int s = 0; s < NS; ++s) f[s] = b * fmaf(alg_entry<D>(V[s], m, lane), first, __shfl_sync(0xffffffffu, tot, (lane & 16) + 4 + 2 * s));
+            if (add && grp == i % ALG_NG) {
+                const float rs = rsqrt_approx(2.f * h);
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) *reinterpret_cast<f32x2 *>(Y + m * D + 32 * q + 2 * c16) = mul2(w[q], pk(rs, rs));
             }
+            if (add && ++m >= D) break;                        // (the same everywhere)
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) {
+                x[q] = fma2(pk(fr, fr), w[q], r[q]);
+#pragma unroll
+                for (int s = 0; s < NS; ++s) V[s][q] = fma2(pk(f[s], f[s]), w[q], V[s][q]);
+            }
+            nn = nr;
+            if (i + 2 < rows) publish(i + 2);
+            __syncthreads();
         }
-        // the flag is written again by the next batch
+        // the reflectors are there, the buffers free
         __syncthreads();
     }
     return m;
@@ -476,14 +523,14 @@ __global__ void __launch_bounds__(ALG_NT) k_obf_rows(const __grid_constant__ Cal
 {
     pdl_wait();
     extern __shared__ __align__(16) float sm[];
-    __shared__ int s_flag[2];
+    __shared__ __align__(16) float s_next[2 * (D + 4)];
     const int g = blockIdx.x;
     int ci, lh;
     locate(p, g, ci, lh);
     const CacheDev &c = p.c[ci];
     const int k = c.k_eff;
     if (c.T <= k) return;
-    const int m = alg_reflectors<TIN, D>(reinterpret_cast<const TIN *>(c.v_out) + (size_t)lh * k * D, k, sm, s_flag);
+    const int m = alg_reflectors<TIN, D>(reinterpret_cast<const TIN *>(c.v_out) + (size_t)lh * k * D, k, sm, s_next);
     float4 *dst = reinterpret_cast<float4 *>(p.rows_y + (size_t)g * p.alg_rows * D);
     for (int e = threadIdx.x; e < m * (D / 4); e += ALG_NT) dst[e] = reinterpret_cast<const float4 *>(sm)[e];
     if (threadIdx.x == 0) p.rows_m[g] = m;
@@ -504,10 +551,9 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
     int *ipq = reinterpret_cast<int *>(tlam + 32), *isel = ipq + D;   // Jacobi: pairs (p, q), selected columns
     float *rows_s = reinterpret_cast<float *>(isel + D);              // a batch of retained rows; then
     float *WS = rows_s;                                               // the workspace of the eigen-solvers
-    __shared__ int s_flag[2];
     __shared__ __align__(16) float kpart[2 * ALG_NG];                 // 2 buffers: the half-warps' shares of v . p
 
-    const int g = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int g = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = warp_uniform(tid >> 5);
     const int grp = tid >> 4, c16 = tid & 15;                         // half-warp and the lane in it
     int ci, lh;
     locate(p, g, ci, lh);
@@ -530,7 +576,7 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
     bool done = false;
 
     // ---- 1. k_eff >= d: the span test kernel has already factorised G_keep --
-    if (k >= D && (p.hflag[g] & HFLAG_SPAN_FULL)) { m = D; done = true; pc = 1.f; status |= OBF_DEV_SKIPPED | OBF_DEV_SPAN_FULL; }
+    if (warp_uniform(k >= D && (p.hflag[g] & HFLAG_SPAN_FULL) != 0u)) { m = D; done = true; pc = 1.f; status |= OBF_DEV_SKIPPED | OBF_DEV_SPAN_FULL; }
 
     if (!done) {
         const TIN *vk = reinterpret_cast<const TIN *>(c.v_out) + (size_t)lh * k * D;
@@ -559,23 +605,23 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
             for (int l = 0; l < U_LEVELS; ++l) uk[l] = 0.f;
 #pragma unroll 1
             for (int b0 = 0; b0 < k; b0 += 32) {
-                const float al = b0 + lane < k ? A[idx[b0 + lane]] : 0.f;
-#pragma unroll 1
-                for (int i0 = 0; i0 < 32; i0 += 16 * NPART) {
-                    float v[16];
+                // (the rows' loads are under way before the masses', which wait for the positions)
+                constexpr int PR = 32 / NPART;
+                float v[PR];
+                const int at = b0 + lane < k ? idx[b0 + lane] : 0;
 #pragma unroll
-                    for (int e = 0; e < 16; ++e) {
-                        const int i = b0 + i0 + e * NPART + part;
-                        v[e] = i < k ? to_f32(vk[(size_t)i * D + col]) : 0.f;
-                    }
+                for (int e = 0; e < PR; ++e) {
+                    const int i = b0 + e * NPART + part;
+                    v[e] = i < k ? to_f32(vk[(size_t)i * D + col]) : 0.f;
+                }
+                const float al = b0 + lane < k ? A[at] : 0.f;
 #pragma unroll
-                    for (int e = 0; e < 16; ++e) {
-                        const float a = __shfl_sync(0xffffffffu, al, i0 + e * NPART + part);
-                        const int lev = u_level(a);
-                        sq = fmaf(v[e], v[e], sq);
+                for (int e = 0; e < PR; ++e) {
+                    const float a = __shfl_sync(0xffffffffu, al, e * NPART + part);
+                    const int lev = u_level(a);
+                    sq = fmaf(v[e], v[e], sq);
 #pragma unroll
-                        for (int l = 0; l < U_LEVELS; ++l) uk[l] = fmaf(l == lev ? a : 0.f, v[e], uk[l]);
-                    }
+                    for (int l = 0; l < U_LEVELS; ++l) uk[l] = fmaf(l == lev ? a : 0.f, v[e], uk[l]);
                 }
             }
 #pragma unroll
@@ -612,12 +658,12 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
         };
         // ---- 2. reflectors of the retained rows, unless k_obf_rows has found them ----
         if (p.rows_y) {
-            m = p.rows_m[g];
+            m = warp_uniform(p.rows_m[g]);
             const float4 *src = reinterpret_cast<const float4 *>(p.rows_y + (size_t)g * p.alg_rows * D);
             for (int e = tid; e < m * (D / 4); e += ALG_NT) reinterpret_cast<float4 *>(Y)[e] = src[e];
             __syncthreads();
         } else {
-            m = alg_reflectors<TIN, D>(vk, k, Y, s_flag);
+            m = alg_reflectors<TIN, D>(vk, k, Y, WS);
         }
         // ---- G into registers, its trace, and the reflectors applied to it from both sides -----------------------
         AlgMat<D> M;
@@ -696,11 +742,11 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
             }
             float trM = block_sum<ALG_NT>(diag_part(m), red);
             rcr = del_negligible ? 0.f : trM / (trG + p.eps);
-            if (!(rcr >= RCR_SKIP_TOL)) { done = true; status |= OBF_DEV_SKIPPED; }
+            if (warp_uniform(!(rcr >= RCR_SKIP_TOL))) { done = true; status |= OBF_DEV_SKIPPED; }
             // What follows squares the block's entries, so a trace far from one (values of 1e-11 or 1e9, say) is brought there by a
             // power of two: exact, and C does not depend on it.  misc[10]: what one stands for from here on (read behind barriers).
             if (tid == 0) misc[10] = 1.f;
-            if (!done && !(trM > 1e-6f && trM < 1e6f)) {
+            if (!done && warp_uniform(!(trM > 1e-6f && trM < 1e6f))) {
                 const uint32_t e = min(max(__float_as_uint(trM) >> 23, 1u), 253u);
                 const float f = __uint_as_float((254u - e) << 23);
 #pragma unroll
@@ -711,92 +757,7 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                 if (tid == 0) misc[10] = __uint_as_float(e << 23);
             }
 
-            // Delta in the rotated coordinates (vx, all d of them, zero below m) -> delta, published and injected (Eq. 6-7).
-            // hi: the reflectors hi .. m + 1 and m - 1 .. 0 lead back.
-            auto finish_delta = [&](int hi) {
-                if (tid < D) pl[tid] = 0.f;
-                __syncthreads();
-                if (warp == 0) {
-                    // four reflectors per step: H_0 H_1 H_2 H_3 x needs the four products with x and the six among the
-                    // reflectors, whose reductions go through the half-warp together
-                    AlgRow<D> x;
-                    alg_load<D>(x, vx, c16);
-#pragma unroll 1
-                    for (int l = (hi > m ? hi - m : 0) + m - 1; l >= 0; l -= 4) {
-                        AlgRow<D> v[4];
-                        float d[16], dv[10];
-                        // v[0] is applied first; past the last one: zeros
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) alg_load<D>(v[e], l - e >= 0 ? Y + (l - e + (l - e >= m ? 1 : 0)) * D : pl, c16);
-#pragma unroll
-                        for (int e = 0; e < 16; ++e) d[e] = 0.f;
-                        // at e (e + 1) / 2: the products of v[e] with v[0] .. v[e - 1] and with x
-#pragma unroll
-                        for (int e = 0; e < 4; ++e)
-#pragma unroll
-                            for (int f = 0; f <= e; ++f) d[e * (e + 1) / 2 + f] = f < e ? alg_dot<D>(v[e], v[f]) : alg_dot<D>(v[e], x);
-                        const float tot = transposed_sum<16, 16>(d, c16);
-#pragma unroll
-                        for (int e = 0; e < 10; ++e) dv[e] = __shfl_sync(0xffffffffu, tot, (lane & 16) + e);
-                        const float s0 = -2.f * dv[0];
-                        const float s1 = -2.f * fmaf(s0, dv[1], dv[2]);
-                        const float s2 = -2.f * fmaf(s1, dv[4], fmaf(s0, dv[3], dv[5]));
-                        const float s3 = -2.f * fmaf(s2, dv[8], fmaf(s1, dv[7], fmaf(s0, dv[6], dv[9])));
-#pragma unroll
-                        for (int q = 0; q < NQ; ++q)
-                            x[q] = fma2(pk(s3, s3), v[3][q], fma2(pk(s2, s2), v[2][q], fma2(pk(s1, s1), v[1][q], fma2(pk(s0, s0), v[0][q], x[q]))));
-                    }
-#pragma unroll
-                    for (int q = 0; q < NQ; ++q) {
-                        x[q] = mul2(x[q], pk(alpha, alpha));
-                        if (grp == 0) *reinterpret_cast<f32x2 *>(vx + 32 * q + 2 * c16) = x[q];
-                    }
-                    const float dn = half_sum(alg_dot<D>(x, x));
-                    if (lane == 0) misc[9] = dn;
-                }
-                __syncthreads();
-                const float dn2 = misc[9];
-                dnorm = sqrtf(dn2);
-                if (!isfinite(dn2)) { status |= OBF_DEV_NONFINITE | OBF_DEV_SKIPPED; dnorm = 0.f; }
-                else if (rho == 0 || dn2 == 0.f) status |= OBF_DEV_SKIPPED;
-                else {
-                    if (tid < D) {
-                        p.delta[(size_t)g * D + tid] = vx[tid];
-                        if (c.delta_out) c.delta_out[(size_t)lh * D + tid] = vx[tid];
-                    }
-                    // Eq. 7: V_out = V_keep + delta on every retained row; the fp32 sum is rounded once.  Attn-inject
-                    // (App. D.2): row t takes k * A_t / (A_keep + eps) times delta instead
-                    constexpr int EPT = 16 / (int)sizeof(TIN);
-                    TIN *rows = reinterpret_cast<TIN *>(c.v_out) + (size_t)lh * k * D;
-                    const float share = (float)k / (a_keep + p.eps);
-                    for (int e0 = tid * EPT; e0 < k * D; e0 += ALG_NT * EPT) {
-                        const float wgt = p.attn_inject ? share * A[idx[e0 / D]] : 1.f;
-                        uint4 raw = *reinterpret_cast<const uint4 *>(rows + e0);
-                        const float *dl = vx + e0 % D;
-                        if constexpr (sizeof(TIN) == 4) {
-                            raw.x = __float_as_uint(fmaf(wgt, dl[0], __uint_as_float(raw.x)));
-                            raw.y = __float_as_uint(fmaf(wgt, dl[1], __uint_as_float(raw.y)));
-                            raw.z = __float_as_uint(fmaf(wgt, dl[2], __uint_as_float(raw.z)));
-                            raw.w = __float_as_uint(fmaf(wgt, dl[3], __uint_as_float(raw.w)));
-                        } else {
-                            uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
-#pragma unroll
-                            for (int q = 0; q < 4; ++q) {
-                                const float lo = fmaf(wgt, dl[2 * q], __uint_as_float(w[q] << 16));
-                                const float hi2 = fmaf(wgt, dl[2 * q + 1], __uint_as_float(w[q] & 0xFFFF0000u));
-                                w[q] = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(lo)) |
-                                       ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(hi2)) << 16);
-                            }
-                            raw = make_uint4(w[0], w[1], w[2], w[3]);
-                        }
-                        *reinterpret_cast<uint4 *>(rows + e0) = raw;
-                    }
-                    // the int8 copy that was made with the gather is of the rows before; every thread reads back what it wrote
-                    if (c.v_q8)
-                        for (int e0 = tid * EPT; e0 < k * D; e0 += ALG_NT * EPT)
-                            quantize16<TIN, D>(*reinterpret_cast<const uint4 *>(rows + e0), c.v_q8, c.v_scale, (size_t)lh * k + e0 / D, e0 % D / EPT);
-                }
-            };
+            int back = -1;                                         // the reflectors back .. m + 1 and m - 1 .. 0 lead back from the rotated coordinates
             const float inv_del = 1.f / (a_del + p.eps);
 
             // ---- 3a. few eigenpairs wanted: tridiagonal form, multisection, inverse iteration ----
@@ -887,6 +848,7 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                 __syncthreads();
                 const float l1 = tlam[0];
                 while (rho < rmax && tlam[rho] > EIG_RANK_TOL * l1 && tlam[rho] > 0.f) ++rho;
+                rho = warp_uniform(rho);
                 const float unit = misc[10];
                 lam1 = l1 * bound * unit;
                 lam_rho = rho > 0 ? tlam[rho - 1] * bound * unit : 0.f;
@@ -895,12 +857,13 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                 revr *= bound * unit / (trM * unit + p.eps);                         // trace of R^T R = sum of all its eigenvalues
                 bool clustered = false;
                 for (int t = 1; t < rho; ++t) clustered = clustered || tlam[t - 1] - tlam[t] <= EIG_CLUSTER_TOL * fabsf(l1);
+                clustered = warp_uniform(clustered);
                 // one warp, in order of the eigenvalues: orthogonal to the neighbours before it that are closer than tol, unit length
                 auto orthogonal = [&](float tol) __attribute__((always_inline)) {
                     for (int j = 1; j < rho; ++j) {
                         float *y = vec + (j * 6 + 5) * D;
                         for (int i2 = 0; i2 < j; ++i2) {
-                            if (fabsf(tlam[i2] - tlam[j]) > tol * fabsf(l1)) continue;
+                            if (warp_uniform(fabsf(tlam[i2] - tlam[j]) > tol * fabsf(l1))) continue;
                             const float *z = vec + (i2 * 6 + 5) * D;
                             float dsum = 0.f;
                             for (int cc = lane; cc < n; cc += 32) dsum = fmaf(y[cc], z[cc], dsum);
@@ -1013,7 +976,7 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                             }
                         }
                         const bool close = (e > 0 && tlam[e - 1] - lam < EIG_NEAR_TOL * l1) || (e + 1 < ne && lam - tlam[e + 1] < EIG_NEAR_TOL * l1);
-                        if (close) {                                   // (the same in every lane)
+                        if (warp_uniform(close)) {
                             // the step of inverse iteration: along both arms to the twist ..
                             float g = 0.f, mn = 0.f;
 #pragma unroll 1
@@ -1059,10 +1022,10 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                         if (lane == 0 && !(best * rsqrtf(n1) <= 2e-7f)) misc[7] = 1.f;
                     }
                     __syncthreads();
-                    clustered = misc[7] != 0.f;
+                    clustered = warp_uniform(misc[7] != 0.f);
                     bool near = false;
                     for (int t = 1; t < rho; ++t) near = near || tlam[t - 1] - tlam[t] < EIG_NEAR_TOL * l1;
-                    if (near && !clustered) {
+                    if (warp_uniform(near) && !clustered) {
                         if (warp == 0) orthogonal(EIG_NEAR_TOL);
                         __syncthreads();
                     }
@@ -1206,7 +1169,7 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                         for (int t = 0; t < rho; ++t) s = fmaf(vc[t], vec[(t * 6 + 5) * D + tid - m], s);
                     vx[tid] = s;
                 }
-                finish_delta(D - 2);
+                back = D - 2;
                 done = true;
             }
 
@@ -1287,7 +1250,7 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
 #pragma unroll
                             for (int q = 0; q < NQ; ++q) n1 = fmaf(y[q], y[q], n1);
                             n1 = warp_sum(n1);
-                            if (n1 > 1e-10f * n0 && n1 > 0.f) {
+                            if (warp_uniform(n1 > 1e-10f * n0 && n1 > 0.f)) {
                                 const float inv = rsqrtf(n1);
 #pragma unroll
                                 for (int q = 0; q < NQ; ++q) C[kept * D + 32 * q + lane] = y[q] * inv;
@@ -1297,7 +1260,7 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                         if (lane == 0) misc[6] = (float)kept;
                     }
                     __syncthreads();
-                    rho_f = (int)misc[6];
+                    rho_f = warp_uniform((int)misc[6]);
                 }
                 rho = rho_f;
                 // Rayleigh quotients of the rows (for the diagnostics), then Delta and delta
@@ -1322,7 +1285,7 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                     for (int t = 0; t < rho; ++t) sacc = fmaf(vc[t], C[t * D + tid], sacc);
                     vx[tid] = sacc;
                 }
-                finish_delta(0);
+                back = 0;
                 done = true;
             }
 
@@ -1479,7 +1442,174 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                     for (int t = 0; t < rho; ++t) s = fmaf(vc[t], U[tid * LD + isel[t]], s);
                     vx[tid] = s;
                 }
-                finish_delta(0);
+                back = 0;
+            }
+            // Delta in the rotated coordinates (vx, all d of them, zero below m) -> delta, published and injected (Eq. 6-7)
+            if (back >= 0) {
+                if (tid < D) pl[tid] = 0.f;
+                __syncthreads();
+                // (Four at a time, the products among them in the chain as well, 21000 cycles for 126 reflectors of 128 channels; so 17000.)
+                // Sixteen reflectors at a time: H_0 .. H_15 x = x + sum_e s_e v_e with s = -2 (I + 2 L)^-1 V x, L the strictly lower
+                // part of V V^T.  The triangular matrices of all groups first, a half-warp each; what is left in the chain of a
+                // group are its products with x, sixteen multiply-adds and the sum.  v[0] is applied first; past the last one: zeros.
+                const int count = (back > m ? back - m : 0) + m;
+                auto reflector = [&](int l) __attribute__((always_inline)) { return l >= 0 ? Y + (l + (l >= m ? 1 : 0)) * D : pl; };
+                constexpr int GR = 16, GSZ = GR * GR;
+                {
+                    float *Lg = WS + grp * GSZ;                    // product of v[e] and v[f] at [f][e]; then the inverse
+                    // the products on the tensor cores, a warp's two groups one after the other: the rows as sums of three bf16 parts (exact),
+                    // the six products of parts that fp32 can tell; a row's channels enter in an order that makes four of them one load
+                    const int fr = lane >> 2, fc = lane & 3;
+#pragma unroll 1
+                    for (int half = 0; half < 2; ++half) {
+                        const int first = 2 * warp + half, top = count - 1 - GR * first;
+                        if (top < 0) break;
+                        const float *r0 = reflector(top - fr) + 4 * fc, *r1 = reflector(top - fr - 8) + 4 * fc;
+                        float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+#pragma unroll 2
+                        for (int k0 = 0; k0 < D; k0 += 16) {
+                            const float4 u = *reinterpret_cast<const float4 *>(r0 + k0), w = *reinterpret_cast<const float4 *>(r1 + k0);
+                            float lo[4] = {u.x, w.x, u.z, w.z}, hi[4] = {u.y, w.y, u.w, w.w};
+                            uint32_t x[3][4];
+#pragma unroll
+                            for (int part = 0; part < 3; ++part)
+#pragma unroll
+                                for (int e = 0; e < 4; ++e) x[part][e] = split_bf16x2(lo[e], hi[e]);
+#pragma unroll
+                            for (int o = 0; o < 6; ++o) {
+                                constexpr int pa[6] = {2, 0, 1, 1, 0, 0}, pb[6] = {0, 2, 1, 0, 1, 0};
+                                mma_bf16(acc[0], x[pa[o]], x[pb[o]][0], x[pb[o]][2]);
+                                mma_bf16(acc[1], x[pa[o]], x[pb[o]][1], x[pb[o]][3]);
+                            }
+                        }
+                        float *to = WS + first * GSZ + fr * GR + 2 * fc;
+#pragma unroll
+                        for (int t = 0; t < 2; ++t) {
+                            *reinterpret_cast<float2 *>(to + 8 * t) = make_float2(acc[t][0], acc[t][1]);
+                            *reinterpret_cast<float2 *>(to + 8 * t + 8 * GR) = make_float2(acc[t][2], acc[t][3]);
+                        }
+                    }
+                    __syncwarp();
+                    // column c16 of the inverse, by forward substitution
+                    float t[GR];
+#pragma unroll
+                    for (int e = 0; e < GR; ++e) t[e] = e == c16 ? 1.f : 0.f;
+#pragma unroll
+                    for (int f = 0; f < GR; ++f) {
+                        t[f] *= -2.f;
+#pragma unroll
+                        for (int e = f + 1; e < GR; ++e) t[e] = fmaf(t[f], Lg[f * GR + e], t[e]);
+                    }
+                    __syncwarp();
+#pragma unroll
+                    for (int e = 0; e < GR; ++e) Lg[e * GR + c16] = t[e];
+                }
+                __syncthreads();
+                if (warp == 0) {
+                    constexpr int PER = D / 32;                    // a lane's entries
+                    typedef typename std::conditional<PER == 4, float4, float2>::type Vec;
+                    float x[PER];
+                    auto load = [&](float (&v)[PER], const float *from) __attribute__((always_inline)) {
+                        *reinterpret_cast<Vec *>(v) = *reinterpret_cast<const Vec *>(from + PER * lane);
+                    };
+                    load(x, vx);
+#pragma unroll 1
+                    for (int g0 = 0; g0 * GR < count; ++g0) {
+                        float v[GR][PER], d[GR], row[GR];
+#pragma unroll
+                        for (int e = 0; e < GR; ++e) load(v[e], reflector(count - 1 - GR * g0 - e));
+#pragma unroll
+                        for (int e = 0; e < GR; e += 4) {
+                            const float4 t = *reinterpret_cast<const float4 *>(WS + g0 * GSZ + (lane >> 1) * GR + e);
+                            row[e] = t.x; row[e + 1] = t.y; row[e + 2] = t.z; row[e + 3] = t.w;
+                        }
+#pragma unroll
+                        for (int e = 0; e < GR; ++e) {
+                            d[e] = 0.f;
+#pragma unroll
+                            for (int q = 0; q < PER; ++q) d[e] = fmaf(v[e][q], x[q], d[e]);
+                        }
+                        const float tot = transposed_sum<GR, 32>(d, lane);         // v[lane / 2] . x
+                        float sa = 0.f, sb = 0.f;
+#pragma unroll
+                        for (int e = 0; e < GR; e += 2) {
+                            sa = fmaf(row[e], __shfl_sync(0xffffffffu, tot, 2 * e), sa);
+                            sb = fmaf(row[e + 1], __shfl_sync(0xffffffffu, tot, 2 * e + 2), sb);
+                        }
+                        sa += sb;
+#pragma unroll
+                        for (int e = 0; e < GR; ++e) {
+                            const float f = __shfl_sync(0xffffffffu, sa, 2 * e);
+#pragma unroll
+                            for (int q = 0; q < PER; ++q) x[q] = fmaf(f, v[e][q], x[q]);
+                        }
+                    }
+                    float dn = 0.f;
+#pragma unroll
+                    for (int q = 0; q < PER; ++q) {
+                        x[q] *= alpha;
+                        dn = fmaf(x[q], x[q], dn);
+                    }
+                    *reinterpret_cast<Vec *>(vx + PER * lane) = *reinterpret_cast<const Vec *>(x);
+                    dn = warp_sum(dn);
+                    if (lane == 0) misc[9] = dn;
+                }
+                __syncthreads();
+                const float dn2 = misc[9];
+                dnorm = sqrtf(dn2);
+                if (!isfinite(dn2)) { status |= OBF_DEV_NONFINITE | OBF_DEV_SKIPPED; dnorm = 0.f; }
+                else if (rho == 0 || dn2 == 0.f) status |= OBF_DEV_SKIPPED;
+                else {
+                    if (tid < D) {
+                        p.delta[(size_t)g * D + tid] = vx[tid];
+                        if (c.delta_out) c.delta_out[(size_t)lh * D + tid] = vx[tid];
+                    }
+                    // Eq. 7: V_out = V_keep + delta on every retained row; the fp32 sum is rounded once.  Attn-inject
+                    // (App. D.2): row t takes k * A_t / (A_keep + eps) times delta instead
+                    constexpr int EPT = 16 / (int)sizeof(TIN);
+                    TIN *rows = reinterpret_cast<TIN *>(c.v_out) + (size_t)lh * k * D;
+                    const float share = (float)k / (a_keep + p.eps);
+                    // (four vectors a thread in flight)
+#pragma unroll 1
+                    for (int b0 = tid * EPT; b0 < k * D; b0 += 4 * ALG_NT * EPT) {
+                        uint4 in[4];
+                        float wgt[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const int e0 = b0 + u * ALG_NT * EPT;
+                            in[u] = e0 < k * D ? *reinterpret_cast<const uint4 *>(rows + e0) : make_uint4(0u, 0u, 0u, 0u);
+                            wgt[u] = p.attn_inject && e0 < k * D ? share * A[idx[e0 / D]] : 1.f;
+                        }
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const int e0 = b0 + u * ALG_NT * EPT;
+                            if (e0 >= k * D) break;
+                            uint4 raw = in[u];
+                            const float *dl = vx + e0 % D;
+                            if constexpr (sizeof(TIN) == 4) {
+                                raw.x = __float_as_uint(fmaf(wgt[u], dl[0], __uint_as_float(raw.x)));
+                                raw.y = __float_as_uint(fmaf(wgt[u], dl[1], __uint_as_float(raw.y)));
+                                raw.z = __float_as_uint(fmaf(wgt[u], dl[2], __uint_as_float(raw.z)));
+                                raw.w = __float_as_uint(fmaf(wgt[u], dl[3], __uint_as_float(raw.w)));
+                            } else {
+                                uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
+#pragma unroll
+                                for (int q = 0; q < 4; ++q) {
+                                    const float lo = fmaf(wgt[u], dl[2 * q], __uint_as_float(w[q] << 16));
+                                    const float hi2 = fmaf(wgt[u], dl[2 * q + 1], __uint_as_float(w[q] & 0xFFFF0000u));
+                                    w[q] = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(lo)) |
+                                           ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(hi2)) << 16);
+                                }
+                                raw = make_uint4(w[0], w[1], w[2], w[3]);
+                            }
+                            *reinterpret_cast<uint4 *>(rows + e0) = raw;
+                        }
+                    }
+                    // the int8 copy that was made with the gather is of the rows before; every thread reads back what it wrote
+                    if (c.v_q8)
+                        for (int e0 = tid * EPT; e0 < k * D; e0 += ALG_NT * EPT)
+                            quantize16<TIN, D>(*reinterpret_cast<const uint4 *>(rows + e0), c.v_q8, c.v_scale, (size_t)lh * k + e0 / D, e0 % D / EPT);
+                }
             }
             }
     }

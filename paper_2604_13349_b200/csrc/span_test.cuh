@@ -53,13 +53,6 @@ constexpr size_t span_smem_bytes(bool from_rows)
     return (panels > rows ? panels : rows) + D * sizeof(float);
 }
 
-__device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
-{
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
 // 16 values as upper, middle and lower bf16 parts (whose sum is the value), 32 bytes each.
 __device__ __forceinline__ void store_parts(uint8_t *dst, const float (&x)[16])
 {
@@ -70,13 +63,7 @@ __device__ __forceinline__ void store_parts(uint8_t *dst, const float (&x)[16])
         for (int e = 0; e < 4; ++e) {
             float a = x[8 * h + 2 * e], b = x[8 * h + 2 * e + 1];
 #pragma unroll
-            for (int part = 0; part < 3; ++part) {
-                uint32_t r;
-                asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(b), "f"(a));
-                w[part][e] = r;
-                a -= __uint_as_float(r << 16);
-                b -= __uint_as_float(r & 0xFFFF0000u);
-            }
+            for (int part = 0; part < 3; ++part) w[part][e] = split_bf16x2(a, b);
         }
 #pragma unroll
         for (int part = 0; part < 3; ++part)
