@@ -20,7 +20,9 @@
 //      reflectors simply go on: H_{m+1} .. H_{d-2} take the trailing block to tridiagonal form (so the basis and the
 //      tridiagonal form together cost the d - 2 steps that the tridiagonal form of the full matrix would), the wanted
 //      eigenvalues come from multisection on Sturm counts, their vectors from twisted factorisations (neighbours closer
-//      than 1e-3 of the largest eigenvalue: from inverse iteration, kept orthogonal during it).  For larger ranks: full
+//      than 1e-3 of the largest eigenvalue: from inverse iteration, kept orthogonal during it).  Heads of 128 channels stop as
+//      soon as the first rows of the tridiagonal form provably hold the wanted eigenvalues and the next one, with their vectors, to
+//      rounding: 24 to 36 rows of 96 where the spectrum falls off, and as many reflectors fewer on the way back.  For larger ranks: full
 //      eigen-decomposition by parallel-order Jacobi rotations run to convergence.
 //   4. Delta = C^T C r_bar (Eq. 5) in the rotated coordinates, taken back through the reflectors as ONE vector,
 //      delta = A_del / (A_keep + eps) * Delta (Eq. 6), V_out = V_keep + delta on the head's retained rows (Eq. 7).
@@ -32,8 +34,11 @@
 // stages of 32 so that finished rows and column pairs cost nothing and every register index is static.  128 threads of
 // 255 registers and less than 113 KB per block: two blocks share a multiprocessor.  What is run once per head is written
 // as small loops: a section's first pass costs about 130 cycles per 128 bytes of its code, more than its arithmetic.
-// Measured on 36 x 8 heads, budget 32, rank 2, head_dim 128 (every head back-filled): 0.141 ms against 0.534 ms for the
-// same algebra on a matrix in shared memory (Gram-Schmidt basis, M = P G P, then the reduction).  Slower were: eight warps
+// Measured on 36 x 8 heads, budget 32, rank 2, head_dim 128 (every head back-filled): 0.534 ms for the
+// same algebra on a matrix in shared memory (Gram-Schmidt basis, M = P G P, then the reduction), 0.142 with all rows of the tridiagonal
+// form, 0.107 (values whose channels fall off; 219 -> 185 us a call; three outlier channels, rank 1 and 2, 217 -> 182 and 220 -> 203; flat
+// values, rank 1, 219 -> 228, for the questions, ranks 2 and 4 the same).  Slower were: one barrier a row of the form, as for the retained rows
+// (622 to 1400 cycles a row against 690 to 1210: more instructions), eight warps
 // with half the registers, the chain of reflectors in a warp of its own beside the matrix warps (the registers it takes cost
 // the others more), one copy of the step's code for all stages, the reflectors on G sixteen at a time in compact form (code
 // that runs twice costs more to fetch than it saves), the auxiliary vector or the next row's norm in one warp only.
@@ -55,6 +60,9 @@ constexpr float EIG_RANK_TOL = 1e-5f;
 constexpr int JACOBI_MAX_SWEEPS = 30;
 constexpr int ALG_TRI_MAX_RANK = 8;     // up to this rank only rank + 1 eigenvalues and rank eigenvectors are computed
 constexpr float EIG_CLUSTER_TOL = 1e-3f; // eigenvalues closer than this (relative to the largest): inverse iteration, kept orthogonal during it
+// Rows of the tridiagonal form after which it is asked whether they suffice, and how many more at least before it is asked again (a
+// quarter of them where that is more, half where the rest is far too large).  The question costs 2000 cycles where the answer is no for the rest's sake, 4500 else, a row 850 to 1600.
+constexpr int ALG_EXIT_FIRST = 18, ALG_EXIT_STEP = 6;
 constexpr float EIG_NEAR_TOL = 5e-2f;    // closer than this: one more step of inverse iteration on the twisted factors, then made orthogonal
 
 // a where the mask is all ones, b where it is zero.  (A conditional between array elements would be a conditional
@@ -493,7 +501,9 @@ __device__ __forceinline__ int alg_reflectors(const TIN *vk, int k, float *Y, fl
 #pragma unroll
             for (int s = 0; s < NS; ++s) f[s] = b * fmaf(alg_entry<D>(V[s], m, lane), first, __shfl_sync(0xffffffffu, tot, (lane & 16) + 4 + 2 * s));
             if (add && grp == i % ALG_NG) {
-                const float rs = rsqrt_approx(2.f * h);
+                // (to the last bit: the rows have met w, whose length is exact, G and the vectors will meet this)
+                float rs = rsqrt_approx(2.f * h);
+                rs *= fmaf(-h * rs, rs, 1.5f);
 #pragma unroll
                 for (int q = 0; q < NQ; ++q) *reinterpret_cast<f32x2 *>(Y + m * D + 32 * q + 2 * c16) = mul2(w[q], pk(rs, rs));
             }
@@ -695,6 +705,19 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
             return s;
         };
 
+        // and of the squares of the trailing block from row and column `from` on
+        auto square_part = [&](int from) __attribute__((always_inline)) {
+            float s = 0.f;
+#pragma unroll
+            for (int r = 0; r < RW; ++r) {
+                AlgRow<D> x;
+                alg_masked<D>(x, M[r], from, c16);
+                const float t = sum2(fma2(x[0], x[0], NQ > 1 ? mul2(x[1], x[1]) : 0ull)), u = NQ > 2 ? sum2(fma2(x[NQ - 2], x[NQ - 2], mul2(x[NQ - 1], x[NQ - 1]))) : 0.f;
+                if (SH::row(grp, r) >= from) s += t + u;
+            }
+            return s;
+        };
+
         const float trAll = block_sum<ALG_NT>(diag_part(0), red);
         // squared Frobenius norm of the deleted values (the denominator of RCR).  As a difference of two fp32 traces
         // it is resolved down to about 1e-6 of the squared norm of all values: below 1e-5 of it the deleted values
@@ -763,7 +786,13 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
             // ---- 3a. few eigenpairs wanted: tridiagonal form, multisection, inverse iteration ----
             if (!done && p.fast_iters == 0 && p.rank <= ALG_TRI_MAX_RANK) {
                 const float tiny2 = 1e-20f * trM * trM;
-                const int n = D - m;                                   // size of the trailing block
+                int n = D - m;                                         // size of the trailing block, then of the tridiagonal form
+                // Whether its first rows suffice is asked first after as many as spectra that fall off take, and never for the last few (heads
+                // of 64 channels, not at all: the code costs them as much as it saves, 16 x 8 heads with 32 rows, rank 2, 116.3 -> 119.7 us).
+                constexpr bool ASKS = D > 64;
+                int last = ASKS ? m + ALG_EXIT_FIRST - 1 + (p.rank > 1 ? ALG_EXIT_STEP : 0) + (p.rank > 2 ? ALG_EXIT_STEP : 0) : D;
+                float m2 = 0.f;                                        // squared Frobenius norm of the block
+                if (ASKS && last <= D - 2 - 2 * ALG_EXIT_STEP) m2 = block_sum<ALG_NT>(square_part(m), red);
                 if (n > 1) {
                     // reflector m + 1 from row m as it stands
                     AlgRow<D> x;
@@ -775,11 +804,13 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                     }
                     alg_row_done<D, 0>(x, m, tiny2, Y, ta, tb, grp, lane);
                 }
-                auto reduce_stage = [&](auto stage) __attribute__((always_inline)) {
+                int J = m + 1;                                         // the next step's reflector
+                auto reduce_stage = [&](auto stage, int last) __attribute__((always_inline)) {
                     constexpr int ST = decltype(stage)::value;
-                    const int j1 = min(32 * ST + 31, D - 2);
+                    const int j1 = min(32 * ST + 31, last);
 #pragma unroll 1
-                    for (int j = max(m + 1, 32 * ST); j <= j1; ++j) {
+                    for (; J <= j1; ++J) {
+                        const int j = J;
                         float *po = pl + (j & 1) * D, *kp = kpart + (j & 1) * ALG_NG;
                         AlgRow<D> v, x;
                         __syncthreads();                               // reflector j is there
@@ -795,13 +826,102 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                         alg_row_done<D, ST>(x, j, tiny2, Y, ta, tb, grp, lane);
                     }
                 };
-                reduce_stage(std::integral_constant<int, 0>{});
-                reduce_stage(std::integral_constant<int, 1>{});
-                if constexpr (D > 64) {
-                    reduce_stage(std::integral_constant<int, D / 32 - 2>{});
-                    reduce_stage(std::integral_constant<int, D / 32 - 1>{});
-                }
-                {
+                float *sa = WS, *sb2 = WS + D + 8, *vec = WS + 2 * (D + 8);   // vec: per wanted eigenvector dd, dl, du, du2, pv, y of D each
+                // Whether the J - m rows of the tridiagonal form so far hold the wanted eigenpairs and the next one (2, else 1, or 0 where it
+                // will take many more).  With sigma just
+                // below the next one, M has as many eigenvalues above sigma as the leading part T (Sylvester, block elimination of T - sigma)
+                // if the rest, R + b b^T / |d|, has none: b is the coupling to the rest, d < 0 the last pivot of T - sigma.  The largest
+                // eigenvalue of R follows from its trace and Frobenius norm, which are those of M less T's:
+                //   lambda <= t / N + sqrt((N - 1) / N (f^2 - t^2 / N)).
+                // And their vectors' last entries, times the coupling, have to be nothing beside rounding: from the recurrence for the
+                // vector upwards from its last entry, at both ends of the interval that holds the eigenvalue.
+                auto leading_part_suffices = [&]() __attribute__((always_inline)) {
+                    const int sz = warp_uniform(J - m), r = min(p.rank, D);
+                    const float *da = ta + m, *db = tb + m;
+                    __syncthreads();                                   // the entries are there
+                    float s1 = 0.f, s2 = 0.f, gb = 0.f;
+                    for (int i = lane; i < sz; i += 32) {
+                        s1 += da[i];
+                        s2 = fmaf(da[i], da[i], fmaf(2.f * db[i], db[i], s2));
+                        gb = fmaxf(gb, fabsf(da[i]) + (i > 0 ? fabsf(db[i - 1]) : 0.f) + (i + 1 < sz ? fabsf(db[i]) : 0.f));
+                    }
+                    s1 = warp_sum(s1);
+                    s2 = warp_sum(s2);
+                    gb = fmaxf(warp_max(gb), 1e-30f);
+                    const float scl = 1.f / gb, nr = (float)(D - J), t = trM - s1, f2 = m2 - s2 + 1e-5f * m2;
+                    const float rest = (t / nr + sqrtf((nr - 1.f) / nr * fmaxf(f2 - t * t / nr, 0.f)) + 1e-5f * trM / nr) * scl, cb = fabsf(db[sz - 1]) * scl;
+                    float *vb = vec + 4, *vi = vb + D + 4;             // couplings (a zero before and after them) and their reciprocals
+                    const int n4 = (sz + 3) / 4;
+                    if (tid < 4 * n4) {
+                        const float b = (tid > 0 && tid < sz) ? db[tid - 1] * scl : 0.f;
+                        sa[tid] = tid < sz ? da[tid] * scl : 2.f;
+                        sb2[tid] = (tid > 0 && tid < sz) ? fmaxf(b * b, 1e-14f) : 0.f;
+                        vb[tid - 1] = b;
+                        if (tid > 0) vi[tid - 1] = 1.f / b;
+                        if (tid + 1 == sz) vb[tid] = 0.f;
+                    }
+                    __syncthreads();
+                    constexpr float STEP = 1.f / (2 * ALG_NT + 1);
+                    uint16_t *cnt = reinterpret_cast<uint16_t *>(ipq);
+                    int c0, c1;
+                    sturm_count2(sa, sb2, n4, STEP * (2 * tid + 1), STEP * (2 * tid + 2), c0, c1);
+                    cnt[tid] = (uint16_t)(c0 | c1 << 8);
+                    __syncthreads();
+                    int nw = 0, nx = 0;                                // shifts not above the last wanted and the next eigenvalue
+#pragma unroll
+                    for (int i = 0; i < ALG_NW; ++i) {
+                        const uint32_t two = cnt[lane + 32 * i];
+                        const int a = two & 255, b = two >> 8;
+                        nw += (a <= sz - r ? 1 : 0) + (b <= sz - r ? 1 : 0);
+                        nx += (a <= sz - 1 - r ? 1 : 0) + (b <= sz - 1 - r ? 1 : 0);
+                    }
+                    nw = __reduce_add_sync(0xffffffffu, nw);
+                    nx = __reduce_add_sync(0xffffffffu, nx);
+                    if (!warp_uniform(nx > 0 && rest * 1.0001f < STEP * (float)nx)) return warp_uniform(rest > 1.3f * STEP * (float)nx) ? 0 : 1;
+                    // lanes 0 .. 3: upwards, at the ends of both intervals; lane 4: downwards at sigma, for the last pivot
+                    const bool down = lane == 4;
+                    const float sg = STEP * (float)(down ? nx : (lane & 2 ? nx : nw) + (lane & 1));
+                    float y1 = 1.f, y0 = 0.f, top = 1.f;
+                    const int by = down ? 1 : -1;
+                    const float *pa = down ? sa : sa + sz - 1, *pb = down ? vb - 1 : vb + sz - 1, *pi = down ? vi : vi + sz - 2;
+#pragma unroll 4
+                    for (int k = 1; k < sz; ++k, pa += by, pb += by, pi += by) {
+                        const float y = -fmaf(*pa - sg, y1, *pb * y0) * *pi;
+                        const float f = down && fabsf(y) > 1e20f ? 1e-20f : 1.f;           // (downwards the quotient counts)
+                        if (top < 1e25f) {
+                            y0 = y1 * f;
+                            y1 = y * f;
+                            top = fmaxf(top, fabsf(y1));
+                        }
+                    }
+                    const float d = (sa[sz - 1] - sg) + vb[sz - 2] * (y0 / y1);
+                    const float d4 = __shfl_sync(0xffffffffu, d, 4), s4 = __shfl_sync(0xffffffffu, sg, 4), t4 = __shfl_sync(0xffffffffu, top, 4);
+                    const bool gone = lane < 2 ? cb <= 1e-9f * top : lane < 4 ? cb <= 3e-5f * top : true;
+                    return warp_uniform(t4 < 1e25f && d4 < 0.f && (rest - cb * cb / d4) * 1.0001f < s4) && __all_sync(0xffffffffu, gone) ? 2 : 1;
+                };
+                int early = 0, more;
+#pragma unroll 1
+                do {
+                    if (last > D - 2 - 2 * ALG_EXIT_STEP) last = D - 2;
+                    reduce_stage(std::integral_constant<int, 0>{}, last);
+                    reduce_stage(std::integral_constant<int, 1>{}, last);
+                    if constexpr (D > 64) {
+                        reduce_stage(std::integral_constant<int, D / 32 - 2>{}, last);
+                        reduce_stage(std::integral_constant<int, D / 32 - 1>{}, last);
+                    }
+                    more = 0;
+                    if (ASKS && last < D - 2) {
+                        const int answer = leading_part_suffices();
+                        early = answer == 2 ? 1 : 0;
+                        more = 1 - early;
+                        last += max(ALG_EXIT_STEP, (J - m) / (answer ? 4 : 2));
+                    }
+                    more = warp_uniform(more);
+                } while (more);
+                early = warp_uniform(early);
+                const int through = warp_uniform(early ? J - 1 : D - 2);     // the last reflector of the form
+                n = warp_uniform(early ? J - m : n);
+                if (!early) {
                     // the last diagonal entry
                     float a, b;
                     upk(M[RW - 1][NQ - 1], a, b);
@@ -820,7 +940,6 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                 float gb = 0.f;
                 if (tid < n) gb = fabsf(da[tid]) + (tid > 0 ? fabsf(db[tid - 1]) : 0.f) + (tid < n - 1 ? fabsf(db[tid]) : 0.f);
                 const float bound = fmaxf(block_max<ALG_NT>(gb, red), 1e-30f), scl = 1.f / bound;
-                float *sa = WS, *sb2 = WS + D + 8, *vec = WS + 2 * (D + 8);   // vec: per wanted eigenvector dd, dl, du, du2, pv, y of D each
                 if (tid < 4 * n4) {
                     sa[tid] = tid < n ? da[tid] * scl : 2.f;
                     const float b = (tid > 0 && tid < n) ? db[tid - 1] * scl : 0.f;        // couples tid - 1 and tid
@@ -891,13 +1010,19 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                     // EIG_NEAR_TOL one step of inverse iteration with the same factors squares that away, down to what T's own
                     // rounding leaves, at two multiply-adds per entry and no division, and wanted neighbours are made orthogonal.
                     // Farther ones leave less than 1e-6.  Each lane's operands lie in the order it needs them, four to a load.
+                    // (Every lane computes, even ones the upper arm and odd ones the lower, and two of them store: a warp that enters a loop
+                    // with two lanes only pays for it at every shuffle behind.)
                     constexpr float PIV = 1e-10f;
+                    constexpr int PL = D / 32;                         // entries a lane holds
+                    const bool lower = lane & 1;
                     if (tid == 0) misc[7] = 0.f;
                     __syncthreads();
                     for (int e = warp; e < rho; e += ALG_NW) {
                         float *pa = vec + e * 6 * D, *pb = pa + D, *qa = pb + D, *qb = qa + D, *y = pa + 5 * D;
                         const float lam = tlam[e];
-                        for (int i = lane; i < 4 * n4; i += 32) {
+#pragma unroll
+                        for (int q = 0; q < PL; ++q) {
+                            const int i = lane + 32 * q;
                             const bool on = i < n - 1;
                             const float bu = on ? db[i] * scl : 0.f, bd = on ? db[n - 2 - i] * scl : 0.f;
                             pa[i] = i < n ? sa[i] - lam : 1.f;
@@ -906,9 +1031,9 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                             qb[i] = bd * bd;
                         }
                         __syncwarp();
-                        if (lane < 2) {
-                            float *a = lane ? qa : pa;
-                            const float *b = lane ? qb : pb;
+                        {
+                            float *a = lower ? qa : pa;
+                            const float *b = lower ? qb : pb;
                             float4 an = *reinterpret_cast<const float4 *>(a);
                             float d = an.x;
 #pragma unroll 1
@@ -923,14 +1048,16 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                                     o[q] = d;
                                     d = fmaf(-bx[q], rcp_approx(d), ax[q]);
                                 }
-                                *reinterpret_cast<float4 *>(a + 4 * t) = make_float4(o[0], o[1], o[2], o[3]);
+                                if (lane < 2) *reinterpret_cast<float4 *>(a + 4 * t) = make_float4(o[0], o[1], o[2], o[3]);
                             }
                         }
                         __syncwarp();
                         float best = INFINITY;
                         int at = 0;
-                        for (int i = lane; i < n; i += 32) {
-                            const float gm = fabsf(pa[i] + qa[n - 1 - i] - (sa[i] - lam));
+#pragma unroll
+                        for (int q = 0; q < PL; ++q) {
+                            const int i = lane + 32 * q;
+                            const float gm = i < n ? fabsf(pa[i] + qa[n - 1 - i] - (sa[i] - lam)) : INFINITY;
                             if (gm < best) { best = gm; at = i; }
                         }
 #pragma unroll
@@ -941,7 +1068,6 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                         }
                         // the multipliers along both arms and the pivots' reciprocals, from the twist outwards
                         const float gam = pa[at] + qa[n - 1 - at] - (sa[at] - lam);
-                        constexpr int PL = D / 32;                     // entries a lane holds
                         float rt[PL], rb[PL];
 #pragma unroll
                         for (int q = 0; q < PL; ++q) {
@@ -959,10 +1085,10 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                             qb[i] = w < n ? -db[w - 1] * scl * rb[q] : 0.f;
                         }
                         __syncwarp();
-                        // lanes 0 and 1 take an arm each (what they learn of one another passes through the whole warp)
-                        const float *mu = lane ? qb : pb, *rc = lane ? qa : pa;
-                        float *x = lane ? y : pa + 4 * D;
-                        const int len = lane > 1 ? 0 : lane ? n - 1 - at : at;
+                        const float *mu = lower ? qb : pb, *rc = lower ? qa : pa;
+                        float *x = lower ? y : pa + 4 * D;
+                        // (both arms as far as the longer one: what lies behind an arm's end is zero)
+                        const int len = warp_uniform(max(n - 1 - at, at));
                         float n1 = 0.f, z = 1.f;                       // n1: squares of the first vector's entries; z: the entry at the twist
                         {
                             float c = 1.f;
@@ -972,7 +1098,7 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                                 float4 o;
                                 o.x = mv.x * c; o.y = mv.y * o.x; o.z = mv.z * o.y; c = o.w = mv.w * o.z;
                                 n1 = fmaf(o.x, o.x, fmaf(o.y, o.y, fmaf(o.z, o.z, fmaf(o.w, o.w, n1))));
-                                *reinterpret_cast<float4 *>(x + t) = o;
+                                if (lane < 2) *reinterpret_cast<float4 *>(x + t) = o;
                             }
                         }
                         const bool close = (e > 0 && tlam[e - 1] - lam < EIG_NEAR_TOL * l1) || (e + 1 < ne && lam - tlam[e + 1] < EIG_NEAR_TOL * l1);
@@ -985,7 +1111,7 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                                 float4 o;
                                 o.w = fmaf(mn, g, xv.w); o.z = fmaf(mv.w, o.w, xv.z); o.y = fmaf(mv.z, o.z, xv.y); g = o.x = fmaf(mv.y, o.y, xv.x);
                                 mn = mv.x;
-                                *reinterpret_cast<float4 *>(x + t) = o;
+                                if (lane < 2) *reinterpret_cast<float4 *>(x + t) = o;
                             }
                             g *= mn;
                             __syncwarp();
@@ -999,7 +1125,7 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                                 float4 o;
                                 o.x = fmaf(mv.x, c, xv.x * rv.x); o.y = fmaf(mv.y, o.x, xv.y * rv.y);
                                 o.z = fmaf(mv.z, o.y, xv.z * rv.z); c = o.w = fmaf(mv.w, o.z, xv.w * rv.w);
-                                *reinterpret_cast<float4 *>(x + t) = o;
+                                if (lane < 2) *reinterpret_cast<float4 *>(x + t) = o;
                             }
                         }
                         __syncwarp();
@@ -1165,11 +1291,11 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                 __syncthreads();
                 if (tid < D) {
                     float s = 0.f;
-                    if (tid >= m)
+                    if (tid >= m && tid < m + n)
                         for (int t = 0; t < rho; ++t) s = fmaf(vc[t], vec[(t * 6 + 5) * D + tid - m], s);
                     vx[tid] = s;
                 }
-                back = D - 2;
+                back = through;
                 done = true;
             }
 
@@ -1445,6 +1571,7 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                 back = 0;
             }
             // Delta in the rotated coordinates (vx, all d of them, zero below m) -> delta, published and injected (Eq. 6-7)
+            back = warp_uniform(back);
             if (back >= 0) {
                 if (tid < D) pl[tid] = 0.f;
                 __syncthreads();
@@ -1453,40 +1580,30 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                 // part of V V^T.  The triangular matrices of all groups first, a half-warp each; what is left in the chain of a
                 // group are its products with x, sixteen multiply-adds and the sum.  v[0] is applied first; past the last one: zeros.
                 const int count = (back > m ? back - m : 0) + m;
-                auto reflector = [&](int l) __attribute__((always_inline)) { return l >= 0 ? Y + (l + (l >= m ? 1 : 0)) * D : pl; };
+                const int zero = algebra_y_rows<D>(p.alg_rows, p.rank, p.fast_iters);       // (pl follows Y)
+                auto reflector = [&](int l) __attribute__((always_inline)) { return Y + (l < 0 ? zero : l + (l >= m ? 1 : 0)) * D; };
                 constexpr int GR = 16, GSZ = GR * GR;
                 {
-                    float *Lg = WS + grp * GSZ;                    // product of v[e] and v[f] at [f][e]; then the inverse
-                    // the products on the tensor cores, a warp's two groups one after the other: the rows as sums of three bf16 parts (exact),
-                    // the six products of parts that fp32 can tell; a row's channels enter in an order that makes four of them one load
-                    const int fr = lane >> 2, fc = lane & 3;
+                    const int first = count - 1 - GR * grp;        // of this half-warp's group
+                    float *Lg = WS + grp * GSZ;                    // product of v[e] and v[f], f < e, at [f][e]; then the inverse
 #pragma unroll 1
-                    for (int half = 0; half < 2; ++half) {
-                        const int first = 2 * warp + half, top = count - 1 - GR * first;
-                        if (top < 0) break;
-                        const float *r0 = reflector(top - fr) + 4 * fc, *r1 = reflector(top - fr - 8) + 4 * fc;
-                        float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-#pragma unroll 2
-                        for (int k0 = 0; k0 < D; k0 += 16) {
-                            const float4 u = *reinterpret_cast<const float4 *>(r0 + k0), w = *reinterpret_cast<const float4 *>(r1 + k0);
-                            float lo[4] = {u.x, w.x, u.z, w.z}, hi[4] = {u.y, w.y, u.w, w.w};
-                            uint32_t x[3][4];
+                    for (int f0 = 0; f0 < GR && 2 * GR * warp < count; f0 += 8) {
+                        AlgRow<D> vf[8];
 #pragma unroll
-                            for (int part = 0; part < 3; ++part)
+                        for (int f = 0; f < 8; ++f) alg_load<D>(vf[f], reflector(first - f0 - f), c16);
+#pragma unroll 1
+                        for (int e = f0 + 1; e < GR; e += 2) {     // two rows at a time: their sums travel together
+                            AlgRow<D> v, w;
+                            float d[16];
+                            alg_load<D>(v, reflector(first - e), c16);
+                            alg_load<D>(w, reflector(first - e - 1), c16);
 #pragma unroll
-                                for (int e = 0; e < 4; ++e) x[part][e] = split_bf16x2(lo[e], hi[e]);
-#pragma unroll
-                            for (int o = 0; o < 6; ++o) {
-                                constexpr int pa[6] = {2, 0, 1, 1, 0, 0}, pb[6] = {0, 2, 1, 0, 1, 0};
-                                mma_bf16(acc[0], x[pa[o]], x[pb[o]][0], x[pb[o]][2]);
-                                mma_bf16(acc[1], x[pa[o]], x[pb[o]][1], x[pb[o]][3]);
+                            for (int f = 0; f < 8; ++f) {
+                                d[f] = alg_dot<D>(v, vf[f]);
+                                d[8 + f] = alg_dot<D>(w, vf[f]);
                             }
-                        }
-                        float *to = WS + first * GSZ + fr * GR + 2 * fc;
-#pragma unroll
-                        for (int t = 0; t < 2; ++t) {
-                            *reinterpret_cast<float2 *>(to + 8 * t) = make_float2(acc[t][0], acc[t][1]);
-                            *reinterpret_cast<float2 *>(to + 8 * t + 8 * GR) = make_float2(acc[t][2], acc[t][3]);
+                            const float tot = transposed_sum<16, 16>(d, c16);
+                            if (e + (c16 >> 3) < GR) Lg[(f0 + (c16 & 7)) * GR + e + (c16 >> 3)] = tot;
                         }
                     }
                     __syncwarp();
@@ -1496,9 +1613,15 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                     for (int e = 0; e < GR; ++e) t[e] = e == c16 ? 1.f : 0.f;
 #pragma unroll
                     for (int f = 0; f < GR; ++f) {
+                        float g[GR];
+#pragma unroll
+                        for (int e = (f + 1) & ~3; e < GR; e += 4) {
+                            const float4 u = *reinterpret_cast<const float4 *>(Lg + f * GR + e);
+                            g[e] = u.x; g[e + 1] = u.y; g[e + 2] = u.z; g[e + 3] = u.w;
+                        }
                         t[f] *= -2.f;
 #pragma unroll
-                        for (int e = f + 1; e < GR; ++e) t[e] = fmaf(t[f], Lg[f * GR + e], t[e]);
+                        for (int e = f + 1; e < GR; ++e) t[e] = fmaf(t[f], g[e], t[e]);
                     }
                     __syncwarp();
 #pragma unroll

@@ -666,6 +666,51 @@ def test_close_eigenvalues_inside_the_principal_subspace(d, rank, gap):
         assert np.linalg.norm(got - ref) <= 32 * par.U32 / (0.2 * 0.8 ** (rank - 2)) * np.linalg.norm(ref), (seed, np.linalg.norm(got - ref) / np.linalg.norm(ref))
 
 
+@pytest.mark.parametrize("d,k", [(128, 24), (128, 70), (64, 20)])
+@pytest.mark.parametrize("rank", [1, 2, 4, 8])
+@pytest.mark.parametrize("spectrum", ["falls", "repeated", "outliers", "flat", "few"])
+def test_tridiagonal_form_that_ends_early(d, k, rank, spectrum):
+    # The reduction ends when its first rows hold the wanted eigenpairs and the next one.  Spectra that fall off end early, flat ones
+    # late; a repeated eigenvalue must not be taken for one (the first rows hold one copy of it each), nor may a residual of
+    # low rank end with fewer.
+    T, n = 500, d - k
+    w = small("early", d=d, dtype="f32", rank=rank, kv_heads=1, caches=((T, k),), seed=131)
+    for seed in range(3):
+        a = synth.gen_cache(w, 0)
+        rng = np.random.default_rng(seed)
+        idx = oracle.topk(oracle.scores(a["K"][0, 0], a["Q"].reshape(1, 1, w.n_q, d)[0, 0]), k)[0]
+        lam = 0.75 ** np.arange(n)
+        if spectrum == "repeated":
+            lam = np.concatenate([np.full(rank, 0.5), 0.2 * 0.75 ** np.arange(n - rank)])
+            lam[0] = 1.0 if rank > 2 else 0.5
+        elif spectrum == "outliers":
+            lam = np.concatenate([np.linspace(1.0, 0.9, rank), np.linspace(0.02, 0.01, n - rank)])
+        elif spectrum == "flat":
+            lam = np.linspace(1.0, 0.5, n)
+            lam[:rank] += 0.2
+        elif spectrum == "few":
+            lam[rank + 1:] = 0.0
+        U = np.linalg.qr(rng.standard_normal((T - k, n)))[0]
+        W = np.linalg.qr(rng.standard_normal((n, n)))[0]
+        V = np.zeros((T, d))
+        dele = np.setdiff1d(np.arange(T), idx)
+        V[idx, :k] = np.linalg.qr(rng.standard_normal((k, k)))[0] * np.sqrt(k)      # (nothing of their own that magnifies roundings)
+        V[dele, k:] = (U * np.sqrt(lam)) @ W * np.sqrt(T)
+        a["V"] = (V @ np.linalg.qr(rng.standard_normal((d, d)))[0]).astype(np.float32)[None, None]
+        out = par.run_gpu(w, [a])[0][0]
+        args = a["K"][0, 0], a["V"][0, 0], out["scores"][0, 0].cpu().numpy().astype(np.float64), out["idx"][0, 0].cpu().numpy()
+        ref, whole = oracle.backfill(*args, rank), oracle.backfill(*args, n)["delta"]
+        got = out["delta"][0, 0].cpu().numpy().astype(np.float64)
+        gap = (lam[rank - 1] - lam[rank]) / lam[0]
+        # some 32 roundings of 2^-24 on the way to the subspace, over its distance from the rest, of the vector that is projected on it
+        err = np.linalg.norm(got - ref["delta"]) / np.linalg.norm(whole)
+        assert err <= 32 * par.U32 / gap, (seed, err)
+        dg, want = P.parse_diag(out["diag"])[0], ref["diag"]
+        for key in ("lam_1", "lam_rho", "lam_next"):
+            # the Gram matrix is a sum of T products, its eigenvalues are resolved to 6e-8 of a bound that is twice the largest at most
+            assert abs(dg[key] - want[key]) <= 32 * par.U32 * want["lam_1"], (key, dg[key], want[key])
+
+
 # ---------------------------------------------------------------------------
 # protected sink prefix: the first s positions are retained besides the budget
 # ---------------------------------------------------------------------------
