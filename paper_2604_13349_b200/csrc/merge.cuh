@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(MGT_NT) k_merge_assign_mma(const __grid_consta
     const CacheDev &c = p.c[ci];
     const int T = c.T, k = c.k_eff, j0 = blockIdx.x * MGT_ROWS;
     if (j0 >= T) return;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gr = lane >> 2, gc = lane & 3;
+    const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31, gr = lane >> 2, gc = lane & 3;
     const uint4 *Kh = reinterpret_cast<const uint4 *>(c.k) + (size_t)lh * T * CH;
     const uint4 *Kr = reinterpret_cast<const uint4 *>(c.k_out) + (size_t)lh * k * CH;
     const uint8_t *keep = p.keep + c.tok_off + (size_t)lh * T;
@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(256) k_merge_apply(const __grid_constant__ Cal
     int ci, lh;
     locate(p, blockIdx.y, ci, lh);
     const CacheDev &c = p.c[ci];
-    const int T = c.T, k = c.k_eff, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int T = c.T, k = c.k_eff, lane = threadIdx.x & 31, warp = warp_uniform((int)threadIdx.x >> 5);
     constexpr int SLOTS = 8 / WPS;                                      // slots of a block
     const int r0 = blockIdx.x * SLOTS, r = r0 + warp / WPS, part = warp % WPS;
     if (r0 >= k) return;

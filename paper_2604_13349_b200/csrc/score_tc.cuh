@@ -231,7 +231,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_score_tc(const __grid_constan
     __shared__ ScoreTab s_tab[OBF_MAX_CACHES];
     __shared__ uint32_t s_tmem, s_abort;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
     const int n_items = p.sc_items, stride = ST_SLOTS * (int)gridDim.x;
     tc::WaitCtx wc{&s_abort, p.status, p.wait_limit_ns};
 
