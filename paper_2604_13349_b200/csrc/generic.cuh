@@ -330,6 +330,11 @@ __global__ void __launch_bounds__(SEL_NT) k_select(const __grid_constant__ CallD
 // Retained rows that the selection copies itself (k_select_smem): with this few a copy of its own costs a launch, 2 us, for
 // what the head's block has in hand a moment after the positions; the block's threads fetch all of them at once.
 constexpr int SEL_GATHER_MAX = 64;
+// and this many where no multiprocessor has more than one head: its block of 1024 threads fetches them while the others would launch the
+// copy: where a span test waits for the values beside the pass over V these only (8 heads, 205 of 2048 rows, 44.1 -> 42.2 us a call; 128 heads,
+// 250 of 2000, 84.1 -> 82.5), without a span test keys and values up to half as many (32 heads, 100 of 1000 rows, 177 -> 173; with 200 rows
+// eviction would go from 24.2 to 25.0).
+constexpr int SEL_GATHER_FEW = 256;
 
 constexpr int SEL_SMEM_MAX_T = 16384;               // keys of a head that fit in shared memory (k_select_smem)
 
@@ -360,8 +365,8 @@ __global__ void __launch_bounds__(256) k_layer_sum(const __grid_constant__ CallD
 // 8 heads, T = 2048: 8.5 -> 6.7 us; 288 heads, T = 4096: 16 -> 11.6; 320 heads, T = 8192, beside the pass over V: 56 -> 40.
 // With LAYER every head's block selects on its layer's summed masses (the layer's heads repeat the same
 // selection side by side rather than one block writing all of them in turn) and writes the demand sums of the head's own.
-// gather_vecs > 0: every budget is at most SEL_GATHER_MAX and the block copies its head's retained rows of K and V too, that
-// many 16-byte vectors each.
+// gather_vecs != 0: the block copies its head's retained rows too (at most SEL_GATHER_FEW), that many 16-byte vectors each: of K and V, or, of
+// V only where it is negative.
 constexpr int SEL_CAND_MAX = 256, SEL_BINS = 2048;
 
 template <int NT, bool LAYER = false>
@@ -377,7 +382,7 @@ __global__ void __launch_bounds__(NT, 2048 / NT) k_select_smem(const __grid_cons
     __shared__ uint32_t s_bin, s_want, s_count, s_listed, s_tau;
     __shared__ uint32_t wtot[32];
     __shared__ float red[3][32];
-    __shared__ int s_idx[SEL_GATHER_MAX];
+    __shared__ int s_idx[SEL_GATHER_FEW];
     int ci, lh;
     locate(p, blockIdx.x, ci, lh);
     const CacheDev &c = p.c[ci];
@@ -568,19 +573,21 @@ __global__ void __launch_bounds__(NT, 2048 / NT) k_select_smem(const __grid_cons
     if (lane == 0) { red[0][warp] = sk; red[1][warp] = sd; red[2][warp] = nx; }
     __syncthreads();
     if (gather_vecs) {
-        const size_t to = (size_t)lh * k * gather_vecs;
-        const uint4 *ks = reinterpret_cast<const uint4 *>(c.k) + (size_t)lh * T * gather_vecs, *vs = reinterpret_cast<const uint4 *>(c.v) + (size_t)lh * T * gather_vecs;
-        for (int e = tid; e < k * gather_vecs; e += NT) {
-            const int r = e / gather_vecs, ch = e - r * gather_vecs;
-            const int j = s_idx[r];
-            if ((unsigned)j >= (unsigned)T) {             // never dereference a position outside the cache
+        // two vectors a thread in flight: of K and V, or two of V
+        const bool both = gather_vecs > 0;
+        const int vecs = both ? gather_vecs : -gather_vecs, n = k * vecs, step = both ? NT : 2 * NT;
+        const size_t to = (size_t)lh * n;
+        const uint4 *vs = reinterpret_cast<const uint4 *>(c.v) + (size_t)lh * T * vecs, *ks = both ? reinterpret_cast<const uint4 *>(c.k) + (size_t)lh * T * vecs : vs;
+        uint4 *vo = reinterpret_cast<uint4 *>(c.v_out) + to, *ko = both ? reinterpret_cast<uint4 *>(c.k_out) + to : vo;
+        for (int e = tid; e < n; e += step) {
+            const int e2 = both ? e : min(e + NT, n - 1), j = s_idx[e / vecs], j2 = s_idx[e2 / vecs];
+            if ((unsigned)j >= (unsigned)T || (unsigned)j2 >= (unsigned)T) {       // never dereference a position outside the cache
                 atomicOr(p.status, OBF_DEV_INTERNAL);
                 continue;
             }
-            const size_t from = (size_t)j * gather_vecs + ch;
-            const uint4 a = ks[from], b = vs[from];
-            reinterpret_cast<uint4 *>(c.k_out)[to + e] = a;
-            reinterpret_cast<uint4 *>(c.v_out)[to + e] = b;
+            const uint4 a = vs[(size_t)j * vecs + e % vecs], b = ks[(size_t)j2 * vecs + e2 % vecs];
+            vo[e] = a;
+            ko[e2] = b;
         }
     }
     if (warp == NW - 1) {

@@ -474,8 +474,11 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
     if (side && !FORK_LATE) OBF_TRY(fork_and_pass());
     bool any_q8 = false;
     for (int i = 0; i < cd.n_caches; ++i) any_q8 = any_q8 || cd.c[i].k_q8 != nullptr;
-    // few retained rows, no int8 copy of them and no span test that waits for them beside the pass over V: the selection copies them itself
-    const int gather_vecs = T_max <= SEL_SMEM_MAX_T && k_max <= SEL_GATHER_MAX && !span && !any_q8 ? D * (int)sizeof(TIN) / 16 : 0;
+    // few retained rows and no int8 copy of them: the selection copies them itself (SEL_GATHER_MAX), the values only (negative) where the
+    // span test waits for them beside the pass over V; where there is a span test and no such pass, the copy is a kernel of its own
+    const bool few = heads <= sm_count();
+    const bool with_selection = T_max <= SEL_SMEM_MAX_T && k_max <= (!few ? SEL_GATHER_MAX : span ? SEL_GATHER_FEW : SEL_GATHER_FEW / 2) && !any_q8 && (!span || (few && side && !FORK_LATE));
+    const int gather_vecs = with_selection ? (span ? -1 : 1) * D * (int)sizeof(TIN) / 16 : 0;
     if (cd.layerwise) {
         // masses of a layer's KV heads added up, then every head's block selects on its layer's sums
         const int n_layers = heads / cd.kv_heads;
@@ -523,15 +526,17 @@ static obf_status_t launch_generic(const CallDev &cd, const Layout &L, int T_max
         return OBF_OK;
     };
     dim3 g4((k_max + GATHER_ROWS - 1) / GATHER_ROWS, heads);
-    if (gather_vecs) {
+    if (gather_vecs > 0) {
         if (side) {
             OBF_TRY(launch_rows(sel));
             OBF_TRY(side_work.join());
         }
     } else if (side) {
         // the values first: the rest of the call needs them
-        OBF_TRY(launch(k_gather<TIN, D, 1>, dim3(g4), 256, 0, sel, cd));
-        mark(sel, "k_gather");
+        if (!gather_vecs) {
+            OBF_TRY(launch(k_gather<TIN, D, 1>, dim3(g4), 256, 0, sel, cd));
+            mark(sel, "k_gather");
+        }
         OBF_CUDA_TRY(cudaEventRecord(side->rows_done, side->stream));
         if constexpr (sizeof(TIN) == 2) if (span) {
             // the span test reads the gathered rows only (it forms G_keep itself): it runs here, beside the pass over

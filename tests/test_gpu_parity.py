@@ -1046,6 +1046,24 @@ def test_retained_rows_are_copied_whoever_copies_them(dtype, d, flags, caches):
                     assert np.array_equal(o["V_out"][l, h].float().cpu().numpy(), par.f32_view(a["V"][l, h], dtype)[idx[l, h]])
 
 
+@pytest.mark.parametrize("dtype,d", [("f32", 64), ("bf16", 64), ("bf16", 128)])
+@pytest.mark.parametrize("budgets", [(127,), (128,), (129, 31), (255, 130), (256,), (257,)])
+def test_retained_rows_of_few_heads_copied_by_the_selection(dtype, d, budgets):
+    # few heads: up to 128 rows of keys and values, up to 256 of the values where a span test waits for them; a full span keeps
+    # the values as they are, so that both outputs are copies
+    w = small("few", layers=2, d=d, dtype=dtype, rank=1, caches=tuple((700, b) for b in budgets), seed=72)
+    arrays = [synth.gen_cache(w, ci) for ci in range(len(w.caches))]
+    for evict in (True, False):
+        outs, _, st = par.run_gpu(w, arrays, evict=evict)
+        assert st & 0xFF == 0
+        for a, o, b in zip(arrays, outs, budgets):
+            idx = o["idx"].cpu().numpy()
+            for l, h in all_heads(w):
+                assert np.array_equal(o["K_out"][l, h].float().cpu().numpy(), par.f32_view(a["K"][l, h], dtype)[idx[l, h]])
+                if evict or b >= d + 60:
+                    assert np.array_equal(o["V_out"][l, h].float().cpu().numpy(), par.f32_view(a["V"][l, h], dtype)[idx[l, h]])
+
+
 # ---------------------------------------------------------------------------
 # selection: masses so close together that one bin of the first count holds most of them (further counts), or spread
 # (the bin's keys are ranked at once)
