@@ -878,26 +878,33 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                     nw = __reduce_add_sync(0xffffffffu, nw);
                     nx = __reduce_add_sync(0xffffffffu, nx);
                     if (!warp_uniform(nx > 0 && rest * 1.0001f < STEP * (float)nx)) return warp_uniform(rest > 1.3f * STEP * (float)nx) ? 0 : 1;
-                    // lanes 0 .. 3: upwards, at the ends of both intervals; lane 4: downwards at sigma, for the last pivot
-                    const bool down = lane == 4;
-                    const float sg = STEP * (float)(down ? nx : (lane & 2 ? nx : nw) + (lane & 1));
-                    float y1 = 1.f, y0 = 0.f, top = 1.f;
+                    // Lanes 0 and 1: upwards, at both ends of the last wanted and of the next eigenvalue's interval, as far as the ends agree in
+                    // sign: where they do not, an eigenvalue of the rows below lies between them and what follows says nothing (a form that
+                    // falls apart, where the eigenvalue belongs to its lower part).  Lane 2: downwards at sigma, for the last pivot.
+                    const bool down = lane == 2;
+                    const float sg = STEP * (float)(lane == 0 ? nw : nx), sh = down ? sg : sg + STEP;
+                    float y1 = 1.f, y0 = 0.f, z1 = 1.f, z0 = 0.f, top = 1.f;
+                    bool live = true;
                     const int by = down ? 1 : -1;
                     const float *pa = down ? sa : sa + sz - 1, *pb = down ? vb - 1 : vb + sz - 1, *pi = down ? vi : vi + sz - 2;
 #pragma unroll 4
                     for (int k = 1; k < sz; ++k, pa += by, pb += by, pi += by) {
-                        const float y = -fmaf(*pa - sg, y1, *pb * y0) * *pi;
+                        const float a = *pa, b = *pb, ib = *pi;
+                        const float y = -fmaf(a - sg, y1, b * y0) * ib, z = -fmaf(a - sh, z1, b * z0) * ib;
+                        live = live && top < 1e25f && (y > 0.f ? z > 0.f : y < 0.f && z < 0.f);
                         const float f = down && fabsf(y) > 1e20f ? 1e-20f : 1.f;           // (downwards the quotient counts)
-                        if (top < 1e25f) {
+                        if (live) {
                             y0 = y1 * f;
                             y1 = y * f;
-                            top = fmaxf(top, fabsf(y1));
+                            z0 = z1 * f;
+                            z1 = z * f;
+                            top = fmaxf(top, fminf(fabsf(y1), fabsf(z1)));
                         }
                     }
                     const float d = (sa[sz - 1] - sg) + vb[sz - 2] * (y0 / y1);
-                    const float d4 = __shfl_sync(0xffffffffu, d, 4), s4 = __shfl_sync(0xffffffffu, sg, 4), t4 = __shfl_sync(0xffffffffu, top, 4);
-                    const bool gone = lane < 2 ? cb <= 1e-9f * top : lane < 4 ? cb <= 3e-5f * top : true;
-                    return warp_uniform(t4 < 1e25f && d4 < 0.f && (rest - cb * cb / d4) * 1.0001f < s4) && __all_sync(0xffffffffu, gone) ? 2 : 1;
+                    const float d2 = __shfl_sync(0xffffffffu, live ? d : 1.f, 2), sig = __shfl_sync(0xffffffffu, sg, 2);
+                    const bool gone = lane == 0 ? cb <= 1e-9f * top : lane == 1 ? cb <= 3e-5f * top : true;
+                    return warp_uniform(d2 < 0.f && (rest - cb * cb / d2) * 1.0001f < sig) && __all_sync(0xffffffffu, gone) ? 2 : 1;
                 };
                 int early = 0, more;
 #pragma unroll 1

@@ -711,6 +711,36 @@ def test_tridiagonal_form_that_ends_early(d, k, rank, spectrum):
             assert abs(dg[key] - want[key]) <= 32 * par.U32 * want["lam_1"], (key, dg[key], want[key])
 
 
+@pytest.mark.parametrize("rank", [1, 2, 4])
+@pytest.mark.parametrize("first", [1, 6, 15])
+@pytest.mark.parametrize("dead", [False, True])
+def test_tridiagonal_form_that_falls_apart(rank, first, dead):
+    # The retained values fill the first channels, the deleted ones two groups of channels on tokens of their own: the residual's Gram
+    # matrix is block diagonal and so is the tridiagonal form, whose first rows hold a block of small eigenvalues (or, dead, of zeros)
+    # and say nothing about how far the second block, with the wanted ones, has come.
+    d, k, T = 128, 24, 500
+    w = small("apart", d=d, dtype="f32", rank=rank, kv_heads=1, caches=((T, k),), seed=137)
+    a = synth.gen_cache(w, 0)
+    rng = np.random.default_rng(first)
+    idx = oracle.topk(oracle.scores(a["K"][0, 0], a["Q"].reshape(1, 1, w.n_q, d)[0, 0]), k)[0]
+    dele = np.setdiff1d(np.arange(T), idx)
+    n = d - k - first
+    lam = 0.9 ** np.arange(n)
+    V = np.zeros((T, d))
+    V[idx, :k] = np.linalg.qr(rng.standard_normal((k, k)))[0] * np.sqrt(k)
+    if not dead:
+        V[dele[:100], k:k + first] = 0.05 * rng.standard_normal((100, first))
+    rows = len(dele) - 100
+    V[dele[100:], k + first:] = (np.linalg.qr(rng.standard_normal((rows, n)))[0] * np.sqrt(lam)) @ np.linalg.qr(rng.standard_normal((n, n)))[0] * np.sqrt(T)
+    a["V"] = V.astype(np.float32)[None, None]
+    out = par.run_gpu(w, [a])[0][0]
+    args = a["K"][0, 0], a["V"][0, 0], out["scores"][0, 0].cpu().numpy().astype(np.float64), out["idx"][0, 0].cpu().numpy()
+    ref, whole = oracle.backfill(*args, rank), oracle.backfill(*args, d)["delta"]
+    gap = (lam[rank - 1] - lam[rank]) / lam[0]
+    # some 32 roundings of 2^-24 on the way to the subspace, over its distance from the rest, of the vector that is projected on it
+    assert np.linalg.norm(out["delta"][0, 0].cpu().numpy().astype(np.float64) - ref["delta"]) <= 32 * par.U32 / gap * np.linalg.norm(whole)
+
+
 # ---------------------------------------------------------------------------
 # protected sink prefix: the first s positions are retained besides the budget
 # ---------------------------------------------------------------------------
