@@ -36,8 +36,8 @@
 // as small loops: a section's first pass costs about 130 cycles per 128 bytes of its code, more than its arithmetic.
 // Measured on 36 x 8 heads, budget 32, rank 2, head_dim 128 (every head back-filled): 0.534 ms for the
 // same algebra on a matrix in shared memory (Gram-Schmidt basis, M = P G P, then the reduction), 0.142 with all rows of the tridiagonal
-// form, 0.107 (values whose channels fall off; 219 -> 185 us a call; three outlier channels, rank 1 and 2, 217 -> 182 and 220 -> 203; flat
-// values, rank 1, 219 -> 228, for the questions, ranks 2 and 4 the same).  Slower were: one barrier a row of the form, as for the retained rows
+// form, 0.110 (values whose channels fall off; 219 -> 187 us a call; three outlier channels, rank 1 and 2, 217 -> 187 and 220 -> 209; flat
+// values, ranks 1, 2 and 4, 219 -> 229, 219 -> 223 and 242 -> 235: the questions cost as much as the last rows).  Slower were: one barrier a row of the form, as for the retained rows
 // (622 to 1400 cycles a row against 690 to 1210: more instructions), eight warps
 // with half the registers, the chain of reflectors in a warp of its own beside the matrix warps (the registers it takes cost
 // the others more), one copy of the step's code for all stages, the reflectors on G sixteen at a time in compact form (code
