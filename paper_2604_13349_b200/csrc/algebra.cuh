@@ -477,6 +477,9 @@ __device__ __forceinline__ int alg_reflectors(const TIN *vk, int k, float *Y, fl
         AlgRow<D> x;                                           // row i as all reflectors before it leave it (the same in every half-warp)
         alg_load<D>(x, next, c16);
         float nn = next[D];
+        // Row i's buffer is written again with row i + 2, in iteration i, behind the barrier after its last read: that is the one that ends
+        // iteration i - 1, where row i was read, and for row 0, read just now, this one.
+        __syncthreads();
 #pragma unroll 1
         for (int i = 0; i < rows; ++i) {
             AlgRow<D> r;

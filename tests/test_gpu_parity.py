@@ -311,6 +311,28 @@ def test_span_subset_deficient_and_all_retained_rows_deficient_too():
     assert torch.all(outs[0]["delta"].norm(dim=-1) > 1e-6)
 
 
+@pytest.mark.parametrize("dtype,d", [("bf16", 128), ("bf16", 64), ("f32", 64)])
+@pytest.mark.parametrize("budget", [1, 2, 3, 4, 32, 33, 34, 35, 36, 61])
+def test_retained_rows_two_apart_do_not_stand_in_for_one_another(dtype, d, budget):
+    # Retained rows pass through two buffers in turn, in batches of 32.  Of every four the first two add a direction each, the third is a
+    # multiple of the first and the fourth of the second: a row read in the place of the one two before or behind it changes the span.
+    # 160 heads, so that two of 128 channels share a multiprocessor.
+    w = small("turns", layers=20, kv_heads=8, d=d, dtype=dtype, rank=1, caches=((97, budget),), heavy=0, seed=150 + budget)
+    arrays = [synth.gen_cache(w, 0)]
+    a = arrays[0]
+    V = par.f32_view(a["V"], dtype).copy()
+    Qv = par.f32_view(a["Q"], dtype).reshape(w.layers, w.kv_heads, w.n_q, d)
+    place = np.arange(budget)
+    source = place - 2 * (place % 4 // 2)
+    for l, h in all_heads(w):
+        idx = oracle.topk(oracle.scores(par.f32_view(a["K"][l, h], dtype), Qv[l, h]), budget)[0]
+        V[l, h, idx] = V[l, h, idx[source]] * np.where(place % 4 < 2, 1.0, -2.0).astype(np.float32)[:, None]
+    a["V"] = synth.to_bf16_bits(V) if dtype == "bf16" else V
+    outs, reps, _ = run_and_check(w, arrays=arrays, heads=[(0, 0), (7, 3), (19, 7)])
+    assert all(dg["span_rank"] == len(set(source)) for dg in P.parse_diag(outs[0]["diag"]))
+    assert all(not r.oracle_skipped for r in reps)
+
+
 def test_retained_rows_with_a_dominant_common_component():
     # budget 24 < head_dim: every value is a common vector plus 3 % of noise, so after the first retained row every
     # further row loses nearly all of its norm to the basis in the first Gram-Schmidt pass and the kernel has to go
