@@ -59,6 +59,7 @@ constexpr float RCR_SKIP_TOL = 1e-6f;
 constexpr float EIG_RANK_TOL = 1e-5f;
 constexpr int JACOBI_MAX_SWEEPS = 30;
 constexpr int ALG_TRI_MAX_RANK = 8;     // up to this rank only rank + 1 eigenvalues and rank eigenvectors are computed
+static_assert(ALG_TRI_MAX_RANK + 1 < 32, "a lane for each of them and one more");
 constexpr float EIG_CLUSTER_TOL = 1e-3f; // eigenvalues closer than this (relative to the largest): inverse iteration, kept orthogonal during it
 // Rows of the tridiagonal form after which it is asked whether they suffice, and how many more at least before it is asked again (a
 // quarter of them where that is more, half where the rest is far too large).  The question costs 2000 cycles where the answer is no for the rest's sake, 4500 else, a row 850 to 1600.
@@ -836,8 +837,10 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                 // if the rest, R + b b^T / |d|, has none: b is the coupling to the rest, d < 0 the last pivot of T - sigma.  The largest
                 // eigenvalue of R follows from its trace and Frobenius norm, which are those of M less T's:
                 //   lambda <= t / N + sqrt((N - 1) / N (f^2 - t^2 / N)).
-                // And their vectors' last entries, times the coupling, have to be nothing beside rounding: from the recurrence for the
-                // vector upwards from its last entry, at both ends of the interval that holds the eigenvalue.
+                // That is a count, and says nothing about which rows the vectors live in: a large eigenvalue may have come into the form after
+                // smaller ones.  So the last entry of every wanted vector and of the next one, times the coupling, has to be nothing
+                // beside rounding: from the recurrence for the vector upwards from its last entry, at both ends of the interval that holds
+                // the eigenvalue, a lane for each.
                 auto leading_part_suffices = [&]() __attribute__((always_inline)) {
                     const int sz = warp_uniform(J - m), r = min(p.rank, D);
                     const float *da = ta + m, *db = tb + m;
@@ -870,22 +873,31 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                     sturm_count2(sa, sb2, n4, STEP * (2 * tid + 1), STEP * (2 * tid + 2), c0, c1);
                     cnt[tid] = (uint16_t)(c0 | c1 << 8);
                     __syncthreads();
-                    int nw = 0, nx = 0;                                // shifts not above the last wanted and the next eigenvalue
+                    // shifts not above eigenvalue e, the largest being number 0
+                    auto shifts_up_to = [&](int e) __attribute__((always_inline)) {
+                        int s = 0;
 #pragma unroll
-                    for (int i = 0; i < ALG_NW; ++i) {
-                        const uint32_t two = cnt[lane + 32 * i];
-                        const int a = two & 255, b = two >> 8;
-                        nw += (a <= sz - r ? 1 : 0) + (b <= sz - r ? 1 : 0);
-                        nx += (a <= sz - 1 - r ? 1 : 0) + (b <= sz - 1 - r ? 1 : 0);
-                    }
-                    nw = __reduce_add_sync(0xffffffffu, nw);
-                    nx = __reduce_add_sync(0xffffffffu, nx);
+                        for (int i = 0; i < ALG_NW; ++i) {
+                            const uint32_t two = cnt[lane + 32 * i];
+                            s += ((int)(two & 255) < sz - e ? 1 : 0) + ((int)(two >> 8) < sz - e ? 1 : 0);
+                        }
+                        return __reduce_add_sync(0xffffffffu, s);
+                    };
+                    const int nx = shifts_up_to(r);
                     if (!warp_uniform(nx > 0 && rest * 1.0001f < STEP * (float)nx)) return warp_uniform(rest > 1.3f * STEP * (float)nx) ? 0 : 1;
-                    // Lanes 0 and 1: upwards, at both ends of the last wanted and of the next eigenvalue's interval, as far as the ends agree in
-                    // sign: where they do not, an eigenvalue of the rows below lies between them and what follows says nothing (a form that
-                    // falls apart, where the eigenvalue belongs to its lower part).  Lane 2: downwards at sigma, for the last pivot.
-                    const bool down = lane == 2;
-                    const float sg = STEP * (float)(lane == 0 ? nw : nx), sh = down ? sg : sg + STEP;
+                    int at = nx;
+#pragma unroll 1
+                    for (int e = 0; e < r; ++e) {
+                        const int s = shifts_up_to(e);
+                        if (lane == e) at = s;
+                    }
+                    // Lanes 0 .. r: upwards, at both ends of their eigenvalue's interval, as far as the ends agree in sign: where they do not, an
+                    // eigenvalue of the rows below lies between them and what follows says nothing (a form that falls apart, where the
+                    // eigenvalue belongs to its lower part).  As far as they do, none lies there (from one row to the next their number
+                    // changes by one at most), and an entry is nowhere between the ends smaller than at the smaller of them: a product of
+                    // distances from points outside.  Last lane: downwards at sigma, for the last pivot.
+                    const bool down = lane == 31;
+                    const float sg = STEP * (float)at, sh = down ? sg : sg + STEP;
                     float y1 = 1.f, y0 = 0.f, z1 = 1.f, z0 = 0.f, top = 1.f;
                     bool live = true;
                     const int by = down ? 1 : -1;
@@ -905,8 +917,8 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                         }
                     }
                     const float d = (sa[sz - 1] - sg) + vb[sz - 2] * (y0 / y1);
-                    const float d2 = __shfl_sync(0xffffffffu, live ? d : 1.f, 2), sig = __shfl_sync(0xffffffffu, sg, 2);
-                    const bool gone = lane == 0 ? cb <= 1e-9f * top : lane == 1 ? cb <= 3e-5f * top : true;
+                    const float d2 = __shfl_sync(0xffffffffu, live ? d : 1.f, 31), sig = __shfl_sync(0xffffffffu, sg, 31);
+                    const bool gone = lane < r ? cb <= 1e-9f * top : lane == r ? cb <= 3e-5f * top : true;
                     return warp_uniform(d2 < 0.f && (rest - cb * cb / d2) * 1.0001f < sig) && __all_sync(0xffffffffu, gone) ? 2 : 1;
                 };
                 int early = 0, more;

@@ -763,6 +763,85 @@ def test_tridiagonal_form_that_falls_apart(rank, first, dead):
     assert np.linalg.norm(out["delta"][0, 0].cpu().numpy().astype(np.float64) - ref["delta"]) <= 32 * par.U32 / gap * np.linalg.norm(whole)
 
 
+def _backfill_of_a_form(a_diag, a_off, rank):
+    """One fp32 head of 128 channels whose residual has the Gram matrix with this diagonal and these couplings: the retained rows fill the
+    first channels, two neighbouring channels a deleted token (a row of the transposed Cholesky factor), so that the reduction
+    leaves the matrix as it is.  (Without couplings a_diag is the whole matrix.)  Error of delta over the norm of what is projected, and
+    the limit: some 32 roundings of 2^-24 over the distance of the wanted eigenvalues from the next."""
+    n = len(a_diag)
+    d, T = 128, 500
+    k = d - n
+    w = small("form", d=d, dtype="f32", rank=rank, kv_heads=1, caches=((T, k),), seed=139)
+    a = synth.gen_cache(w, 0)
+    rng = np.random.default_rng(n)
+    idx = oracle.topk(oracle.scores(a["K"][0, 0], a["Q"].reshape(1, 1, w.n_q, d)[0, 0]), k)[0]
+    dele = np.setdiff1d(np.arange(T), idx)
+    M = a_diag if a_off is None else np.diag(a_diag) + np.diag(a_off, 1) + np.diag(a_off, -1)
+    V = np.zeros((T, d))
+    V[idx, :k] = np.linalg.qr(rng.standard_normal((k, k)))[0] * np.sqrt(k)
+    V[rng.choice(dele, n, replace=False), k:] = np.linalg.cholesky(M).T * np.sqrt(T)
+    a["V"] = V.astype(np.float32)[None, None]
+    out = par.run_gpu(w, [a])[0][0]
+    args = a["K"][0, 0], a["V"][0, 0], out["scores"][0, 0].cpu().numpy().astype(np.float64), out["idx"][0, 0].cpu().numpy()
+    ref, whole = oracle.backfill(*args, rank), oracle.backfill(*args, d)["delta"]
+    lam = np.linalg.eigvalsh(M)[::-1]
+    err = np.linalg.norm(out["delta"][0, 0].cpu().numpy().astype(np.float64) - ref["delta"]) / np.linalg.norm(whole)
+    return err, 32 * par.U32 * lam[0] / (lam[rank - 1] - lam[rank])
+
+
+@pytest.mark.parametrize("rank,first", [(2, 19), (2, 20), (2, 21), (2, 22), (2, 33), (3, 26), (3, 27), (4, 26), (4, 27), (8, 26), (8, 27)])
+@pytest.mark.parametrize("coupling", [1e-8, 1e-5, 1e-3])
+def test_largest_eigenvalue_that_enters_the_tridiagonal_form_late(rank, first, coupling):
+    # Two groups of rows, hardly coupled.  The first holds all wanted eigenvalues but the largest, and the next one, and is complete (or has its
+    # vectors settled) when the form's first rows are looked at; the second, with the largest eigenvalue, has only begun.
+    for seed in range(3):
+        rng = np.random.default_rng(seed)
+        diag, off = np.zeros(104), np.full(103, coupling)
+        small_ones = lambda n, by: 0.002 + 0.25 * by ** np.arange(n)
+        for at, lam in ((0, np.concatenate([0.6 - 0.2 * np.arange(rank) / rank, small_ones(first - rank, 0.7)])),
+                        (first, np.concatenate([[1.0], small_ones(103 - first, 0.8)]))):
+            # the form of a dense matrix with these eigenvalues, by Lanczos' recurrence with all vectors kept orthogonal
+            n = len(lam)
+            q = [rng.standard_normal(n)]
+            q[0] /= np.linalg.norm(q[0])
+            for i in range(n):
+                y = lam * q[i]
+                diag[at + i] = q[i] @ y
+                for _ in range(2):
+                    y -= np.array(q).T @ (np.array(q) @ y)
+                if i + 1 < n:
+                    off[at + i] = np.linalg.norm(y)
+                    q.append(y / off[at + i])
+        err, limit = _backfill_of_a_form(diag, off, rank)
+        assert err <= limit, (seed, err, limit)
+
+
+@pytest.mark.parametrize("coupling", [0.05, 0.2])
+def test_largest_eigenvalue_two_rows_before_the_end_of_the_leading_part(coupling):
+    # no wanted eigenvalue's neighbourhood looks unsettled but the largest one's
+    diag, off = np.full(104, 0.06), np.zeros(103)
+    diag[[0, 1, 22]] = 0.6, 0.5, 1.0
+    off[:30] = 0.02
+    off[22], diag[23] = coupling, 0.06 + coupling ** 2
+    err, limit = _backfill_of_a_form(diag, off, 2)
+    assert err <= limit, (err, limit)
+
+
+@pytest.mark.parametrize("rank", [2, 8])
+@pytest.mark.parametrize("leakage", [1e-9, 1e-7, 1e-6])
+def test_two_groups_of_channels_that_hardly_mix(rank, leakage):
+    for seed, first in enumerate((10, 18, 20, 25, 40)):
+        rng = np.random.default_rng(seed)
+        # (an eigenvalue of the second group, then one of the first, and so on, down to a floor)
+        M = leakage * rng.standard_normal((104, 104))
+        M += M.T
+        for lo, hi, lead in ((0, first, 0.8), (first, 104, 1.0)):
+            Q = np.linalg.qr(rng.standard_normal((hi - lo, hi - lo)))[0]
+            M[lo:hi, lo:hi] = (Q * (1e-3 + lead * 0.7 ** np.arange(hi - lo))) @ Q.T
+        err, limit = _backfill_of_a_form(M, None, rank)
+        assert err <= limit, (seed, err, limit)
+
+
 # ---------------------------------------------------------------------------
 # protected sink prefix: the first s positions are retained besides the budget
 # ---------------------------------------------------------------------------
