@@ -36,11 +36,10 @@
 // as small loops: a section's first pass costs about 130 cycles per 128 bytes of its code, more than its arithmetic.
 // Measured on 36 x 8 heads, budget 32, rank 2, head_dim 128 (every head back-filled): 0.534 ms for the
 // same algebra on a matrix in shared memory (Gram-Schmidt basis, M = P G P, then the reduction), 0.142 with all rows of the tridiagonal
-// form, 0.110 (values whose channels fall off; 219 -> 187 us a call; three outlier channels, rank 1 and 2, 217 -> 187 and 220 -> 209; flat
-// values, ranks 1, 2 and 4, 219 -> 229, 219 -> 223 and 242 -> 235: the questions cost as much as the last rows).  Slower were: one barrier a row of the form, as for the retained rows
-// (622 to 1400 cycles a row against 690 to 1210: more instructions), eight warps
-// with half the registers, the chain of reflectors in a warp of its own beside the matrix warps (the registers it takes cost
-// the others more), one copy of the step's code for all stages, the reflectors on G sixteen at a time in compact form (code
+// form, 0.110 (values whose channels fall off; how much the early end brings for other spectra stands at ALG_EXIT_FIRST).  Slower
+// were: one barrier a row of the form, as for the retained rows (622 to 1400 cycles a row against 690 to 1210: more instructions),
+// eight warps with half the registers, the chain of reflectors in a warp of its own beside the matrix warps (the registers it takes
+// cost the others more), one copy of the step's code for all stages, the reflectors on G sixteen at a time in compact form (code
 // that runs twice costs more to fetch than it saves), the auxiliary vector or the next row's norm in one warp only.
 #pragma once
 
@@ -62,8 +61,18 @@ constexpr int ALG_TRI_MAX_RANK = 8;     // up to this rank only rank + 1 eigenva
 static_assert(ALG_TRI_MAX_RANK + 1 < 32, "a lane for each of them and one more");
 constexpr float EIG_CLUSTER_TOL = 1e-3f; // eigenvalues closer than this (relative to the largest): inverse iteration, kept orthogonal during it
 // Rows of the tridiagonal form after which it is asked whether they suffice, and how many more at least before it is asked again (a
-// quarter of them where that is more, half where the rest is far too large).  The question costs 2000 cycles where the answer is no for the rest's sake, 4500 else, a row 850 to 1600.
+// quarter of them where that is more, half where the rest is far too large).  A question costs 400 cycles where the rest's bound exceeds
+// all that the rows so far can hold, else 2000 to 4500 after 30 rows and twice that after 70; a row costs 850 to 1600.  So it is given up
+// where the rest comes down too slowly: when a line through its last two bounds, half as far again, ends behind three quarters of all
+// rows.  36 x 8 heads of 1024 positions, budget 32, ranks 1, 2 and 4, us a call:
+//   values' channels             all rows         asked to the end   given up so
+//   flat                         212  213  224    229  223  235      216  216  226
+//   flat, three 8 times as large 211  213  222    199  208  234      200  208  226
+//   0.985 each of the last       212  213  224    224  213  230      222  212  224
+//   0.97 each of the last        212  213  225    201  204  213      201  205  216
+//   inverse root of their number 211  213  222    182  187  199      179  187  199
 constexpr int ALG_EXIT_FIRST = 18, ALG_EXIT_STEP = 6;
+constexpr float ALG_EXIT_BEND = 1.5f, ALG_EXIT_SHARE = 0.75f;
 constexpr float EIG_NEAR_TOL = 5e-2f;    // closer than this: one more step of inverse iteration on the twisted factors, then made orthogonal
 
 // a where the mask is all ones, b where it is zero.  (A conditional between array elements would be a conditional
@@ -831,16 +840,17 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                     }
                 };
                 float *sa = WS, *sb2 = WS + D + 8, *vec = WS + 2 * (D + 8);   // vec: per wanted eigenvector dd, dl, du, du2, pv, y of D each
-                // Whether the J - m rows of the tridiagonal form so far hold the wanted eigenpairs and the next one (2, else 1, or 0 where it
-                // will take many more).  With sigma just
-                // below the next one, M has as many eigenvalues above sigma as the leading part T (Sylvester, block elimination of T - sigma)
-                // if the rest, R + b b^T / |d|, has none: b is the coupling to the rest, d < 0 the last pivot of T - sigma.  The largest
-                // eigenvalue of R follows from its trace and Frobenius norm, which are those of M less T's:
+                // Whether the J - m rows of the tridiagonal form so far hold the wanted eigenpairs and the next one: 0, else in how many rows to
+                // ask again (D: not at all).  With sigma just below the next one, M has as many eigenvalues above sigma as the leading part T
+                // (Sylvester, block elimination of T - sigma) if the rest, R + b b^T / |d|, has none: b is the coupling to the rest, d < 0 the
+                // last pivot of T - sigma.  The largest eigenvalue of R follows from its trace and Frobenius norm, which are those of M less T's:
                 //   lambda <= t / N + sqrt((N - 1) / N (f^2 - t^2 / N)).
                 // That is a count, and says nothing about which rows the vectors live in: a large eigenvalue may have come into the form after
                 // smaller ones.  So the last entry of every wanted vector and of the next one, times the coupling, has to be nothing
                 // beside rounding: from the recurrence for the vector upwards from its last entry, at both ends of the interval that holds
                 // the eigenvalue, a lane for each.
+                float *was = misc + 12 + 2 * warp;                     // a warp's: the rest's bound when last asked, and after how many rows
+                if (lane == 0) was[1] = 0.f;
                 auto leading_part_suffices = [&]() __attribute__((always_inline)) {
                     const int sz = warp_uniform(J - m), r = min(p.rank, D);
                     const float *da = ta + m, *db = tb + m;
@@ -857,69 +867,87 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                     const float scl = 1.f / gb, nr = (float)(D - J), t = trM - s1, f2 = m2 - s2 + 1e-5f * m2;
                     const float rest = (t / nr + sqrtf((nr - 1.f) / nr * fmaxf(f2 - t * t / nr, 0.f)) + 1e-5f * trM / nr) * scl, cb = fabsf(db[sz - 1]) * scl;
                     float *vb = vec + 4, *vi = vb + D + 4;             // couplings (a zero before and after them) and their reciprocals
-                    const int n4 = (sz + 3) / 4;
-                    if (tid < 4 * n4) {
-                        const float b = (tid > 0 && tid < sz) ? db[tid - 1] * scl : 0.f;
-                        sa[tid] = tid < sz ? da[tid] * scl : 2.f;
-                        sb2[tid] = (tid > 0 && tid < sz) ? fmaxf(b * b, 1e-14f) : 0.f;
-                        vb[tid - 1] = b;
-                        if (tid > 0) vi[tid - 1] = 1.f / b;
-                        if (tid + 1 == sz) vb[tid] = 0.f;
-                    }
-                    __syncthreads();
-                    constexpr float STEP = 1.f / (2 * ALG_NT + 1);
-                    uint16_t *cnt = reinterpret_cast<uint16_t *>(ipq);
-                    int c0, c1;
-                    sturm_count2(sa, sb2, n4, STEP * (2 * tid + 1), STEP * (2 * tid + 2), c0, c1);
-                    cnt[tid] = (uint16_t)(c0 | c1 << 8);
-                    __syncthreads();
-                    // shifts not above eigenvalue e, the largest being number 0
-                    auto shifts_up_to = [&](int e) __attribute__((always_inline)) {
-                        int s = 0;
+                    bool suffice = false;
+                    float sigma = 1.f;                                 // (T's eigenvalues are at most one, in units of gb)
+                    if (warp_uniform(rest < 1.f)) {
+                        const int n4 = (sz + 3) / 4;
+                        if (tid < 4 * n4) {
+                            const float b = (tid > 0 && tid < sz) ? db[tid - 1] * scl : 0.f;
+                            sa[tid] = tid < sz ? da[tid] * scl : 2.f;
+                            sb2[tid] = (tid > 0 && tid < sz) ? fmaxf(b * b, 1e-14f) : 0.f;
+                            vb[tid - 1] = b;
+                            if (tid > 0) vi[tid - 1] = 1.f / b;
+                            if (tid + 1 == sz) vb[tid] = 0.f;
+                        }
+                        __syncthreads();
+                        constexpr float STEP = 1.f / (2 * ALG_NT + 1);
+                        uint16_t *cnt = reinterpret_cast<uint16_t *>(ipq);
+                        int c0, c1;
+                        sturm_count2(sa, sb2, n4, STEP * (2 * tid + 1), STEP * (2 * tid + 2), c0, c1);
+                        cnt[tid] = (uint16_t)(c0 | c1 << 8);
+                        __syncthreads();
+                        // shifts not above eigenvalue e, the largest being number 0
+                        auto shifts_up_to = [&](int e) __attribute__((always_inline)) {
+                            int s = 0;
 #pragma unroll
-                        for (int i = 0; i < ALG_NW; ++i) {
-                            const uint32_t two = cnt[lane + 32 * i];
-                            s += ((int)(two & 255) < sz - e ? 1 : 0) + ((int)(two >> 8) < sz - e ? 1 : 0);
-                        }
-                        return __reduce_add_sync(0xffffffffu, s);
-                    };
-                    const int nx = shifts_up_to(r);
-                    if (!warp_uniform(nx > 0 && rest * 1.0001f < STEP * (float)nx)) return warp_uniform(rest > 1.3f * STEP * (float)nx) ? 0 : 1;
-                    int at = nx;
+                            for (int i = 0; i < ALG_NW; ++i) {
+                                const uint32_t two = cnt[lane + 32 * i];
+                                s += ((int)(two & 255) < sz - e ? 1 : 0) + ((int)(two >> 8) < sz - e ? 1 : 0);
+                            }
+                            return __reduce_add_sync(0xffffffffu, s);
+                        };
+                        const int nx = shifts_up_to(r);
+                        sigma = STEP * (float)nx;
+                        if (warp_uniform(nx > 0 && rest * 1.0001f < sigma)) {
+                            int at = nx;
 #pragma unroll 1
-                    for (int e = 0; e < r; ++e) {
-                        const int s = shifts_up_to(e);
-                        if (lane == e) at = s;
-                    }
-                    // Lanes 0 .. r: upwards, at both ends of their eigenvalue's interval, as far as the ends agree in sign: where they do not, an
-                    // eigenvalue of the rows below lies between them and what follows says nothing (a form that falls apart, where the
-                    // eigenvalue belongs to its lower part).  As far as they do, none lies there (from one row to the next their number
-                    // changes by one at most), and an entry is nowhere between the ends smaller than at the smaller of them: a product of
-                    // distances from points outside.  Last lane: downwards at sigma, for the last pivot.
-                    const bool down = lane == 31;
-                    const float sg = STEP * (float)at, sh = down ? sg : sg + STEP;
-                    float y1 = 1.f, y0 = 0.f, z1 = 1.f, z0 = 0.f, top = 1.f;
-                    bool live = true;
-                    const int by = down ? 1 : -1;
-                    const float *pa = down ? sa : sa + sz - 1, *pb = down ? vb - 1 : vb + sz - 1, *pi = down ? vi : vi + sz - 2;
+                            for (int e = 0; e < r; ++e) {
+                                const int s = shifts_up_to(e);
+                                if (lane == e) at = s;
+                            }
+                            // Lanes 0 .. r: upwards, at both ends of their eigenvalue's interval, as far as the ends agree in sign: where they do not, an
+                            // eigenvalue of the rows below lies between them and what follows says nothing (a form that falls apart, where the
+                            // eigenvalue belongs to its lower part).  As far as they do, none lies there (from one row to the next their number
+                            // changes by one at most), and an entry is nowhere between the ends smaller than at the smaller of them: a product of
+                            // distances from points outside.  Last lane: downwards at sigma, for the last pivot.
+                            const bool down = lane == 31;
+                            const float sg = STEP * (float)at, sh = down ? sg : sg + STEP;
+                            float y1 = 1.f, y0 = 0.f, z1 = 1.f, z0 = 0.f, top = 1.f;
+                            bool live = true;
+                            const int by = down ? 1 : -1;
+                            const float *pa = down ? sa : sa + sz - 1, *pb = down ? vb - 1 : vb + sz - 1, *pi = down ? vi : vi + sz - 2;
 #pragma unroll 4
-                    for (int k = 1; k < sz; ++k, pa += by, pb += by, pi += by) {
-                        const float a = *pa, b = *pb, ib = *pi;
-                        const float y = -fmaf(a - sg, y1, b * y0) * ib, z = -fmaf(a - sh, z1, b * z0) * ib;
-                        live = live && top < 1e25f && (y > 0.f ? z > 0.f : y < 0.f && z < 0.f);
-                        const float f = down && fabsf(y) > 1e20f ? 1e-20f : 1.f;           // (downwards the quotient counts)
-                        if (live) {
-                            y0 = y1 * f;
-                            y1 = y * f;
-                            z0 = z1 * f;
-                            z1 = z * f;
-                            top = fmaxf(top, fminf(fabsf(y1), fabsf(z1)));
+                            for (int k = 1; k < sz; ++k, pa += by, pb += by, pi += by) {
+                                const float a = *pa, b = *pb, ib = *pi;
+                                const float y = -fmaf(a - sg, y1, b * y0) * ib, z = -fmaf(a - sh, z1, b * z0) * ib;
+                                live = live && top < 1e25f && (y > 0.f ? z > 0.f : y < 0.f && z < 0.f);
+                                const float f = down && fabsf(y) > 1e20f ? 1e-20f : 1.f;           // (downwards the quotient counts)
+                                if (live) {
+                                    y0 = y1 * f;
+                                    y1 = y * f;
+                                    z0 = z1 * f;
+                                    z1 = z * f;
+                                    top = fmaxf(top, fminf(fabsf(y1), fabsf(z1)));
+                                }
+                            }
+                            const float d = (sa[sz - 1] - sg) + vb[sz - 2] * (y0 / y1);
+                            const float d2 = __shfl_sync(0xffffffffu, live ? d : 1.f, 31);
+                            const bool gone = lane < r ? cb <= 1e-9f * top : lane == r ? cb <= 3e-5f * top : true;
+                            suffice = d2 < 0.f && (rest - cb * cb / d2) * 1.0001f < sigma && __all_sync(0xffffffffu, gone);
                         }
                     }
-                    const float d = (sa[sz - 1] - sg) + vb[sz - 2] * (y0 / y1);
-                    const float d2 = __shfl_sync(0xffffffffu, live ? d : 1.f, 31), sig = __shfl_sync(0xffffffffu, sg, 31);
-                    const bool gone = lane < r ? cb <= 1e-9f * top : lane == r ? cb <= 3e-5f * top : true;
-                    return warp_uniform(d2 < 0.f && (rest - cb * cb / d2) * 1.0001f < sig) && __all_sync(0xffffffffu, gone) ? 2 : 1;
+                    if (warp_uniform(suffice)) return 0;
+                    // A line through the last two bounds of the rest, which comes down ever more slowly, tells when it will be down at sigma.
+                    const float now = rest * gb, above = now - sigma * gb;
+                    int rows = max(ALG_EXIT_STEP, rest > 1.3f * sigma ? sz / 2 : sz / 4);
+                    if (was[1] > 0.f && above > 0.f &&
+                        (float)sz + ALG_EXIT_BEND * above * ((float)sz - was[1]) / fmaxf(was[0] - now, 1e-3f * now) > ALG_EXIT_SHARE * (float)(D - m)) rows = D;
+                    __syncwarp();
+                    if (lane == 0) {
+                        was[0] = now;
+                        was[1] = (float)sz;
+                    }
+                    return warp_uniform(rows);
                 };
                 int early = 0, more;
 #pragma unroll 1
@@ -933,10 +961,9 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                     }
                     more = 0;
                     if (ASKS && last < D - 2) {
-                        const int answer = leading_part_suffices();
-                        early = answer == 2 ? 1 : 0;
-                        more = 1 - early;
-                        last += max(ALG_EXIT_STEP, (J - m) / (answer ? 4 : 2));
+                        more = leading_part_suffices();
+                        early = more ? 0 : 1;
+                        last += more;
                     }
                     more = warp_uniform(more);
                 } while (more);
