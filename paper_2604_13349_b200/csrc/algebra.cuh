@@ -464,13 +464,19 @@ __device__ __forceinline__ int alg_reflectors(const TIN *vk, int k, float *Y, fl
         for (int s = 0; s < NS; ++s) {
             n0[s] = half_sum(alg_dot<D>(V[s], V[s]));
             // a reflector depends on its row's direction alone: rows whose squares leave the range of fp32's normal numbers
-            // are brought back by a power of two
-            const bool far = n0[s] > 0.f && !(n0[s] > 1e-24f && n0[s] < 1e24f);
+            // are brought back by a power of two.  A row that is not finite adds no direction and is a row of zeros from here on: it
+            // meets the others with a factor of zero, which would not be zero
+            const bool far = n0[s] != 0.f && !(n0[s] > 1e-24f && n0[s] < 1e24f);
             if (warp_uniform(far)) {                           // (any of them: the sum below takes the whole warp)
                 const float f = !far ? 1.f : n0[s] < 1.f ? 1.8446744e19f : 5.421011e-20f;   // 2^64, 2^-64
 #pragma unroll
                 for (int q = 0; q < NQ; ++q) V[s][q] = mul2(V[s][q], pk(f, f));
                 n0[s] = half_sum(alg_dot<D>(V[s], V[s]));
+                if (!(n0[s] < INFINITY)) {
+                    n0[s] = 0.f;
+#pragma unroll
+                    for (int q = 0; q < NQ; ++q) V[s][q] = 0ull;
+                }
             }
         }
         // (the reflectors that earlier batches found, all published behind a barrier)

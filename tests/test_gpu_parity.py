@@ -333,6 +333,27 @@ def test_retained_rows_two_apart_do_not_stand_in_for_one_another(dtype, d, budge
     assert all(not r.oracle_skipped for r in reps)
 
 
+@pytest.mark.parametrize("dtype,d,flags", [("f32", 64, 0), ("f32", 128, 0), ("bf16", 64, 0), ("f32", 64, P.binding.OBF_FLAG_FAST_PATH)])
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+def test_retained_row_that_is_not_finite_stays_out_of_the_others(dtype, d, flags, bad):
+    # such a row adds no direction, like a row of zeros: the head's other rows get the delta that they would get beside that
+    # (bf16 heads of 128 channels sum over all rows and skip the head)
+    for row in (0, 1, 5, 33):
+        w = small("notfinite", d=d, dtype=dtype, rank=1, kv_heads=1, caches=((300, 34),), seed=3)
+        a = synth.gen_cache(w, 0)
+        idx = oracle.topk(oracle.scores(par.f32_view(a["K"][0, 0], dtype), par.f32_view(a["Q"], dtype).reshape(w.n_q, d)), 34)[0]
+        got = []
+        for value in (0.0, bad):
+            V = par.f32_view(a["V"], dtype).copy()
+            V[0, 0, idx[row]] = 0.0
+            V[0, 0, idx[row], 3] = value
+            out, _, st = par.run_gpu(w, [dict(a, V=synth.to_bf16_bits(V) if dtype == "bf16" else V)], flags=flags)
+            assert P.parse_diag(out[0]["diag"])[0]["span_rank"] == 33
+            assert torch.all(out[0]["delta"].isfinite()) and torch.any(out[0]["delta"] != 0)
+            got.append((out[0]["delta"][0, 0].cpu().numpy(), np.delete(out[0]["V_out"][0, 0].float().cpu().numpy(), row, axis=0)))
+        assert np.array_equal(got[0][0], got[1][0]) and np.array_equal(got[0][1], got[1][1]), row
+
+
 def test_retained_rows_with_a_dominant_common_component():
     # budget 24 < head_dim: every value is a common vector plus 3 % of noise, so after the first retained row every
     # further row loses nearly all of its norm to the basis in the first Gram-Schmidt pass and the kernel has to go
