@@ -938,7 +938,7 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                             }
                             const float d = (sa[sz - 1] - sg) + vb[sz - 2] * (y0 / y1);
                             const float d2 = __shfl_sync(0xffffffffu, live ? d : 1.f, 31);
-                            const bool gone = lane < r ? cb <= 1e-9f * top : lane == r ? cb <= 3e-5f * top : true;
+                            const bool gone = lane < r ? cb <= 1e-9f * top : lane == r ? cb <= 1e-6f * top : true;
                             suffice = d2 < 0.f && (rest - cb * cb / d2) * 1.0001f < sigma && __all_sync(0xffffffffu, gone);
                         }
                     }

@@ -808,6 +808,10 @@ def _backfill_of_a_form(a_diag, a_off, rank):
     args = a["K"][0, 0], a["V"][0, 0], out["scores"][0, 0].cpu().numpy().astype(np.float64), out["idx"][0, 0].cpu().numpy()
     ref, whole = oracle.backfill(*args, rank), oracle.backfill(*args, d)["delta"]
     lam = np.linalg.eigvalsh(M)[::-1]
+    # (the eigenvalues are resolved to 6e-8 of a bound that is twice the largest at most)
+    dg, want = P.parse_diag(out["diag"])[0], ref["diag"]
+    for key in ("lam_1", "lam_rho", "lam_next"):
+        assert abs(dg[key] - want[key]) <= 32 * par.U32 * want["lam_1"], (key, dg[key], want[key])
     err = np.linalg.norm(out["delta"][0, 0].cpu().numpy().astype(np.float64) - ref["delta"]) / np.linalg.norm(whole)
     return err, 32 * par.U32 * lam[0] / (lam[rank - 1] - lam[rank])
 
@@ -847,6 +851,21 @@ def test_largest_eigenvalue_two_rows_before_the_end_of_the_leading_part(coupling
     off[:30] = 0.02
     off[22], diag[23] = coupling, 0.06 + coupling ** 2
     err, limit = _backfill_of_a_form(diag, off, 2)
+    assert err <= limit, (err, limit)
+
+
+def test_next_eigenvalue_close_to_one_outside_the_leading_part():
+    # The first row holds the wanted eigenvalue, rows 16 and 17 the next one, with a coupling of 2e-5 to a row behind them whose own
+    # eigenvalue is 8e-5 smaller: as much as the leading part and the rest may share without the rest's bound showing it.
+    diag, off = np.full(104, 1e-3), np.zeros(103)
+    diag[0], diag[1:16], diag[17] = 1.0, 0.06, 0.06
+    off[:15], off[15], off[16], off[17] = 0.02, 1e-3, 1e-3, 9e-3
+    shift = 129 / 257 * 1.02                                  # the one just below the next eigenvalue
+    diag[16], diag[18] = shift, shift - 2.5e-4
+    for _ in range(5):
+        T = np.diag(diag[:18]) + np.diag(off[:17], 1) + np.diag(off[:17], -1)
+        diag[16] += shift + 1e-5 - np.linalg.eigvalsh(T)[-2]
+    err, limit = _backfill_of_a_form(diag, off, 1)
     assert err <= limit, (err, limit)
 
 
