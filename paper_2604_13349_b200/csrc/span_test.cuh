@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(ST_NT, 3) k_span_test(const __grid_constant__ 
         for (int sp = 0; sp < n_part; ++sp) {
 #pragma unroll
             for (int i = 0; i < PAIRS; ++i) {
-                if (D == 64 && i > warp) continue;
+                // (heads of 64 channels read the blocks above the diagonal too, without a branch between their loads)
 #pragma unroll
                 for (int t = 0; t < 2; ++t)
 #pragma unroll
