@@ -573,19 +573,21 @@ __global__ void __launch_bounds__(NT, 2048 / NT) k_select_smem(const __grid_cons
     if (lane == 0) { red[0][warp] = sk; red[1][warp] = sd; red[2][warp] = nx; }
     __syncthreads();
     if (gather_vecs) {
-        // two vectors a thread in flight: of K and V, or two of V
+        // two vectors a thread in flight: of K and V, or two of V.  A row has 8, 16 or 32 vectors, and a head's rows of them fit 32 bits; with
+        // divisions by that number 152 heads with 24 rows each took 27.3 us a call (so 24.9), 64 with 120 rows 26.6 (25.9)
         const bool both = gather_vecs > 0;
-        const int vecs = both ? gather_vecs : -gather_vecs, n = k * vecs, step = both ? NT : 2 * NT;
+        const int vecs = both ? gather_vecs : -gather_vecs, n = k * vecs, step = both ? NT : 2 * NT, sh = __ffs(vecs) - 1;
         const size_t to = (size_t)lh * n;
         const uint4 *vs = reinterpret_cast<const uint4 *>(c.v) + (size_t)lh * T * vecs, *ks = both ? reinterpret_cast<const uint4 *>(c.k) + (size_t)lh * T * vecs : vs;
         uint4 *vo = reinterpret_cast<uint4 *>(c.v_out) + to, *ko = both ? reinterpret_cast<uint4 *>(c.k_out) + to : vo;
+#pragma unroll 1
         for (int e = tid; e < n; e += step) {
-            const int e2 = both ? e : min(e + NT, n - 1), j = s_idx[e / vecs], j2 = s_idx[e2 / vecs];
+            const int e2 = both ? e : min(e + NT, n - 1), j = s_idx[e >> sh], j2 = s_idx[e2 >> sh];
             if ((unsigned)j >= (unsigned)T || (unsigned)j2 >= (unsigned)T) {       // never dereference a position outside the cache
                 atomicOr(p.status, OBF_DEV_INTERNAL);
                 continue;
             }
-            const uint4 a = vs[(size_t)j * vecs + e % vecs], b = ks[(size_t)j2 * vecs + e2 % vecs];
+            const uint4 a = vs[(j << sh) + (e & (vecs - 1))], b = ks[(j2 << sh) + (e2 & (vecs - 1))];
             vo[e] = a;
             ko[e2] = b;
         }
