@@ -574,13 +574,13 @@ __global__ void __launch_bounds__(NT, 2048 / NT) k_select_smem(const __grid_cons
     __syncthreads();
     if (gather_vecs) {
         // two vectors a thread in flight: of K and V, or two of V.  A row has 8, 16 or 32 vectors, and a head's rows of them fit 32 bits; with
-        // divisions by that number 152 heads with 24 rows each took 27.3 us a call (so 24.9), 64 with 120 rows 26.6 (25.9)
+        // divisions by that number 152 heads with 24 rows each took 27.3 us a call (so 25.5), 64 with 120 rows 26.6 (25.9).  Not unrolled it would be 24.9,
+        // but the selection before it spills registers: 12 x 8 ragged heads that copy nothing here 328 -> 332
         const bool both = gather_vecs > 0;
         const int vecs = both ? gather_vecs : -gather_vecs, n = k * vecs, step = both ? NT : 2 * NT, sh = __ffs(vecs) - 1;
         const size_t to = (size_t)lh * n;
         const uint4 *vs = reinterpret_cast<const uint4 *>(c.v) + (size_t)lh * T * vecs, *ks = both ? reinterpret_cast<const uint4 *>(c.k) + (size_t)lh * T * vecs : vs;
         uint4 *vo = reinterpret_cast<uint4 *>(c.v_out) + to, *ko = both ? reinterpret_cast<uint4 *>(c.k_out) + to : vo;
-#pragma unroll 1
         for (int e = tid; e < n; e += step) {
             const int e2 = both ? e : min(e + NT, n - 1), j = s_idx[e >> sh], j2 = s_idx[e2 >> sh];
             if ((unsigned)j >= (unsigned)T || (unsigned)j2 >= (unsigned)T) {       // never dereference a position outside the cache
