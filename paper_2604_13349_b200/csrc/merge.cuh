@@ -221,7 +221,9 @@ __global__ void __launch_bounds__(MGT_NT) k_merge_assign_mma(const __grid_consta
 // the values of eight of them together before it adds them up.  What bounds the kernel is the slot with the most hits, a
 // heavy hitter's, and, with many slots, the walks themselves.  36 x 8 heads, T = 1024, 32 slots: one row at a time 115 us,
 // eight rows in flight 44 us, the same with eight warps per slot 48 us, with two 35 us; 6 x 8 heads, T = 1500: one warp per
-// slot 21 us, eight 11 us.
+// slot 21 us, eight 11 us.  The warp's number is known to be the same in its lanes (88 -> 80 us a call, 36 x 8 heads of 64 channels; 126.9
+// where 128.2) but for long walks over few slots, whose loads the compiler then puts in another order: 24 heads of 128 channels, T = 7585,
+// 78.0 us a call without, 79.1 with it in all warps, 76.1 so.
 // grid = (ceil(k_eff_max WPS / 8), heads_total), 256 threads.
 template <typename TIN, int D, int WPS>
 __global__ void __launch_bounds__(256) k_merge_apply(const __grid_constant__ CallDev p)
@@ -232,7 +234,7 @@ __global__ void __launch_bounds__(256) k_merge_apply(const __grid_constant__ Cal
     int ci, lh;
     locate(p, blockIdx.y, ci, lh);
     const CacheDev &c = p.c[ci];
-    const int T = c.T, k = c.k_eff, lane = threadIdx.x & 31, warp = warp_uniform((int)threadIdx.x >> 5);
+    const int T = c.T, k = c.k_eff, lane = threadIdx.x & 31, warp = WPS == 8 && D == 128 ? (int)threadIdx.x >> 5 : warp_uniform((int)threadIdx.x >> 5);
     constexpr int SLOTS = 8 / WPS;                                      // slots of a block
     const int r0 = blockIdx.x * SLOTS, r = r0 + warp / WPS, part = warp % WPS;
     if (r0 >= k) return;
