@@ -66,11 +66,11 @@ constexpr float EIG_CLUSTER_TOL = 1e-3f; // eigenvalues closer than this (relati
 // where the rest comes down too slowly: when a line through its last two bounds, half as far again, ends behind three quarters of all
 // rows.  36 x 8 heads of 1024 positions, budget 32, ranks 1, 2 and 4, us a call:
 //   values' channels             all rows         asked to the end   given up so
-//   flat                         212  213  224    229  223  235      216  216  226
-//   flat, three 8 times as large 211  213  222    199  208  234      200  208  226
-//   0.985 each of the last       212  213  224    224  213  230      222  212  224
-//   0.97 each of the last        212  213  225    201  204  213      201  205  216
-//   inverse root of their number 211  213  222    182  187  199      179  187  199
+//   flat                         212  213  224    228  224  236      215  216  228
+//   flat, three 8 times as large 211  213  222    198  207  234      199  207  226
+//   0.985 each of the last       212  213  224    224  213  230      221  220  228
+//   0.97 each of the last        212  213  225    201  203  213      199  203  212
+//   inverse root of their number 211  213  222    182  187  199      181  187  199
 constexpr int ALG_EXIT_FIRST = 18, ALG_EXIT_STEP = 6;
 constexpr float ALG_EXIT_BEND = 1.5f, ALG_EXIT_SHARE = 0.75f;
 constexpr float EIG_NEAR_TOL = 5e-2f;    // closer than this: one more step of inverse iteration on the twisted factors, then made orthogonal
@@ -945,7 +945,7 @@ __global__ void __launch_bounds__(ALG_NT, 2) k_obf_algebra(const __grid_constant
                     if (warp_uniform(suffice)) return 0;
                     // A line through the last two bounds of the rest, which comes down ever more slowly, tells when it will be down at sigma.
                     const float now = rest * gb, above = now - sigma * gb;
-                    int rows = max(ALG_EXIT_STEP, rest > 1.3f * sigma ? sz / 2 : sz / 4);
+                    int rows = max(ALG_EXIT_STEP, rest > fminf(1.3f * sigma, 1.f) ? sz / 2 : sz / 4);
                     if (was[1] > 0.f && above > 0.f &&
                         (float)sz + ALG_EXIT_BEND * above * ((float)sz - was[1]) / fmaxf(was[0] - now, 1e-3f * now) > ALG_EXIT_SHARE * (float)(D - m)) rows = D;
                     __syncwarp();
