@@ -472,11 +472,10 @@ __device__ __forceinline__ int alg_reflectors(const TIN *vk, int k, float *Y, fl
 #pragma unroll
                 for (int q = 0; q < NQ; ++q) V[s][q] = mul2(V[s][q], pk(f, f));
                 n0[s] = half_sum(alg_dot<D>(V[s], V[s]));
-                if (!(n0[s] < INFINITY)) {
-                    n0[s] = 0.f;
+                const bool finite = n0[s] < INFINITY;
+                n0[s] = finite ? n0[s] : 0.f;
 #pragma unroll
-                    for (int q = 0; q < NQ; ++q) V[s][q] = 0ull;
-                }
+                for (int q = 0; q < NQ; ++q) V[s][q] &= mask2(finite);
             }
         }
         // (the reflectors that earlier batches found, all published behind a barrier)
