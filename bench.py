@@ -175,17 +175,26 @@ def run_reference(args):
     return 0
 
 
+def algebra_constant(name: str) -> int:
+    """An integer constant of the dense algebra, from the kernel's source."""
+    import re
+    with open(os.path.join(ROOT, "paper_2604_13349_b200", "csrc", "algebra.cuh")) as f:
+        return int(re.search(r"constexpr int [^;]*\b%s = (\d+)" % name, f.read()).group(1))
+
+
 # fp32 work of the dense algebra per (layer, KV head) whose retained values do not span R^d, as the kernel
 # formulates it (Eq. 2-6): a reflector per retained row, taken to the rows after it; every reflector to the Gram matrix from both
 # sides (a product and a rank-two update of the block it reaches, both triangles); on the exact route the trailing block's further
 # reflectors to tridiagonal form; on the fixed-iteration route three products with the block instead; one vector back through the
 # reflectors.  (What the eigenpairs of the tridiagonal form cost is of order rank * d.)  Heads of 128 channels end the tridiagonal form
-# when its first rows hold the wanted eigenpairs, after 18 rows (24, 30) at the earliest: what they cannot do without is counted.
+# when its first rows hold the wanted eigenpairs, after ALG_EXIT_FIRST rows (one or two ALG_EXIT_STEP more for larger ranks) at the
+# earliest: what they cannot do without is counted.
 def algebra_flops(d: int, k: int, rank: int, fast: bool = False) -> float:
+    first, step, max_rank = (algebra_constant(c) for c in ("ALG_EXIT_FIRST", "ALG_EXIT_STEP", "ALG_TRI_MAX_RANK"))
     m = min(k, d)
     rows = 4.0 * d * sum(min(i, m) for i in range(k))
-    asked = m + 18 + 6 * (rank > 1) + 6 * (rank > 2)
-    last = m if fast else asked if d > 64 and rank <= 8 and asked <= d - 13 else d - 1
+    asked = m + first + step * (rank > 1) + step * (rank > 2)
+    last = m if fast else asked if d > 64 and rank <= max_rank and asked < d - 2 * step else d - 1
     two_sided = sum(6.0 * (d - j) ** 2 for j in range(last))
     iterations = 3 * min(rank, d - m) * 2.0 * (d - m) ** 2 if fast else 0.0
     return rows + two_sided + iterations + 4.0 * d * last
